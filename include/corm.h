@@ -80,9 +80,9 @@ typedef struct {
                                                         attended_keys is the sparsity figure of Section 3.1 */
     int64_t near_threshold;                          /* verdicts (Definition 3.1) whose reduced-precision logit fell
                                                         inside the proven error bound around its threshold and was
-                                                        formed again in fp64 before it was decided: only the tiled
-                                                        prompt pass places logits in fp32; decode logits are fp64
-                                                        throughout and add nothing here */
+                                                        formed again in fp64 before it was decided: only the prompt
+                                                        pass of bf16 caches places logits in fp32; decode logits are
+                                                        fp64 throughout and add nothing here */
 } corm_stats_t;
 
 /* Bytes of device memory a cache with this configuration needs (host, pure). 0 if the configuration is invalid. */
@@ -262,10 +262,9 @@ corm_status_t corm_cache_set_tuning(corm_cache_t* cache, int32_t split_len, int3
 corm_status_t corm_cache_set_similarity_monitor(corm_cache_t* cache, int32_t enabled);
 corm_status_t corm_cache_similarity(corm_cache_t* cache, double* sum_host, int64_t* count_host, void* stream);
 
-/* The tiled prompt pass (bf16, head_dim 128) places each logit of its second launch on one side of its exact
- * threshold with an fp32 dot product wherever a proven bound on the fp32 accumulation error allows, and forms the
- * logit again in fp64 where it does not, so results never depend on this. `scale` >= 1 multiplies the bound
- * (default 1): larger values send more logits through the exact path, which is how the tests exercise it.
+/* The prompt pass of bf16 caches forms its logits on the tensor cores with proven bounds on their errors; a verdict
+ * that a bound leaves open is decided in fp64, so results never depend on it. `scale` >= 1 multiplies the bounds
+ * (default 1): larger values send more logits and rows through the exact path, which is how the tests exercise it.
  * Errors: INVALID_ARG. */
 corm_status_t corm_cache_set_bound_scale(corm_cache_t* cache, double scale);
 

@@ -1,5 +1,5 @@
 // Host side of the C-ABI library: arena layout, argument checks, launch configuration. Every step of the hot
-// path runs in the kernels of corm_fast.cuh / corm_balanced.cuh / corm_verdict.cuh / corm_prompt_fast.cuh /
+// path runs in the kernels of corm_fast.cuh / corm_balanced.cuh / corm_verdict.cuh / corm_prompt.cuh /
 // corm_generic.cuh; nothing
 // here touches tensor data on the CPU.
 #include <cuda_runtime.h>
@@ -20,7 +20,7 @@
 #include "corm_fast.cuh"
 #include "corm_balanced.cuh"
 #include "corm_generic.cuh"
-#include "corm_prompt_fast.cuh"
+#include "corm_prompt.cuh"
 
 using namespace corm;
 
@@ -32,7 +32,7 @@ constexpr int kMinSplit = 64;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-    size_t K, V, word, pos, live, base_tokens, base_obs, ticket, ticket2, ticket3, move_info, unit_stamp, counters, status, maxlive, sim_acc, page_table, page_bits, page_room, q_prev, stash, partials, keepmask, unit_rec;
+    size_t K, V, word, pos, live, base_tokens, base_obs, ticket, ticket2, unit_stamp, counters, status, maxlive, sim_acc, page_table, page_bits, page_room, q_prev, stash, partials, keepmask, unit_rec;
     size_t stage_q, stage_k, stage_v, stage_out, total, bookkeeping_begin, bookkeeping_end;
 };
 
@@ -97,8 +97,6 @@ Layout make_layout(const corm_config_t& c, int pool_pages) {
     L.base_obs = take(Ltot * c.batch * 4);
     L.ticket = take(Ltot * U * 4);
     L.ticket2 = take(Ltot * U * 4);
-    L.ticket3 = take(Ltot * U * 4);
-    L.move_info = take(Ltot * U * 8);
     L.unit_stamp = take(Ltot * U * 8);
     L.counters = take(Ltot * CNT_COUNT * 8);
     L.status = take(4);
@@ -342,8 +340,6 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     p.base_obs = reinterpret_cast<int32_t*>(layer_ptr(c, c->lay.base_obs, (size_t)cf.batch * 4, layer));
     p.ticket = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.ticket, U * 4, layer));
     p.ticket2 = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.ticket2, U * 4, layer));
-    p.ticket3 = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.ticket3, U * 4, layer));
-    p.move_info = reinterpret_cast<unsigned long long*>(layer_ptr(c, c->lay.move_info, U * 8, layer));
     p.counters = reinterpret_cast<unsigned long long*>(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer));
     p.status = reinterpret_cast<int32_t*>(c->arena + c->lay.status);
     p.maxlive = maxlive_ptr(c, layer);
@@ -552,13 +548,11 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     if (!layer_ok(c, layer) || !prompt_lens_host || p_max < 0) return CORM_ERR_INVALID_ARG;
     const corm_config_t& cf = c->cfg;
     int max_p = 0;
-    std::vector<int32_t> obs(cf.batch);
     for (int b = 0; b < cf.batch; ++b) {
         const int P = prompt_lens_host[b];
         if (P < 0 || P > p_max) return CORM_ERR_INVALID_ARG;
         if (P > cf.max_tokens) return CORM_ERR_CAPACITY;
         max_p = std::max(max_p, P);
-        obs[b] = std::min(P, cf.window_w);
     }
     if (max_p > 0 && (!k_prompt || !v_prompt || !q_last)) return CORM_ERR_INVALID_ARG;
     if (max_p > 0 && ((reinterpret_cast<uintptr_t>(k_prompt) | reinterpret_cast<uintptr_t>(v_prompt) |
@@ -566,20 +560,26 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     DeviceGuard guard(cf.device);
     if (!guard.ok) return CORM_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t C = cf.max_tokens, D = cf.head_dim, U = c->U;
+    const size_t C = cf.max_tokens, U = c->U;
     int32_t* base_tokens = reinterpret_cast<int32_t*>(layer_ptr(c, c->lay.base_tokens, (size_t)cf.batch * 4, layer));
     int32_t* base_obs = reinterpret_cast<int32_t*>(layer_ptr(c, c->lay.base_obs, (size_t)cf.batch * 4, layer));
-    // pageable sources are staged by the runtime before these calls return
-    CORM_CUDA(cudaMemcpyAsync(base_tokens, prompt_lens_host, (size_t)cf.batch * 4, cudaMemcpyHostToDevice, st));
-    CORM_CUDA(cudaMemcpyAsync(base_obs, obs.data(), (size_t)cf.batch * 4, cudaMemcpyHostToDevice, st));
-    CORM_CUDA(cudaMemsetAsync(layer_ptr(c, c->lay.ticket, U * 4, layer), 0, U * 4, st));
-    CORM_CUDA(cudaMemsetAsync(layer_ptr(c, c->lay.ticket2, U * 4, layer), 0, U * 4, st));
-    CORM_CUDA(cudaMemsetAsync(layer_ptr(c, c->lay.ticket3, U * 4, layer), 0, U * 4, st));
-    CORM_CUDA(cudaMemsetAsync(layer_ptr(c, c->lay.move_info, U * 8, layer), 0, U * 8, st));
-    CORM_CUDA(cudaMemsetAsync(layer_ptr(c, c->lay.unit_stamp, U * 8, layer), 0, U * 8, st));   // step counts restart
+    PromptBeginParams bp{};
+    bp.w = cf.window_w; bp.base_tokens = base_tokens; bp.base_obs = base_obs;
+    int n_clear = 0;
+    auto clear = [&](void* ptr, size_t bytes) { bp.clear[n_clear++] = {static_cast<uint32_t*>(ptr), bytes / 4}; };
+    clear(layer_ptr(c, c->lay.ticket, U * 4, layer), U * 4);
+    clear(layer_ptr(c, c->lay.ticket2, U * 4, layer), U * 4);
+    clear(layer_ptr(c, c->lay.unit_stamp, U * 8, layer), U * 8);        // step counts restart
+    clear(maxlive_ptr(c, layer), 8);
+    clear(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer), CNT_COUNT * 8);   // a new prompt restarts the layer's statistics
+    if (c->pool_pages) {   // whatever the layer held is replaced: all its pages return to the pool
+        clear(page_table_ptr(c, layer), U * c->pt_stride * 4);
+        clear(page_bits_ptr(c, layer), (size_t)(c->pool_pages / 32) * 4);
+        clear(page_room_ptr(c, layer), U * 4);
+    }
+    int n_begin = 0;
+    CORM_CUDA(launch_prompt_begin(bp, prompt_lens_host, cf.batch, st, &n_begin));
     c->chain_ok[layer] = 0;
-    CORM_CUDA(cudaMemsetAsync(maxlive_ptr(c, layer), 0, 8, st));
-    CORM_CUDA(cudaMemsetAsync(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer), 0, CNT_COUNT * 8, st));   // a new prompt restarts the layer's statistics
     c->readback_pending[layer] = 0;   // an older read-back no longer describes this layer
     PromptParams p{};
     p.k_prompt = k_prompt; p.v_prompt = v_prompt; p.q_last = q_last;
@@ -587,11 +587,6 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     p.K = layer_ptr(c, c->lay.K, kv_layer_bytes(c), layer);
     p.V = layer_ptr(c, c->lay.V, kv_layer_bytes(c), layer);
     set_paging(c, layer, p);
-    if (c->pool_pages) {   // whatever the layer held is replaced: all its pages return to the pool
-        CORM_CUDA(cudaMemsetAsync(p.page_table, 0, U * c->pt_stride * 4, st));
-        CORM_CUDA(cudaMemsetAsync(p.page_bits, 0, (size_t)(c->pool_pages / 32) * 4, st));
-        CORM_CUDA(cudaMemsetAsync(p.page_room, 0, U * 4, st));
-    }
     p.word = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.word, U * C * 4, layer));
     p.pos = reinterpret_cast<int32_t*>(layer_ptr(c, c->lay.pos, U * C * 4, layer));
     p.live_out = live_buf(c, layer, 0);
@@ -602,32 +597,13 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     p.U = (int)U; p.Hkv = cf.n_kv_heads; p.C = cf.max_tokens; p.p_max = p_max; p.w = cf.window_w; p.r = cf.recent_r;
     p.log_alpha = log_alpha_of(c);
     p.bound_scale = c->bound_scale;
-    corm_status_t rc = CORM_ERR_UNSUPPORTED;
-    int n_launched = 1;
-    if (cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->allow_fast) {     // two-launch tiled pass
-        PromptFastParams fp{};
-        fp.p = p;
-        fp.partials = c->arena + c->lay.partials;
-        fp.ticket = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.ticket, U * 4, layer));
-        const size_t cap = U * (size_t)max_splits_of(cf) * c->G * partial_stride((int)D);   // one layer's share is enough here
-        rc = launch_prompt_fast(fp, c->G, max_p, c->sm_count, cap, st);
-        n_launched = prompt_fast_launches(c->G, cf.window_w);
-    }
-    if (rc == CORM_ERR_UNSUPPORTED) {
-        n_launched = 1;
-        rc = dispatch(c, [&](auto* tp, auto dd, auto gg) -> corm_status_t {
-            using T = std::remove_pointer_t<decltype(tp)>;
-            constexpr int DD = decltype(dd)::value, GG = decltype(gg)::value;
-            const size_t smem = prompt_smem(GG, cf.window_w, cf.max_tokens);
-            auto kern = prompt_generic_kernel<T, DD, GG>;
-            CORM_CUDA(ensure_dynamic_smem(reinterpret_cast<const void*>(kern), smem));
-            kern<<<(unsigned)U, kPromptThreads, smem, st>>>(p);
-            CORM_CUDA(cudaGetLastError());
-            return CORM_OK;
-        });
-    }
+    p.keepmask = reinterpret_cast<uint32_t*>(c->arena + c->lay.keepmask);
+    const bool bf = cf.kv_dtype == CORM_BF16;
+    const corm_status_t rc =
+        cf.head_dim == 128 ? (bf ? launch_prompt_cluster<bf16_t, 128>(p, c->G, max_p, c->sm_count, st) : launch_prompt_cluster<float, 128>(p, c->G, max_p, c->sm_count, st))
+                           : (bf ? launch_prompt_cluster<bf16_t, 64>(p, c->G, max_p, c->sm_count, st) : launch_prompt_cluster<float, 64>(p, c->G, max_p, c->sm_count, st));
     if (rc != CORM_OK) return rc;
-    c->launches += n_launched;
+    c->launches += n_begin + 1;
     c->parity[layer] = 0; c->steps[layer] = 0; c->ready[layer] = 1; c->live_upper[layer] = max_p; c->live_mean[layer] = 0;
     c->have_q_prev[layer] = 0;                    // the previous decode query belonged to the old text
     c->step_group[layer] = -1;

@@ -37,11 +37,6 @@ inline cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes) {
     return e;
 }
 
-// |fp32 dot - exact dot| <= kDotErr * |q| * |k| for a 128-term dot product of bf16 values formed the way the fast
-// kernels fold it (bf16 x bf16 products are exact in fp32): 7 roundings in a lane's 8-term FMA chain and 5 in the
-// cross-lane fold make 12 * 2^-24 to first order; 16 * 2^-24 leaves a third of slack for the higher-order terms and
-// for the rounding of the fp32 key norm itself.
-constexpr double kDotErr = 16.0 / 16777216.0;
 // 1 / sqrt(head_dim), the scale of Eq. 2's exponent
 __host__ __device__ constexpr double inv_root_dim(int D) { return D == 128 ? 0.088388347648318440550 : 0.125; }
 
@@ -59,8 +54,6 @@ struct DecodeParams {
     const int32_t* base_obs;     // [B] verdict rows recorded at that time
     uint32_t* ticket;         // [U] arrival counters of the splits of a unit (zero between steps)
     uint32_t* ticket2;        // [U] second arrival counters (balanced kernel: blocks done with their verdicts)
-    uint32_t* ticket3;        // [U] third arrival counters (balanced kernel: blocks done with their share of the row moves)
-    unsigned long long* move_info;   // [U] balanced kernel: the unit's move word (zero between steps)
     unsigned long long* counters;  // [CNT_COUNT]
     int32_t* status;          // sticky device status
     unsigned long long* maxlive;  // (steps done << 32 | longest live length after that step), atomicMax; may be null
@@ -101,9 +94,10 @@ struct PromptParams {
     int32_t* status;
     unsigned long long* maxlive;
     double* stash;            // scratch, reused for temporary registers
+    uint32_t* keepmask;       // [U][ceil(C/32)+2] keep bits (scratch)
     int32_t U, Hkv, C, p_max, w, r;
     double log_alpha;
-    double bound_scale;       // multiplies the proven fp32 error bound of the tiled pass (1; tests raise it)
+    double bound_scale;       // multiplies the proven error bounds of the bf16 pass (1; tests raise it)
     int32_t* page_table;      // paged caches only, as in DecodeParams
     uint32_t* page_bits;
     int32_t* page_room;

@@ -1,6 +1,6 @@
 // Generic kernels: any supported dtype / head_dim / group size, written for clarity. One warp per key, lanes
-// split the head dimension, fp64 logits. The bf16 / head_dim 128 decode path has a faster kernel of its own;
-// this one serves fp32 caches, head_dim 64 and the prompt-end pass.
+// split the head dimension, fp64 logits. The bf16 / head_dim 128 decode path has faster kernels of its own;
+// this one serves fp32 caches, head_dim 64 and groups of eight.
 #pragma once
 
 #include "corm_common.cuh"
@@ -8,7 +8,6 @@
 namespace corm {
 
 constexpr int kGenericThreads = 128;
-constexpr int kPromptThreads = 256;
 
 __host__ __device__ inline size_t generic_decode_smem(int D, int G, int C, bool paged) {
     const size_t warps = kGenericThreads / 32;
@@ -139,161 +138,6 @@ __global__ void __launch_bounds__(kGenericThreads) decode_generic_kernel(const _
     __syncthreads();
     if (!s_last) return;
     finalize_unit<T, D, G, NT>(p, u, b, l, n_act, t, smem);
-}
-
-// window slots handled per pass of the generic prompt kernel (at most 64 (slot, head) rows at a time)
-__host__ __device__ inline int prompt_chunk_slots(int G, int w) { const int s = 64 / G; return s < w ? s : w; }
-
-__host__ __device__ inline size_t prompt_smem(int G, int w, int C) {
-    const size_t warps = kPromptThreads / 32, rows = (size_t)G * prompt_chunk_slots(G, w);
-    size_t a = warps * rows * 16 + rows * 8;
-    size_t b = (size_t)2 * ((C + 31) / 32 + 2) * 4;
-    return a + b;
-}
-
-// Prompt-end pass, one block per unit. Pass 1: log-sum-exp of every recorded causal row; pass 2: verdict bits of
-// every key for those rows -> registers; then keep flags, prefix sums and an ordered gather into the slab.
-template <typename T, int D, int G>
-__global__ void __launch_bounds__(kPromptThreads) prompt_generic_kernel(const __grid_constant__ PromptParams p) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ int s_scan[kPromptThreads];
-    constexpr int NT = kPromptThreads, NW = NT / 32, NPL = D / 32;
-    const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int b = u / p.Hkv;
-    const int P = __ldg(p.prompt_lens + b);
-    if (P > p.C) {
-        if (tid == 0) { report_status(p.status, CORM_ERR_CAPACITY); p.live_out[u] = 0; }
-        return;
-    }
-    if (P == 0) {
-        if (tid == 0) {
-            p.live_out[u] = 0;
-            if (p.page_table) {  // an empty unit still owns the page its first append goes to
-                const int pg = claim_page(p.page_bits, p.pool_pages, p.U, u, 0);
-                p.page_table[(size_t)u * p.pt_stride] = pg + 1;
-                p.page_room[u] = pg >= 0;
-            }
-        }
-        return;
-    }
-    const int w = p.w, wp = min(P, w);
-    const int cs = prompt_chunk_slots(G, w), rows = G * cs;           // window slots per pass, rows per pass
-    double* sm_mz = reinterpret_cast<double*>(smem);                   // [NW][rows][2], row = g * cs + (slot - slot0)
-    double* sm_thr = sm_mz + (size_t)NW * rows * 2;                    // [rows]
-    uint32_t* keepmask = reinterpret_cast<uint32_t*>(sm_thr + rows);
-    int* prefix = reinterpret_cast<int*>(keepmask + (p.C + 31) / 32 + 2);
-    const T* Kp = reinterpret_cast<const T*>(p.k_prompt) + (size_t)u * p.p_max * D;
-    const T* Vp = reinterpret_cast<const T*>(p.v_prompt) + (size_t)u * p.p_max * D;
-    const T* Q = reinterpret_cast<const T*>(p.q_last) + (size_t)u * G * w * D;   // [G][w][D]
-    const int c0 = lane * NPL;
-    const double root_d = sqrt((double)D);
-    uint32_t* tmp_word = reinterpret_cast<uint32_t*>(p.stash + (size_t)u * G * p.C);
-
-    // the recorded queries are taken oldest first, a few window slots per pass over the keys
-    for (int slot0 = w - wp; slot0 < w; slot0 += cs) {
-        const int slot1 = min(w, slot0 + cs);
-        for (int i = tid; i < NW * rows; i += NT) { sm_mz[2 * i] = -INFINITY; sm_mz[2 * i + 1] = 0.0; }
-        __syncthreads();
-        // pass 1: running max / sum of every row, per warp (only lane 0 owns the warp's entries)
-        for (int j = warp; j < P; j += NW) {
-            float kf[NPL];
-            load_slice<T, NPL>(Kp + (size_t)j * D + c0, kf);
-            for (int row = slot0; row < slot1; ++row) {
-                const int i = P - (w - 1 - row);          // position of this query; it sees keys 1..i
-                if (j + 1 > i) continue;
-                for (int g = 0; g < G; ++g) {
-                    float qf[NPL];
-                    load_slice<T, NPL>(Q + ((size_t)g * w + row) * D + c0, qf);
-                    double part = 0.0;
-#pragma unroll
-                    for (int k = 0; k < NPL; ++k) part += (double)qf[k] * (double)kf[k];
-                    const double s = warp_sum(part) / root_d;
-                    if (lane == 0) {
-                        double* mz = sm_mz + ((size_t)warp * rows + g * cs + (row - slot0)) * 2;
-                        if (s > mz[0]) { mz[1] = mz[1] * exp(mz[0] - s) + 1.0; mz[0] = s; }
-                        else mz[1] += exp(s - mz[0]);
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        for (int rr = tid; rr < rows; rr += NT) {
-            const int row = slot0 + rr % cs;
-            if (row >= slot1) { sm_thr[rr] = INFINITY; continue; }
-            double M = -INFINITY, Z = 0.0;
-            for (int x = 0; x < NW; ++x) M = fmax(M, sm_mz[((size_t)x * rows + rr) * 2]);
-            for (int x = 0; x < NW; ++x)
-                Z += sm_mz[((size_t)x * rows + rr) * 2 + 1] * exp(sm_mz[((size_t)x * rows + rr) * 2] - M);
-            const int i = P - (w - 1 - row);
-            sm_thr[rr] = M + log(Z) + p.log_alpha - log((double)i);  // Definition 3.1 in log form, threshold alpha/i
-        }
-        __syncthreads();
-        // pass 2: verdicts of these queries enter the registers (shift register: the query at position P ends in
-        // bit 0; wide windows: the position of the newest query that found the key important)
-        for (int j = warp; j < P; j += NW) {
-            float kf[NPL];
-            load_slice<T, NPL>(Kp + (size_t)j * D + c0, kf);
-            uint32_t wd = slot0 == w - wp ? 0u : tmp_word[j];          // written by this same thread in the previous pass
-            for (int row = slot0; row < slot1; ++row) {
-                const int i = P - (w - 1 - row);
-                bool bit = false;
-                if (j + 1 <= i) {
-                    for (int g = 0; g < G; ++g) {
-                        float qf[NPL];
-                        load_slice<T, NPL>(Q + ((size_t)g * w + row) * D + c0, qf);
-                        double part = 0.0;
-#pragma unroll
-                        for (int k = 0; k < NPL; ++k) part += (double)qf[k] * (double)kf[k];
-                        const double s = warp_sum(part) / root_d;
-                        bit |= (s >= sm_thr[g * cs + (row - slot0)]);
-                    }
-                }
-                wd = update_register(wd, bit, w, i);
-            }
-            if (lane == 0) tmp_word[j] = wd;
-        }
-        __syncthreads();
-    }
-    const bool evict_on = wp >= w;
-    for (int base = 0; base < P; base += NT) {
-        const int j = base + tid;
-        bool keep = false;
-        if (j < P) keep = !evict_on || register_needed(tmp_word[j], w, P) || (j + 1) > P - p.r;
-        const uint32_t ballot = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0 && base + warp * 32 < P) keepmask[(base >> 5) + warp] = ballot;
-    }
-    __syncthreads();
-    const int nwords = (P + 31) / 32;
-    block_popc_scan<NT>(keepmask, prefix, nwords, s_scan);
-    const int kept_total = prefix[nwords];
-    const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
-    if (!claim_unit_pages<NT>(p.page_table, p.page_bits, p.page_room, p.pool_pages, p.pt_stride, p.U, u, kept_total)) {
-        if (tid == 0) { report_status(p.status, CORM_ERR_CAPACITY); p.live_out[u] = 0; }   // the pool is too small
-        return;
-    }
-    T* Kl = reinterpret_cast<T*>(p.K);
-    T* Vl = reinterpret_cast<T*>(p.V);
-    constexpr int kChunks = D * Elem<T>::kBytes / 16;
-    for (int j = warp; j < P; j += NW) {
-        if (!((keepmask[j >> 5] >> (j & 31)) & 1u)) continue;
-        const int dst = kept_before(keepmask, prefix, j);
-        const uint4* ks = reinterpret_cast<const uint4*>(Kp + (size_t)j * D);
-        const uint4* vs = reinterpret_cast<const uint4*>(Vp + (size_t)j * D);
-        const size_t drow = kv_row(pt_u, (size_t)u * p.C, dst, p.pool_pages, p.status);
-        uint4* kd = reinterpret_cast<uint4*>(Kl + drow * D);
-        uint4* vd = reinterpret_cast<uint4*>(Vl + drow * D);
-        for (int c = lane; c < 2 * kChunks; c += 32) {
-            if (c < kChunks) kd[c] = ks[c];
-            else vd[c - kChunks] = vs[c - kChunks];
-        }
-        if (lane == 0) { p.word[(size_t)u * p.C + dst] = tmp_word[j]; p.pos[(size_t)u * p.C + dst] = j + 1; }
-    }
-    if (tid == 0) {
-        p.live_out[u] = kept_total;
-        publish_live(p.maxlive, 0, kept_total);
-        atomicAdd(p.counters + CNT_APPENDED, (unsigned long long)P);
-        if (kept_total < P) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(P - kept_total));
-    }
 }
 
 }  // namespace corm

@@ -111,6 +111,48 @@ def test_prompt_pass_fp32_placement_and_exact_path(G, w, scale):
     assert orc.counters()["near_threshold"] == 0 and orc.counters()["evicted"] > 0
 
 
+# prompt lengths at the edges of words, ring buffers (128 keys) and of what the blocks of a cluster keep on chip; windows
+# below, at and beyond a register; row counts that leave warps without rows or share them
+PROMPT_EDGES = [
+    # dtype, head_dim, group, prompt range, w, planted scale, seed (no probability of the oracle's within 1e-6 of a threshold)
+    ("bf16", 128, 1, (1, 33), 1, 4.0, 91),
+    ("bf16", 128, 1, (127, 129), 8, 4.0, 91),
+    ("bf16", 128, 4, (1023, 1025), 3, 4.0, 91),
+    ("bf16", 128, 8, (250, 420), 33, 4.0, 93),
+    ("bf16", 64, 2, (3071, 3073), 16, 4.0, 92),
+    ("bf16", 64, 1, (600, 700), 256, 4.0, 91),
+    ("bf16", 128, 8, (40, 60), 256, 4.0, 91),
+    ("f32", 128, 1, (20, 30), 40, 4.0, 91),
+    ("f32", 128, 2, (2047, 2049), 5, 4.0, 91),
+    ("f32", 64, 8, (255, 300), 64, 4.0, 91),
+    ("bf16", 128, 4, (4200, 4200), 8, 4.0, 91),
+    ("bf16", 128, 4, (300, 300), 8, 400.0, 91),       # logits beyond the plain sum of exponentials: the exact rows
+    ("bf16", 64, 1, (300, 300), 8, 2.0 ** 42, 91),     # keys beyond the range of the exact pieces
+    ("f32", 64, 2, (300, 300), 8, 400.0, 91),
+]
+
+
+@pytest.mark.parametrize("case", PROMPT_EDGES, ids=lambda c: "-".join(str(x) for x in c))
+def test_prompt_pass_edges(case):
+    """Registers, positions and rows after the prompt pass are the oracle's, bit for bit, on slabs and on pages."""
+    dtype, d, G, (pmin, pmax), w, scale, seed = case
+    cfg = CONFIGS[1].with_(name="edges", batch=3, n_q_heads=2 * G, n_kv_heads=2, head_dim=d, dtype=dtype, prompt_min=pmin,
+                           prompt_max=pmax, steps=4, window_w=w, recent_r=16, gqa_rho=0.7 if G > 1 else 0.0, hh_min=2,
+                           hh_max=6, hh_scale=scale, seed=seed)
+    data = generate(cfg)
+    orc = make_oracle(cfg, 3, 2)
+    orc.compress_prompt(0, data.k_prompt, data.v_prompt, data.q_last, data.prompt_lens)
+    if pmin >= w:                      # a query at position 1 sits on its threshold by construction (p = 1 = 1 / t)
+        assert orc.counters()["near_threshold"] == 0
+    pages = -(-6 * (cfg.max_tokens // 32 + 2) // 32) * 32
+    for pool in (0, pages):
+        gpu = make_gpu_cache(cfg, 3, 2, pool_pages=pool)
+        gpu.corm_compress_prompt(0, to_dev(data.k_prompt, dtype), to_dev(data.v_prompt, dtype), to_dev(data.q_last, dtype),
+                                 data.prompt_lens)
+        assert_states_equal(gpu, orc, 0, 3, 2, f"pool {pool}")
+        assert gpu.corm_cache_stats()["device_status"] == 0
+
+
 def test_alpha_zero_never_evicts():
     cfg = CONFIGS[1].with_(prompt_min=100, prompt_max=100, steps=20, alpha=0.0, dtype="bf16")
     data = generate(cfg)
