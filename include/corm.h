@@ -80,9 +80,8 @@ typedef struct {
                                                         attended_keys is the sparsity figure of Section 3.1 */
     int64_t near_threshold;                          /* verdicts (Definition 3.1) whose reduced-precision logit fell
                                                         inside the proven error bound around its threshold and was
-                                                        formed again in fp64 before it was decided: only the prompt
-                                                        pass of bf16 caches places logits in fp32; decode logits are
-                                                        fp64 throughout and add nothing here */
+                                                        formed again in fp64 before it was decided: the prompt pass of
+                                                        bf16 caches and the decode kernels that keep logits in fp32 */
 } corm_stats_t;
 
 /* Bytes of device memory a cache with this configuration needs (host, pure). 0 if the configuration is invalid. */
@@ -243,7 +242,8 @@ corm_status_t corm_cache_import_state(corm_cache_t* cache, int32_t layer, int32_
 
 /* Tuning knobs (performance only; live lists and registers do not depend on them, outputs only within rounding):
  * keys per split of the block-per-split decode kernel (multiple of 32, 0 = automatic) and which kernels may be used:
- * allow_fast_path 0 = the generic kernels only; 1 = automatic (default): for bf16 / head_dim 128, one query head per
+ * allow_fast_path 0 = the generic kernel only; 1 = automatic (default): a cluster of blocks per unit for fp32 caches,
+ * head_dim 64 and groups of eight; for bf16 / head_dim 128, one query head per
  * KV head takes the block-per-split kernel, which finishes a unit of several splits inside the decode launch when the
  * launch has many units and by a second, verdict launch when it has few, and grouped heads take the balanced
  * kernel (every block an equal share of the step's keys) followed by the verdict launch; 2 / 3 = the block-per-split

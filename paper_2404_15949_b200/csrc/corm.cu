@@ -19,6 +19,7 @@
 #include "corm_common.cuh"
 #include "corm_fast.cuh"
 #include "corm_balanced.cuh"
+#include "corm_cluster.cuh"
 #include "corm_generic.cuh"
 #include "corm_prompt.cuh"
 
@@ -172,6 +173,9 @@ struct corm_cache {
     std::vector<CUtensorMap> vmaps;               // per layer: the V storage as a tiled tensor (balanced kernel); empty = unavailable
     CUtensorMap vmap_all;                         // the V storage of all layers of a slab cache as one tensor (layers stepped together)
     bool have_vmap_all = false;
+    // per layer: K and V as tensors of 16-row boxes (cluster kernel; empty = unavailable); a slab layer's reach to the end
+    // of the last layer, for layers stepped together
+    std::vector<CUtensorMap> kmaps_row, vmaps_row;
     // per layer: the group of layers (first layer * 65536 + count) it has been stepped with ever since its prompt pass
     // (-1: not stepped yet, -2: alone or in different groups); only then does the group's length read-back describe it
     std::vector<int> step_group;
@@ -305,6 +309,21 @@ corm_status_t monitor_similarity(corm_cache* c, int layer, const void* q, cudaSt
     return CORM_OK;
 }
 
+// which caches the cluster kernel steps: whatever the bf16 / head_dim-128 kernels do not cover
+bool takes_cluster(const corm_cache* c) {
+    const bool covered = c->cfg.kv_dtype == CORM_BF16 && c->cfg.head_dim == 128 && c->G <= 4;
+    return c->allow_fast == 1 && !c->kmaps_row.empty() && !covered;
+}
+
+// whether several layers from first_layer on may run as one launch as far as the kernels are concerned
+bool can_fuse(const corm_cache* c, int first_layer) {
+    const corm_config_t& cf = c->cfg;
+    if (fused_layers_of(cf, c->pool_pages) <= 1 || !c->allow_fast || c->monitor_similarity) return false;
+    if (takes_cluster(c)) return true;
+    return cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4 &&
+           ((c->allow_fast != 6 && (c->G == 1 || c->allow_fast == 2 || c->allow_fast == 3)) || (c->have_vmap_all && first_layer == 0));
+}
+
 // One decode step of layers [layer, layer + n_fused) as ONE launch (pair): the layers' units are consecutive in every
 // per-unit array of the arena, so n_fused layers of U units are one array of n_fused * U units to the kernels. The
 // caller has checked that the layers are at the same step with the same buffer parity and that q, k_new, v_new and
@@ -360,7 +379,8 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     }
     const int upper = std::min(cf.max_tokens, bound + 1);   // no unit can hold more live keys
 
-    const bool fast = c->allow_fast && cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4;
+    const bool cluster = takes_cluster(c);
+    const bool fast = !cluster && c->allow_fast && cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4;
     corm_status_t rc;
     int n_launched = 1;
     // Grouped query heads take the balanced streaming kernel followed by the verdict launch (measured against the
@@ -381,8 +401,20 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     bool chain_ok_before = chain && !c->monitor_similarity;
     for (int i = 0; i < n_fused; ++i) chain_ok_before &= c->chain_ok[layer + i] != 0;
     bool self_finishing = false;
-    if (!(fast && !balanced) && !units) p.unit_stamp = nullptr;    // only the block-per-split kernels keep stamps
-    if (units) {
+    if (!(fast && !balanced) && !units && !cluster) p.unit_stamp = nullptr;    // only kernels that finish a unit in one launch keep stamps
+    if (cluster) {
+        DecodeClusterParams dp{};
+        dp.p = p;
+        dp.G = c->G;
+        dp.bound_scale = (float)c->bound_scale;
+        const bool may_chain = !c->monitor_similarity && (c->G == 1 || (long long)upper <= 96ll * (long long)p.U);
+        if (!may_chain || !(chain || more)) dp.p.unit_stamp = nullptr;
+        dp.p.chain_wait = chain_ok_before && may_chain ? 1 : 0;
+        dp.p.early_trigger = more && may_chain ? 1 : 0;
+        rc = launch_decode_cluster(dp, cf.kv_dtype == CORM_BF16, cf.head_dim, c->kmaps_row[layer], c->vmaps_row[layer], upper, c->tune_split_len, c->sm_count, st);
+        self_finishing = rc == CORM_OK && dp.p.unit_stamp;
+        if (rc == CORM_OK && dp.p.chain_wait) c->chained_launches += 1;
+    } else if (units) {
         const int typical = mean_known ? std::min(upper, mean_sum / n_fused + c->steps[layer] - c->last_readback_step[layer] + 1) : 0;
         rc = launch_decode_balanced_units(p, n_fused > 1 ? c->vmap_all : c->vmaps[layer], c->G, upper, typical, c->tune_split_len,
                                           c->sm_count, partial_records_of(cf, c->pool_pages), st, &n_launched,
@@ -504,6 +536,21 @@ corm_status_t corm_cache_create_paged(const corm_config_t* cfg, int32_t pool_pag
             }
         if (!c->vmaps.empty() && !pool_pages && cfg->n_layers > 1)
             c->have_vmap_all = make_v_tensor_map(&c->vmap_all, layer_ptr(c, lay.V, kv_layer_bytes(c), 0), rows * cfg->n_layers) == CORM_OK;
+    }
+    {
+        const bool bf = cfg->kv_dtype == CORM_BF16;
+        const unsigned long long rows = pool_pages ? (unsigned long long)pool_pages * kPageKeys : (unsigned long long)c->U * cfg->max_tokens;
+        auto map = [&](CUtensorMap* m, size_t at, int l, unsigned long long n) {
+            return make_row_tensor_map(m, layer_ptr(c, at, kv_layer_bytes(c), l), n, cfg->head_dim, bf) == CORM_OK;
+        };
+        bool ok = rows * cfg->n_layers < (1ull << 31);
+        c->kmaps_row.resize(cfg->n_layers);
+        c->vmaps_row.resize(cfg->n_layers);
+        for (int l = 0; ok && l < cfg->n_layers; ++l) {
+            const unsigned long long n = rows * (pool_pages ? 1 : cfg->n_layers - l);
+            ok = map(&c->kmaps_row[l], lay.K, l, n) && map(&c->vmaps_row[l], lay.V, l, n);
+        }
+        if (!ok) { c->kmaps_row.clear(); c->vmaps_row.clear(); }
     }
     cudaError_t e = cudaMemset(c->arena + lay.bookkeeping_begin, 0, lay.bookkeeping_end - lay.bookkeeping_begin);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -645,9 +692,7 @@ corm_status_t corm_decode_step_layers(corm_cache_t* c, int32_t first_layer, int3
     // starts at layer 0.)
     const corm_config_t& cf = c->cfg;
     const size_t qb = (size_t)cf.batch * cf.n_q_heads * cf.head_dim * c->e, kb = (size_t)c->U * cf.head_dim * c->e;
-    bool fuse = n_layers > 1 && fused_layers_of(cf, c->pool_pages) > 1 && c->allow_fast && cf.kv_dtype == CORM_BF16 &&
-                cf.head_dim == 128 && c->G <= 4 && !c->monitor_similarity &&
-                ((c->allow_fast != 6 && (c->G == 1 || c->allow_fast == 2 || c->allow_fast == 3)) || (c->have_vmap_all && first_layer == 0));
+    bool fuse = n_layers > 1 && can_fuse(c, first_layer);
     for (int i = 1; fuse && i < n_layers; ++i) {
         const auto at = [](const void* ptr, size_t off) { return static_cast<const unsigned char*>(ptr) + off; };
         fuse = c->steps[first_layer + i] == c->steps[first_layer] && c->parity[first_layer + i] == c->parity[first_layer] &&
@@ -682,9 +727,7 @@ corm_status_t decode_steps_impl(corm_cache_t* c, int32_t first_layer, int32_t n_
     const size_t qb = (size_t)cf.batch * cf.n_q_heads * cf.head_dim * c->e, kb = (size_t)c->U * cf.head_dim * c->e;
     // all layers of a step as one launch under the same conditions as corm_decode_step_layers (the buffers are
     // contiguous by this call's layout)
-    bool fuse = n_layers > 1 && fused_layers_of(cf, c->pool_pages) > 1 && c->allow_fast && cf.kv_dtype == CORM_BF16 &&
-                cf.head_dim == 128 && c->G <= 4 && !c->monitor_similarity &&
-                ((c->allow_fast != 6 && (c->G == 1 || c->allow_fast == 2 || c->allow_fast == 3)) || (c->have_vmap_all && first_layer == 0));
+    bool fuse = n_layers > 1 && can_fuse(c, first_layer);
     for (int i = 1; fuse && i < n_layers; ++i)
         fuse = c->steps[first_layer + i] == c->steps[first_layer] && c->parity[first_layer + i] == c->parity[first_layer];
     const auto at = [](const void* ptr, size_t off) { return static_cast<const unsigned char*>(ptr) + off; };

@@ -1,0 +1,1032 @@
+// Decode step: one launch, a thread-block cluster per unit, any dtype, head_dim and group size.
+//
+// The cluster's blocks share the unit's live slots (whole 32-slot words each) and do the whole of Algorithm 1:
+//   1. every warp streams 16-key tiles of K and V through its own ring of shared-memory stages (2-D tensor-map copies
+//      with the 128-byte swizzle, mbarriers, bounded waits): logits, probabilities, P.V; no block-wide step in the loop;
+//   -- the blocks exchange {m, Z, acc} per head through distributed shared memory: log-sum-exp, thresholds, outputs
+//   2. verdicts of the block's slots, register update, keep bits;
+//   -- the blocks exchange their counts of kept slots: new length, places of holes and movers
+//   3. hole filling, shared over the cluster; the first block publishes the unit's new length.
+//
+// bf16 logits on the tensor cores (corm_mma.cuh): keys cut into pieces k1, k2, r2, queries into q1, q2, q3. An
+// mma.m16n8k16 has eight columns, so the pieces of several heads share one: for a group of up to four heads the columns
+// are (q1, q2) of each, and the accumulators of different columns are different numbers, so every product of pieces is
+// summed apart (exactly, where the pieces allow). Per 16 keys and 16 channels: 3 mma for one or two heads (the q3's take
+// the other columns), 5 for four, 8 for eight. P.V on the tensor cores as well: A = V^T (ldmatrix.trans), B = the
+// probabilities, each split into two bf16.
+// fp32: a key per lane (its channels shared by two half-warps), fp64 products on the CUDA cores, P.V by fp32 FMAs.
+//
+// What bounds it: the chain of round trips (about 20 us of 30) on units of a few hundred keys, which is what it is used
+// on. Measured against one warp per key and the last-arriving split finishing the unit alone, us per step:
+//   64 units x 970 keys, G 8, bf16   253 -> 31      128 units x 1090 keys, G 4, 64 channels   143 -> 34
+//   20 units x 250 keys, G 2, fp32    64 -> 15      8 units x 170 keys, G 1, fp32            37.7 -> 14
+//
+// Verdicts are the fp64 ones: a slot's logit is kept in fp32, and one that lies within the proven error of its threshold
+// is formed again in fp64. If it then lies within the error of the log-sum-exp itself, the head is marked and the
+// cluster forms that head's log-sum-exp and verdicts in fp64 once more before anything is evicted (rare).
+#pragma once
+
+#include <cuda.h>
+
+#include "corm_balanced.cuh"
+#include "corm_mma.cuh"
+
+namespace corm {
+
+constexpr int kDcMaxCluster = 8;
+constexpr int kDcKeys = 16;                       // keys per tile
+constexpr int kDcMaxWords = 4096;                 // 32-slot words a block may own (its keep bits and prefix sums lie in the ring)
+
+struct DecodeClusterParams {
+    DecodeParams p;
+    int32_t G;
+    int32_t lcap;                                 // logits that fit on chip, per block (a longer block's go to p.stash)
+    float bound_scale;
+};
+
+template <typename T, int D, int GP> struct DcShape {
+    static constexpr bool kBf16 = Elem<T>::kBytes == 2;
+    static constexpr int kRow = D * Elem<T>::kBytes;
+    static constexpr int kBoxes = kRow / 128;     // 128-byte wide boxes of the swizzled copies
+    static constexpr int kBox = kDcKeys * 128;
+    static constexpr int kTile = kDcKeys * kRow;
+    static constexpr int kKs = kTile >= 8192 ? 1 : kTile == 4096 ? 2 : 4;
+    static constexpr int kVs = kTile >= 4096 ? 1 : 2;
+    static constexpr int kStages = kKs + kVs;
+    static constexpr int kWarpRing = kStages * kTile;
+    static constexpr int kProb = kBf16 ? kDcKeys * (GP == 8 ? 32 : 16) : kDcKeys * GP * 4;   // a warp's probabilities
+};
+// resident blocks per SM the register budget is set for
+template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int dc_blocks() {
+    return Elem<T>::kBytes == 4 ? (D == 128 ? 12 : 16) / NW : (GP == 8 ? 12 : 16) / NW;
+}
+
+template <int NW> struct DcMisc {
+    unsigned long long stamp;
+    double wM[NW][8], wZ[NW][8];                  // per warp and head
+    double M[8], Z[8];                            // the block's, read by its peers
+    double thr[8], Zt[8];
+    double red[NW][2], mz[2];                     // exact heads
+    float wsc[NW][8], sc[8][kDcMaxCluster], qe[8], thr_f[8], slack[8];
+    uint32_t amax, flags, unit_amax;
+    int mode, any_mode;                           // 0: fine; 1: a wait expired; 2: the unit cannot take the token
+    int bad, any_bad;
+    int count, n_imp;                             // kept slots, important keys of the block
+    int warp_cnt[NW], warp_imp[NW];
+    int scan[NW * 32];
+};
+
+struct DcSmem { int prob, q, newrow, logits, bars, misc, total; };
+template <typename T, int D, int GP, int NW>
+__host__ __device__ inline DcSmem dc_smem_layout(int lcap) {
+    using S = DcShape<T, D, GP>;
+    DcSmem s{};
+    int off = NW * S::kWarpRing;
+    auto take = [&](int bytes) { int at = off; off = (off + bytes + 127) / 128 * 128; return at; };
+    s.prob = take(NW * S::kProb);
+    s.q = take(GP * D * (S::kBf16 ? 2 : 8));      // fp32: widened to fp64
+    s.newrow = take(2 * S::kRow);
+    s.bars = take(NW * S::kStages * 8);
+    s.misc = take((int)sizeof(DcMisc<NW>));
+    s.logits = take(lcap * 4);
+    s.total = off;
+    return s;
+}
+
+// N contiguous elements of the cache past the L1 (rows move between launches that may overlap)
+template <typename T, int N> __device__ __forceinline__ void load_slice_cg(const T* p, float (&out)[N]) {
+    if constexpr (Elem<T>::kBytes == 2) {
+        uint32_t w[N / 2];
+        if constexpr (N == 4) { const uint2 v = __ldcg(reinterpret_cast<const uint2*>(p)); w[0] = v.x; w[1] = v.y; }
+        else w[0] = __ldcg(reinterpret_cast<const uint32_t*>(p));
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) { out[2 * i] = __uint_as_float(w[i] << 16); out[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u); }
+    } else if constexpr (N == 4) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+        out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
+    } else {
+        const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+        out[0] = v.x; out[1] = v.y;
+    }
+}
+
+// exact q.k of a slot by four lanes (sub = lane & 3): fp64, a fixed order; before the 1/sqrt(d)
+template <typename T, int D>
+__device__ __forceinline__ double quad_exact_dot(const T* q, const T* k, int sub) {
+    double part = 0.0;
+#pragma unroll 4
+    for (int i = 0; i < D / 16; ++i) {
+        float a[4], b[4];
+        load_slice<T, 4>(q + (i * 4 + sub) * 4, a);
+        load_slice_cg<T, 4>(k + (i * 4 + sub) * 4, b);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) part = fma((double)a[e], (double)b[e], part);
+    }
+    part += __shfl_xor_sync(0xffffffffu, part, 1);
+    part += __shfl_xor_sync(0xffffffffu, part, 2);
+    return part;
+}
+// ... and by a whole warp
+template <typename T, int D>
+__device__ __forceinline__ double warp_exact_dot_cg(const T* q, const T* k, int lane) {
+    constexpr int NPL = D / 32;
+    float a[NPL], b[NPL];
+    load_slice<T, NPL>(q + lane * NPL, a);
+    load_slice_cg<T, NPL>(k + lane * NPL, b);
+    double part = 0.0;
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) part = fma((double)a[i], (double)b[i], part);
+    return warp_sum(part);
+}
+
+// The marked heads, exactly: log-sum-exp with a running maximum and verdicts in fp64 from global memory, by the whole
+// cluster. A verdict that was sure before holds for the exact threshold too, so adding importance is enough: the
+// register gets its newest bit (or stamp), the keep bit is set.
+template <typename T, int D, int NW>
+__device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G, int t, int k_begin, int k_end, uint32_t heads,
+                                            uint32_t* keep, DcMisc<NW>* misc, int cs) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & 3;
+    const double inv_root_d = inv_root_dim(D);
+    const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
+    const T* Kl = reinterpret_cast<const T*>(p.K);
+    const uint32_t mz_addr = smem_addr(misc->mz);
+    uint32_t* wordu = p.word + (size_t)u * p.C;
+    int added = 0, added_imp = 0;
+    for (int h = 0; h < G; ++h) {
+        if (!((heads >> h) & 1u)) continue;
+        const T* q = reinterpret_cast<const T*>(p.q) + ((size_t)u * G + h) * D;
+        double m = -INFINITY, Z = 0.0;
+        for (int j0 = k_begin + warp * 8; j0 < k_end; j0 += NW * 8) {
+            const int j = j0 + (lane >> 2);
+            const size_t row = kv_row(pt_u, (size_t)u * p.C, min(j, k_end - 1), p.pool_pages, p.status);
+            const double s = quad_exact_dot<T, D>(q, Kl + row * D, sub) * inv_root_d;
+            if (j < k_end) {
+                if (s > m) { Z = Z * exp(m - s) + 1.0; m = s; }
+                else Z += exp(s - m);
+            }
+        }
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            const double mo = __shfl_xor_sync(0xffffffffu, m, o), Zo = __shfl_xor_sync(0xffffffffu, Z, o), mn = fmax(m, mo);
+            Z = (m == mn ? Z : Z > 0.0 ? Z * exp(m - mn) : 0.0) + (mo == mn ? Zo : Zo > 0.0 ? Zo * exp(mo - mn) : 0.0);
+            m = mn;
+        }
+        if (lane == 0) { misc->red[warp][0] = m; misc->red[warp][1] = Z; }
+        __syncthreads();
+        if (tid == 0) {
+            double mb = -INFINITY, Zb = 0.0;
+            for (int x = 0; x < NW; ++x) mb = fmax(mb, misc->red[x][0]);
+            for (int x = 0; x < NW; ++x)
+                if (misc->red[x][1] > 0.0) Zb += misc->red[x][1] * exp(misc->red[x][0] - mb);
+            misc->mz[0] = mb; misc->mz[1] = Zb;
+        }
+        cluster_sync();
+        double M = -INFINITY, Zt = 0.0;
+        for (int x = 0; x < cs; ++x) M = fmax(M, ld_peer_f64(map_rank(mz_addr, x)));
+        for (int x = 0; x < cs; ++x) {
+            const double z = ld_peer_f64(map_rank(mz_addr + 8, x));
+            if (z > 0.0) Zt += z * exp(ld_peer_f64(map_rank(mz_addr, x)) - M);
+        }
+        const double thr = M + log(Zt) + p.log_alpha - log((double)t);
+        for (int j0 = k_begin + warp * 8; j0 < k_end; j0 += NW * 8) {
+            const int j = j0 + (lane >> 2);
+            const size_t row = kv_row(pt_u, (size_t)u * p.C, min(j, k_end - 1), p.pool_pages, p.status);
+            const double s = quad_exact_dot<T, D>(q, Kl + row * D, sub) * inv_root_d;
+            if (sub == 0 && j < k_end && s >= thr) {
+                const uint32_t reg = __ldcg(wordu + j), bit = 1u << (j & 31);
+                const bool had = p.w <= 32 ? (reg & 1u) : reg == (uint32_t)t;
+                if (!had) {
+                    wordu[j] = p.w <= 32 ? (reg | 1u) : (uint32_t)t;
+                    added_imp += 1;
+                    if (!(atomicOr(keep + ((j - k_begin) >> 5), bit) & bit)) added += 1;
+                }
+            }
+        }
+        cluster_sync();                                       // everybody has read mz; the registers of this head are written
+    }
+    if (added) atomicAdd(&misc->count, added);
+    if (added_imp) atomicAdd(&misc->n_imp, added_imp);
+}
+
+template <typename T, int D, int GP, int NW>
+__global__ void __launch_bounds__(NW * 32, dc_blocks<T, D, GP, NW>())
+decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    using S = DcShape<T, D, GP>;
+    constexpr bool kBf16 = S::kBf16;
+    constexpr int NT = NW * 32, kKs = S::kKs, kVs = S::kVs;
+    constexpr int NH = kBf16 ? (GP == 8 ? 2 : 1) : GP;        // heads a thread handles logits of
+    constexpr int NK = kBf16 ? 2 : 1;                         // keys of a tile a thread handles
+    const DecodeParams& p = dp.p;
+    const int G = kBf16 && GP == 2 ? dp.G : GP;               // one or two heads share an instance
+    const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int cs = (int)cluster_size(), rank = (int)cluster_rank();
+    const DcSmem lay = dc_smem_layout<T, D, GP, NW>(0);       // the logits come last: every other offset is a constant
+    unsigned char* ring = smem + warp * S::kWarpRing;
+    unsigned char* prob = smem + lay.prob + warp * S::kProb;
+    unsigned char* newrow = smem + lay.newrow;
+    const uint32_t bars = smem_addr(smem + lay.bars) + warp * S::kStages * 8;
+    DcMisc<NW>* misc = reinterpret_cast<DcMisc<NW>*>(smem + lay.misc);
+
+    // ---- set-up that reads nothing of the previous launch ----
+    if (tid == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&kmap)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&vmap)) : "memory");
+        misc->amax = 0u; misc->flags = 0u; misc->mode = 0; misc->bad = 0;
+        if (smem_addr(smem) & 1023u) { report_status(p.status, CORM_ERR_INTERNAL); misc->mode = 1; }   // never expected
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int s = 0; s < S::kStages; ++s) mbar_init(bars + s * 8, 1);
+        fence_mbar_init();
+        fence_async_smem();
+    }
+    int l_old, mode = 0;
+    if (p.chain_wait) {                                       // this unit's previous step, not the whole previous launch
+        if (tid == 0) misc->stamp = wait_unit_stamp(p.unit_stamp + u, (uint32_t)p.step, p.status);
+        __syncthreads();
+        const unsigned long long sw = misc->stamp;
+        const bool ok = (uint32_t)(sw >> 32) == (uint32_t)p.step;
+        l_old = ok ? (int)(uint32_t)sw : 0;
+        if (!ok) mode = 1;
+        asm volatile("fence.proxy.async.global;" ::: "memory");   // the tile copies read rows that ordinary stores wrote
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        l_old = __ldcg(p.live_in + u);
+    }
+    const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
+    const int room = pt_u ? __ldcg(p.page_room + u) : 1;
+    const int b = u / p.Hkv;
+    const int t = __ldcg(p.base_tokens + b) + p.step + 1;
+    const bool evict_on = min(p.w, __ldcg(p.base_obs + b) + p.step + 1) >= p.w;
+    if (p.early_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // every block has its length by now
+    const int l = l_old + 1;
+    if (l > p.C || !room) mode = max(mode, 2);
+    // the block's slots: whole words, shared out evenly
+    const int n_words = mode ? 0 : (l + 31) >> 5;
+    const int w0 = (int)((long long)n_words * rank / cs), w1 = (int)((long long)n_words * (rank + 1) / cs);
+    const int k_begin = w0 * 32, k_end = mode ? 0 : min(l, w1 * 32), n_keys = max(0, k_end - k_begin);
+    const int n_tiles = (n_keys + kDcKeys - 1) / kDcKeys;
+    const int my_n = n_tiles > warp ? (n_tiles - warp + NW - 1) / NW : 0;       // tiles warp, warp + NW, ...
+    const bool fits = n_keys * G <= dp.lcap;
+    float* lg = fits ? reinterpret_cast<float*>(smem + lay.logits)
+                     : reinterpret_cast<float*>(p.stash) + ((size_t)u * p.C + k_begin) * G;
+    int my_page = 0;
+    if (pt_u) {                                               // lane i keeps the page entry of the warp's tile i
+        const int j = k_begin + (warp + lane * NW) * kDcKeys;
+        if (j < k_end) my_page = __ldcg(pt_u + (j >> 5));
+    }
+    auto tile_row0 = [&](int it) -> int {                     // first row of a tile in the layer's K / V storage (all lanes call)
+        const int j = k_begin + (warp + it * NW) * kDcKeys;
+        if (!pt_u) return (int)((size_t)u * p.C) + j;
+        const int pg = it < 32 ? __shfl_sync(0xffffffffu, my_page, it) : __ldcg(pt_u + (j >> 5));
+        return (int)page_row(pg, j, p.pool_pages, p.status);
+    };
+    auto issue = [&](const CUtensorMap& map, int row0, int stage) {             // lane 0
+        const uint32_t bar = bars + stage * 8, dst = smem_addr(ring + stage * S::kTile);
+        mbar_expect_tx(bar, S::kTile);
+#pragma unroll
+        for (int x = 0; x < S::kBoxes; ++x) tma_load_2d(dst + x * S::kBox, &map, x * (128 / Elem<T>::kBytes), row0, bar);
+    };
+#pragma unroll
+    for (int it = 0; it < kKs; ++it)
+        if (it < my_n) {
+            const int r0 = tile_row0(it);
+            if (lane == 0) { issue(kmap, r0, it); if (it < kVs) issue(vmap, r0, kKs + it); }
+        }
+    // queries and the appended rows (their latency is a bus round trip when the caller's buffers are host memory)
+    const bool new_here = !mode && l_old >= k_begin && l_old < k_end;
+    {
+        const unsigned char* qg = reinterpret_cast<const unsigned char*>(p.q) + (size_t)u * G * S::kRow;
+        if constexpr (kBf16) {
+            for (int x = tid; x < G * (S::kRow / 16); x += NT) cp_async16(smem_addr(smem + lay.q + x * 16), qg + x * 16);
+        } else {
+            double* qd = reinterpret_cast<double*>(smem + lay.q);
+            for (int x = tid; x < G * D; x += NT) qd[x] = (double)reinterpret_cast<const float*>(qg)[x];
+        }
+        if (new_here)
+            for (int x = tid; x < 2 * (S::kRow / 16); x += NT) {
+                const int c = x % (S::kRow / 16);
+                cp_async16(smem_addr(newrow + x * 16), reinterpret_cast<const unsigned char*>(x < S::kRow / 16 ? p.k_new : p.v_new) + (size_t)u * S::kRow + c * 16);
+            }
+        cp_async_wait_all();
+    }
+    __syncthreads();
+
+    // ---- 1. streaming ----
+    const double inv_root_d = inv_root_dim(D);
+    unsigned char* Kl = reinterpret_cast<unsigned char*>(p.K);
+    unsigned char* Vl = reinterpret_cast<unsigned char*>(p.V);
+    uint32_t* wordu = p.word + (size_t)u * p.C;
+    int32_t* posu = p.pos + (size_t)u * p.C;
+    bool failed = false;
+    double Zl[NH];
+    float Mref[NH];
+#pragma unroll
+    for (int x = 0; x < NH; ++x) { Zl[x] = 0.0; Mref[x] = -INFINITY; }
+    // the appended token's row replaces whatever the copy fetched for its slot; rows past the unit's end become zero
+    auto patch_tile = [&](unsigned char* tile, int j0, int n_valid, int which, int it) {
+        auto chunk_at = [&](int r, int c) { return tile + (c >> 3) * S::kBox + r * 128 + ((((c & 7) ^ r) & 7) << 4); };
+        if (l_old >= j0 && l_old < j0 + kDcKeys) {
+            const int row0 = tile_row0(it);
+            if (lane < S::kRow / 16) {
+                const uint4 x = *reinterpret_cast<const uint4*>(newrow + which * S::kRow + lane * 16);
+                *reinterpret_cast<uint4*>(chunk_at(l_old - j0, lane)) = x;
+                reinterpret_cast<uint4*>((which ? Vl : Kl) + (size_t)(row0 + (l_old - j0)) * S::kRow)[lane] = x;
+            }
+            if (which == 0 && lane == 0) { wordu[l_old] = 0u; posu[l_old] = t; }
+        }
+        if (n_valid < kDcKeys)
+            for (int x = lane; x < (kDcKeys - n_valid) * (S::kRow / 16); x += 32)
+                *reinterpret_cast<uint4*>(chunk_at(n_valid + x / (S::kRow / 16), x % (S::kRow / 16))) = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+    };
+    float* rec = reinterpret_cast<float*>(ring);              // the warp's record [G][D], once its tiles are done
+
+    if constexpr (kBf16) {
+        // pieces of the queries, as B fragments: column n = lane / 4
+        constexpr int KK = D / 16;
+        uint32_t b1[KK][2], b2[GP == 2 ? 1 : KK][2], b3[GP == 8 ? KK : 1][2];
+        {
+            const int n = lane >> 2;
+            const int hq = GP == 8 ? n : GP == 4 ? n >> 1 : (n & 3) >> 1;
+            const bool on = hq < G;
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(smem + lay.q) + (on ? hq : 0) * (D / 2) + (lane & 3);
+            uint32_t mx = 0u;
+#pragma unroll
+            for (int kk = 0; kk < KK; ++kk) {
+                b1[kk][0] = on ? src[kk * 8] : 0u;
+                b1[kk][1] = on ? src[kk * 8 + 4] : 0u;
+                mx = max_abs_bf16x2(max_abs_bf16x2(mx, b1[kk][0]), b1[kk][1]);
+            }
+            uint32_t m16 = max(mx & 0xffffu, mx >> 16);
+            m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 1));
+            m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 2));
+            const bool ok = m16 < kSplitMaxBits;
+            if (!ok) misc->bad = 1;
+            const float c = split_query_const(ok ? __uint_as_float(m16 << 16) : 1.f);
+            float n1 = 0.f, n2 = 0.f, n3 = 0.f;
+#pragma unroll
+            for (int kk = 0; kk < KK; ++kk)
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    const float a[2] = {__uint_as_float(b1[kk][hf] << 16), __uint_as_float(b1[kk][hf] & 0xffff0000u)};
+                    uint32_t y1[2], y2[2], y3[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        float x1, x2, x3;
+                        split_query(a[e], c, x1, x2, x3);
+                        n1 += fabsf(a[e]); n2 += fabsf(x2); n3 += fabsf(x3);
+                        y1[e] = __float_as_uint(x1); y2[e] = __float_as_uint(x2); y3[e] = __float_as_uint(x3);
+                    }
+                    auto pack = [](const uint32_t (&y)[2]) { return (y[0] >> 16) | (y[1] & 0xffff0000u); };   // exact: bf16 numbers
+                    if constexpr (GP == 8) {
+                        b1[kk][hf] = pack(y1); b2[kk][hf] = pack(y2); b3[kk][hf] = pack(y3);
+                    } else if constexpr (GP == 4) {
+                        b1[kk][hf] = n & 1 ? pack(y2) : pack(y1);
+                        b2[kk][hf] = n & 1 ? 0u : pack(y3);
+                    } else {
+                        b1[kk][hf] = n & 4 ? (n & 1 ? 0u : pack(y3)) : n & 1 ? pack(y2) : pack(y1);
+                    }
+                }
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+                n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+                n3 += __shfl_xor_sync(0xffffffffu, n3, o);
+            }
+            // Error of a logit (before the 1/sqrt(d)) per unit of the unit's largest key magnitude A. r2.q: 34 roundings
+            // of 2^-23 per 16 channels (two products of 16 terms and their accumulators; half of that for four heads or
+            // fewer) and 8 of 2^-24 in fp32, on terms of at most A/8192 |q|; k.q3: at most 2 * 8 * 17 roundings of 2^-23;
+            // r2.q3 <= A/8192 |q3| (left out for eight and four heads); the sum of the small parts (k2.q2 <= A/64 |q2|
+            // among them) rounds three times.
+            if (on && (lane & 3) == 0)
+                misc->qe[hq] = dp.bound_scale * 1.05f * (4.6e-6f * (n1 * 1.01f) * (1.f / 8192.f) + (3.3e-5f + 1.3e-4f) * n3 + 2.4e-7f * n2 * (1.f / 64.f));
+        }
+        float accd[D / 16][4];
+#pragma unroll
+        for (int cb = 0; cb < D / 16; ++cb)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) accd[cb][e] = 0.f;
+        uint32_t amax_w = 0u;
+        const int h0 = GP == 8 ? 2 * (lane & 3) : (lane & 3);                    // the thread's head(s)
+        bool first = true;
+        for (int it = 0; it < my_n; ++it) {
+            const int j0 = k_begin + (warp + it * NW) * kDcKeys, n_valid = min(kDcKeys, k_end - j0);
+            const int ks = it % kKs, vs = it % kVs;
+            unsigned char* ktile = ring + ks * S::kTile;
+            unsigned char* vtile = ring + (kKs + vs) * S::kTile;
+            const bool edge = n_valid < kDcKeys || (l_old >= j0 && l_old < j0 + kDcKeys);
+            if (!failed && !mbar_wait(bars + ks * 8, (it / kKs) & 1)) failed = true;   // once one wait has expired the rest are skipped
+            if (edge) patch_tile(ktile, j0, n_valid, 0, it);
+            uint32_t a[KK][4];
+            {
+                const uint32_t arow = smem_addr(ktile) + (lane & 15) * 128;
+#pragma unroll
+                for (int kk = 0; kk < KK; ++kk) ldmatrix_x4(a[kk], arow + (kk >> 2) * S::kBox + ((((kk & 3) * 2 + (lane >> 4)) ^ (lane & 7)) << 4));
+            }
+            __syncwarp();
+            if (it + kKs < my_n) {                            // the whole tile is in registers: its stage is free
+                const int r0 = tile_row0(it + kKs);
+                if (lane == 0) { fence_async_smem(); issue(kmap, r0, ks); }
+            }
+            uint32_t mx = a[0][0];
+#pragma unroll
+            for (int kk = 0; kk < KK; ++kk)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) mx = max_mag_bf16x2(mx, a[kk][e]);
+            mx &= 0x7fff7fffu;
+            const uint32_t am = __reduce_max_sync(0xffffffffu, max(mx & 0xffffu, mx >> 16));
+            amax_w = max(amax_w, am);
+            const SplitGrid g = split_grid(min(am, kSplitMaxBits));
+            // sums of the products of pieces; see the head of the file
+            float x1[4] = {0.f, 0.f, 0.f, 0.f}, x2[4] = {0.f, 0.f, 0.f, 0.f}, x3[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+            float x4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int kk = 0; kk < KK; ++kk) {
+                uint32_t k1[4], k2[4], r2[4];
+                split_key(a[kk], g, k1, k2, r2);
+                float tt[4] = {0.f, 0.f, 0.f, 0.f};
+                mma16816(x1, k1, b1[kk][0], b1[kk][1]);
+                mma16816(tt, r2, b1[kk][0], b1[kk][1]);
+                if constexpr (GP == 8) {
+                    mma16816(x2, k1, b2[kk][0], b2[kk][1]);   // k1.q2 + k2.q1: exact together
+                    mma16816(x2, k2, b1[kk][0], b1[kk][1]);
+                    mma16816(x4, k2, b2[kk][0], b2[kk][1]);   // exact
+                    mma16816(tt, r2, b2[kk][0], b2[kk][1]);
+                    mma16816(x3, k1, b3[kk][0], b3[kk][1]);
+                    mma16816(x3, k2, b3[kk][0], b3[kk][1]);
+                } else {
+                    mma16816(x2, k2, b1[kk][0], b1[kk][1]);
+                    if constexpr (GP == 4) {
+                        mma16816(x3, k1, b2[kk][0], b2[kk][1]);
+                        mma16816(x3, k2, b2[kk][0], b2[kk][1]);
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) lo[e] += tt[e];
+            }
+            // Eq. 2's exponent, thread's keys lane / 4 and + 8
+            double s[NK][NH];
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                if constexpr (GP == 8) {
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        const int e = 2 * y + x;
+                        s[y][x] = (((double)x1[e] + (double)x2[e]) + (double)(x4[e] + (lo[e] + x3[e]))) * inv_root_d;
+                    }
+                } else {
+                    // columns: (.q1, .q2) of the thread's head; two heads: the q3 products two lanes further on
+                    float small = x2[2 * y + 1] + (lo[2 * y] + lo[2 * y + 1]);
+                    if constexpr (GP == 4) small += x3[2 * y];
+                    else small += __shfl_xor_sync(0xffffffffu, x1[2 * y] + (x2[2 * y] + lo[2 * y]), 2);
+                    s[y][0] = (((double)x1[2 * y] + (double)(x1[2 * y + 1] + x2[2 * y])) + (double)small) * inv_root_d;
+                }
+            }
+            bool on[NK][NH];
+            bool over = first;
+#pragma unroll
+            for (int y = 0; y < 2; ++y)
+#pragma unroll
+                for (int x = 0; x < NH; ++x) {
+                    on[y][x] = (lane >> 2) + 8 * y < n_valid && h0 + x < G;
+                    over |= on[y][x] && (float)s[y][x] > Mref[x] + 16.f;
+                }
+            if (__any_sync(0xffffffffu, over)) {              // the reference moves: first tile, or a logit far above it (rare)
+                float scf[NH];
+#pragma unroll
+                for (int x = 0; x < NH; ++x) {
+                    float mt = fmaxf(on[0][x] ? (float)s[0][x] : -INFINITY, on[1][x] ? (float)s[1][x] : -INFINITY);
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+                    const float mn = fmaxf(Mref[x], mt);
+                    const double sc = first || mn == -INFINITY ? 0.0 : exp_nonpos((double)Mref[x] - (double)mn);
+                    Zl[x] *= sc;
+                    scf[x] = (float)sc;
+                    Mref[x] = mn;
+                }
+#pragma unroll
+                for (int cb = 0; cb < D / 16; ++cb)           // the accumulators' columns are the thread's own heads
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) accd[cb][e] *= GP == 8 ? scf[(e & 1) % NH] : scf[0];
+                first = false;
+            }
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const int kq = (lane >> 2) + 8 * y;
+                float hi_f[NH], lo_f[NH];
+#pragma unroll
+                for (int x = 0; x < NH; ++x) {
+                    const double ex = on[y][x] ? exp_nonpos(s[y][x] - (double)Mref[x]) : 0.0;
+                    Zl[x] += ex;
+                    const float pf = (float)ex;
+                    hi_f[x] = __uint_as_float(pack_bf16x2(0.f, pf) << 16);
+                    lo_f[x] = pf - hi_f[x];
+                    if (on[y][x]) lg[(j0 - k_begin + kq) * G + h0 + x] = (float)s[y][x];
+                }
+                if constexpr (GP == 8) {                      // [key][8 heads] high parts, then low parts
+                    *reinterpret_cast<uint32_t*>(prob + kq * 16 + (lane & 3) * 4) = pack_bf16x2(hi_f[1 % NH], hi_f[0]);
+                    *reinterpret_cast<uint32_t*>(prob + 256 + kq * 16 + (lane & 3) * 4) = pack_bf16x2(lo_f[1 % NH], lo_f[0]);
+                } else {
+                    *reinterpret_cast<uint32_t*>(prob + kq * 16 + (lane & 3) * 4) = pack_bf16x2(lo_f[0], hi_f[0]);   // [key][head x (high, low)]
+                }
+            }
+            __syncwarp();
+            if (!failed && !mbar_wait(bars + (kKs + vs) * 8, (it / kVs) & 1)) failed = true;
+            if (edge) patch_tile(vtile, j0, n_valid, 1, it);
+            {
+                uint32_t bf[4];
+                ldmatrix_x4_trans(bf, smem_addr(prob) + (GP == 8 ? lane : lane & 15) * 16);       // keys 0-7 | 8-15 (| the low parts)
+                const int row = ((lane >> 4) << 3) + (lane & 7);
+                const uint32_t vrow = smem_addr(vtile) + row * 128;
+#pragma unroll
+                for (int cb = 0; cb < D / 16; ++cb) {
+                    uint32_t va[4];
+                    ldmatrix_x4_trans(va, vrow + (cb >> 2) * S::kBox + ((((cb & 3) * 2 + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
+                    mma16816(accd[cb], va, bf[0], bf[1]);     // Eq. 1
+                    if constexpr (GP == 8) mma16816(accd[cb], va, bf[2], bf[3]);
+                }
+            }
+            __syncwarp();
+            if (it + kVs < my_n) {
+                const int r0 = tile_row0(it + kVs);
+                if (lane == 0) { fence_async_smem(); issue(vmap, r0, kKs + vs); }
+            }
+        }
+#pragma unroll
+        for (int x = 0; x < NH; ++x) {
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) Zl[x] += __shfl_xor_sync(0xffffffffu, Zl[x], o);
+            if ((lane >> 2) == 0 && h0 + x < G) { misc->wM[warp][h0 + x] = (double)Mref[x]; misc->wZ[warp][h0 + x] = Zl[x]; }
+        }
+#pragma unroll
+        for (int cb = 0; cb < D / 16; ++cb) {
+            if constexpr (GP == 8) {
+                rec[h0 * D + cb * 16 + (lane >> 2)] = accd[cb][0];
+                rec[(h0 + 1) * D + cb * 16 + (lane >> 2)] = accd[cb][1];
+                rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][2];
+                rec[(h0 + 1) * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][3];
+            } else if (h0 < G) {
+                rec[h0 * D + cb * 16 + (lane >> 2)] = accd[cb][0] + accd[cb][1];       // high + low parts
+                rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][2] + accd[cb][3];
+            }
+        }
+        if (lane == 0) {
+            if (amax_w >= kSplitMaxBits) misc->bad = 1;
+            atomicMax(&misc->amax, amax_w);
+        }
+    } else {
+        const double* qd = reinterpret_cast<const double*>(smem + lay.q);
+        float* pr = reinterpret_cast<float*>(prob);           // [key][GP]
+        constexpr int NC = D / 32;                            // channels a lane accumulates
+        float acc[GP][NC];
+#pragma unroll
+        for (int x = 0; x < GP; ++x)
+#pragma unroll
+            for (int e = 0; e < NC; ++e) acc[x][e] = 0.f;
+        const int key = lane & 15, half = lane >> 4;
+        bool first = true;
+        for (int it = 0; it < my_n; ++it) {
+            const int j0 = k_begin + (warp + it * NW) * kDcKeys, n_valid = min(kDcKeys, k_end - j0);
+            const int ks = it % kKs, vs = it % kVs;
+            unsigned char* ktile = ring + ks * S::kTile;
+            unsigned char* vtile = ring + (kKs + vs) * S::kTile;
+            const bool edge = n_valid < kDcKeys || (l_old >= j0 && l_old < j0 + kDcKeys);
+            if (!failed && !mbar_wait(bars + ks * 8, (it / kKs) & 1)) failed = true;
+            if (edge) patch_tile(ktile, j0, n_valid, 0, it);
+            double s[GP];
+#pragma unroll
+            for (int x = 0; x < GP; ++x) s[x] = 0.0;
+#pragma unroll
+            for (int bx = 0; bx < S::kBoxes / 2; ++bx) {
+                const int box = half * (S::kBoxes / 2) + bx;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float4 kv = *reinterpret_cast<const float4*>(ktile + box * S::kBox + key * 128 + ((c ^ (key & 7)) << 4));
+                    const double k4[4] = {(double)kv.x, (double)kv.y, (double)kv.z, (double)kv.w};
+#pragma unroll
+                    for (int x = 0; x < GP; ++x) {
+                        const double2 qa = *reinterpret_cast<const double2*>(qd + x * D + box * 32 + c * 4);
+                        const double2 qb = *reinterpret_cast<const double2*>(qd + x * D + box * 32 + c * 4 + 2);
+                        s[x] = fma(qa.x, k4[0], s[x]); s[x] = fma(qa.y, k4[1], s[x]);
+                        s[x] = fma(qb.x, k4[2], s[x]); s[x] = fma(qb.y, k4[3], s[x]);
+                    }
+                }
+            }
+            __syncwarp();
+            if (it + kKs < my_n) {
+                const int r0 = tile_row0(it + kKs);
+                if (lane == 0) { fence_async_smem(); issue(kmap, r0, ks); }
+            }
+            const bool on = key < n_valid;
+            bool over = first;
+#pragma unroll
+            for (int x = 0; x < GP; ++x) {
+                s[x] = (s[x] + __shfl_xor_sync(0xffffffffu, s[x], 16)) * inv_root_d;
+                over |= on && (float)s[x] > Mref[x] + 16.f;
+            }
+            if (__any_sync(0xffffffffu, over)) {
+#pragma unroll
+                for (int x = 0; x < GP; ++x) {
+                    float mt = on ? (float)s[x] : -INFINITY;
+#pragma unroll
+                    for (int o = 1; o < 16; o <<= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+                    const float mn = fmaxf(Mref[x], mt);
+                    const double sc = first || mn == -INFINITY ? 0.0 : exp_nonpos((double)Mref[x] - (double)mn);
+                    Zl[x] *= sc;
+                    Mref[x] = mn;
+#pragma unroll
+                    for (int e = 0; e < NC; ++e) acc[x][e] *= (float)sc;
+                }
+                first = false;
+            }
+#pragma unroll
+            for (int x = 0; x < GP; ++x) {
+                if (GP > 1 && (x & 1) != half) continue;      // the half-warps share the heads
+                const double ex = on ? exp_nonpos(s[x] - (double)Mref[x]) : 0.0;
+                if (GP > 1 || half == 0) {
+                    Zl[x] += ex;
+                    pr[key * GP + x] = (float)ex;
+                    if (on) lg[(j0 - k_begin + key) * GP + x] = (float)s[x];
+                }
+            }
+            __syncwarp();
+            if (!failed && !mbar_wait(bars + (kKs + vs) * 8, (it / kVs) & 1)) failed = true;
+            if (edge) patch_tile(vtile, j0, n_valid, 1, it);
+#pragma unroll 4
+            for (int r = 0; r < kDcKeys; ++r) {
+                const int c = NC == 4 ? lane : lane >> 1;     // 16-byte chunk of the lane's channels
+                const unsigned char* src = vtile + (c >> 3) * S::kBox + r * 128 + ((((c & 7) ^ r) & 7) << 4) + (NC == 2 ? (lane & 1) * 8 : 0);
+                float v[NC];
+                load_slice<float, NC>(reinterpret_cast<const float*>(src), v);
+#pragma unroll
+                for (int x = 0; x < GP; ++x) {
+                    const float pj = pr[r * GP + x];
+#pragma unroll
+                    for (int e = 0; e < NC; ++e) acc[x][e] = fmaf(pj, v[e], acc[x][e]);
+                }
+            }
+            __syncwarp();
+            if (it + kVs < my_n) {
+                const int r0 = tile_row0(it + kVs);
+                if (lane == 0) { fence_async_smem(); issue(vmap, r0, kKs + vs); }
+            }
+        }
+#pragma unroll
+        for (int x = 0; x < GP; ++x) {
+            Zl[x] = warp_sum(Zl[x]);
+            if (lane == 0) { misc->wM[warp][x] = (double)Mref[x]; misc->wZ[warp][x] = Zl[x]; }
+#pragma unroll
+            for (int e = 0; e < NC; ++e) rec[x * D + lane * NC + e] = acc[x][e];
+        }
+        if (warp == 0 && lane < GP) misc->qe[lane] = 0.f;
+    }
+    if (failed) mode = max(mode, 1);
+    if (mode) { if (mode == 1) report_status(p.status, CORM_ERR_TIMEOUT); misc->mode = mode; }
+    // the next launch may become resident while this one judges and compacts (it waits for this one to complete)
+    if (!p.early_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    __syncthreads();
+
+    // the block's record: warps merged, in place of the first warp's
+    if (tid < 8 * NW) {
+        const int h = tid / NW, w = tid % NW;
+        const double m = h < G ? misc->wM[w][h] : -INFINITY, z = h < G ? misc->wZ[w][h] : 0.0;
+        double mb = m;
+#pragma unroll
+        for (int o = 1; o < NW; o <<= 1) mb = fmax(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+        const double sc = m == -INFINITY ? 0.0 : exp_nonpos(m - mb);
+        double zb = z * sc;
+#pragma unroll
+        for (int o = 1; o < NW; o <<= 1) zb += __shfl_xor_sync(0xffffffffu, zb, o);
+        misc->wsc[w][h] = (float)sc;
+        if (w == 0) { misc->M[h] = mb; misc->Z[h] = zb; }
+    }
+    __syncthreads();
+    float* blk_rec = reinterpret_cast<float*>(smem);
+    for (int x = tid; x < G * D; x += NT) {
+        const int h = x / D;
+        float acc = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const float sc = misc->wsc[w][h];
+            acc += sc != 0.f ? reinterpret_cast<const float*>(smem + w * S::kWarpRing)[x] * sc : 0.f;
+        }
+        blk_rec[x] = acc;
+    }
+    // registers and positions of the first slots this thread judges are requested before the blocks meet
+    constexpr int kB = 4;                                     // slots per thread and batch
+    uint32_t wv[kB];
+    int32_t pv[kB];
+    auto load_regs = [&](int base) {
+#pragma unroll
+        for (int k = 0; k < kB; ++k) {
+            const int j = k_begin + base + k * NT + tid;
+            wv[k] = 0u; pv[k] = t;                            // the token appended by this step
+            if (j < k_end && j < l_old) { wv[k] = __ldcg(wordu + j); pv[k] = __ldcg(posu + j); }
+        }
+    };
+    load_regs(0);
+    cluster_sync();                                           // records are complete (the block's logits, too)
+
+    // ---- thresholds of Definition 3.1 in log form, the same in every block ----
+    if (tid < 64) {
+        const int h = tid >> 3, x = tid & 7;
+        const bool on = h < G && x < cs;
+        const double m = on ? ld_peer_f64(map_rank(smem_addr(&misc->M[h]), x)) : -INFINITY;
+        const double z = on ? ld_peer_f64(map_rank(smem_addr(&misc->Z[h]), x)) : 0.0;
+        double M = m;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
+        const double sc = m == -INFINITY ? 0.0 : exp_nonpos(m - M);
+        double Z = z * sc;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
+        misc->sc[h][x] = (float)sc;
+        if (x == 0) {
+            const double thr = M + log(Z) + p.log_alpha - log((double)t);
+            misc->thr[h] = thr; misc->Zt[h] = Z; misc->thr_f[h] = (float)thr;
+        }
+    } else if (tid < 96) {
+        const int x = lane;
+        const int md = x < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->mode), x)) : 0;
+        const int bd = x < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->bad), x)) : 0;
+        const uint32_t am = x < cs ? ld_peer_u32(map_rank(smem_addr(&misc->amax), x)) : 0u;
+        const int any_m = __reduce_max_sync(0xffffffffu, md), any_b = __reduce_max_sync(0xffffffffu, bd);
+        const uint32_t any_a = __reduce_max_sync(0xffffffffu, am);
+        if (lane == 0) { misc->any_mode = any_m; misc->any_bad = any_b; misc->unit_amax = any_a; }
+    }
+    __syncthreads();
+    if (misc->any_mode) {                                     // an expired wait, or a unit that cannot take the token: it is left as it is
+        cluster_sync();
+        if (rank == 0 && tid == 0) {
+            if (misc->any_mode == 2) report_status(p.status, CORM_ERR_CAPACITY);
+            p.live_out[u] = l_old;
+            if (misc->any_mode == 2) publish_unit_stamp(p, u, l_old);
+            publish_live(p.maxlive, p.step + 1, l_old);
+        }
+        return;
+    }
+    // error of a head's log-sum-exp (every logit of it is off by at most this much)
+    const float eps_a = kBf16 ? split_amax(min(misc->unit_amax, kSplitMaxBits)) * (float)inv_root_d * 1.0001f : 0.f;
+    if (tid < G) {
+        const float th = fabsf(misc->thr_f[tid]);
+        misc->slack[tid] = 2.f * eps_a * misc->qe[tid] + (th < 3e38f ? th : 0.f) * 1.3e-7f + 1e-12f;
+    }
+    __syncthreads();
+
+    // ---- 2. verdicts, register update, keep bits ----
+    uint32_t* keep = reinterpret_cast<uint32_t*>(smem + 8192);                  // the ring is free behind the block's record
+    int* prefix = reinterpret_cast<int*>(smem + 8192) + kDcMaxWords;
+    {
+        int n_imp = 0, n_keep = 0;
+        for (int base0 = 0; base0 < n_keys; base0 += kB * NT) {
+            if (base0) load_regs(base0);
+#pragma unroll
+            for (int k = 0; k < kB; ++k) {
+                const int base = base0 + k * NT;
+                if (base >= n_keys) break;                    // uniform
+                const int i = base + tid, j = k_begin + i;
+                const bool on = i < n_keys;
+                bool imp = false;
+                uint32_t open = 0u;
+#pragma unroll
+                for (int h = 0; h < GP; ++h) {
+                    if (h >= G || !on) continue;
+                    const float sf = fits ? lg[i * G + h] : __ldcg(lg + (size_t)i * G + h), margin = sf - misc->thr_f[h];
+                    const float err = fabsf(sf) * 6.1e-8f + misc->slack[h];
+                    if (margin >= err) imp = true;
+                    else if (margin > -err) open |= 1u << h;
+                }
+                uint32_t who = __ballot_sync(0xffffffffu, open != 0u && !imp);
+                while (who) {                                 // formed again in fp64, one slot after the other, by the whole warp
+                    const int src = __ffs(who) - 1;
+                    who &= who - 1u;
+                    const int js = __shfl_sync(0xffffffffu, j, src);
+                    uint32_t os = __shfl_sync(0xffffffffu, open, src);
+                    const size_t row = kv_row(pt_u, (size_t)u * p.C, js, p.pool_pages, p.status);
+                    bool yes = false;
+                    int n_near = 0;
+                    while (os) {
+                        const int h = __ffs(os) - 1;
+                        os &= os - 1u;
+                        const double s = warp_exact_dot_cg<T, D>(reinterpret_cast<const T*>(p.q) + ((size_t)u * G + h) * D,
+                                                                 reinterpret_cast<const T*>(p.K) + row * D, lane) * inv_root_d;
+                        const double th = misc->thr[h], e = (double)(eps_a * misc->qe[h]) + 1e-13 * (1.0 + fabs(th));
+                        yes |= s - th > e;
+                        if (lane == 0 && fabs(s - th) <= e) atomicOr(&misc->flags, 1u << h);   // left to the exact heads
+                        ++n_near;
+                    }
+                    if (lane == 0) atomicAdd(p.counters + CNT_NEAR, (unsigned long long)n_near);
+                    if (lane == src) imp = yes;
+                }
+                bool kp = false;
+                if (on) {
+                    const uint32_t wd = update_register(wv[k], imp, p.w, t);
+                    if (CORM_IN_RANGE(j < p.C, p.status)) wordu[j] = wd;
+                    kp = !evict_on || register_needed(wd, p.w, t) || pv[k] > t - p.r;
+                }
+                const uint32_t ballot = __ballot_sync(0xffffffffu, kp);
+                n_imp += __popc(__ballot_sync(0xffffffffu, imp));
+                n_keep += __popc(ballot);
+                if (lane == 0 && base + warp * 32 < n_keys && CORM_IN_RANGE((base >> 5) + warp < kDcMaxWords, p.status))
+                    keep[(base >> 5) + warp] = ballot;
+            }
+        }
+        if (lane == 0) { misc->warp_cnt[warp] = n_keep; misc->warp_imp[warp] = n_imp; }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int c = 0, m = 0;
+#pragma unroll
+        for (int x = 0; x < NW; ++x) { c += misc->warp_cnt[x]; m += misc->warp_imp[x]; }
+        misc->count = c; misc->n_imp = m;
+        if (misc->any_bad) misc->flags = (1u << G) - 1u;      // magnitudes beyond the pieces' range: every head exactly
+    }
+    __syncthreads();
+    cluster_arrive();
+    // outputs (Eq. 1): the unit's G x D values are shared out over the blocks, two channels per thread
+    {
+        const int np = G * D / 2, x0 = np * rank / cs, x1 = np * (rank + 1) / cs;
+        for (int x = x0 + tid; x < x1; x += NT) {
+            const int h = x / (D / 2);
+            float a0 = 0.f, a1 = 0.f;
+            const uint32_t at = smem_addr(blk_rec + 2 * x);
+            float v[kDcMaxCluster][2];
+#pragma unroll
+            for (int y = 0; y < kDcMaxCluster; ++y)
+                if (y < cs) {
+                    const double d = ld_peer_f64(map_rank(at, y));
+                    v[y][0] = __uint_as_float((uint32_t)__double2loint(d)); v[y][1] = __uint_as_float((uint32_t)__double2hiint(d));
+                }
+#pragma unroll
+            for (int y = 0; y < kDcMaxCluster; ++y)
+                if (y < cs) { const float sc = misc->sc[h][y]; a0 = fmaf(v[y][0], sc, a0); a1 = fmaf(v[y][1], sc, a1); }
+            const float o0 = (float)((double)a0 / misc->Zt[h]), o1 = (float)((double)a1 / misc->Zt[h]);
+            if constexpr (kBf16) reinterpret_cast<uint32_t*>(p.out)[(size_t)u * np + x] = (uint32_t)float_to_bf16_bits(o0) | ((uint32_t)float_to_bf16_bits(o1) << 16);
+            else reinterpret_cast<float2*>(p.out)[(size_t)u * np + x] = make_float2(o0, o1);
+        }
+    }
+    cluster_wait();
+    {
+        uint32_t marks = lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->flags), lane)) : 0u;
+        marks = __reduce_or_sync(0xffffffffu, marks);
+        if (marks) {                                          // uniform in the cluster
+            cluster_sync();
+            dc_exact_heads<T, D, NW>(p, u, G, t, k_begin, k_end, marks, keep, misc, cs);
+            cluster_sync();
+        }
+    }
+    // ---- 3. compaction: kept slots at or above the new length move into the holes below it ----
+    int before = 0, total = 0, imp_total = 0;
+    {
+        const int c = lane < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->count), lane)) : 0;
+        total = __reduce_add_sync(0xffffffffu, c);
+        before = __reduce_add_sync(0xffffffffu, lane < rank ? c : 0);
+        if (rank == 0) imp_total = __reduce_add_sync(0xffffffffu, lane < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->n_imp), lane)) : 0);
+    }
+    const int new_len = evict_on ? total : l;
+    int n_moved = 0;
+    if (new_len < l) {
+        // Lists in scratch: hole number = evicted slots before it; mover number = kept slots behind it, so that both follow
+        // from the counts of the blocks before.
+        int* holes = reinterpret_cast<int*>(p.stash) + (size_t)p.U * p.C * G + (size_t)u * p.C;
+        int* movers = holes + p.C / 2;
+        const int nw = (n_keys + 31) >> 5;
+        block_popc_scan<NT>(keep, prefix, nw, misc->scan);
+        for (int i = tid; i < nw; i += NT) {
+            const uint32_t m = keep[i];
+            const int s0 = k_begin + i * 32, kb = before + prefix[i];            // kept slots before this word
+            const uint32_t valid = k_end - s0 >= 32 ? 0xffffffffu : (1u << (k_end - s0)) - 1u;
+            const uint32_t below = new_len - s0 >= 32 ? 0xffffffffu : (new_len > s0 ? (1u << (new_len - s0)) - 1u : 0u);
+            uint32_t hm = ~m & valid & below;                 // evicted slots below the new length
+            while (hm) {
+                const int bit = __ffs(hm) - 1;
+                hm &= hm - 1u;
+                const int x = s0 + bit - kb - __popc(m & ((1u << bit) - 1u));
+                if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) holes[x] = s0 + bit;
+            }
+            uint32_t km = m & valid & ~below;                 // kept slots at or above it
+            while (km) {
+                const int bit = __ffs(km) - 1;
+                km &= km - 1u;
+                const int x = total - 1 - kb - __popc(m & ((1u << bit) - 1u));
+                if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) movers[x] = s0 + bit;
+            }
+            if (new_len >= s0 && new_len < s0 + 32 && new_len < k_end)           // how many: evicted slots below the new length
+                p.unit_rec[u] = make_int2(new_len - kb - __popc(m & below), 0);
+        }
+        cluster_sync();
+        n_moved = __ldcg(&p.unit_rec[u].x);
+        const size_t slab_row0 = (size_t)u * p.C;
+        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V),
+                                  [&](int slot) -> size_t {
+                                      return pt_u ? page_row(__ldcg(pt_u + (slot >> 5)), slot, p.pool_pages, p.status) : slab_row0 + (size_t)slot;
+                                  }, wordu, posu, movers, holes, n_moved, rank, cs, l, p.status);
+    }
+    // every block's row moves come before released pages and the stamp; and a block's shared memory stays until its peers
+    // have read it
+    if (new_len == l || pt_u || p.unit_stamp) cluster_sync();
+    if (rank != 0) return;
+    if (pt_u) settle_pages<NT>(p.page_table, p.page_bits, p.page_room, p.pool_pages, p.pt_stride, p.U, u, l_old, new_len);
+    if (pt_u && p.unit_stamp) __syncthreads();
+    if (tid == 0) {
+        p.live_out[u] = new_len;
+        publish_unit_stamp(p, u, new_len);
+        publish_live(p.maxlive, p.step + 1, new_len);
+        atomicAdd(p.counters + CNT_APPENDED, 1ull);
+        atomicAdd(p.counters + CNT_ATTENDED, (unsigned long long)l);
+        if (imp_total) atomicAdd(p.counters + CNT_IMPORTANT, (unsigned long long)imp_total);
+        if (new_len < l) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(l - new_len));
+        if (n_moved) atomicAdd(p.counters + CNT_MOVED, (unsigned long long)n_moved);
+    }
+}
+
+// One layer's (or, from it on, all layers') K or V storage as a 2-D tensor [rows][D] with boxes of 16 rows x 128 bytes and
+// the 128-byte swizzle. The map only ever covers memory of the cache's own device.
+inline corm_status_t make_row_tensor_map(CUtensorMap* out, void* base, unsigned long long rows, int D, bool bf16) {
+    typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                 const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                 CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn ||
+        q != cudaDriverEntryPointSuccess) {
+        (void)cudaGetLastError();
+        return CORM_ERR_UNSUPPORTED;
+    }
+    const int e = bf16 ? 2 : 4;
+    const cuuint64_t dims[2] = {(cuuint64_t)D, rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)(D * e)};
+    const cuuint32_t box[2] = {(cuuint32_t)(128 / e), kDcKeys};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = reinterpret_cast<EncodeFn>(fn)(
+        out, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? CORM_OK : CORM_ERR_CUDA;
+}
+
+constexpr int kDcWarps = 4;
+
+template <typename T, int D, int GP>
+inline corm_status_t launch_decode_cluster_as(DecodeClusterParams& dp, const CUtensorMap& kmap, const CUtensorMap& vmap, int upper,
+                                              int tune_split_len, int sm_count, cudaStream_t st) {
+    constexpr int NW = kDcWarps;
+    const DecodeParams& p = dp.p;
+    const int sms = sm_count > 0 ? sm_count : 148;
+    constexpr int kBlocks = dc_blocks<T, D, GP, NW>();
+    // as many blocks per unit as fill the resident slots once, but at least two 32-slot words each ...
+    long long cs = (long long)sms * kBlocks / p.U;
+    if (tune_split_len) cs = (upper + tune_split_len - 1) / tune_split_len;
+    if (cs > (upper + 63) / 64) cs = (upper + 63) / 64;
+    // ... and no more words than a block can keep track of
+    const long long least = ((p.C + 31) / 32 + kDcMaxWords - 1) / kDcMaxWords;
+    cs = std::max(std::max(cs, least), 1ll);
+    if (cs > kDcMaxCluster) cs = kDcMaxCluster;
+    if (least > kDcMaxCluster) return CORM_ERR_UNSUPPORTED;
+    const int base = dc_smem_layout<T, D, GP, NW>(0).total;
+    const int budget = (228 * 1024) / kBlocks - 1024;
+    const int need = (int)std::min<long long>(((upper + 31) / 32 + cs - 1) / cs * 32 * (long long)dp.G, 1 << 20);
+    dp.lcap = std::max(0, std::min(need, (budget - base) / 128 * 32));
+    const size_t smem = (size_t)dc_smem_layout<T, D, GP, NW>(dp.lcap).total;
+    auto kern = decode_cluster_kernel<T, D, GP, NW>;
+    cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), (size_t)std::max(budget, base));
+    if (e == cudaSuccess) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)p.U, (unsigned)cs);
+        cfg.blockDim = dim3(NW * 32);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = (unsigned)cs;
+        attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // set-up overlaps the previous launch's tail
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        e = cudaLaunchKernelEx(&cfg, kern, dp, kmap, vmap);
+        if (e == cudaSuccess) e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) { std::fprintf(stderr, "corm: decode launch: %s\n", cudaGetErrorString(e)); return CORM_ERR_CUDA; }
+    return CORM_OK;
+}
+
+inline corm_status_t launch_decode_cluster(DecodeClusterParams& dp, bool bf16, int D, const CUtensorMap& kmap, const CUtensorMap& vmap,
+                                           int upper, int tune_split_len, int sm_count, cudaStream_t st) {
+    const int G = dp.G;
+#define CORM_DC(TT, DD, GG) return launch_decode_cluster_as<TT, DD, GG>(dp, kmap, vmap, upper, tune_split_len, sm_count, st)
+    if (bf16) {
+        if (D == 128) { if (G <= 2) CORM_DC(bf16_t, 128, 2); if (G == 4) CORM_DC(bf16_t, 128, 4); if (G == 8) CORM_DC(bf16_t, 128, 8); }
+        else { if (G <= 2) CORM_DC(bf16_t, 64, 2); if (G == 4) CORM_DC(bf16_t, 64, 4); if (G == 8) CORM_DC(bf16_t, 64, 8); }
+    } else {
+        if (D == 128) { if (G == 1) CORM_DC(float, 128, 1); if (G == 2) CORM_DC(float, 128, 2); if (G == 4) CORM_DC(float, 128, 4); if (G == 8) CORM_DC(float, 128, 8); }
+        else { if (G == 1) CORM_DC(float, 64, 1); if (G == 2) CORM_DC(float, 64, 2); if (G == 4) CORM_DC(float, 64, 4); if (G == 8) CORM_DC(float, 64, 8); }
+    }
+#undef CORM_DC
+    return CORM_ERR_UNSUPPORTED;
+}
+
+}  // namespace corm

@@ -1,6 +1,6 @@
-// Generic kernels: any supported dtype / head_dim / group size, written for clarity. One warp per key, lanes
-// split the head dimension, fp64 logits. The bf16 / head_dim 128 decode path has faster kernels of its own;
-// this one serves fp32 caches, head_dim 64 and groups of eight.
+// Generic decode kernel: any supported dtype / head_dim / group size, written for clarity. One warp per key, lanes
+// split the head dimension, fp64 logits. It serves corm_decode_step_static, whose scratch is a fixed array, and tuning
+// value 0; every other step has a faster kernel.
 #pragma once
 
 #include "corm_common.cuh"

@@ -44,8 +44,8 @@ __device__ __forceinline__ uint32_t sub_bf16x2(uint32_t a, uint32_t b) {
     return r;
 }
 
-// Keys of larger magnitude than 2^40 (or not finite) leave the range in which products of pieces are safe in fp32.
-constexpr uint32_t kSplitMaxBits = (127u + 40u) << 7;          // bf16 bits of 2^40
+// Elements of larger magnitude than 2^56 (or not finite) leave the range in which products of pieces are safe in fp32.
+constexpr uint32_t kSplitMaxBits = (127u + 56u) << 7;          // bf16 bits of 2^56
 constexpr uint32_t kSplitMinExp = 127u - 40u;                  // smaller tiles are cut on the grid of 2^-40
 
 // The two grid constants (192 g and 192 g/128, each twice in a word) of a key tile whose largest magnitude has the
@@ -77,7 +77,7 @@ __device__ __forceinline__ void split_query(float q, float c, float& q1, float& 
     q2 = __fsub_rn(__fadd_rn(r, c2), c2);
     q3 = __fsub_rn(r, q2);
 }
-// c of split_query for a row whose largest magnitude is aq (finite, below 2^40)
+// c of split_query for a row whose largest magnitude is aq (finite, below 2^56)
 __device__ __forceinline__ float split_query_const(float aq) {
     const int ex = max((int)((__float_as_uint(aq) >> 23) & 255u), 127 - 40);
     return __uint_as_float((uint32_t)(ex - 7 + 23) << 23) * 1.5f;
@@ -92,11 +92,18 @@ __device__ __forceinline__ float split_error(float n1, float n2, float n3) {
 // words of two bf16 -> the larger magnitude of each half, as bits
 __device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t m, uint32_t x) { return __vmaxu2(m, x & 0x7fff7fffu); }
 
+// running maximum of magnitudes, two at a time (signs of the result are meaningless), NaN stays
+__device__ __forceinline__ uint32_t max_mag_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.NaN.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 // ---- clusters ----
 __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ uint32_t cluster_size() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 // shared-memory address of the same variable in the cluster's block `rank`
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {

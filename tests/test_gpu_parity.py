@@ -127,7 +127,7 @@ PROMPT_EDGES = [
     ("f32", 64, 8, (255, 300), 64, 4.0, 91),
     ("bf16", 128, 4, (4200, 4200), 8, 4.0, 91),
     ("bf16", 128, 4, (300, 300), 8, 400.0, 91),       # logits beyond the plain sum of exponentials: the exact rows
-    ("bf16", 64, 1, (300, 300), 8, 2.0 ** 42, 91),     # keys beyond the range of the exact pieces
+    ("bf16", 64, 1, (300, 300), 8, 2.0 ** 58, 91),     # keys beyond the range of the exact pieces
     ("f32", 64, 2, (300, 300), 8, 400.0, 91),
 ]
 
@@ -151,6 +151,57 @@ def test_prompt_pass_edges(case):
                                  data.prompt_lens)
         assert_states_equal(gpu, orc, 0, 3, 2, f"pool {pool}")
         assert gpu.corm_cache_stats()["device_status"] == 0
+
+
+# the cluster kernel where it can go wrong: units of one slot, tiles of 16 and words of 32 slots at their edges, blocks
+# without slots, eight blocks per unit, heads formed again in fp64 (bound scale), pages, layers stepped as one launch
+CLUSTER = [
+    # dtype, head_dim, group, n_kv, batch, layers, prompt range, steps, w, r, bound scale, pool_pages, seed
+    ("f32", 128, 1, 2, 2, 1, (0, 3), 70, 2, 1, 1.0, 0, 50),
+    ("f32", 64, 4, 2, 1, 1, (500, 560), 40, 8, 16, 1e6, 64, 50),
+    ("f32", 128, 8, 1, 2, 1, (31, 33), 36, 4, 8, 1.0, 0, 51),
+    ("bf16", 64, 1, 3, 2, 1, (15, 17), 40, 4, 8, 1.0, 64, 50),
+    ("bf16", 64, 2, 2, 1, 2, (1000, 1100), 24, 8, 16, 1.0, 0, 50),
+    ("bf16", 64, 8, 2, 2, 1, (100, 300), 40, 33, 16, 1e4, 64, 50),
+    ("bf16", 64, 4, 1, 1, 1, (3000, 3000), 12, 8, 64, 1e9, 0, 51),
+    ("bf16", 128, 8, 1, 1, 3, (700, 700), 20, 8, 32, 1.0, 0, 51),
+    ("bf16", 128, 8, 2, 1, 1, (60, 70), 30, 8, 4, 1e6, 32, 50),
+]
+
+
+@pytest.mark.parametrize("case", CLUSTER, ids=lambda c: "-".join(str(x) for x in c))
+def test_cluster_decode_edges(case):
+    """Free-running parity through one call per step, then the same steps through multi-step calls of 1, 5 and the rest
+    (chained launches) on a second cache."""
+    dtype, d, G, nkv, B, L, (pmin, pmax), steps, w, r, scale, pool, seed = case
+    cfg = CONFIGS[1].with_(name="cluster", n_layers=L, batch=B, n_q_heads=nkv * G, n_kv_heads=nkv, head_dim=d, dtype=dtype,
+                           prompt_min=pmin, prompt_max=pmax, steps=steps, window_w=w, recent_r=r,
+                           gqa_rho=0.7 if G > 1 else 0.0, hh_min=2, hh_max=6, seed=seed)
+    datas = [generate(cfg, layer=l) for l in range(L)]
+    one, many = (make_gpu_cache(cfg, B, nkv, n_layers=L, pool_pages=pool) for _ in range(2))
+    orc = make_oracle(cfg, B, nkv, n_layers=L)
+    for g in (one, many):
+        g.corm_cache_set_bound_scale(scale)
+        for l, dat in enumerate(datas):
+            g.corm_compress_prompt(l, to_dev(dat.k_prompt, dtype), to_dev(dat.v_prompt, dtype), to_dev(dat.q_last, dtype),
+                                   dat.prompt_lens)
+    for l, dat in enumerate(datas):
+        orc.compress_prompt(l, dat.k_prompt, dat.v_prompt, dat.q_last, dat.prompt_lens)
+    q, k, v = (torch.stack([to_dev(getattr(dat, n), dtype) for dat in datas], dim=1).contiguous() for n in ("q", "k_new", "v_new"))
+    outs = torch.cat([many.corm_decode_steps(0, L, q[a:b], k[a:b], v[a:b]) for a, b in ((0, 1), (1, 6), (6, steps))])
+    for s in range(steps):
+        for l, dat in enumerate(datas):
+            ref = orc.decode_step(l, dat.q[s], dat.k_new[s], dat.v_new[s])
+            out = one.corm_decode_step(l, q[s, l], k[s, l], v[s, l])
+            assert np.abs(out.float().cpu().numpy() - ref).max() <= OUT_TOL[dtype], (s, l)
+            assert np.abs(outs[s, l].float().cpu().numpy() - ref).max() <= OUT_TOL[dtype], (s, l)
+            if s % 7 == 0 or s == steps - 1:
+                assert_states_equal(one, orc, l, B, nkv, f"step {s} layer {l}")
+    for l in range(L):
+        assert_states_equal(many, orc, l, B, nkv, f"multi-step, layer {l}")
+    assert one.corm_cache_stats()["device_status"] == many.corm_cache_stats()["device_status"] == 0
+    if G == 1 or pmax + steps <= 96 * B * nkv * L:
+        assert many.corm_cache_chained_launches() >= steps // 2
 
 
 def test_alpha_zero_never_evicts():
