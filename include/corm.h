@@ -175,9 +175,8 @@ corm_status_t corm_decode_step_layers(corm_cache_t* cache, int32_t first_layer, 
  * Every input must be complete in stream order before the call; the result is that of calling corm_decode_step_layers
  * once per step (registers, live lists and positions identical, outputs within rounding).
  * What the call adds: the units of a cache are independent (Algorithm 1 runs "on each head at every layer"), so
- * step s + 1 of a unit needs step s of that unit only. When a step's launch finishes every unit inside the streaming
- * kernel (one query head per KV head; grouped heads inside this call, which take a block per split unless units are
- * few and long; tuning values 2 and 6), the next step's launch is chained to it: its blocks start
+ * step s + 1 of a unit needs step s of that unit only. When a step's launch finishes every unit inside itself (all but
+ * tuning values 3 and 5, and few long units of grouped heads), the next step's launch is chained to it: its blocks start
  * as soon as a multiprocessor has room and each waits (bounded, like every wait here) for its own unit's previous
  * step instead of the whole previous launch, so consecutive steps fill one another's last waves. Steps that need the
  * verdict launch, and caches with the similarity monitor on, run as with the per-step calls.
@@ -242,15 +241,13 @@ corm_status_t corm_cache_import_state(corm_cache_t* cache, int32_t layer, int32_
 
 /* Tuning knobs (performance only; live lists and registers do not depend on them, outputs only within rounding):
  * keys per split of the block-per-split decode kernel (multiple of 32, 0 = automatic) and which kernels may be used:
- * allow_fast_path 0 = the generic kernel only; 1 = automatic (default): a cluster of blocks per unit for fp32 caches,
- * head_dim 64 and groups of eight; for bf16 / head_dim 128, one query head per
- * KV head takes the block-per-split kernel, which finishes a unit of several splits inside the decode launch when the
- * launch has many units and by a second, verdict launch when it has few, and grouped heads take the balanced
- * kernel (every block an equal share of the step's keys) followed by the verdict launch; 2 / 3 = the block-per-split
+ * allow_fast_path 0 = the generic kernel only; 1 = automatic (default): a cluster of blocks per unit, and for bf16 /
+ * head_dim 128 with one query head per KV head, where units fit one block, are many or lose nothing to eviction, the
+ * block-per-split kernel, which finishes a unit of several splits inside the decode launch when the launch has many units
+ * and by a second, verdict launch when it has few; 2 / 3 = the block-per-split
  * kernel with the first / the second way always; 4 / 5 = the balanced kernel for every group size it covers,
  * finishing inside its own launch / with the verdict launch; 6 = the balanced kernel's streaming loop with a block per
- * split, each unit finished by its last-arriving split (what automatic picks for grouped heads inside
- * corm_decode_steps unless units are few and long, because such launches can be chained). Errors: INVALID_ARG. */
+ * split, each unit finished by its last-arriving split. Errors: INVALID_ARG. */
 corm_status_t corm_cache_set_tuning(corm_cache_t* cache, int32_t split_len, int32_t allow_fast_path);
 
 /* Opt-in monitor of the method's premise (Sections 3.2-3.3: the current query resembles recent ones, which is what

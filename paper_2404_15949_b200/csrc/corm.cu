@@ -33,7 +33,7 @@ constexpr int kMinSplit = 64;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-    size_t K, V, word, pos, live, base_tokens, base_obs, ticket, ticket2, unit_stamp, counters, status, maxlive, sim_acc, page_table, page_bits, page_room, q_prev, stash, partials, keepmask, unit_rec;
+    size_t K, V, word, pos, live, base_tokens, base_obs, ticket, ticket2, kmax, unit_stamp, counters, status, maxlive, sim_acc, page_table, page_bits, page_room, q_prev, stash, partials, keepmask, unit_rec;
     size_t stage_q, stage_k, stage_v, stage_out, total, bookkeeping_begin, bookkeeping_end;
 };
 
@@ -98,6 +98,7 @@ Layout make_layout(const corm_config_t& c, int pool_pages) {
     L.base_obs = take(Ltot * c.batch * 4);
     L.ticket = take(Ltot * U * 4);
     L.ticket2 = take(Ltot * U * 4);
+    L.kmax = take(Ltot * U * 4);
     L.unit_stamp = take(Ltot * U * 8);
     L.counters = take(Ltot * CNT_COUNT * 8);
     L.status = take(4);
@@ -309,17 +310,24 @@ corm_status_t monitor_similarity(corm_cache* c, int layer, const void* q, cudaSt
     return CORM_OK;
 }
 
-// which caches the cluster kernel steps: whatever the bf16 / head_dim-128 kernels do not cover
-bool takes_cluster(const corm_cache* c) {
-    const bool covered = c->cfg.kv_dtype == CORM_BF16 && c->cfg.head_dim == 128 && c->G <= 4;
-    return c->allow_fast == 1 && !c->kmaps_row.empty() && !covered;
+// Whether the cluster kernel takes a step of units of up to `upper` keys. Everything but one query head per KV head on
+// bf16 / head_dim 128, and that too when units are longer than a block of the block-per-split kernel finishes on chip and
+// eviction is at work (us per step, block-per-split -> cluster, 16000-key prompts: 32 units 61 -> 37, 128 units 130 -> 95,
+// 4000-key prompts: 32 units 26 -> 22, 256 units 61 -> 54; but 1000-key prompts: 32 units 17.7 -> 19.3, 512 units 32 -> 46;
+// 4000-key prompts: 512 units 87 -> 89).
+// Where nothing or little is evicted (alpha 0, windows beyond a register) its finish is cheap and its loop, which widens
+// keys to fp64 instead of cutting them into pieces, streams faster (128 units x 3400 keys 54 -> 62).
+bool takes_cluster(const corm_cache* c, int upper, int n_units) {
+    if (c->allow_fast != 1 || c->kmaps_row.empty()) return false;
+    if (c->cfg.kv_dtype != CORM_BF16 || c->cfg.head_dim != 128 || c->G >= 2) return true;
+    return upper > 1024 && n_units <= 256 && c->cfg.window_w <= 32 && c->cfg.alpha > 0.f;
 }
 
 // whether several layers from first_layer on may run as one launch as far as the kernels are concerned
 bool can_fuse(const corm_cache* c, int first_layer) {
     const corm_config_t& cf = c->cfg;
     if (fused_layers_of(cf, c->pool_pages) <= 1 || !c->allow_fast || c->monitor_similarity) return false;
-    if (takes_cluster(c)) return true;
+    if (c->allow_fast == 1 && !c->kmaps_row.empty()) return true;
     return cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4 &&
            ((c->allow_fast != 6 && (c->G == 1 || c->allow_fast == 2 || c->allow_fast == 3)) || (c->have_vmap_all && first_layer == 0));
 }
@@ -367,6 +375,7 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     p.keepmask = reinterpret_cast<uint32_t*>(c->arena + c->lay.keepmask);
     p.unit_rec = reinterpret_cast<int2*>(c->arena + c->lay.unit_rec);
     p.unit_stamp = reinterpret_cast<unsigned long long*>(layer_ptr(c, c->lay.unit_stamp, U * 8, layer));
+    p.kmax = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.kmax, U * 4, layer));
     p.q = q; p.k_new = k_new; p.v_new = v_new; p.out = out;
     p.U = (int)U * n_fused; p.Hkv = cf.n_kv_heads; p.C = cf.max_tokens; p.max_splits = max_splits_of(cf);
     p.step = c->steps[layer]; p.w = cf.window_w; p.r = cf.recent_r;
@@ -379,24 +388,13 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     }
     const int upper = std::min(cf.max_tokens, bound + 1);   // no unit can hold more live keys
 
-    const bool cluster = takes_cluster(c);
+    const bool cluster = takes_cluster(c, upper, p.U);
     const bool fast = !cluster && c->allow_fast && cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4;
     corm_status_t rc;
     int n_launched = 1;
-    // Grouped query heads take the balanced streaming kernel followed by the verdict launch (measured against the
-    // block-per-split kernels on one GPU, us per step: 53 against 55 in the steady state of the grouped workload, 122
-    // against 136 in its first steps, 174 against 190 on 24k-key units, 157 against 177 on 8k-key units without
-    // evictions); one query head per KV head stays on the block-per-split kernel, whose loop is lighter (three
-    // blocks per SM). Tuning values 4 / 5 force the balanced kernel finishing in the launch / with the verdict launch.
-    // Inside a call of several steps (corm_decode_steps) grouped heads take that kernel's loop with a block per split
-    // and the unit finished by its last split instead, because such launches can be chained: 43 against 51 us per step
-    // on 128 units of 1660 keys, 132 against 142 on 8200-key units. Not with few long units, whose finishing block
-    // walks the whole unit alone (32 units of 12-24k keys: 133 against 103 us). Tuning value 6 forces it.
-    const bool units = fast && !c->vmaps.empty() &&
-                       (c->allow_fast == 6 || (c->allow_fast == 1 && c->G >= 2 && (chain || more) && !c->monitor_similarity &&
-                                               (long long)upper <= 96ll * (long long)p.U));
-    const bool balanced = !units && fast && !c->vmaps.empty() &&
-                          (c->allow_fast == 4 || c->allow_fast == 5 || (c->allow_fast == 1 && c->G >= 2));
+    // Tuning values 4 / 5 / 6 force the balanced kernel's three forms.
+    const bool units = fast && !c->vmaps.empty() && c->allow_fast == 6;
+    const bool balanced = fast && !c->vmaps.empty() && (c->allow_fast == 4 || c->allow_fast == 5);
     const bool balanced_verdict = c->allow_fast != 4;
     bool chain_ok_before = chain && !c->monitor_similarity;
     for (int i = 0; i < n_fused; ++i) chain_ok_before &= c->chain_ok[layer + i] != 0;
@@ -616,6 +614,7 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     auto clear = [&](void* ptr, size_t bytes) { bp.clear[n_clear++] = {static_cast<uint32_t*>(ptr), bytes / 4}; };
     clear(layer_ptr(c, c->lay.ticket, U * 4, layer), U * 4);
     clear(layer_ptr(c, c->lay.ticket2, U * 4, layer), U * 4);
+    clear(layer_ptr(c, c->lay.kmax, U * 4, layer), U * 4);
     clear(layer_ptr(c, c->lay.unit_stamp, U * 8, layer), U * 8);        // step counts restart
     clear(maxlive_ptr(c, layer), 8);
     clear(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer), CNT_COUNT * 8);   // a new prompt restarts the layer's statistics
@@ -645,6 +644,7 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     p.log_alpha = log_alpha_of(c);
     p.bound_scale = c->bound_scale;
     p.keepmask = reinterpret_cast<uint32_t*>(c->arena + c->lay.keepmask);
+    p.kmax = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.kmax, U * 4, layer));
     const bool bf = cf.kv_dtype == CORM_BF16;
     const corm_status_t rc =
         cf.head_dim == 128 ? (bf ? launch_prompt_cluster<bf16_t, 128>(p, c->G, max_p, c->sm_count, st) : launch_prompt_cluster<float, 128>(p, c->G, max_p, c->sm_count, st))
@@ -913,6 +913,7 @@ corm_status_t corm_decode_step_static(corm_cache_t* c, int32_t layer, const void
     p.stash = reinterpret_cast<double*>(scratch);
     p.partials = scratch + stash_bytes;
     p.ticket = reinterpret_cast<uint32_t*>(scratch + stash_bytes + partial_bytes);
+    p.kmax = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.kmax, U * 4, layer));
     p.q = q; p.k_new = k_new; p.v_new = v_new; p.out = out;
     p.U = (int)U; p.Hkv = cf.n_kv_heads; p.C = cf.max_tokens; p.max_splits = n_splits; p.split_len = split_len;
     p.step = c->steps[layer]; p.w = cf.window_w; p.r = cf.recent_r;
@@ -1078,6 +1079,10 @@ corm_status_t corm_cache_import_state(corm_cache_t* c, int32_t layer, int32_t se
         CORM_CUDA(cudaMemcpyAsync(layer_ptr(c, c->lay.word, U * C * 4, layer) + u * C * 4, word_host, n * 4, cudaMemcpyHostToDevice, st));
         CORM_CUDA(cudaMemcpyAsync(layer_ptr(c, c->lay.pos, U * C * 4, layer) + u * C * 4, pos_host, n * 4, cudaMemcpyHostToDevice, st));
     }
+    uint32_t kmax = 0u;                           // largest magnitude among the imported keys
+    if (cf.kv_dtype == CORM_BF16)
+        for (size_t i = 0; i < n * D; ++i) kmax = std::max<uint32_t>(kmax, static_cast<const uint16_t*>(k_host)[i] & 0x7fffu);
+    CORM_CUDA(cudaMemcpyAsync(layer_ptr(c, c->lay.kmax, U * 4, layer) + u * 4, &kmax, 4, cudaMemcpyHostToDevice, st));
     // the kernels see tokens = base + steps and rows = min(w, base + steps): rebase this sequence
     const int32_t bt = n_tokens - c->steps[layer], bo = n_obs - c->steps[layer], lv = live_len;
     CORM_CUDA(cudaMemcpyAsync(live_buf(c, layer, c->parity[layer]) + u, &lv, 4, cudaMemcpyHostToDevice, st));

@@ -768,6 +768,7 @@ decode_balanced_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
                     if (!failed && !mbar_wait(my_bars + kslot * 8, (n_consumed / kBalKStages) & 1)) failed = true;   // once one wait has expired the rest are skipped
                     if (has_new) {   // append: the new row goes to the cache and into the arriving tile
                         const long long row0 = tile_row0(sg, ti);
+                        note_key_magnitude(p.kmax + u, lane < 16 ? new_row(0) : make_uint4(0, 0, 0, 0));
                         if (row0 >= 0 && lane < 16) {
                             const uint4 newk = new_row(0);
                             *reinterpret_cast<uint4*>(ktile + (l_old - k0) * kRowBytes + lane * 16) = newk;

@@ -16,10 +16,15 @@
 // probabilities, each split into two bf16.
 // fp32: a key per lane (its channels shared by two half-warps), fp64 products on the CUDA cores, P.V by fp32 FMAs.
 //
-// What bounds it: the chain of round trips (about 20 us of 30) on units of a few hundred keys, which is what it is used
-// on. Measured against one warp per key and the last-arriving split finishing the unit alone, us per step:
-//   64 units x 970 keys, G 8, bf16   253 -> 31      128 units x 1090 keys, G 4, 64 channels   143 -> 34
-//   20 units x 250 keys, G 2, fp32    64 -> 15      8 units x 170 keys, G 1, fp32            37.7 -> 14
+// What bounds it: on units of a few hundred keys the chain of round trips (set-up 2 us, first tiles 2, exchange and
+// thresholds 3, verdicts 2, exchange 1, moves 2, launch 2); on long units HBM, shared out unevenly where units differ in
+// length. Measured, us per step from one call per step, before -> now:
+//   64 units x 970 keys, G 8, bf16          253 -> 32     128 units x 1090 keys, G 4, 64 channels   143 -> 30
+//   20 units x 250 keys, G 2, fp32           64 -> 16     8 units x 170 keys, G 1, fp32            37.7 -> 14
+//   128 units x 2800 keys, G 4, bf16         86 -> 68     32 units x 21400 keys, G 4, bf16          133 -> 103
+//   32 units x 8200 keys, G 4, no eviction   55 -> 47     32 units x 1160 keys, G 1, bf16            35 -> 24
+// (from one warp per key and the last-arriving split finishing the unit, from the balanced kernel and its verdict launch,
+// from the block-per-split kernel).
 //
 // Verdicts are the fp64 ones: a slot's logit is kept in fp32, and one that lies within the proven error of its threshold
 // is formed again in fp64. If it then lies within the error of the log-sum-exp itself, the head is marked and the
@@ -35,7 +40,7 @@ namespace corm {
 
 constexpr int kDcMaxCluster = 8;
 constexpr int kDcKeys = 16;                       // keys per tile
-constexpr int kDcMaxWords = 4096;                 // 32-slot words a block may own (its keep bits and prefix sums lie in the ring)
+constexpr int kDcMaxWords = 4096;                 // 32-slot words a block may own (its keep bits and prefix sums lie in the ring: 41 KB)
 
 struct DecodeClusterParams {
     DecodeParams p;
@@ -61,20 +66,23 @@ template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int d
     return Elem<T>::kBytes == 4 ? (D == 128 ? 12 : 16) / NW : (GP == 8 ? 12 : 16) / NW;
 }
 
+constexpr int kDcListCap = 1024;                  // slots a step may evict from a unit for its moves to be listed on chip
+
 template <int NW> struct DcMisc {
     unsigned long long stamp;
-    double wM[NW][8], wZ[NW][8];                  // per warp and head
-    double M[8], Z[8];                            // the block's, read by its peers
-    double thr[8], Zt[8];
+    double wZ[NW][8];                             // per warp and head, read by the cluster
+    double thr[8], Zt[8], log_t;
     double red[NW][2], mz[2];                     // exact heads
-    float wsc[NW][8], sc[8][kDcMaxCluster], qe[8], thr_f[8], slack[8];
-    uint32_t amax, flags, unit_amax;
-    int mode, any_mode;                           // 0: fine; 1: a wait expired; 2: the unit cannot take the token
-    int bad, any_bad;
-    int count, n_imp;                             // kept slots, important keys of the block
-    int warp_cnt[NW], warp_imp[NW];
+    float wM[NW][8];
+    float sc[8][kDcMaxCluster * NW], qe[8], thr_f[8], slack[8];
+    // largest key magnitude (bf16 bits), 1 << 16 if a magnitude is beyond the pieces' range, 1 << 17 if a wait expired,
+    // 1 << 18 if the unit cannot take the token
+    uint32_t state;
+    uint32_t flags;                               // heads to be formed exactly
+    int count, n_imp, n_moved;                    // kept slots and important keys of the block; row moves of the unit
     int scan[NW * 32];
 };
+constexpr uint32_t kDcBad = 1u << 16, kDcExpired = 1u << 17, kDcFull = 1u << 18;
 
 struct DcSmem { int prob, q, newrow, logits, bars, misc, total; };
 template <typename T, int D, int GP, int NW>
@@ -208,6 +216,36 @@ __device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G,
     if (added_imp) atomicAdd(&misc->n_imp, added_imp);
 }
 
+// Verdicts that the error bounds leave open, by a whole warp: lane's slot j, heads `open`; true where a head is sure to
+// find the key important. Heads whose threshold is too close to tell are marked in misc->flags.
+template <typename T, int D, int NW>
+__device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int G, int j, uint32_t open, float eps_a, DcMisc<NW>* misc) {
+    const int lane = threadIdx.x & 31;
+    const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
+    bool imp = false;
+    uint32_t who = __ballot_sync(0xffffffffu, open != 0u);
+    int n_near = 0;
+    while (who) {
+        const int src = __ffs(who) - 1;
+        who &= who - 1u;
+        const int js = __shfl_sync(0xffffffffu, j, src);
+        uint32_t os = __shfl_sync(0xffffffffu, open, src);
+        const size_t row = kv_row(pt_u, (size_t)u * p.C, js, p.pool_pages, p.status);
+        while (os) {
+            const int h = __ffs(os) - 1;
+            os &= os - 1u;
+            const double s = warp_exact_dot_cg<T, D>(reinterpret_cast<const T*>(p.q) + ((size_t)u * G + h) * D,
+                                                     reinterpret_cast<const T*>(p.K) + row * D, lane) * inv_root_dim(D);
+            const double th = misc->thr[h], e = (double)(eps_a * misc->qe[h]) + 1e-13 * (1.0 + fabs(th));
+            if (lane == src && s - th > e) imp = true;
+            if (lane == 0 && fabs(s - th) <= e) atomicOr(&misc->flags, 1u << h);
+            ++n_near;
+        }
+    }
+    if (lane == 0) atomicAdd(p.counters + CNT_NEAR, (unsigned long long)n_near);
+    return imp;
+}
+
 template <typename T, int D, int GP, int NW>
 __global__ void __launch_bounds__(NW * 32, dc_blocks<T, D, GP, NW>())
 decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap) {
@@ -232,8 +270,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     if (tid == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&kmap)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&vmap)) : "memory");
-        misc->amax = 0u; misc->flags = 0u; misc->mode = 0; misc->bad = 0;
-        if (smem_addr(smem) & 1023u) { report_status(p.status, CORM_ERR_INTERNAL); misc->mode = 1; }   // never expected
+        misc->state = 0u; misc->flags = 0u; misc->count = 0; misc->n_imp = 0;
     }
     if (lane == 0) {
 #pragma unroll
@@ -241,36 +278,51 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         fence_mbar_init();
         fence_async_smem();
     }
-    int l_old, mode = 0;
+    int l_old;
+    uint32_t state = smem_addr(smem) & 1023u ? kDcExpired : 0u;          // swizzled tiles need the alignment; never expected
     if (p.chain_wait) {                                       // this unit's previous step, not the whole previous launch
+        if (p.early_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         if (tid == 0) misc->stamp = wait_unit_stamp(p.unit_stamp + u, (uint32_t)p.step, p.status);
         __syncthreads();
         const unsigned long long sw = misc->stamp;
         const bool ok = (uint32_t)(sw >> 32) == (uint32_t)p.step;
         l_old = ok ? (int)(uint32_t)sw : 0;
-        if (!ok) mode = 1;
+        if (!ok) state = kDcExpired;
         asm volatile("fence.proxy.async.global;" ::: "memory");   // the tile copies read rows that ordinary stores wrote
     } else {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         l_old = __ldcg(p.live_in + u);
     }
+    // queries, and in the block that will own the last slot the appended rows: requested next to the length (their latency
+    // is a bus round trip when the caller's buffers are host memory)
+    const float* q_raw = reinterpret_cast<const float*>(p.q) + (size_t)u * G * D;
+    if constexpr (kBf16)
+        for (int x = tid; x < G * (S::kRow / 16); x += NT)
+            cp_async16(smem_addr(smem + lay.q + x * 16), reinterpret_cast<const unsigned char*>(p.q) + ((size_t)u * G * (S::kRow / 16) + x) * 16);
+    if (rank == cs - 1)
+        for (int x = tid; x < 2 * (S::kRow / 16); x += NT) {
+            const int c = x % (S::kRow / 16);
+            cp_async16(smem_addr(newrow + x * 16), reinterpret_cast<const unsigned char*>(x < S::kRow / 16 ? p.k_new : p.v_new) + (size_t)u * S::kRow + c * 16);
+        }
+    const uint32_t kmax_old = kBf16 ? __ldcg(p.kmax + u) : 0u;
     const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
     const int room = pt_u ? __ldcg(p.page_room + u) : 1;
     const int b = u / p.Hkv;
     const int t = __ldcg(p.base_tokens + b) + p.step + 1;
     const bool evict_on = min(p.w, __ldcg(p.base_obs + b) + p.step + 1) >= p.w;
-    if (p.early_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // every block has its length by now
+    if (p.early_trigger && !p.chain_wait) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the block has its length
     const int l = l_old + 1;
-    if (l > p.C || !room) mode = max(mode, 2);
+    if (l > p.C || !room) state |= kDcFull;
+    if (tid == NT - 1) misc->log_t = log((double)t);
     // the block's slots: whole words, shared out evenly
-    const int n_words = mode ? 0 : (l + 31) >> 5;
+    const int n_words = state ? 0 : (l + 31) >> 5;
     const int w0 = (int)((long long)n_words * rank / cs), w1 = (int)((long long)n_words * (rank + 1) / cs);
-    const int k_begin = w0 * 32, k_end = mode ? 0 : min(l, w1 * 32), n_keys = max(0, k_end - k_begin);
+    const int k_begin = w0 * 32, k_end = state ? 0 : min(l, w1 * 32), n_keys = max(0, k_end - k_begin);
     const int n_tiles = (n_keys + kDcKeys - 1) / kDcKeys;
     const int my_n = n_tiles > warp ? (n_tiles - warp + NW - 1) / NW : 0;       // tiles warp, warp + NW, ...
     const bool fits = n_keys * G <= dp.lcap;
     float* lg = fits ? reinterpret_cast<float*>(smem + lay.logits)
-                     : reinterpret_cast<float*>(p.stash) + ((size_t)u * p.C + k_begin) * G;
+                     : reinterpret_cast<float*>(p.stash + (size_t)u * G * p.C) + (size_t)k_begin * G;   // the unit's own scratch: launches overlap
     int my_page = 0;
     if (pt_u) {                                               // lane i keeps the page entry of the warp's tile i
         const int j = k_begin + (warp + lane * NW) * kDcKeys;
@@ -289,27 +341,15 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         for (int x = 0; x < S::kBoxes; ++x) tma_load_2d(dst + x * S::kBox, &map, x * (128 / Elem<T>::kBytes), row0, bar);
     };
 #pragma unroll
-    for (int it = 0; it < kKs; ++it)
+    for (int it = 0; it < (kKs > kVs ? kKs : kVs); ++it)
         if (it < my_n) {
             const int r0 = tile_row0(it);
-            if (lane == 0) { issue(kmap, r0, it); if (it < kVs) issue(vmap, r0, kKs + it); }
+            if (lane == 0) { if (it < kKs) issue(kmap, r0, it); if (it < kVs) issue(vmap, r0, kKs + it); }
         }
-    // queries and the appended rows (their latency is a bus round trip when the caller's buffers are host memory)
-    const bool new_here = !mode && l_old >= k_begin && l_old < k_end;
-    {
-        const unsigned char* qg = reinterpret_cast<const unsigned char*>(p.q) + (size_t)u * G * S::kRow;
-        if constexpr (kBf16) {
-            for (int x = tid; x < G * (S::kRow / 16); x += NT) cp_async16(smem_addr(smem + lay.q + x * 16), qg + x * 16);
-        } else {
-            double* qd = reinterpret_cast<double*>(smem + lay.q);
-            for (int x = tid; x < G * D; x += NT) qd[x] = (double)reinterpret_cast<const float*>(qg)[x];
-        }
-        if (new_here)
-            for (int x = tid; x < 2 * (S::kRow / 16); x += NT) {
-                const int c = x % (S::kRow / 16);
-                cp_async16(smem_addr(newrow + x * 16), reinterpret_cast<const unsigned char*>(x < S::kRow / 16 ? p.k_new : p.v_new) + (size_t)u * S::kRow + c * 16);
-            }
-        cp_async_wait_all();
+    cp_async_wait_all();
+    if (!kBf16) {
+        double* qd = reinterpret_cast<double*>(smem + lay.q);
+        for (int x = tid; x < G * D; x += NT) qd[x] = q_raw[x];
     }
     __syncthreads();
 
@@ -363,7 +403,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 1));
             m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 2));
             const bool ok = m16 < kSplitMaxBits;
-            if (!ok) misc->bad = 1;
+            if (!ok) state |= kDcBad;
             const float c = split_query_const(ok ? __uint_as_float(m16 << 16) : 1.f);
             float n1 = 0.f, n2 = 0.f, n3 = 0.f;
 #pragma unroll
@@ -408,7 +448,20 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         for (int cb = 0; cb < D / 16; ++cb)
 #pragma unroll
             for (int e = 0; e < 4; ++e) accd[cb][e] = 0.f;
-        uint32_t amax_w = 0u;
+        // The keys are cut on a grid of the unit's, kept in p.kmax: the largest magnitude it has ever held (scanning every
+        // tile for its own cost 96 instructions of 550 per tile and a chain of 32 dependent ones).
+        uint32_t kmax = kmax_old;
+        if (rank == cs - 1) {
+            uint32_t m = 0u;
+            if (lane < S::kRow / 16) {
+                const uint4 x = *reinterpret_cast<const uint4*>(newrow + lane * 16);
+                m = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(m, x.x), x.y), x.z), x.w);
+            }
+            kmax = max(kmax, __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16)));
+            if (tid == 0 && kmax > kmax_old && !state) p.kmax[u] = kmax;
+        }
+        if (kmax >= kSplitMaxBits) { state |= kDcBad; kmax = kSplitMaxBits; }
+        const SplitGrid g = split_grid(kmax);
         const int h0 = GP == 8 ? 2 * (lane & 3) : (lane & 3);                    // the thread's head(s)
         bool first = true;
         for (int it = 0; it < my_n; ++it) {
@@ -430,15 +483,6 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 const int r0 = tile_row0(it + kKs);
                 if (lane == 0) { fence_async_smem(); issue(kmap, r0, ks); }
             }
-            uint32_t mx = a[0][0];
-#pragma unroll
-            for (int kk = 0; kk < KK; ++kk)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) mx = max_mag_bf16x2(mx, a[kk][e]);
-            mx &= 0x7fff7fffu;
-            const uint32_t am = __reduce_max_sync(0xffffffffu, max(mx & 0xffffu, mx >> 16));
-            amax_w = max(amax_w, am);
-            const SplitGrid g = split_grid(min(am, kSplitMaxBits));
             // sums of the products of pieces; see the head of the file
             float x1[4] = {0.f, 0.f, 0.f, 0.f}, x2[4] = {0.f, 0.f, 0.f, 0.f}, x3[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
             float x4[4] = {0.f, 0.f, 0.f, 0.f};
@@ -460,7 +504,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                     mma16816(x2, k2, b1[kk][0], b1[kk][1]);
                     if constexpr (GP == 4) {
                         mma16816(x3, k1, b2[kk][0], b2[kk][1]);
-                        mma16816(x3, k2, b2[kk][0], b2[kk][1]);
+                        mma16816(x4, k2, b2[kk][0], b2[kk][1]);
                     }
                 }
 #pragma unroll
@@ -479,7 +523,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 } else {
                     // columns: (.q1, .q2) of the thread's head; two heads: the q3 products two lanes further on
                     float small = x2[2 * y + 1] + (lo[2 * y] + lo[2 * y + 1]);
-                    if constexpr (GP == 4) small += x3[2 * y];
+                    if constexpr (GP == 4) small += x3[2 * y] + x4[2 * y];
                     else small += __shfl_xor_sync(0xffffffffu, x1[2 * y] + (x2[2 * y] + lo[2 * y]), 2);
                     s[y][0] = (((double)x1[2 * y] + (double)(x1[2 * y + 1] + x2[2 * y])) + (double)small) * inv_root_d;
                 }
@@ -558,7 +602,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         for (int x = 0; x < NH; ++x) {
 #pragma unroll
             for (int o = 4; o < 32; o <<= 1) Zl[x] += __shfl_xor_sync(0xffffffffu, Zl[x], o);
-            if ((lane >> 2) == 0 && h0 + x < G) { misc->wM[warp][h0 + x] = (double)Mref[x]; misc->wZ[warp][h0 + x] = Zl[x]; }
+            if ((lane >> 2) == 0 && h0 + x < G) { misc->wM[warp][h0 + x] = Mref[x]; misc->wZ[warp][h0 + x] = Zl[x]; }
         }
 #pragma unroll
         for (int cb = 0; cb < D / 16; ++cb) {
@@ -572,10 +616,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][2] + accd[cb][3];
             }
         }
-        if (lane == 0) {
-            if (amax_w >= kSplitMaxBits) misc->bad = 1;
-            atomicMax(&misc->amax, amax_w);
-        }
+        state = (state & ~0xffffu) | kmax;
     } else {
         const double* qd = reinterpret_cast<const double*>(smem + lay.q);
         float* pr = reinterpret_cast<float*>(prob);           // [key][GP]
@@ -676,201 +717,158 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
 #pragma unroll
         for (int x = 0; x < GP; ++x) {
             Zl[x] = warp_sum(Zl[x]);
-            if (lane == 0) { misc->wM[warp][x] = (double)Mref[x]; misc->wZ[warp][x] = Zl[x]; }
+            if (lane == 0) { misc->wM[warp][x] = Mref[x]; misc->wZ[warp][x] = Zl[x]; }
 #pragma unroll
             for (int e = 0; e < NC; ++e) rec[x * D + lane * NC + e] = acc[x][e];
         }
         if (warp == 0 && lane < GP) misc->qe[lane] = 0.f;
     }
-    if (failed) mode = max(mode, 1);
-    if (mode) { if (mode == 1) report_status(p.status, CORM_ERR_TIMEOUT); misc->mode = mode; }
+    if (failed) state |= kDcExpired;
+    state = __reduce_or_sync(0xffffffffu, state);             // the magnitude is the same in every lane
+    if (lane == 0) {
+        if (state & kDcExpired) report_status(p.status, CORM_ERR_TIMEOUT);
+        atomicMax(&misc->state, state);
+    }
     // the next launch may become resident while this one judges and compacts (it waits for this one to complete)
     if (!p.early_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __syncthreads();
-
-    // the block's record: warps merged, in place of the first warp's
-    if (tid < 8 * NW) {
-        const int h = tid / NW, w = tid % NW;
-        const double m = h < G ? misc->wM[w][h] : -INFINITY, z = h < G ? misc->wZ[w][h] : 0.0;
-        double mb = m;
-#pragma unroll
-        for (int o = 1; o < NW; o <<= 1) mb = fmax(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-        const double sc = m == -INFINITY ? 0.0 : exp_nonpos(m - mb);
-        double zb = z * sc;
-#pragma unroll
-        for (int o = 1; o < NW; o <<= 1) zb += __shfl_xor_sync(0xffffffffu, zb, o);
-        misc->wsc[w][h] = (float)sc;
-        if (w == 0) { misc->M[h] = mb; misc->Z[h] = zb; }
-    }
-    __syncthreads();
-    float* blk_rec = reinterpret_cast<float*>(smem);
-    for (int x = tid; x < G * D; x += NT) {
-        const int h = x / D;
-        float acc = 0.f;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const float sc = misc->wsc[w][h];
-            acc += sc != 0.f ? reinterpret_cast<const float*>(smem + w * S::kWarpRing)[x] * sc : 0.f;
-        }
-        blk_rec[x] = acc;
-    }
     // registers and positions of the first slots this thread judges are requested before the blocks meet
-    constexpr int kB = 4;                                     // slots per thread and batch
+    constexpr int kB = GP == 8 ? 4 : 8;                       // slots per thread and batch
     uint32_t wv[kB];
     int32_t pv[kB];
+    float sv[kB][GP];
     auto load_regs = [&](int base) {
 #pragma unroll
         for (int k = 0; k < kB; ++k) {
-            const int j = k_begin + base + k * NT + tid;
+            const int i = base + k * NT + tid, j = k_begin + i;
             wv[k] = 0u; pv[k] = t;                            // the token appended by this step
             if (j < k_end && j < l_old) { wv[k] = __ldcg(wordu + j); pv[k] = __ldcg(posu + j); }
+#pragma unroll
+            for (int h = 0; h < GP; ++h)
+                sv[k][h] = i < n_keys && h < G ? (fits ? lg[i * G + h] : __ldcg(lg + (size_t)i * G + h)) : 0.f;
         }
     };
+    __syncthreads();                                          // the appended slot's row, word and position are stored
     load_regs(0);
-    cluster_sync();                                           // records are complete (the block's logits, too)
+    cluster_sync();                                           // every warp's record is complete (and the block's logits)
 
-    // ---- thresholds of Definition 3.1 in log form, the same in every block ----
-    if (tid < 64) {
-        const int h = tid >> 3, x = tid & 7;
-        const bool on = h < G && x < cs;
-        const double m = on ? ld_peer_f64(map_rank(smem_addr(&misc->M[h]), x)) : -INFINITY;
-        const double z = on ? ld_peer_f64(map_rank(smem_addr(&misc->Z[h]), x)) : 0.0;
-        double M = m;
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
-        const double sc = m == -INFINITY ? 0.0 : exp_nonpos(m - M);
-        double Z = z * sc;
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
-        misc->sc[h][x] = (float)sc;
-        if (x == 0) {
-            const double thr = M + log(Z) + p.log_alpha - log((double)t);
-            misc->thr[h] = thr; misc->Zt[h] = Z; misc->thr_f[h] = (float)thr;
-        }
-    } else if (tid < 96) {
-        const int x = lane;
-        const int md = x < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->mode), x)) : 0;
-        const int bd = x < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->bad), x)) : 0;
-        const uint32_t am = x < cs ? ld_peer_u32(map_rank(smem_addr(&misc->amax), x)) : 0u;
-        const int any_m = __reduce_max_sync(0xffffffffu, md), any_b = __reduce_max_sync(0xffffffffu, bd);
-        const uint32_t any_a = __reduce_max_sync(0xffffffffu, am);
-        if (lane == 0) { misc->any_mode = any_m; misc->any_bad = any_b; misc->unit_amax = any_a; }
-    }
-    __syncthreads();
-    if (misc->any_mode) {                                     // an expired wait, or a unit that cannot take the token: it is left as it is
+    // ---- thresholds of Definition 3.1 in log form, the same in every block: warp h reduces head h over the cluster's warps ----
+    const uint32_t unit_state = __reduce_max_sync(0xffffffffu, lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->state), lane)) : 0u);
+    if (unit_state & (kDcExpired | kDcFull)) {                // the unit is left as it is
         cluster_sync();
         if (rank == 0 && tid == 0) {
-            if (misc->any_mode == 2) report_status(p.status, CORM_ERR_CAPACITY);
+            const bool full = !(unit_state & kDcExpired) || l > p.C || !room;
+            if (full) report_status(p.status, CORM_ERR_CAPACITY);
             p.live_out[u] = l_old;
-            if (misc->any_mode == 2) publish_unit_stamp(p, u, l_old);
+            if (full) publish_unit_stamp(p, u, l_old);
             publish_live(p.maxlive, p.step + 1, l_old);
         }
         return;
     }
-    // error of a head's log-sum-exp (every logit of it is off by at most this much)
-    const float eps_a = kBf16 ? split_amax(min(misc->unit_amax, kSplitMaxBits)) * (float)inv_root_d * 1.0001f : 0.f;
-    if (tid < G) {
-        const float th = fabsf(misc->thr_f[tid]);
-        misc->slack[tid] = 2.f * eps_a * misc->qe[tid] + (th < 3e38f ? th : 0.f) * 1.3e-7f + 1e-12f;
+    // error of a head's log-sum-exp per unit of qe (every logit of it is off by at most this much)
+    const float eps_a = kBf16 ? split_amax(min(unit_state & 0xffffu, kSplitMaxBits)) * (float)inv_root_d * 1.0001f : 0.f;
+    for (int h = warp; h < G; h += NW) {
+        constexpr int kEnt = kDcMaxCluster * NW / 32;         // (block, warp) entries per lane
+        float m[kEnt], M = -INFINITY;
+        double z[kEnt], Z = 0.0;
+#pragma unroll
+        for (int y = 0; y < kEnt; ++y) {
+            const int e = y * 32 + lane, blk = e / NW, w = e % NW;
+            m[y] = blk < cs ? __uint_as_float(ld_peer_u32(map_rank(smem_addr(&misc->wM[w][h]), blk))) : -INFINITY;
+            z[y] = blk < cs ? ld_peer_f64(map_rank(smem_addr(&misc->wZ[w][h]), blk)) : 0.0;
+        }
+#pragma unroll
+        for (int y = 0; y < kEnt; ++y) M = fmaxf(M, m[y]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+#pragma unroll
+        for (int y = 0; y < kEnt; ++y) {
+            const double sc = m[y] == -INFINITY ? 0.0 : exp_nonpos((double)m[y] - (double)M);
+            Z = fma(z[y], sc, Z);
+            misc->sc[h][y * 32 + lane] = (float)sc;
+        }
+        Z = warp_sum(Z);                                      // a fixed tree: every block gets the same bits
+        if (lane == 0) {
+            const double thr = (double)M + log(Z) + p.log_alpha - misc->log_t;
+            const float tf = (float)thr, ta = fabsf(tf);
+            misc->thr[h] = thr; misc->Zt[h] = Z; misc->thr_f[h] = tf;
+            misc->slack[h] = 2.f * eps_a * misc->qe[h] + (ta < 3e38f ? ta : 0.f) * 1.3e-7f + 1e-12f;
+        }
     }
     __syncthreads();
 
     // ---- 2. verdicts, register update, keep bits ----
     uint32_t* keep = reinterpret_cast<uint32_t*>(smem + 8192);                  // the ring is free behind the block's record
-    int* prefix = reinterpret_cast<int*>(smem + 8192) + kDcMaxWords;
     {
+        // first the block's record of the outputs' numerators (Eq. 1): its warps' merged, in place of the first warp's
+        for (int x = tid; x < G * D; x += NT) {
+            const int h = x / D;
+            float acc = 0.f;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                const float sc = misc->sc[h][rank * NW + w];
+                acc += sc != 0.f ? reinterpret_cast<const float*>(smem + w * S::kWarpRing)[x] * sc : 0.f;
+            }
+            reinterpret_cast<float*>(smem)[x] = acc;
+        }
+        __syncthreads();                                      // the other warps' records give way to the keep bits
         int n_imp = 0, n_keep = 0;
+#pragma unroll 1
         for (int base0 = 0; base0 < n_keys; base0 += kB * NT) {
             if (base0) load_regs(base0);
+            uint32_t imp = 0u, open[kB];
 #pragma unroll
             for (int k = 0; k < kB; ++k) {
-                const int base = base0 + k * NT;
-                if (base >= n_keys) break;                    // uniform
-                const int i = base + tid, j = k_begin + i;
-                const bool on = i < n_keys;
-                bool imp = false;
-                uint32_t open = 0u;
+                const int i = base0 + k * NT + tid;
+                open[k] = 0u;
+                if (i >= n_keys) continue;
 #pragma unroll
                 for (int h = 0; h < GP; ++h) {
-                    if (h >= G || !on) continue;
-                    const float sf = fits ? lg[i * G + h] : __ldcg(lg + (size_t)i * G + h), margin = sf - misc->thr_f[h];
+                    if (h >= G) continue;
+                    const float sf = sv[k][h], margin = sf - misc->thr_f[h];
                     const float err = fabsf(sf) * 6.1e-8f + misc->slack[h];
-                    if (margin >= err) imp = true;
-                    else if (margin > -err) open |= 1u << h;
+                    if (margin >= err) imp |= 1u << k;
+                    else if (margin > -err) open[k] |= 1u << h;
                 }
-                uint32_t who = __ballot_sync(0xffffffffu, open != 0u && !imp);
-                while (who) {                                 // formed again in fp64, one slot after the other, by the whole warp
-                    const int src = __ffs(who) - 1;
-                    who &= who - 1u;
-                    const int js = __shfl_sync(0xffffffffu, j, src);
-                    uint32_t os = __shfl_sync(0xffffffffu, open, src);
-                    const size_t row = kv_row(pt_u, (size_t)u * p.C, js, p.pool_pages, p.status);
-                    bool yes = false;
-                    int n_near = 0;
-                    while (os) {
-                        const int h = __ffs(os) - 1;
-                        os &= os - 1u;
-                        const double s = warp_exact_dot_cg<T, D>(reinterpret_cast<const T*>(p.q) + ((size_t)u * G + h) * D,
-                                                                 reinterpret_cast<const T*>(p.K) + row * D, lane) * inv_root_d;
-                        const double th = misc->thr[h], e = (double)(eps_a * misc->qe[h]) + 1e-13 * (1.0 + fabs(th));
-                        yes |= s - th > e;
-                        if (lane == 0 && fabs(s - th) <= e) atomicOr(&misc->flags, 1u << h);   // left to the exact heads
-                        ++n_near;
-                    }
-                    if (lane == 0) atomicAdd(p.counters + CNT_NEAR, (unsigned long long)n_near);
-                    if (lane == src) imp = yes;
+                if ((imp >> k) & 1u) open[k] = 0u;
+            }
+            uint32_t any_open = 0u;
+#pragma unroll
+            for (int k = 0; k < kB; ++k) any_open |= open[k];
+            if (__any_sync(0xffffffffu, any_open != 0u)) {    // rare
+#pragma unroll 1
+                for (int k = 0; k < kB; ++k) {
+                    uint32_t ok = 0u;
+#pragma unroll
+                    for (int x = 0; x < kB; ++x) ok = x == k ? open[x] : ok;
+                    if (dc_open_verdicts<T, D, NW>(p, u, G, k_begin + base0 + k * NT + tid, ok, eps_a, misc)) imp |= 1u << k;
                 }
+            }
+#pragma unroll
+            for (int k = 0; k < kB; ++k) {
+                const int base = base0 + k * NT, i = base + tid;
+                if (base + warp * 32 >= n_keys) break;        // uniform in the warp
+                const bool on = i < n_keys, im = (imp >> k) & 1u;
                 bool kp = false;
                 if (on) {
-                    const uint32_t wd = update_register(wv[k], imp, p.w, t);
-                    if (CORM_IN_RANGE(j < p.C, p.status)) wordu[j] = wd;
+                    const uint32_t wd = update_register(wv[k], im, p.w, t);
+                    if (CORM_IN_RANGE(k_begin + i < p.C, p.status)) wordu[k_begin + i] = wd;
                     kp = !evict_on || register_needed(wd, p.w, t) || pv[k] > t - p.r;
                 }
                 const uint32_t ballot = __ballot_sync(0xffffffffu, kp);
-                n_imp += __popc(__ballot_sync(0xffffffffu, imp));
+                n_imp += __popc(__ballot_sync(0xffffffffu, im));
                 n_keep += __popc(ballot);
-                if (lane == 0 && base + warp * 32 < n_keys && CORM_IN_RANGE((base >> 5) + warp < kDcMaxWords, p.status))
-                    keep[(base >> 5) + warp] = ballot;
+                if (lane == 0 && CORM_IN_RANGE((base >> 5) + warp < kDcMaxWords, p.status)) keep[(base >> 5) + warp] = ballot;
             }
         }
-        if (lane == 0) { misc->warp_cnt[warp] = n_keep; misc->warp_imp[warp] = n_imp; }
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int c = 0, m = 0;
-#pragma unroll
-        for (int x = 0; x < NW; ++x) { c += misc->warp_cnt[x]; m += misc->warp_imp[x]; }
-        misc->count = c; misc->n_imp = m;
-        if (misc->any_bad) misc->flags = (1u << G) - 1u;      // magnitudes beyond the pieces' range: every head exactly
-    }
-    __syncthreads();
-    cluster_arrive();
-    // outputs (Eq. 1): the unit's G x D values are shared out over the blocks, two channels per thread
-    {
-        const int np = G * D / 2, x0 = np * rank / cs, x1 = np * (rank + 1) / cs;
-        for (int x = x0 + tid; x < x1; x += NT) {
-            const int h = x / (D / 2);
-            float a0 = 0.f, a1 = 0.f;
-            const uint32_t at = smem_addr(blk_rec + 2 * x);
-            float v[kDcMaxCluster][2];
-#pragma unroll
-            for (int y = 0; y < kDcMaxCluster; ++y)
-                if (y < cs) {
-                    const double d = ld_peer_f64(map_rank(at, y));
-                    v[y][0] = __uint_as_float((uint32_t)__double2loint(d)); v[y][1] = __uint_as_float((uint32_t)__double2hiint(d));
-                }
-#pragma unroll
-            for (int y = 0; y < kDcMaxCluster; ++y)
-                if (y < cs) { const float sc = misc->sc[h][y]; a0 = fmaf(v[y][0], sc, a0); a1 = fmaf(v[y][1], sc, a1); }
-            const float o0 = (float)((double)a0 / misc->Zt[h]), o1 = (float)((double)a1 / misc->Zt[h]);
-            if constexpr (kBf16) reinterpret_cast<uint32_t*>(p.out)[(size_t)u * np + x] = (uint32_t)float_to_bf16_bits(o0) | ((uint32_t)float_to_bf16_bits(o1) << 16);
-            else reinterpret_cast<float2*>(p.out)[(size_t)u * np + x] = make_float2(o0, o1);
+        if (lane == 0) {
+            atomicAdd(&misc->count, n_keep);
+            atomicAdd(&misc->n_imp, n_imp);
+            if (unit_state & kDcBad) atomicOr(&misc->flags, (1u << G) - 1u);    // magnitudes beyond the pieces' range: every head exactly
         }
     }
-    cluster_wait();
+    cluster_sync();
     {
-        uint32_t marks = lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->flags), lane)) : 0u;
-        marks = __reduce_or_sync(0xffffffffu, marks);
+        const uint32_t marks = __reduce_or_sync(0xffffffffu, lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->flags), lane)) : 0u);
         if (marks) {                                          // uniform in the cluster
             cluster_sync();
             dc_exact_heads<T, D, NW>(p, u, G, t, k_begin, k_end, marks, keep, misc, cs);
@@ -878,6 +876,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         }
     }
     // ---- 3. compaction: kept slots at or above the new length move into the holes below it ----
+    // Hole number = evicted slots before it, mover number = kept slots behind it, so both follow from the blocks' counts.
     int before = 0, total = 0, imp_total = 0;
     {
         const int c = lane < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->count), lane)) : 0;
@@ -886,47 +885,119 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         if (rank == 0) imp_total = __reduce_add_sync(0xffffffffu, lane < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->n_imp), lane)) : 0);
     }
     const int new_len = evict_on ? total : l;
-    int n_moved = 0;
-    if (new_len < l) {
-        // Lists in scratch: hole number = evicted slots before it; mover number = kept slots behind it, so that both follow
-        // from the counts of the blocks before.
-        int* holes = reinterpret_cast<int*>(p.stash) + (size_t)p.U * p.C * G + (size_t)u * p.C;
-        int* movers = holes + p.C / 2;
+    auto row_of = [&](int slot) -> size_t {
+        return pt_u ? page_row(__ldcg(pt_u + (slot >> 5)), slot, p.pool_pages, p.status) : (size_t)u * p.C + (size_t)slot;
+    };
+    int* holes = reinterpret_cast<int*>(smem + 8192) + kDcMaxWords;             // [kDcListCap] each, behind the keep bits
+    int* movers = holes + kDcListCap;
+    auto hole_words = [&](int i, uint32_t& m, uint32_t& hm) {                   // word i of the block: kept slots, holes
+        m = keep[i];
+        const int s0 = k_begin + i * 32;
+        const uint32_t valid = k_end - s0 >= 32 ? 0xffffffffu : (1u << (k_end - s0)) - 1u;
+        const uint32_t below = new_len - s0 >= 32 ? 0xffffffffu : (new_len > s0 ? (1u << (new_len - s0)) - 1u : 0u);
+        hm = ~m & valid & below;
+        m &= ~below;                                          // kept slots at or above the new length
+    };
+    if (new_len < l && l - new_len <= kDcListCap) {
+        // The usual step: every block fills its own holes; the last words of the unit, where the movers are, are read from
+        // the blocks that own them. Warp 0 lists the block's holes, warp 1 the movers that go there.
+        const int nw = (n_keys + 31) >> 5, k_lo = max(0, k_begin - before);     // number of the block's first hole
+        if (warp == 0) {
+            int base = 0;
+            for (int i0 = 0; i0 < nw && k_begin + i0 * 32 < new_len; i0 += 32) {
+                uint32_t m = 0u, hm = 0u;
+                if (i0 + lane < nw) hole_words(i0 + lane, m, hm);
+                int at = __popc(hm);
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xffffffffu, at, o); if (lane >= o) at += up; }
+                const int all = __shfl_sync(0xffffffffu, at, 31);
+                at += base - __popc(hm);
+                base += all;
+                for (; hm; hm &= hm - 1u) holes[at++] = k_begin + (i0 + lane) * 32 + __ffs(hm) - 1;
+            }
+        } else if (warp == 1) {
+            const int first_w = new_len >> 5;                 // the unit's words that hold movers: [first_w, n_words), from the end
+            const int k_hi = k_begin < new_len ? k_lo + n_keys - misc->count : k_lo;
+            int base = 0;
+            for (int i0 = 0; n_words - 1 - i0 >= first_w; i0 += 32) {
+                const int wd = n_words - 1 - i0 - lane;
+                uint32_t km = 0u;
+                if (wd >= first_w) {
+                    int o = 0;                                // the block that owns the word
+                    while (o + 1 < cs && (int)((long long)n_words * (o + 1) / cs) <= wd) ++o;
+                    km = ld_peer_u32(map_rank(smem_addr(keep + (wd - (int)((long long)n_words * o / cs))), o));
+                    if (wd == first_w) km &= ~((1u << (new_len & 31)) - 1u);
+                }
+                int at = __popc(km);
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xffffffffu, at, o); if (lane >= o) at += up; }
+                const int all = __shfl_sync(0xffffffffu, at, 31);
+                at += base - __popc(km);
+                base += all;
+                while (km) {                                  // from the last slot down
+                    const int bit = 31 - __clz(km);
+                    km &= ~(1u << bit);
+                    if (at >= k_lo && at < k_hi) movers[at - k_lo] = wd * 32 + bit;
+                    ++at;
+                }
+            }
+            if (lane == 0) misc->n_moved = base;
+        }
+        __syncthreads();
+        const int n_moved = misc->n_moved;
+        const int mine = k_begin < new_len ? min(n_moved, k_lo + n_keys - misc->count) - k_lo : 0;
+        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, movers, holes, mine, 0, 1, l, p.status);
+    } else if (new_len < l) {
+        // many: the lists go to scratch and the moves are shared out evenly
+        int* gholes = reinterpret_cast<int*>(p.stash + (size_t)u * G * p.C) + (size_t)G * p.C;   // behind the unit's logits
+        int* gmovers = gholes + p.C / 2;
+        int* prefix = holes;                                  // [kDcMaxWords + 1]
         const int nw = (n_keys + 31) >> 5;
         block_popc_scan<NT>(keep, prefix, nw, misc->scan);
         for (int i = tid; i < nw; i += NT) {
+            uint32_t km, hm;
+            hole_words(i, km, hm);
             const uint32_t m = keep[i];
             const int s0 = k_begin + i * 32, kb = before + prefix[i];            // kept slots before this word
-            const uint32_t valid = k_end - s0 >= 32 ? 0xffffffffu : (1u << (k_end - s0)) - 1u;
-            const uint32_t below = new_len - s0 >= 32 ? 0xffffffffu : (new_len > s0 ? (1u << (new_len - s0)) - 1u : 0u);
-            uint32_t hm = ~m & valid & below;                 // evicted slots below the new length
-            while (hm) {
-                const int bit = __ffs(hm) - 1;
-                hm &= hm - 1u;
-                const int x = s0 + bit - kb - __popc(m & ((1u << bit) - 1u));
-                if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) holes[x] = s0 + bit;
-            }
-            uint32_t km = m & valid & ~below;                 // kept slots at or above it
-            while (km) {
-                const int bit = __ffs(km) - 1;
-                km &= km - 1u;
-                const int x = total - 1 - kb - __popc(m & ((1u << bit) - 1u));
-                if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) movers[x] = s0 + bit;
-            }
             if (new_len >= s0 && new_len < s0 + 32 && new_len < k_end)           // how many: evicted slots below the new length
-                p.unit_rec[u] = make_int2(new_len - kb - __popc(m & below), 0);
+                p.unit_rec[u] = make_int2(new_len - kb - __popc(m & ~km), 0);
+            for (; hm; hm &= hm - 1u) {
+                const int bit = __ffs(hm) - 1, x = s0 + bit - kb - __popc(m & ((1u << bit) - 1u));
+                if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) gholes[x] = s0 + bit;
+            }
+            for (; km; km &= km - 1u) {
+                const int bit = __ffs(km) - 1, x = total - 1 - kb - __popc(m & ((1u << bit) - 1u));
+                if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) gmovers[x] = s0 + bit;
+            }
         }
         cluster_sync();
-        n_moved = __ldcg(&p.unit_rec[u].x);
-        const size_t slab_row0 = (size_t)u * p.C;
-        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V),
-                                  [&](int slot) -> size_t {
-                                      return pt_u ? page_row(__ldcg(pt_u + (slot >> 5)), slot, p.pool_pages, p.status) : slab_row0 + (size_t)slot;
-                                  }, wordu, posu, movers, holes, n_moved, rank, cs, l, p.status);
+        if (tid == 0) misc->n_moved = __ldcg(&p.unit_rec[u].x);
+        __syncthreads();
+        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, gmovers, gholes, misc->n_moved, rank, cs, l, p.status);
+    }
+    // outputs (Eq. 1): the unit's G x D values are shared out over the blocks, two channels per thread
+    {
+        const int np = G * D / 2, x0 = np * rank / cs, x1 = np * (rank + 1) / cs;
+        for (int x = x0 + tid; x < x1; x += NT) {
+            const uint32_t at = smem_addr(smem) + x * 8;
+            double v[kDcMaxCluster];
+#pragma unroll
+            for (int y = 0; y < kDcMaxCluster; ++y) v[y] = y < cs ? ld_peer_f64(map_rank(at, y)) : 0.0;
+            float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+            for (int y = 0; y < kDcMaxCluster; ++y) {
+                a0 += __uint_as_float((uint32_t)__double2loint(v[y]));
+                a1 += __uint_as_float((uint32_t)__double2hiint(v[y]));
+            }
+            const double Z = misc->Zt[x / (D / 2)];
+            const float o0 = (float)((double)a0 / Z), o1 = (float)((double)a1 / Z);
+            if constexpr (kBf16) reinterpret_cast<uint32_t*>(p.out)[(size_t)u * np + x] = (uint32_t)float_to_bf16_bits(o0) | ((uint32_t)float_to_bf16_bits(o1) << 16);
+            else reinterpret_cast<float2*>(p.out)[(size_t)u * np + x] = make_float2(o0, o1);
+        }
     }
     // every block's row moves come before released pages and the stamp; and a block's shared memory stays until its peers
     // have read it
-    if (new_len == l || pt_u || p.unit_stamp) cluster_sync();
+    cluster_sync();
     if (rank != 0) return;
     if (pt_u) settle_pages<NT>(p.page_table, p.page_bits, p.page_room, p.pool_pages, p.pt_stride, p.U, u, l_old, new_len);
     if (pt_u && p.unit_stamp) __syncthreads();
@@ -938,7 +1009,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         atomicAdd(p.counters + CNT_ATTENDED, (unsigned long long)l);
         if (imp_total) atomicAdd(p.counters + CNT_IMPORTANT, (unsigned long long)imp_total);
         if (new_len < l) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(l - new_len));
-        if (n_moved) atomicAdd(p.counters + CNT_MOVED, (unsigned long long)n_moved);
+        if (new_len < l && misc->n_moved) atomicAdd(p.counters + CNT_MOVED, (unsigned long long)misc->n_moved);
     }
 }
 
@@ -948,31 +1019,36 @@ inline corm_status_t make_row_tensor_map(CUtensorMap* out, void* base, unsigned 
     typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || !fn ||
-        q != cudaDriverEntryPointSuccess) {
-        (void)cudaGetLastError();
-        return CORM_ERR_UNSUPPORTED;
-    }
+    static const EncodeFn encode = [] {                       // looked up once per process
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+            (void)cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<EncodeFn>(fn);
+    }();
+    if (!encode) return CORM_ERR_UNSUPPORTED;
     const int e = bf16 ? 2 : 4;
     const cuuint64_t dims[2] = {(cuuint64_t)D, rows};
     const cuuint64_t strides[1] = {(cuuint64_t)(D * e)};
     const cuuint32_t box[2] = {(cuuint32_t)(128 / e), kDcKeys};
     const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = reinterpret_cast<EncodeFn>(fn)(
+    const CUresult r = encode(
         out, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? CORM_OK : CORM_ERR_CUDA;
 }
 
-constexpr int kDcWarps = 4;
+// Warps per block: eight where rows are short (units of a few hundred keys get more warps from eight blocks), four for
+// fp32, whose tiles are twice as large (20 units x 250 keys 23 -> 15 us per step).
+template <typename T> constexpr int dc_warps() { return Elem<T>::kBytes == 4 ? 4 : 8; }
 
 template <typename T, int D, int GP>
 inline corm_status_t launch_decode_cluster_as(DecodeClusterParams& dp, const CUtensorMap& kmap, const CUtensorMap& vmap, int upper,
                                               int tune_split_len, int sm_count, cudaStream_t st) {
-    constexpr int NW = kDcWarps;
+    constexpr int NW = dc_warps<T>();
     const DecodeParams& p = dp.p;
     const int sms = sm_count > 0 ? sm_count : 148;
     constexpr int kBlocks = dc_blocks<T, D, GP, NW>();

@@ -60,6 +60,7 @@ struct DecodeParams {
     double* stash;            // [U*G][C] scaled logits of this step (scratch)
     unsigned char* partials;  // [U][max_splits][G] records {double m, double Z, float acc[D]} (scratch)
     uint32_t* keepmask;       // [U][ceil(C/32)+2] keep bits of the verdict launch (scratch)
+    uint32_t* kmax;           // [U] bf16 caches: bits of the largest key magnitude the unit has held since its prompt pass
     int2* unit_rec;           // [U] balanced kernel -> verdict launch: a unit's first record and its record count (scratch)
     unsigned long long* unit_stamp;  // [U] (decode steps the unit has finished << 32 | its live length after the last of them),
                                      // written by the block that finishes a unit inside the streaming launch; null = not kept
@@ -95,6 +96,7 @@ struct PromptParams {
     unsigned long long* maxlive;
     double* stash;            // scratch, reused for temporary registers
     uint32_t* keepmask;       // [U][ceil(C/32)+2] keep bits (scratch)
+    uint32_t* kmax;           // [U] as in DecodeParams
     int32_t U, Hkv, C, p_max, w, r;
     double log_alpha;
     double bound_scale;       // multiplies the proven error bounds of the bf16 pass (1; tests raise it)
@@ -188,6 +190,17 @@ __device__ __forceinline__ double warp_sum(double x) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
+}
+
+// words of two bf16 -> the larger magnitude of each half, as bits
+__device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t m, uint32_t x) { return __vmaxu2(m, x & 0x7fff7fffu); }
+
+// A row appended to a bf16 cache enters the unit's largest magnitude. x: 16 bytes of the row per lane (zero in lanes
+// without any); the whole warp calls.
+__device__ __forceinline__ void note_key_magnitude(uint32_t* kmax_u, uint4 x) {
+    const uint32_t m = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(0u, x.x), x.y), x.z), x.w);
+    const uint32_t all = __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16));
+    if ((threadIdx.x & 31) == 0) atomicMax(kmax_u, all);
 }
 
 // Publishes a unit's new live length for the host's launch sizing: the word holds the latest step in its high half,

@@ -313,6 +313,7 @@ __global__ void __launch_bounds__(kFastThreads, fast_blocks_per_sm(G)) decode_fa
     int l_old;
     if (p.chain_wait) {
         __shared__ unsigned long long s_stamp;
+        if (p.early_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         if (tid == 0) s_stamp = wait_unit_stamp(p.unit_stamp + u, (uint32_t)p.step, p.status);
         __syncthreads();
         const unsigned long long sw = s_stamp;
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(kFastThreads, fast_blocks_per_sm(G)) decode_fa
     // From here on the next launch may become resident (a chained one: its blocks wait for their units' stamps). Not
     // earlier: an unchained block takes its unit's length from the double-buffered array, whose other half the next
     // step rewrites, so every block has its length (the branch above depends on it) before a block of the next step runs.
-    if (p.early_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (p.early_trigger && !p.chain_wait) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool single = (n_act == 1 && l <= p.single_cap);
     const int t = __ldg(p.base_tokens + b) + p.step + 1;
     const int begin = split * p.split_len, end = min(l, begin + p.split_len);
@@ -461,6 +462,7 @@ __global__ void __launch_bounds__(kFastThreads, fast_blocks_per_sm(G)) decode_fa
         if (has_new) {   // append: the new row goes to the slab and replaces whatever the copy fetched for that slot
             cp_async_wait_all();
             __syncwarp();
+            note_key_magnitude(p.kmax + u, lane < 16 ? *reinterpret_cast<const uint4*>(newrow + lane * 16) : make_uint4(0, 0, 0, 0));
             if (lane < 16) {
                 const uint4 x = *reinterpret_cast<const uint4*>(newrow + lane * 16);
                 *reinterpret_cast<uint4*>(ktile + (l_old - k0) * kRowBytes + lane * 16) = x;

@@ -45,6 +45,8 @@ __global__ void __launch_bounds__(kGenericThreads) decode_generic_kernel(const _
         const T* vn = reinterpret_cast<const T*>(p.v_new) + (size_t)u * D;
         const size_t row = kv_row(pt_u, slab_row0, l_old, p.pool_pages, p.status);
         for (int c = tid; c < D; c += NT) { Kl[row * D + c] = kn[c]; Vl[row * D + c] = vn[c]; }
+        if (Elem<T>::kBytes == 2 && warp == 0)
+            note_key_magnitude(p.kmax + u, lane < D / 8 ? reinterpret_cast<const uint4*>(kn)[lane % (D / 8)] : make_uint4(0, 0, 0, 0));
         if (tid == 0) { p.word[(size_t)u * p.C + l_old] = 0u; p.pos[(size_t)u * p.C + l_old] = t; }
         __syncthreads();
     }

@@ -89,16 +89,6 @@ __device__ __forceinline__ float split_error(float n1, float n2, float n3) {
     return 7.62939453125e-6f * (n2 * (1.f / 64.f) + n1 * (1.f / 8192.f) + n3) * 1.2f + n3 * (1.f / 60.f);
 }
 
-// words of two bf16 -> the larger magnitude of each half, as bits
-__device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t m, uint32_t x) { return __vmaxu2(m, x & 0x7fff7fffu); }
-
-// running maximum of magnitudes, two at a time (signs of the result are meaningless), NaN stays
-__device__ __forceinline__ uint32_t max_mag_bf16x2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("max.NaN.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-
 // ---- clusters ----
 __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ uint32_t cluster_size() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }

@@ -27,7 +27,7 @@
 // out); for wide windows the tensor pipe's mma.sync rate in phase A (R P d multiply-adds, seven times).
 // Measured against the two-launch pass this replaces (fp64 logits on the CUDA cores; one block per unit gathering) and,
 // for fp32 or 64 channels, a pass with one block per unit; us, w = queries in the window, G = heads per group:
-//   1024 units x 3250 keys, G 1, w 8    1597 -> 1387      128 units x 3390 keys, G 1, w 256    5341 -> 1735
+//   1024 units x 3250 keys, G 1, w 8    1597 -> 1033      128 units x 3390 keys, G 1, w 256    5341 -> 1735
 //   128 units x 8192 keys, G 4, w 8     1821 ->  785      32 units x 8192 keys, G 4, w 128     6736 -> 2235
 //   32 units x 32768 keys, G 4, w 16    4618 -> 2363      32 units x 4096 keys, G 1, w 8        259 ->   77
 //   fp32: 20 units x 1300 keys, G 2     2787 ->  111      64 channels: 128 units x 2000, G 4  11037 ->  287
@@ -686,6 +686,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         }
     }
     if (rank == 0 && tid == 0) {
+        if (kBf16) p.kmax[u] = amax_unit;
         p.live_out[u] = kept_total;
         publish_live(p.maxlive, 0, kept_total);
         atomicAdd(p.counters + CNT_APPENDED, (unsigned long long)P);
@@ -704,7 +705,7 @@ struct PromptBeginParams {
     int32_t first, n, w;                                  // sequences [first, first + n)
     int32_t* base_tokens;
     int32_t* base_obs;
-    struct Span { uint32_t* ptr; unsigned long long words; } clear[8];    // 32-bit words to zero
+    struct Span { uint32_t* ptr; unsigned long long words; } clear[9];    // 32-bit words to zero
 };
 __global__ void __launch_bounds__(kPbThreads) prompt_begin_kernel(const __grid_constant__ PromptBeginParams p) {
     const unsigned long long at = (unsigned long long)blockIdx.x * kPbThreads + threadIdx.x, step = (unsigned long long)gridDim.x * kPbThreads;
@@ -713,7 +714,7 @@ __global__ void __launch_bounds__(kPbThreads) prompt_begin_kernel(const __grid_c
         p.base_obs[p.first + at] = min(p.lens[at], p.w);
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 9; ++i)
         for (unsigned long long x = at; x < p.clear[i].words; x += step) p.clear[i].ptr[x] = 0u;
 }
 
@@ -741,10 +742,12 @@ inline corm_status_t launch_prompt_cluster(const PromptParams& p, int G, int max
     while ((1 << pp.log2g) < G) ++pp.log2g;
     pp.rows8 = (p.w * G + 7) / 8 * 8;
     const int n_words = std::max(1, (max_p + 31) / 32);
-    // eight blocks per unit spread its keys, its gather and its latency; fewer when a block would be left with less than
-    // a ring buffer of keys although the machine is full without it
-    int cs = kPcMaxCluster;
-    while (cs > 1 && ((n_words * 32 < cs * kPcKeys && (long long)p.U * cs > 2ll * sm_count) || cs > n_words)) cs /= 2;
+    // As many blocks per unit as make the launch at least five waves of resident blocks: fewer leave the machine
+    // to the longest units, more pay each block's fixed chain of round trips more often. us per pass with 1 / 2 / 4 / 8:
+    // 1024 units x 3250 keys 969-1353 (with the slab's stride) / 956-1033 / 1073 / 1365, 128 units x 8192 keys (G 4) 2152 / 1281 / 811 / 752, 32 units x
+    // 4096 keys 350 / 192 / 120 / 93.
+    int cs = 1;
+    while (cs < kPcMaxCluster && cs * 2 <= n_words && (long long)p.U * cs < 1500ll * sm_count / 148) cs *= 2;
     const PcSmem lay = pc_smem_layout<T, D>(pp.rows8);
     if (lay.total > 227 * 1024) return CORM_ERR_UNSUPPORTED;
     auto kern = prompt_cluster_kernel<T, D>;
