@@ -140,10 +140,11 @@ corm_status_t corm_compress_prompt(corm_cache_t* cache, int32_t layer, const voi
  *   q      device [batch, n_q_heads, head_dim]
  *   k_new  device [batch, n_kv_heads, head_dim], v_new likewise
  *   out    device [batch, n_q_heads, head_dim]
- * The call enqueues one or two launches and returns; it sizes them from the longest and the mean live length the
- * kernels last reported, which it reads back asynchronously every 8 steps (batch * n_kv_heads integers). A host that has run 24 steps past a read-back that
- * has not landed waits for it here (the GPU still has those steps queued), so the call can block briefly, and a
- * layer's decode steps cannot be recorded into a CUDA graph.
+ * The call enqueues one or two launches and returns; it sizes them from the live lengths the kernels last reported (every
+ * 8 steps, written to pinned host memory). Where the grid follows the longest unit (bf16 / head_dim 128 with one query head
+ * per KV head, and tuning values other than 1), a host that has run 24 steps past a report that has not landed waits for
+ * it here, at most 20 ms (the GPU still has those steps queued). A layer's decode steps cannot be recorded into a CUDA
+ * graph.
  * Errors: STATE if the layer has had no corm_compress_prompt since create/reset; INVALID_ARG. */
 corm_status_t corm_decode_step(corm_cache_t* cache, int32_t layer, const void* q, const void* k_new,
                                const void* v_new, void* out, void* stream);

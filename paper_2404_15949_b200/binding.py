@@ -113,8 +113,14 @@ def _check(call, rc):
 
 
 def _stream_ptr(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    """Address of the stream, by default torch's current one on the current device (asked for directly: building the
+    Stream object takes 3.5 us, a third of a decode call's host time)."""
+    if stream is not None:
+        return stream.cuda_stream
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _torch_dtype(kv_dtype):

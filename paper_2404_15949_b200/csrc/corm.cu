@@ -6,8 +6,8 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cmath>
-#include <climits>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -33,7 +33,7 @@ constexpr int kMinSplit = 64;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-    size_t K, V, word, pos, live, base_tokens, base_obs, ticket, ticket2, kmax, unit_stamp, counters, status, maxlive, sim_acc, page_table, page_bits, page_room, q_prev, stash, partials, keepmask, unit_rec;
+    size_t K, V, word, pos, live, base_tokens, base_obs, ticket, ticket2, kmax, unit_stamp, counters, status, sim_acc, page_table, page_bits, page_room, q_prev, stash, partials, keepmask, unit_rec;
     size_t stage_q, stage_k, stage_v, stage_out, total, bookkeeping_begin, bookkeeping_end;
 };
 
@@ -102,7 +102,6 @@ Layout make_layout(const corm_config_t& c, int pool_pages) {
     L.unit_stamp = take(Ltot * U * 8);
     L.counters = take(Ltot * CNT_COUNT * 8);
     L.status = take(4);
-    L.maxlive = take(Ltot * 8);
     L.sim_acc = take(16);
     L.page_table = take(pool_pages ? Ltot * U * pt_stride_of(c) * 4 : 0);
     L.page_bits = take(pool_pages ? Ltot * (size_t)(pool_pages / 32) * 4 : 0);
@@ -158,12 +157,11 @@ struct corm_cache {
     int U, G;
     size_t e;
     std::vector<int> parity, steps, ready, live_upper;
-    // sizing feedback: the kernels publish the longest live length, the host reads it back without ever waiting
-    unsigned long long* maxlive_host = nullptr;   // pinned, [n_layers] words followed by [n_layers][U] live lengths
-    int32_t* live_host = nullptr;                 // the second part of that buffer
-    std::vector<int> live_mean;                   // mean live length at the last read-back that landed (0 = unknown)
-    std::vector<cudaEvent_t> readback_ev;
-    std::vector<int> readback_pending, last_readback_step;
+    // sizing feedback: when asked to, the kernels write every unit's length to pinned host memory, which the host looks at
+    unsigned long long* report_host = nullptr;    // [n_layers][U], report_live's words
+    std::vector<int> live_mean;                   // mean live length at the last report that landed (0 = unknown)
+    std::vector<int> report_pending, last_report_step;
+    std::vector<unsigned> report_epoch;           // 1..4095: reports of before a prompt pass, an import or a reset do not count
     int tune_split_len = 0, allow_fast = 1;
     double bound_scale = 1.0;
     int monitor_similarity = 0;
@@ -177,13 +175,6 @@ struct corm_cache {
     // per layer: K and V as tensors of 16-row boxes (cluster kernel; empty = unavailable); a slab layer's reach to the end
     // of the last layer, for layers stepped together
     std::vector<CUtensorMap> kmaps_row, vmaps_row;
-    // per layer: the group of layers (first layer * 65536 + count) it has been stepped with ever since its prompt pass
-    // (-1: not stepped yet, -2: alone or in different groups); only then does the group's length read-back describe it
-    std::vector<int> step_group;
-    // per layer, meaningful for the first layer of a group: bound on the longest unit of ALL the group's layers, taken
-    // from a length word that a launch over the whole group wrote (INT_MAX = none yet). The first layer's own
-    // live_upper may be smaller: right after the prompt pass it describes that layer alone.
-    std::vector<int> group_upper;
     // per layer: its latest decode launch finished every unit inside the streaming kernel and left the units' stamps,
     // so the next step's launch may be chained to it (corm_decode_steps)
     std::vector<int> chain_ok;
@@ -245,45 +236,44 @@ bool layer_ok(const corm_cache* c, int layer) { return c && layer >= 0 && layer 
 
 double log_alpha_of(const corm_cache* c) { return c->cfg.alpha > 0.f ? std::log((double)c->cfg.alpha) : -INFINITY; }
 
-unsigned long long* maxlive_ptr(const corm_cache* c, int layer) {
-    return reinterpret_cast<unsigned long long*>(c->arena + c->lay.maxlive) + layer;
-}
-
-// If an earlier read-back has landed, tighten the bound on this layer's longest unit: a unit grows by at most one
-// key per step, so (length after step s) + (steps since s) bounds every unit now.
-// A host that enqueues steps much faster than the GPU runs them would otherwise size its launches from a bound that
-// is hundreds of steps stale (every step adds one key to it): once it is kMaxRunAhead steps past a read-back that
-// has not landed it waits for that one, which leaves the GPU that many steps of queued work and costs it nothing.
+// If the report asked for earlier has landed, tighten the bound on this layer's longest unit: a unit grows by at most one
+// key per step, so (length after step s) + (steps since s) bounds it now.
+// Kernels whose grids follow the bound (`sized`) would be sized from one that is hundreds of steps stale when the host
+// enqueues steps much faster than the GPU runs them: once it is kMaxRunAhead steps past a report that has not landed it
+// waits for it, which leaves the GPU that many steps of queued work and costs it nothing. The wait is bounded (the queue
+// may be held up by other work): after it the old bound, which only grows, still holds.
 constexpr int kMaxRunAhead = 24;
-void poll_live_bound(corm_cache* c, int layer) {
-    if (!c->readback_pending[layer]) return;
-    if (c->steps[layer] - c->last_readback_step[layer] >= kMaxRunAhead) {
-        if (cudaEventSynchronize(c->readback_ev[layer]) != cudaSuccess) return;
-    } else if (cudaEventQuery(c->readback_ev[layer]) != cudaSuccess) {
-        (void)cudaGetLastError();   // cudaErrorNotReady is not an error
-        return;
+constexpr double kReportWaitSeconds = 0.02;
+bool take_report(corm_cache* c, int layer) {
+    const volatile unsigned long long* r = c->report_host + (size_t)layer * c->U;
+    long long sum = 0;
+    int bound = 0;
+    for (int u = 0; u < c->U; ++u) {
+        const unsigned long long v = r[u];
+        const int steps = (int)((v >> kReportLenBits) & ((1ull << kReportStepBits) - 1)), len = (int)(v & ((1ull << kReportLenBits) - 1));
+        if ((unsigned)(v >> (kReportLenBits + kReportStepBits)) != c->report_epoch[layer] || steps < c->last_report_step[layer]) return false;
+        bound = std::max(bound, len + c->steps[layer] - steps);
+        sum += len;
     }
-    c->readback_pending[layer] = 0;
-    const unsigned long long v = c->maxlive_host[layer];
-    const int steps_done = (int)(v >> 32), len = (int)(v & 0xffffffffu);
-    if (steps_done > c->steps[layer]) return;   // stale word from before a reset / new prompt
-    const int bound = len + (c->steps[layer] - steps_done);
-    if (bound < c->live_upper[layer]) c->live_upper[layer] = bound;
-    // a word written by a decode launch over the layer's group covers every layer of the group
-    if (steps_done >= 1 && c->step_group[layer] >= 0 && bound < c->group_upper[layer]) c->group_upper[layer] = bound;
-    long long sum = 0;                            // the lengths themselves came with the same read-back
-    for (int u = 0; u < c->U; ++u) sum += c->live_host[(size_t)layer * c->U + u];
+    c->report_pending[layer] = 0;
+    c->live_upper[layer] = std::min(c->live_upper[layer], bound);
     c->live_mean[layer] = (int)(sum / c->U);
+    return true;
 }
-
-void schedule_live_readback(corm_cache* c, int layer, cudaStream_t st) {
-    if (c->readback_pending[layer] || !c->maxlive_host) return;
-    if (cudaMemcpyAsync(c->maxlive_host + layer, maxlive_ptr(c, layer), 8, cudaMemcpyDeviceToHost, st) != cudaSuccess) return;
-    if (cudaMemcpyAsync(c->live_host + (size_t)layer * c->U, live_buf(c, layer, c->parity[layer]), (size_t)c->U * 4,
-                        cudaMemcpyDeviceToHost, st) != cudaSuccess) return;
-    if (cudaEventRecord(c->readback_ev[layer], st) != cudaSuccess) return;
-    c->readback_pending[layer] = 1;
-    c->last_readback_step[layer] = c->steps[layer];
+void wait_report(corm_cache* c, int layer) {
+    const auto start = std::chrono::steady_clock::now();
+    while (!take_report(c, layer))
+        if (std::chrono::duration<double>(std::chrono::steady_clock::now() - start).count() > kReportWaitSeconds) return;
+}
+void poll_live_bound(corm_cache* c, int layer, bool sized) {
+    if (!c->report_pending[layer]) return;
+    if (sized && c->steps[layer] - c->last_report_step[layer] >= kMaxRunAhead) wait_report(c, layer);
+    else (void)take_report(c, layer);
+}
+// Reports of launches before this call do not count any more.
+void forget_reports(corm_cache* c, int layer) {
+    c->report_pending[layer] = 0;
+    c->report_epoch[layer] = c->report_epoch[layer] % 4095 + 1;
 }
 
 // Eq. 3 between this step's queries and the layer's previous decode queries (opt-in; one small launch), after any
@@ -308,6 +298,11 @@ corm_status_t monitor_similarity(corm_cache* c, int layer, const void* q, cudaSt
     c->have_q_prev[layer] = 1;
     c->launches += 1;
     return CORM_OK;
+}
+
+// The cluster kernel works out its shares on the device; the other kernels' grids are sized from the host's bound.
+bool grids_follow_bound(const corm_cache* c) {
+    return c->allow_fast != 1 || c->kmaps_row.empty() || (c->cfg.kv_dtype == CORM_BF16 && c->cfg.head_dim == 128 && c->G == 1);
 }
 
 // Whether the cluster kernel takes a step of units of up to `upper` keys. Everything but one query head per KV head on
@@ -340,19 +335,7 @@ bool can_fuse(const corm_cache* c, int first_layer) {
 // this step's inputs were complete before that; more: the next step follows in the same way.
 corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void* k_new, const void* v_new, void* out,
                             cudaStream_t st, int n_fused = 1, bool chain = false, bool more = false) {
-    for (int i = 0; i < n_fused; ++i) poll_live_bound(c, layer + i);
-    {   // A launch publishes its longest unit in its first layer's word. That bounds every layer of the group, but only
-        // while that word has only ever been written by launches over this same group of layers.
-        const int now = n_fused > 1 ? layer * 65536 + n_fused : -2;           // this launch's group (solo launches: none)
-        bool same_group = n_fused > 1;
-        for (int i = 0; i < n_fused; ++i) {
-            int& g = c->step_group[layer + i];
-            g = (g == -1 || g == now) ? now : -2;
-            same_group &= g == now && now != -2;
-        }
-        if (same_group && c->group_upper[layer] != INT_MAX)
-            for (int i = 0; i < n_fused; ++i) c->live_upper[layer + i] = std::min(c->live_upper[layer + i], c->group_upper[layer]);
-    }
+    for (int i = 0; i < n_fused; ++i) poll_live_bound(c, layer + i, grids_follow_bound(c));
     const corm_config_t& cf = c->cfg;
     const size_t C = cf.max_tokens, D = cf.head_dim, U = c->U;
     DecodeParams p{};
@@ -369,7 +352,11 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     p.ticket2 = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.ticket2, U * 4, layer));
     p.counters = reinterpret_cast<unsigned long long*>(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer));
     p.status = reinterpret_cast<int32_t*>(c->arena + c->lay.status);
-    p.maxlive = maxlive_ptr(c, layer);
+    bool ask = true;                              // every 8 steps, all of the launch's layers together
+    for (int i = 0; i < n_fused; ++i)
+        ask &= !c->report_pending[layer + i] && c->steps[layer + i] + 1 - c->last_report_step[layer + i] >= 8 && c->report_epoch[layer + i] == c->report_epoch[layer];
+    p.report = ask ? c->report_host + (size_t)layer * U : nullptr;
+    p.report_tag = c->report_epoch[layer];
     p.stash = reinterpret_cast<double*>(c->arena + c->lay.stash);
     p.partials = c->arena + c->lay.partials;
     p.keepmask = reinterpret_cast<uint32_t*>(c->arena + c->lay.keepmask);
@@ -413,7 +400,7 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
         self_finishing = rc == CORM_OK && dp.p.unit_stamp;
         if (rc == CORM_OK && dp.p.chain_wait) c->chained_launches += 1;
     } else if (units) {
-        const int typical = mean_known ? std::min(upper, mean_sum / n_fused + c->steps[layer] - c->last_readback_step[layer] + 1) : 0;
+        const int typical = mean_known ? std::min(upper, mean_sum / n_fused + c->steps[layer] - c->last_report_step[layer] + 1) : 0;
         rc = launch_decode_balanced_units(p, n_fused > 1 ? c->vmap_all : c->vmaps[layer], c->G, upper, typical, c->tune_split_len,
                                           c->sm_count, partial_records_of(cf, c->pool_pages), st, &n_launched,
                                           chain_ok_before, more && !c->monitor_similarity);
@@ -423,7 +410,7 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
         rc = launch_decode_balanced(p, n_fused > 1 ? c->vmap_all : c->vmaps[layer], c->G, upper, c->sm_count, partial_records_of(cf, c->pool_pages), balanced_verdict, st, &n_launched);
     } else if (fast) {
         // the mean grows by at most one key per step, like the bound
-        const int typical = mean_known ? std::min(upper, mean_sum / n_fused + c->steps[layer] - c->last_readback_step[layer] + 1) : 0;
+        const int typical = mean_known ? std::min(upper, mean_sum / n_fused + c->steps[layer] - c->last_report_step[layer] + 1) : 0;
         rc = launch_decode_fast(p, c->G, upper, typical, c->tune_split_len, c->sm_count, st, &n_launched, c->allow_fast,
                                 chain_ok_before, more && !c->monitor_similarity, &self_finishing);
         if (rc == CORM_OK && p.chain_wait) c->chained_launches += 1;
@@ -449,8 +436,7 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
         c->parity[l] ^= 1;
         c->steps[l] += 1;
         c->live_upper[l] = std::min(cf.max_tokens, c->live_upper[l] + 1);
-        if (c->group_upper[l] != INT_MAX) c->group_upper[l] += 1;
-        if (c->steps[l] - c->last_readback_step[l] >= 8) schedule_live_readback(c, l, st);
+        if (ask) { c->report_pending[l] = 1; c->last_report_step[l] = c->steps[l]; }
     }
     return n_fused == 1 ? monitor_similarity(c, layer, q, st) : CORM_OK;
 }
@@ -499,28 +485,17 @@ corm_status_t corm_cache_create_paged(const corm_config_t* cfg, int32_t pool_pag
     c->live_upper.assign(cfg->n_layers, 0);
     c->live_mean.assign(cfg->n_layers, 0);
     c->have_q_prev.assign(cfg->n_layers, 0);
-    c->step_group.assign(cfg->n_layers, -1);
-    c->group_upper.assign(cfg->n_layers, INT_MAX);
     c->chain_ok.assign(cfg->n_layers, 0);
-    c->readback_pending.assign(cfg->n_layers, 0);
-    c->last_readback_step.assign(cfg->n_layers, 0);
-    c->readback_ev.assign(cfg->n_layers, nullptr);
-    bool host_ok = cudaHostAlloc(reinterpret_cast<void**>(&c->maxlive_host),
-                                 sizeof(unsigned long long) * cfg->n_layers + sizeof(int32_t) * (size_t)cfg->n_layers * c->U,
-                                 cudaHostAllocDefault) == cudaSuccess;   // pinned HOST memory; device memory stays the caller's
-    if (host_ok) {
-        c->live_host = reinterpret_cast<int32_t*>(c->maxlive_host + cfg->n_layers);
-        std::memset(c->maxlive_host, 0, sizeof(unsigned long long) * cfg->n_layers + sizeof(int32_t) * (size_t)cfg->n_layers * c->U);
-    }
-    for (int l = 0; host_ok && l < cfg->n_layers; ++l)
-        host_ok = cudaEventCreateWithFlags(&c->readback_ev[l], cudaEventDisableTiming) == cudaSuccess;
-    if (!host_ok) {
-        std::fprintf(stderr, "corm: could not set up the host-side read-back buffer\n");
-        for (cudaEvent_t ev : c->readback_ev) if (ev) cudaEventDestroy(ev);
-        if (c->maxlive_host) cudaFreeHost(c->maxlive_host);
+    c->report_pending.assign(cfg->n_layers, 0);
+    c->last_report_step.assign(cfg->n_layers, 0);
+    c->report_epoch.assign(cfg->n_layers, 1);
+    const size_t report_bytes = sizeof(unsigned long long) * (size_t)cfg->n_layers * c->U;
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->report_host), report_bytes, cudaHostAllocMapped) != cudaSuccess) {   // pinned HOST memory
+        std::fprintf(stderr, "corm: could not set up the host-side report buffer\n");
         delete c;
         return CORM_ERR_CUDA;
     }
+    std::memset(c->report_host, 0, report_bytes);
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cfg->device) == cudaSuccess && sms > 0) c->sm_count = sms;
     if (cfg->kv_dtype == CORM_BF16 && cfg->head_dim == 128 && c->G <= 4 && cfg->max_tokens <= kBalMaxTokens) {
@@ -554,8 +529,7 @@ corm_status_t corm_cache_create_paged(const corm_config_t* cfg, int32_t pool_pag
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         std::fprintf(stderr, "corm: clearing the arena failed: %s\n", cudaGetErrorString(e));
-        for (cudaEvent_t ev : c->readback_ev) if (ev) cudaEventDestroy(ev);
-        cudaFreeHost(c->maxlive_host);
+        cudaFreeHost(c->report_host);
         delete c;
         return CORM_ERR_CUDA;
     }
@@ -567,8 +541,9 @@ corm_status_t corm_cache_destroy(corm_cache_t* cache) {
     if (!cache) return CORM_ERR_INVALID_ARG;
     {
         DeviceGuard guard(cache->cfg.device);
-        for (cudaEvent_t ev : cache->readback_ev) if (ev) cudaEventDestroy(ev);
-        if (cache->maxlive_host) cudaFreeHost(cache->maxlive_host);
+        for (int pending : cache->report_pending)
+            if (pending) { cudaDeviceSynchronize(); break; }      // a launch may still write its report
+        cudaFreeHost(cache->report_host);
     }
     delete cache;
     return CORM_OK;
@@ -582,7 +557,8 @@ corm_status_t corm_cache_reset(corm_cache_t* c, void* stream) {
                               static_cast<cudaStream_t>(stream)));
     for (int l = 0; l < c->cfg.n_layers; ++l) {
         c->parity[l] = 0; c->steps[l] = 0; c->ready[l] = 0; c->live_upper[l] = 0; c->live_mean[l] = 0; c->have_q_prev[l] = 0;
-        c->readback_pending[l] = 0; c->last_readback_step[l] = 0; c->step_group[l] = -1; c->chain_ok[l] = 0; c->group_upper[l] = INT_MAX;
+        c->last_report_step[l] = 0; c->chain_ok[l] = 0;
+        forget_reports(c, l);
     }
     return CORM_OK;
 }
@@ -616,7 +592,6 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     clear(layer_ptr(c, c->lay.ticket2, U * 4, layer), U * 4);
     clear(layer_ptr(c, c->lay.kmax, U * 4, layer), U * 4);
     clear(layer_ptr(c, c->lay.unit_stamp, U * 8, layer), U * 8);        // step counts restart
-    clear(maxlive_ptr(c, layer), 8);
     clear(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer), CNT_COUNT * 8);   // a new prompt restarts the layer's statistics
     if (c->pool_pages) {   // whatever the layer held is replaced: all its pages return to the pool
         clear(page_table_ptr(c, layer), U * c->pt_stride * 4);
@@ -626,7 +601,7 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     int n_begin = 0;
     CORM_CUDA(launch_prompt_begin(bp, prompt_lens_host, cf.batch, st, &n_begin));
     c->chain_ok[layer] = 0;
-    c->readback_pending[layer] = 0;   // an older read-back no longer describes this layer
+    forget_reports(c, layer);                     // older ones no longer describe this layer
     PromptParams p{};
     p.k_prompt = k_prompt; p.v_prompt = v_prompt; p.q_last = q_last;
     p.prompt_lens = base_tokens;
@@ -638,7 +613,8 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     p.live_out = live_buf(c, layer, 0);
     p.counters = reinterpret_cast<unsigned long long*>(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer));
     p.status = reinterpret_cast<int32_t*>(c->arena + c->lay.status);
-    p.maxlive = maxlive_ptr(c, layer);
+    p.report = c->report_host + (size_t)layer * U;
+    p.report_tag = c->report_epoch[layer];
     p.stash = reinterpret_cast<double*>(c->arena + c->lay.stash);
     p.U = (int)U; p.Hkv = cf.n_kv_heads; p.C = cf.max_tokens; p.p_max = p_max; p.w = cf.window_w; p.r = cf.recent_r;
     p.log_alpha = log_alpha_of(c);
@@ -653,10 +629,8 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     c->launches += n_begin + 1;
     c->parity[layer] = 0; c->steps[layer] = 0; c->ready[layer] = 1; c->live_upper[layer] = max_p; c->live_mean[layer] = 0;
     c->have_q_prev[layer] = 0;                    // the previous decode query belonged to the old text
-    c->step_group[layer] = -1;
-    c->group_upper[layer] = INT_MAX;
-    c->last_readback_step[layer] = 0;
-    schedule_live_readback(c, layer, st);
+    c->last_report_step[layer] = 0;
+    c->report_pending[layer] = 1;
     return CORM_OK;
 }
 
@@ -732,16 +706,15 @@ corm_status_t decode_steps_impl(corm_cache_t* c, int32_t first_layer, int32_t n_
         fuse = c->steps[first_layer + i] == c->steps[first_layer] && c->parity[first_layer + i] == c->parity[first_layer];
     const auto at = [](const void* ptr, size_t off) { return static_cast<const unsigned char*>(ptr) + off; };
     const auto at_out = [](void* ptr, size_t off) { return static_cast<unsigned char*>(ptr) + off; };
-    // A call that enqueues many steps at once would size all of them from whatever the host knew on entry. If a length
-    // read-back is still in flight (typically the prompt pass's: without it the bound is the prompt length, several
-    // times the survivors), wait for it here, once: the GPU is busy with what precedes it anyway.
-    if (n_steps > 1)
+    // A call that enqueues many steps at once would size all of them from whatever the host knew on entry. If a report is
+    // still on its way (typically the prompt pass's: without it the bound is the prompt length, several times the
+    // survivors) and grids follow the bound, wait for it here, once: the GPU is busy with what precedes it anyway.
+    if (n_steps > 1 && grids_follow_bound(c))
         for (int i = 0; i < n_layers; ++i)
-            if (c->readback_pending[first_layer + i]) (void)cudaEventSynchronize(c->readback_ev[first_layer + i]);
+            if (c->report_pending[first_layer + i]) wait_report(c, first_layer + i);
     for (int s = 0; s < n_steps; ++s) {
         // A step is chained to the one before it when that one was enqueued by this call (nothing of the caller's can
-        // sit between them on the stream, and every step's inputs precede the call) and neither is the last word on
-        // its units' lengths for the host: a length read-back between two launches separates them anyway.
+        // sit between them on the stream, and every step's inputs precede the call).
         const bool chain = s > 0, more = s + 1 < n_steps;
         if (fuse || n_layers == 1) {
             const size_t i0 = (size_t)s * n_layers;
@@ -1090,11 +1063,9 @@ corm_status_t corm_cache_import_state(corm_cache_t* c, int32_t layer, int32_t se
     CORM_CUDA(cudaMemcpyAsync(layer_ptr(c, c->lay.base_obs, (size_t)cf.batch * 4, layer) + (size_t)seq * 4, &bo, 4, cudaMemcpyHostToDevice, st));
     CORM_CUDA(cudaStreamSynchronize(st));
     c->ready[layer] = 1;
-    c->readback_pending[layer] = 0;   // a read-back enqueued before this import knows nothing of it
+    forget_reports(c, layer);         // a report asked for before this import knows nothing of it
     c->live_upper[layer] = std::max(c->live_upper[layer], live_len);
-    c->live_mean[layer] = 0;                      // unknown until the next read-back
-    c->step_group[layer] = -2;                    // lengths changed behind the kernels' backs: the layer keeps its own bound
-    c->group_upper[layer] = INT_MAX;
+    c->live_mean[layer] = 0;                      // unknown until the next report
     c->chain_ok[layer] = 0;                       // ... and its units' stamps no longer describe them
     return CORM_OK;
 }

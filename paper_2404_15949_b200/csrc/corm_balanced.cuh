@@ -466,7 +466,7 @@ __device__ void bal_finish_block(const DecodeParams& p, const BalSeg* segs, int 
         if (tid == 0) {
             p.live_out[u] = new_len;
             if (UNIT) publish_unit_stamp(p, u, new_len);
-            publish_live(p.maxlive, p.step + 1, new_len);
+            report_live(p, u, p.step + 1, new_len);
             atomicAdd(p.counters + CNT_APPENDED, 1ull);
             atomicAdd(p.counters + CNT_ATTENDED, (unsigned long long)l);
             if (new_len < l) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(l - new_len));
@@ -538,7 +538,7 @@ decode_balanced_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
                 report_status(p.status, CORM_ERR_CAPACITY);
                 p.live_out[u] = l_old;
                 publish_unit_stamp(p, u, l_old);
-                publish_live(p.maxlive, p.step + 1, l_old);
+                report_live(p, u, p.step + 1, l_old);
             }
             return;
         }
@@ -588,7 +588,7 @@ decode_balanced_kernel(const __grid_constant__ DecodeParams p, const __grid_cons
             const int l_old = __ldcg(p.live_in + v);
             report_status(p.status, CORM_ERR_CAPACITY);
             p.live_out[v] = l_old;
-            publish_live(p.maxlive, p.step + 1, l_old);
+            report_live(p, v, p.step + 1, l_old);
         }
         sum += (l + kTileKeys - 1) / kTileKeys;
     }

@@ -760,7 +760,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             if (full) report_status(p.status, CORM_ERR_CAPACITY);
             p.live_out[u] = l_old;
             if (full) publish_unit_stamp(p, u, l_old);
-            publish_live(p.maxlive, p.step + 1, l_old);
+            report_live(p, u, p.step + 1, l_old);
         }
         return;
     }
@@ -875,8 +875,36 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             cluster_sync();
         }
     }
+    // outputs (Eq. 1): the unit's G x D values are shared out over the blocks, two channels per thread
+    auto write_outputs = [&](int first, int step) {
+        const int np = G * D / 2, x0 = np * rank / cs, x1 = np * (rank + 1) / cs;
+        for (int x = x0 + first; x < x1; x += step) {
+            const uint32_t at = smem_addr(smem) + x * 8;
+            double v[kDcMaxCluster];
+#pragma unroll
+            for (int y = 0; y < kDcMaxCluster; ++y) v[y] = y < cs ? ld_peer_f64(map_rank(at, y)) : 0.0;
+            float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+            for (int y = 0; y < kDcMaxCluster; ++y) {
+                a0 += __uint_as_float((uint32_t)__double2loint(v[y]));
+                a1 += __uint_as_float((uint32_t)__double2hiint(v[y]));
+            }
+            const double Z = misc->Zt[x / (D / 2)];
+            const float o0 = (float)((double)a0 / Z), o1 = (float)((double)a1 / Z);
+            if constexpr (kBf16) reinterpret_cast<uint32_t*>(p.out)[(size_t)u * np + x] = (uint32_t)float_to_bf16_bits(o0) | ((uint32_t)float_to_bf16_bits(o1) << 16);
+            else reinterpret_cast<float2*>(p.out)[(size_t)u * np + x] = make_float2(o0, o1);
+        }
+    };
     // ---- 3. compaction: kept slots at or above the new length move into the holes below it ----
     // Hole number = evicted slots before it, mover number = kept slots behind it, so both follow from the blocks' counts.
+    // the kept slots of the unit's word `wd`, from the block that owns it
+    auto peer_keep = [&](int wd) -> uint32_t {
+        int o = 0;
+        while (o + 1 < cs && (int)((long long)n_words * (o + 1) / cs) <= wd) ++o;
+        return ld_peer_u32(map_rank(smem_addr(keep + (wd - (int)((long long)n_words * o / cs))), o));
+    };
+    uint32_t last_keep = 0u;                                  // of the last 32 words, requested next to the counts
+    if (warp == 1 && n_words - 1 - lane >= 0) last_keep = peer_keep(n_words - 1 - lane);
     int before = 0, total = 0, imp_total = 0;
     {
         const int c = lane < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->count), lane)) : 0;
@@ -923,9 +951,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 const int wd = n_words - 1 - i0 - lane;
                 uint32_t km = 0u;
                 if (wd >= first_w) {
-                    int o = 0;                                // the block that owns the word
-                    while (o + 1 < cs && (int)((long long)n_words * (o + 1) / cs) <= wd) ++o;
-                    km = ld_peer_u32(map_rank(smem_addr(keep + (wd - (int)((long long)n_words * o / cs))), o));
+                    km = i0 == 0 ? last_keep : peer_keep(wd);
                     if (wd == first_w) km &= ~((1u << (new_len & 31)) - 1u);
                 }
                 int at = __popc(km);
@@ -942,12 +968,17 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 }
             }
             if (lane == 0) misc->n_moved = base;
+        } else {
+            write_outputs(tid - 64, NT - 64);
         }
         __syncthreads();
         const int n_moved = misc->n_moved;
         const int mine = k_begin < new_len ? min(n_moved, k_lo + n_keys - misc->count) - k_lo : 0;
         block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, movers, holes, mine, 0, 1, l, p.status);
-    } else if (new_len < l) {
+    } else {
+        write_outputs(tid, NT);
+    }
+    if (new_len < l && l - new_len > kDcListCap) {
         // many: the lists go to scratch and the moves are shared out evenly
         int* gholes = reinterpret_cast<int*>(p.stash + (size_t)u * G * p.C) + (size_t)G * p.C;   // behind the unit's logits
         int* gmovers = gholes + p.C / 2;
@@ -975,26 +1006,6 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         __syncthreads();
         block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, gmovers, gholes, misc->n_moved, rank, cs, l, p.status);
     }
-    // outputs (Eq. 1): the unit's G x D values are shared out over the blocks, two channels per thread
-    {
-        const int np = G * D / 2, x0 = np * rank / cs, x1 = np * (rank + 1) / cs;
-        for (int x = x0 + tid; x < x1; x += NT) {
-            const uint32_t at = smem_addr(smem) + x * 8;
-            double v[kDcMaxCluster];
-#pragma unroll
-            for (int y = 0; y < kDcMaxCluster; ++y) v[y] = y < cs ? ld_peer_f64(map_rank(at, y)) : 0.0;
-            float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-            for (int y = 0; y < kDcMaxCluster; ++y) {
-                a0 += __uint_as_float((uint32_t)__double2loint(v[y]));
-                a1 += __uint_as_float((uint32_t)__double2hiint(v[y]));
-            }
-            const double Z = misc->Zt[x / (D / 2)];
-            const float o0 = (float)((double)a0 / Z), o1 = (float)((double)a1 / Z);
-            if constexpr (kBf16) reinterpret_cast<uint32_t*>(p.out)[(size_t)u * np + x] = (uint32_t)float_to_bf16_bits(o0) | ((uint32_t)float_to_bf16_bits(o1) << 16);
-            else reinterpret_cast<float2*>(p.out)[(size_t)u * np + x] = make_float2(o0, o1);
-        }
-    }
     // every block's row moves come before released pages and the stamp; and a block's shared memory stays until its peers
     // have read it
     cluster_sync();
@@ -1004,7 +1015,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     if (tid == 0) {
         p.live_out[u] = new_len;
         publish_unit_stamp(p, u, new_len);
-        publish_live(p.maxlive, p.step + 1, new_len);
+        report_live(p, u, p.step + 1, new_len);
         atomicAdd(p.counters + CNT_APPENDED, 1ull);
         atomicAdd(p.counters + CNT_ATTENDED, (unsigned long long)l);
         if (imp_total) atomicAdd(p.counters + CNT_IMPORTANT, (unsigned long long)imp_total);

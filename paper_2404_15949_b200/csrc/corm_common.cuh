@@ -56,7 +56,8 @@ struct DecodeParams {
     uint32_t* ticket2;        // [U] second arrival counters (balanced kernel: blocks done with their verdicts)
     unsigned long long* counters;  // [CNT_COUNT]
     int32_t* status;          // sticky device status
-    unsigned long long* maxlive;  // (steps done << 32 | longest live length after that step), atomicMax; may be null
+    unsigned long long* report;   // [U] mapped host memory: units report their new lengths there (report_live); null = not asked for
+    unsigned long long report_tag;
     double* stash;            // [U*G][C] scaled logits of this step (scratch)
     unsigned char* partials;  // [U][max_splits][G] records {double m, double Z, float acc[D]} (scratch)
     uint32_t* keepmask;       // [U][ceil(C/32)+2] keep bits of the verdict launch (scratch)
@@ -93,7 +94,8 @@ struct PromptParams {
     int32_t* live_out;        // [U]
     unsigned long long* counters;
     int32_t* status;
-    unsigned long long* maxlive;
+    unsigned long long* report;   // as in DecodeParams
+    unsigned long long report_tag;
     double* stash;            // scratch, reused for temporary registers
     uint32_t* keepmask;       // [U][ceil(C/32)+2] keep bits (scratch)
     uint32_t* kmax;           // [U] as in DecodeParams
@@ -203,10 +205,14 @@ __device__ __forceinline__ void note_key_magnitude(uint32_t* kmax_u, uint4 x) {
     if ((threadIdx.x & 31) == 0) atomicMax(kmax_u, all);
 }
 
-// Publishes a unit's new live length for the host's launch sizing: the word holds the latest step in its high half,
-// so the maximum over all units of the most recent step wins.
-__device__ __forceinline__ void publish_live(unsigned long long* maxlive, int steps_done, int live) {
-    if (maxlive) atomicMax(maxlive, ((unsigned long long)(unsigned)steps_done << 32) | (unsigned)live);
+// A unit's new live length for the host's launch sizing: one word written straight to mapped host memory (tag in the top
+// 12 bits, steps done, length), so that neither a copy nor an event stands between two launches (two copies and an event
+// every 8 steps cost 1.2 us per step and broke the overlap of consecutive launches).
+constexpr int kReportLenBits = 24, kReportStepBits = 28;
+template <typename P> __device__ __forceinline__ void report_live(const P& p, int u, int steps_done, int live) {
+    if (p.report)
+        *reinterpret_cast<volatile unsigned long long*>(p.report + u) =
+            (p.report_tag << (kReportLenBits + kReportStepBits)) | ((unsigned long long)(unsigned)steps_done << kReportLenBits) | (unsigned)live;
 }
 
 __device__ __forceinline__ uint32_t window_mask(int w) { return w >= 32 ? 0xffffffffu : ((1u << w) - 1u); }
@@ -543,7 +549,7 @@ __device__ void finalize_unit(const DecodeParams& p, int u, int b, int l, int n_
     if (tid == 0) {
         p.live_out[u] = new_len;
         publish_unit_stamp(p, u, new_len);
-        publish_live(p.maxlive, p.step + 1, new_len);
+        report_live(p, u, p.step + 1, new_len);
         atomicAdd(p.counters + CNT_APPENDED, 1ull);
         atomicAdd(p.counters + CNT_ATTENDED, (unsigned long long)l);
         if (new_len < l) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(l - new_len));

@@ -279,7 +279,7 @@ __device__ void finalize_single(const DecodeParams& p, int u, int b, int l, int 
     if (tid == 0) {
         p.live_out[u] = new_len;
         publish_unit_stamp(p, u, new_len);
-        publish_live(p.maxlive, p.step + 1, new_len);
+        report_live(p, u, p.step + 1, new_len);
         atomicAdd(p.counters + CNT_APPENDED, 1ull);
         atomicAdd(p.counters + CNT_ATTENDED, (unsigned long long)l);
         if (new_len < l) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(l - new_len));
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kFastThreads, fast_blocks_per_sm(G)) decode_fa
             report_status(p.status, CORM_ERR_CAPACITY);
             p.live_out[u] = l_old;
             publish_unit_stamp(p, u, l_old);
-            publish_live(p.maxlive, p.step + 1, l_old);
+            report_live(p, u, p.step + 1, l_old);
         }
         return;
     }
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(kFastThreads, fast_blocks_per_sm(G)) decode_fa
     }
     __syncthreads();                       // every warp is done with its tiles: the tile area becomes scratch
     if (s_failed) {                        // a bounded wait expired: reported through the status word; the unit keeps its
-        if (split == 0 && tid == 0) { p.live_out[u] = l_old; publish_live(p.maxlive, p.step + 1, l_old); }   // old length
+        if (split == 0 && tid == 0) { p.live_out[u] = l_old; report_live(p, u, p.step + 1, l_old); }   // old length
         return;                            // (its arrival counter is not taken: the cache must be reset after this status)
     }
     unsigned char* merge = smem + lay.tiles;                      // [NW][G] records {double M, double Z, float acc[128]}

@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(kGenericThreads) decode_generic_kernel(const _
     const int room = pt_u ? __ldcg(p.page_room + u) : 1;
     const int l_old = __ldcg(p.live_in + u), l = l_old + 1;
     if (l > p.C || !room) {   // the slab is full (paged: no page for the new row): report, leave the unit untouched
-        if (split == 0 && tid == 0) { report_status(p.status, CORM_ERR_CAPACITY); p.live_out[u] = l_old; publish_live(p.maxlive, p.step + 1, l_old); }
+        if (split == 0 && tid == 0) { report_status(p.status, CORM_ERR_CAPACITY); p.live_out[u] = l_old; report_live(p, u, p.step + 1, l_old); }
         return;
     }
     const int n_act = (l + p.split_len - 1) / p.split_len;

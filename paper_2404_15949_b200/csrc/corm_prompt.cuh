@@ -242,7 +242,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     }
     if (P == 0) {
         if (rank == 0 && tid == 0) {
-            p.live_out[u] = 0; publish_live(p.maxlive, 0, 0);
+            p.live_out[u] = 0; report_live(p, u, 0, 0);
             if (p.page_table) {  // an empty unit still owns the page its first append goes to
                 const int pg = claim_page(p.page_bits, p.pool_pages, p.U, u, 0);
                 p.page_table[(size_t)u * p.pt_stride] = pg + 1;
@@ -633,7 +633,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         for (int x = 0; x < cs; ++x) failed |= (int)ld_peer_u32(map_rank(smem_addr(&misc->fail), x));
         if (rank == 0 && tid == 0) p.page_room[u] = failed ? 0 : 1;
         if (failed) {                                         // the pool is too small: the unit is left empty
-            if (rank == 0 && tid == 0) { report_status(p.status, CORM_ERR_CAPACITY); p.live_out[u] = 0; publish_live(p.maxlive, 0, 0); }
+            if (rank == 0 && tid == 0) { report_status(p.status, CORM_ERR_CAPACITY); p.live_out[u] = 0; report_live(p, u, 0, 0); }
             cluster_sync();
             return;
         }
@@ -688,7 +688,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     if (rank == 0 && tid == 0) {
         if (kBf16) p.kmax[u] = amax_unit;
         p.live_out[u] = kept_total;
-        publish_live(p.maxlive, 0, kept_total);
+        report_live(p, u, 0, kept_total);
         atomicAdd(p.counters + CNT_APPENDED, (unsigned long long)P);
         if (kept_total < P) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(P - kept_total));
     }
