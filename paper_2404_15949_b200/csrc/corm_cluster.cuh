@@ -68,6 +68,7 @@ template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int d
 
 constexpr int kDcListCap = 1024;                  // slots a step may evict from a unit for its moves to be listed on chip
 
+constexpr int kDcOpenCap = 32;
 template <int NW> struct DcMisc {
     unsigned long long stamp;
     double wZ[NW][8];                             // per warp and head, read by the cluster
@@ -79,6 +80,8 @@ template <int NW> struct DcMisc {
     // 1 << 18 if the unit cannot take the token
     uint32_t state;
     uint32_t flags;                               // heads to be formed exactly
+    int n_open;                                   // open verdicts of marked heads: slot << 3 | head
+    uint32_t open[kDcOpenCap];
     int count, n_imp, n_moved;                    // kept slots and important keys of the block; row moves of the unit
     int scan[NW * 32];
 };
@@ -118,23 +121,7 @@ template <typename T, int N> __device__ __forceinline__ void load_slice_cg(const
     }
 }
 
-// exact q.k of a slot by four lanes (sub = lane & 3): fp64, a fixed order; before the 1/sqrt(d)
-template <typename T, int D>
-__device__ __forceinline__ double quad_exact_dot(const T* q, const T* k, int sub) {
-    double part = 0.0;
-#pragma unroll 4
-    for (int i = 0; i < D / 16; ++i) {
-        float a[4], b[4];
-        load_slice<T, 4>(q + (i * 4 + sub) * 4, a);
-        load_slice_cg<T, 4>(k + (i * 4 + sub) * 4, b);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) part = fma((double)a[e], (double)b[e], part);
-    }
-    part += __shfl_xor_sync(0xffffffffu, part, 1);
-    part += __shfl_xor_sync(0xffffffffu, part, 2);
-    return part;
-}
-// ... and by a whole warp
+// exact q.k of a slot by a whole warp: fp64, before the 1/sqrt(d)
 template <typename T, int D>
 __device__ __forceinline__ double warp_exact_dot_cg(const T* q, const T* k, int lane) {
     constexpr int NPL = D / 32;
@@ -147,38 +134,34 @@ __device__ __forceinline__ double warp_exact_dot_cg(const T* q, const T* k, int 
     return warp_sum(part);
 }
 
-// The marked heads, exactly: log-sum-exp with a running maximum and verdicts in fp64 from global memory, by the whole
-// cluster. A verdict that was sure before holds for the exact threshold too, so adding importance is enough: the
-// register gets its newest bit (or stamp), the keep bit is set.
+// The marked heads, exactly, by the whole cluster: their log-sum-exp in fp64 with a running maximum, then the verdicts
+// that were left open (misc->open, or every slot of the block where those did not fit or magnitudes are beyond the pieces'
+// range). A verdict that was sure before holds for the exact threshold too, so adding importance is enough: the register
+// gets its newest bit (or stamp), the keep bit is set. About one step in ten of 32 units x 21000 keys comes here: 16 keys
+// per warp at a time instead of 8, and no second pass over the keys, took 100 us of such a step to 20.
 template <typename T, int D, int NW>
-__device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G, int t, int k_begin, int k_end, uint32_t heads,
+__device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G, int t, int k_begin, int k_end, uint32_t heads, bool all_slots,
                                             uint32_t* keep, DcMisc<NW>* misc, int cs) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & 3;
-    const double inv_root_d = inv_root_dim(D);
     const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
     const T* Kl = reinterpret_cast<const T*>(p.K);
     const uint32_t mz_addr = smem_addr(misc->mz);
     uint32_t* wordu = p.word + (size_t)u * p.C;
+    auto row_of = [&](int j) -> const T* { return Kl + kv_row(pt_u, (size_t)u * p.C, j, p.pool_pages, p.status) * D; };
     int added = 0, added_imp = 0;
+    auto add_importance = [&](int j) {
+        const uint32_t reg = __ldcg(wordu + j), bit = 1u << (j & 31);
+        if (p.w <= 32 ? (reg & 1u) : reg == (uint32_t)t) return;
+        wordu[j] = p.w <= 32 ? (reg | 1u) : (uint32_t)t;
+        added_imp += 1;
+        if (!(atomicOr(keep + ((j - k_begin) >> 5), bit) & bit)) added += 1;
+    };
+    const int n_open = all_slots || misc->n_open > kDcOpenCap ? -1 : misc->n_open;
     for (int h = 0; h < G; ++h) {
         if (!((heads >> h) & 1u)) continue;
         const T* q = reinterpret_cast<const T*>(p.q) + ((size_t)u * G + h) * D;
-        double m = -INFINITY, Z = 0.0;
-        for (int j0 = k_begin + warp * 8; j0 < k_end; j0 += NW * 8) {
-            const int j = j0 + (lane >> 2);
-            const size_t row = kv_row(pt_u, (size_t)u * p.C, min(j, k_end - 1), p.pool_pages, p.status);
-            const double s = quad_exact_dot<T, D>(q, Kl + row * D, sub) * inv_root_d;
-            if (j < k_end) {
-                if (s > m) { Z = Z * exp(m - s) + 1.0; m = s; }
-                else Z += exp(s - m);
-            }
-        }
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-            const double mo = __shfl_xor_sync(0xffffffffu, m, o), Zo = __shfl_xor_sync(0xffffffffu, Z, o), mn = fmax(m, mo);
-            Z = (m == mn ? Z : Z > 0.0 ? Z * exp(m - mn) : 0.0) + (mo == mn ? Zo : Zo > 0.0 ? Zo * exp(mo - mn) : 0.0);
-            m = mn;
-        }
+        double m, Z;
+        warp_exact_lse<T, D>(q, row_of, k_begin + warp * 16, k_end, NW * 16, m, Z);
         if (lane == 0) { misc->red[warp][0] = m; misc->red[warp][1] = Z; }
         __syncthreads();
         if (tid == 0) {
@@ -196,19 +179,17 @@ __device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G,
             if (z > 0.0) Zt += z * exp(ld_peer_f64(map_rank(mz_addr, x)) - M);
         }
         const double thr = M + log(Zt) + p.log_alpha - log((double)t);
-        for (int j0 = k_begin + warp * 8; j0 < k_end; j0 += NW * 8) {
-            const int j = j0 + (lane >> 2);
-            const size_t row = kv_row(pt_u, (size_t)u * p.C, min(j, k_end - 1), p.pool_pages, p.status);
-            const double s = quad_exact_dot<T, D>(q, Kl + row * D, sub) * inv_root_d;
-            if (sub == 0 && j < k_end && s >= thr) {
-                const uint32_t reg = __ldcg(wordu + j), bit = 1u << (j & 31);
-                const bool had = p.w <= 32 ? (reg & 1u) : reg == (uint32_t)t;
-                if (!had) {
-                    wordu[j] = p.w <= 32 ? (reg | 1u) : (uint32_t)t;
-                    added_imp += 1;
-                    if (!(atomicOr(keep + ((j - k_begin) >> 5), bit) & bit)) added += 1;
-                }
-            }
+        QuadRow<T, D> qr;
+        qr.load(q, sub);
+        const int n = n_open < 0 ? k_end - k_begin : n_open;
+        for (int i0 = warp * 8; i0 < n; i0 += NW * 8) {       // eight slots per warp, the same sums as above
+            const int i = i0 + (lane >> 2);
+            const bool on = i < n && (n_open < 0 || (misc->open[i] & 7u) == (uint32_t)h);
+            const int j = on ? (n_open < 0 ? k_begin + i : (int)(misc->open[i] >> 3)) : k_begin;
+            const T* const rows[1] = {row_of(j)};
+            double s[1];
+            quad_exact_dots<T, D, 1>(qr, rows, sub, s);
+            if (on && sub == 0 && s[0] * inv_root_dim(D) >= thr) add_importance(j);
         }
         cluster_sync();                                       // everybody has read mz; the registers of this head are written
     }
@@ -238,7 +219,11 @@ __device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int 
                                                      reinterpret_cast<const T*>(p.K) + row * D, lane) * inv_root_dim(D);
             const double th = misc->thr[h], e = (double)(eps_a * misc->qe[h]) + 1e-13 * (1.0 + fabs(th));
             if (lane == src && s - th > e) imp = true;
-            if (lane == 0 && fabs(s - th) <= e) atomicOr(&misc->flags, 1u << h);
+            if (lane == 0 && fabs(s - th) <= e) {
+                atomicOr(&misc->flags, 1u << h);
+                const int at = atomicAdd(&misc->n_open, 1);
+                if (at < kDcOpenCap) misc->open[at] = ((uint32_t)js << 3) | (uint32_t)h;
+            }
             ++n_near;
         }
     }
@@ -270,7 +255,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     if (tid == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&kmap)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&vmap)) : "memory");
-        misc->state = 0u; misc->flags = 0u; misc->count = 0; misc->n_imp = 0;
+        misc->state = 0u; misc->flags = 0u; misc->count = 0; misc->n_imp = 0; misc->n_open = 0;
     }
     if (lane == 0) {
 #pragma unroll
@@ -435,13 +420,13 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 n2 += __shfl_xor_sync(0xffffffffu, n2, o);
                 n3 += __shfl_xor_sync(0xffffffffu, n3, o);
             }
-            // Error of a logit (before the 1/sqrt(d)) per unit of the unit's largest key magnitude A. r2.q: 34 roundings
-            // of 2^-23 per 16 channels (two products of 16 terms and their accumulators; half of that for four heads or
-            // fewer) and 8 of 2^-24 in fp32, on terms of at most A/8192 |q|; k.q3: at most 2 * 8 * 17 roundings of 2^-23;
+            // Error of a logit (before the 1/sqrt(d)) per unit of the unit's largest key magnitude A. r2.q: per 16 channels 17
+            // roundings of 2^-23 (a product of 16 terms and its accumulator; twice that for eight heads, whose two products
+            // share one) and 8 of 2^-24 in fp32, on terms of at most A/8192 |q|; k.q3: at most 2 * 8 * 17 roundings of 2^-23;
             // r2.q3 <= A/8192 |q3| (left out for eight and four heads); the sum of the small parts (k2.q2 <= A/64 |q2|
             // among them) rounds three times.
             if (on && (lane & 3) == 0)
-                misc->qe[hq] = dp.bound_scale * 1.05f * (4.6e-6f * (n1 * 1.01f) * (1.f / 8192.f) + (3.3e-5f + 1.3e-4f) * n3 + 2.4e-7f * n2 * (1.f / 64.f));
+                misc->qe[hq] = dp.bound_scale * 1.05f * ((GP == 8 ? 4.6e-6f : 2.6e-6f) * (n1 * 1.01f) * (1.f / 8192.f) + (3.3e-5f + 1.3e-4f) * n3 + 2.4e-7f * n2 * (1.f / 64.f));
         }
         float accd[D / 16][4];
 #pragma unroll
@@ -871,7 +856,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         const uint32_t marks = __reduce_or_sync(0xffffffffu, lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->flags), lane)) : 0u);
         if (marks) {                                          // uniform in the cluster
             cluster_sync();
-            dc_exact_heads<T, D, NW>(p, u, G, t, k_begin, k_end, marks, keep, misc, cs);
+            dc_exact_heads<T, D, NW>(p, u, G, t, k_begin, k_end, marks, (unit_state & kDcBad) != 0u, keep, misc, cs);
             cluster_sync();
         }
     }

@@ -89,6 +89,88 @@ __device__ __forceinline__ float split_error(float n1, float n2, float n3) {
     return 7.62939453125e-6f * (n2 * (1.f / 64.f) + n1 * (1.f / 8192.f) + n3) * 1.2f + n3 * (1.f / 60.f);
 }
 
+// ---- exact logits ----
+// A quarter of a row (lane's sub = lane & 3: the 16-byte chunks sub, sub + 4, ...) in registers, widened.
+template <typename T, int D> struct QuadRow {
+    static constexpr int kN = D / 4, kVec = 16 / Elem<T>::kBytes, kLoads = kN / kVec;
+    double v[kN];
+    __device__ __forceinline__ void load(const T* row, int sub) {
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) widen(__ldcg(reinterpret_cast<const uint4*>(row) + i * 4 + sub), i);
+    }
+    __device__ __forceinline__ void widen(const uint4& x, int i) {
+        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if constexpr (kVec == 8) {
+                v[i * 8 + 2 * e] = (double)__uint_as_float(w[e] << 16);
+                v[i * 8 + 2 * e + 1] = (double)__uint_as_float(w[e] & 0xffff0000u);
+            } else {
+                v[i * 4 + e] = (double)__uint_as_float(w[e]);
+            }
+        }
+    }
+};
+// N rows of the cache against one query, four lanes to a row: fp64, a fixed order (every caller gets the same bits for the
+// same pair), before the 1/sqrt(d). Rows are read past the L1 (they move between launches that may overlap).
+template <typename T, int D, int N>
+__device__ __forceinline__ void quad_exact_dots(const QuadRow<T, D>& q, const T* const (&rows)[N], int sub, double (&s)[N]) {
+    using Q = QuadRow<T, D>;
+    uint4 x[N][Q::kLoads];
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+#pragma unroll
+        for (int i = 0; i < Q::kLoads; ++i) x[n][i] = __ldcg(reinterpret_cast<const uint4*>(rows[n]) + i * 4 + sub);
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+        double part = 0.0;
+#pragma unroll
+        for (int i = 0; i < Q::kLoads; ++i) {
+            const uint32_t w[4] = {x[n][i].x, x[n][i].y, x[n][i].z, x[n][i].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if constexpr (Q::kVec == 8) {
+                    part = fma(q.v[i * 8 + 2 * e], (double)__uint_as_float(w[e] << 16), part);
+                    part = fma(q.v[i * 8 + 2 * e + 1], (double)__uint_as_float(w[e] & 0xffff0000u), part);
+                } else {
+                    part = fma(q.v[i * 4 + e], (double)__uint_as_float(w[e]), part);
+                }
+            }
+        }
+        part += __shfl_xor_sync(0xffffffffu, part, 1);
+        part += __shfl_xor_sync(0xffffffffu, part, 2);
+        s[n] = part;
+    }
+}
+// Log-sum-exp of one query over the slots [begin + first, end) in steps of `step` by a whole warp, 16 slots at a time;
+// row_of(j) gives a slot's row. All lanes return the same (m, Z).
+template <typename T, int D, typename RowOf>
+__device__ __forceinline__ void warp_exact_lse(const T* q, RowOf row_of, int begin, int end, int step, double& m, double& Z) {
+    const int lane = threadIdx.x & 31, sub = lane & 3;
+    QuadRow<T, D> qr;
+    qr.load(q, sub);
+    m = -INFINITY; Z = 0.0;
+    for (int j0 = begin; j0 < end; j0 += step) {
+        const int ja = j0 + (lane >> 2), jb = ja + 8;
+        const T* const rows[2] = {row_of(min(ja, end - 1)), row_of(min(jb, end - 1))};
+        double s[2];
+        quad_exact_dots<T, D, 2>(qr, rows, sub, s);
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            if ((y ? jb : ja) >= end) continue;
+            const double x = s[y] * inv_root_dim(D);
+            if (x > m) { Z = Z * exp(m - x) + 1.0; m = x; }
+            else Z += exp(x - m);
+        }
+    }
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) {
+        const double mo = __shfl_xor_sync(0xffffffffu, m, o), Zo = __shfl_xor_sync(0xffffffffu, Z, o), mn = fmax(m, mo);
+        Z = (m == mn ? Z : Z > 0.0 ? Z * exp(m - mn) : 0.0) + (mo == mn ? Zo : Zo > 0.0 ? Zo * exp(mo - mn) : 0.0);
+        m = mn;
+    }
+}
+
 // ---- clusters ----
 __device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ uint32_t cluster_size() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }

@@ -9,28 +9,29 @@
 //   B. verdicts of the block's keys for every row -> verdict registers;
 //   -- the blocks exchange their counts of surviving keys
 //   C. every block gathers its own survivors (K, V rows, registers, positions) to their place in token order.
-// Keys stream through a ring of shared-memory buffers of 128 keys (asynchronous copies, two buffers ahead); a block
-// whose keys fit the ring reads K once, otherwise phase B finds it in L2 (a unit's K is a few MB and only as many units
-// are in flight as fit the machine).
+// Keys stream through a ring of shared-memory buffers of 128 keys (asynchronous copies); a block whose keys fit the ring
+// reads K once, otherwise later passes find it in L2 (a unit's K is a few MB and only as many units are in flight as fit the
+// machine).
 //
 // bf16: both contractions run on the tensor cores. Phase A needs fp64-grade logits: operands cut into exact pieces
-// (corm_mma.cuh), 7 mma.m16n8k16 per 16 channels for 16 keys x 8 rows. Phase B only has to place a logit on one side of
-// its threshold: one plain mma per 16 channels, whose rounding is at most 2^-23 per term; the few logits inside that
-// bound are formed again in fp64 by the whole warp (counted in corm_stats_t.near_threshold). If such a logit falls
-// within the error of phase A's log-sum-exp itself, it is left undecided and the row is marked; after phase B the
-// cluster forms the marked rows' log-sum-exps and verdicts again entirely in fp64 (about one row in 10^4..10^5). So
-// every verdict is the fp64 one.
+// (corm_mma.cuh), 7 mma.m16n8k16 per 16 channels for 16 keys x 8 rows; the rows' pieces lie on chip for 32 rows at a time,
+// and a warp's tile of keys is cut once for 16 of them. Phase B only has to place a logit on one side of its threshold: one
+// plain mma per 16 channels, whose rounding is at most 2^-23 per term; the few logits inside that bound are formed again in
+// fp64 by the whole warp (counted in corm_stats_t.near_threshold). If such a logit falls within the error of phase A's
+// log-sum-exp itself, it is left open and the row is marked; after phase B the cluster forms the marked rows' log-sum-exps
+// in fp64 and decides what was left open (about one row in 10^4..10^5). So every verdict is the fp64 one.
 // fp32: fp64 arithmetic on the CUDA cores, lane = key, 4 rows at a time; only ties (1e-13) go to the exact rows, whose
 // sums keep the largest logit apart, so that a query at position 1 stays exactly on its threshold.
 //
 // What bounds it: for windows of a few queries HBM and the latency of the gather (K once, the survivors' V in, K and V
 // out); for wide windows the tensor pipe's mma.sync rate in phase A (R P d multiply-adds, seven times).
-// Measured against the two-launch pass this replaces (fp64 logits on the CUDA cores; one block per unit gathering) and,
-// for fp32 or 64 channels, a pass with one block per unit; us, w = queries in the window, G = heads per group:
-//   1024 units x 3250 keys, G 1, w 8    1597 -> 1033      128 units x 3390 keys, G 1, w 256    5341 -> 1735
-//   128 units x 8192 keys, G 4, w 8     1821 ->  785      32 units x 8192 keys, G 4, w 128     6736 -> 2235
-//   32 units x 32768 keys, G 4, w 16    4618 -> 2363      32 units x 4096 keys, G 1, w 8        259 ->   77
-//   fp32: 20 units x 1300 keys, G 2     2787 ->  111      64 channels: 128 units x 2000, G 4  11037 ->  287
+// Measured, us per pass: a two-launch pass (fp64 logits on the CUDA cores; one block per unit gathering; for fp32 or 64
+// channels one block per unit for everything) -> a first cluster pass (a warp per octet of rows, every warp cutting every
+// key; marked rows a key at a time) -> now:
+//   1024 units x 3250 keys, G 1, w 8    1597 -> 1036 ->  842    128 units x 3390 keys, G 1, w 256    5341 -> 1709 -> 1630
+//   128 units x 8192 keys, G 4, w 8     1821 ->  769 ->  607    32 units x 8192 keys, G 4, w 128     6736 -> 2206 -> 1747
+//   32 units x 32768 keys, G 4, w 16    4618 -> 2375 -> 1072    32 units x 4096 keys, G 1, w 8        259 ->   65 ->   61
+//   fp32: 20 units x 1300 keys, G 2     2787 ->  103            64 channels: 128 units x 2000, G 4  11037 ->  273 ->  247
 #pragma once
 
 #include "corm_fast.cuh"
@@ -41,7 +42,12 @@ namespace corm {
 constexpr int kPcThreads = 256;
 constexpr int kPcWarps = kPcThreads / 32;
 constexpr int kPcKeys = 128;                    // keys per ring buffer
-template <typename T, int D> __host__ __device__ constexpr int pc_bufs() { return D * Elem<T>::kBytes <= 256 ? 3 : 2; }
+// ring buffers: three, two where rows are long or the row pieces of a group take the room
+template <typename T, int D> __host__ __device__ constexpr int pc_bufs(int rows8) {
+    return D * Elem<T>::kBytes > 256 || (Elem<T>::kBytes == 2 && D == 128 && rows8 > 16) ? 2 : 3;
+}
+constexpr int kPcGroup = 4;                     // octets of rows (bf16) whose pieces lie on chip at a time in phase A
+constexpr int kPcGroupB = 8;                    // ... whose raw values do in phase B
 constexpr int kPcMaxCluster = 8;
 constexpr double kPcLogitLimit = 650.0;         // exp of anything below stays finite in fp64, also summed over 2^19 keys
 
@@ -51,28 +57,36 @@ struct PromptClusterParams {
     int32_t rows8;           // w G rounded up to a multiple of 8
 };
 
-struct PcSmem { int ring, zs, thr, n1, qe, flags, words, list, stage, misc, total; };
+struct PcSmem { int ring, zs, thr, n1, qe, flags, words, list, stage, frag, misc, total; };
+constexpr int kPcOpenCap = 64;
 struct PcMisc {
     double red[kPcWarps][2];
     double mz[2];
+    double zw[kPcWarps][kPcGroup * 8];          // phase A: the warps' sums of a group's rows
     int count, bad, warp_sum[kPcWarps], fail;
+    int n_open;                                 // verdicts that phase B left open: (row, key)
+    int2 open[kPcOpenCap];
     uint32_t amax;                              // largest magnitude (bf16 bits) of the block's keys
-    uint16_t tile_amax[3 * kPcKeys / 16];       // ... of every 16-key tile in the ring
+    float thr_f[kPcGroupB * 8], err_f[kPcGroupB * 8], slack[kPcGroupB * 8];      // phase B: a group's rows
 };
 template <typename T, int D>
 __host__ __device__ inline PcSmem pc_smem_layout(int rows8) {
     PcSmem s{};
     int off = 0;
     auto take = [&](int bytes) { int at = off; off = (off + bytes + 127) / 128 * 128; return at; };
-    s.ring = take(pc_bufs<T, D>() * kPcKeys * D * Elem<T>::kBytes);
+    s.ring = take(pc_bufs<T, D>(rows8) * kPcKeys * D * Elem<T>::kBytes);
     s.zs = take((rows8 > 64 ? rows8 : 64) * 8);
     s.thr = take(rows8 * 8);
     s.n1 = take(rows8 * 4);
     s.qe = take(rows8 * 4);
     s.flags = take((rows8 + 31) / 32 * 4);
-    s.words = take(kPcKeys * 4);
+    s.words = take(Elem<T>::kBytes == 4 ? kPcKeys * 4 : 0);
     s.list = take(kPcWarps * 32);               // gather: the kept lanes of a warp's word
     s.stage = take(Elem<T>::kBytes == 4 ? kPcWarps * 4 * D * 8 : 0);
+    // bf16: pieces of a group's octets (three of 256 bytes per 16 channels), or raw values of twice as many (one)
+    const int octets = rows8 / 8, even = octets == 1 ? 1 : (octets + 1) / 2 * 2;
+    const int fa = (even < kPcGroup ? even : kPcGroup) * (D / 16) * 3 * 256, fb = (octets < kPcGroupB ? octets : kPcGroupB) * (D / 16) * 256;
+    s.frag = take(Elem<T>::kBytes == 2 ? (fa > fb ? fa : fb) : 0);
     s.misc = take((int)sizeof(PcMisc));
     s.total = off;
     return s;
@@ -119,27 +133,25 @@ struct PcRows {
 __device__ __forceinline__ uint32_t pc_mark(int w, int rho, int qpos) { return w <= 32 ? 1u << (w - 1 - rho) : (uint32_t)qpos; }
 __device__ __forceinline__ uint32_t pc_join(int w, uint32_t a, uint32_t b) { return w <= 32 ? (a | b) : max(a, b); }
 
-// The marked rows, exactly: log-sum-exp with a running maximum and every verdict in fp64 straight from global memory.
-// Rare (or asked for by an inflated bound); all blocks of the cluster take it together. Verdicts that phase B was sure
-// of hold for the exact threshold too, so adding marks is enough.
+// The marked rows, exactly, by all blocks of the cluster: log-sum-exp in fp64 with a running maximum, then the verdicts that
+// phase B left open (misc->open, or every key where those did not fit or `all_keys`). Verdicts that phase B was sure of hold
+// for the exact threshold too, so adding marks is enough. Rare, but a launch is as long as its longest unit: with a key at a
+// time per warp and a second pass over the keys for the verdicts this took 714 us of 1592 on 32768-key prompts.
 template <typename T, int D>
-__device__ __noinline__ void pc_exact_rows(const PromptParams& p, const PcRows& R, const T* Qu, const T* Ku, int k_begin, int k_end,
+__device__ __noinline__ void pc_exact_rows(const PromptParams& p, const PcRows& R, const T* Qu, const T* Ku, int k_begin, int k_end, bool all_keys,
                                            const uint32_t* flags, uint32_t* words_g, PcMisc* misc, int cs) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const double inv_root_d = inv_root_dim(D);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & 3;
     const uint32_t mz_addr = smem_addr(misc->mz);
+    auto row_of = [&](int j) -> const T* { return Ku + (size_t)j * D; };
+    const int n_open = all_keys || misc->n_open > kPcOpenCap ? -1 : misc->n_open;
     for (int r = 0; r < R.rows; ++r) {
         if (!((flags[r >> 5] >> (r & 31)) & 1u)) continue;
         const int qpos = R.pos(r);
         if (!qpos) continue;
         const T* qr = R.q<T, D>(Qu, r);
         const int end = min(k_end, qpos);                     // causal row: keys 1..position of the query
-        double m = -INFINITY, Z = 0.0;
-        for (int j = k_begin + warp; j < end; j += kPcWarps) {
-            const double s = warp_exact_dot<T, D>(qr, Ku + (size_t)j * D, lane) * inv_root_d;
-            if (s > m) { Z = Z * exp(m - s) + 1.0; m = s; }
-            else Z += exp(s - m);
-        }
+        double m, Z;
+        warp_exact_lse<T, D>(qr, row_of, k_begin + warp * 16, end, kPcWarps * 16, m, Z);
         if (lane == 0) { misc->red[warp][0] = m; misc->red[warp][1] = Z; }
         __syncthreads();
         if (tid == 0) {
@@ -157,17 +169,23 @@ __device__ __noinline__ void pc_exact_rows(const PromptParams& p, const PcRows& 
             if (z > 0.0) Zt += z * exp(ld_peer_f64(map_rank(mz_addr, x)) - M);
         }
         const double thr = M + log(Zt) + p.log_alpha - log((double)qpos);
-        for (int j = k_begin + warp; j < end; j += kPcWarps) {
-            const double s = warp_exact_dot<T, D>(qr, Ku + (size_t)j * D, lane) * inv_root_d;
-            if (lane == 0 && s >= thr) words_g[j] = pc_join(p.w, words_g[j], pc_mark(p.w, R.rho(r), qpos));
+        QuadRow<T, D> q;
+        q.load(qr, sub);
+        const int n = n_open < 0 ? max(0, end - k_begin) : n_open;
+        for (int i0 = warp * 8; i0 < n; i0 += kPcWarps * 8) {  // eight keys per warp, the same sums as above
+            const int i = i0 + (lane >> 2);
+            const bool on = i < n && (n_open < 0 || misc->open[i].x == r);
+            const int j = on ? (n_open < 0 ? k_begin + i : misc->open[i].y) : k_begin;
+            const T* const rows[1] = {row_of(j)};
+            double s[1];
+            quad_exact_dots<T, D, 1>(q, rows, sub, s);
+            if (on && sub == 0 && s[0] * inv_root_dim(D) >= thr) words_g[j] = pc_join(p.w, __ldcg(words_g + j), pc_mark(p.w, R.rho(r), qpos));
         }
-        cluster_sync();                                       // everybody has read mz
+        cluster_sync();                                       // everybody has read mz; the marks of this row are written
     }
 }
 
-// Query pieces of 8 rows in the B operand's layout (row n = lane / 4), held in registers.
-template <int D> struct PcFrag { uint32_t b1[D / 16][2], b2[D / 16][2], b3[D / 16][2]; };
-
+// Raw values of 8 rows in the B operand's layout (row n = lane / 4); zeros for rows that do not exist.
 template <int D>
 __device__ __forceinline__ void pc_load_raw(const PcRows& R, const bf16_t* Qu, int octet, int lane, uint32_t (&raw)[D / 16][2]) {
     const int r = 8 * octet + (lane >> 2);
@@ -180,9 +198,10 @@ __device__ __forceinline__ void pc_load_raw(const PcRows& R, const bf16_t* Qu, i
     }
 }
 
-// The pieces, and the row's norms for the error bounds. Returns false if the row leaves the safe range.
+// The pieces of 8 rows (b1 and b2 as one 16-byte word per lane and 16 channels, b3 as one of 8), and the rows' norms for
+// the error bounds. Returns false if a row leaves the safe range.
 template <int D>
-__device__ __forceinline__ bool pc_load_frag(const PcRows& R, const bf16_t* Qu, int octet, int lane, PcFrag<D>& f, float* n1_sm, float* qe_sm) {
+__device__ __noinline__ bool pc_store_pieces(const PcRows& R, const bf16_t* Qu, int octet, int lane, uint4* f12, uint2* f3, float* n1_sm, float* qe_sm) {
     uint32_t raw[D / 16][2];
     pc_load_raw<D>(R, Qu, octet, lane, raw);
     uint32_t mx = 0u;
@@ -195,7 +214,8 @@ __device__ __forceinline__ bool pc_load_frag(const PcRows& R, const bf16_t* Qu, 
     const float c = split_query_const(ok ? __uint_as_float(m16 << 16) : 1.f);
     float n1 = 0.f, n2 = 0.f, n3 = 0.f;
 #pragma unroll
-    for (int kk = 0; kk < D / 16; ++kk)
+    for (int kk = 0; kk < D / 16; ++kk) {
+        uint32_t b[2][3];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             float a[2] = {__uint_as_float(raw[kk][h] << 16), __uint_as_float(raw[kk][h] & 0xffff0000u)}, x1[2], x2[2], x3[2];
@@ -204,21 +224,115 @@ __device__ __forceinline__ bool pc_load_frag(const PcRows& R, const bf16_t* Qu, 
                 split_query(a[e], c, x1[e], x2[e], x3[e]);
                 n1 += fabsf(a[e]); n2 += fabsf(x2[e]); n3 += fabsf(x3[e]);
             }
-            f.b1[kk][h] = (__float_as_uint(x1[0]) >> 16) | (__float_as_uint(x1[1]) & 0xffff0000u);   // exact: bf16 numbers
-            f.b2[kk][h] = (__float_as_uint(x2[0]) >> 16) | (__float_as_uint(x2[1]) & 0xffff0000u);
-            f.b3[kk][h] = (__float_as_uint(x3[0]) >> 16) | (__float_as_uint(x3[1]) & 0xffff0000u);
+            b[h][0] = (__float_as_uint(x1[0]) >> 16) | (__float_as_uint(x1[1]) & 0xffff0000u);   // exact: bf16 numbers
+            b[h][1] = (__float_as_uint(x2[0]) >> 16) | (__float_as_uint(x2[1]) & 0xffff0000u);
+            b[h][2] = (__float_as_uint(x3[0]) >> 16) | (__float_as_uint(x3[1]) & 0xffff0000u);
         }
+        f12[kk * 32 + lane] = make_uint4(b[0][0], b[1][0], b[0][1], b[1][1]);
+        f3[kk * 32 + lane] = make_uint2(b[0][2], b[1][2]);
+    }
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) {
         n1 += __shfl_xor_sync(0xffffffffu, n1, o);
         n2 += __shfl_xor_sync(0xffffffffu, n2, o);
         n3 += __shfl_xor_sync(0xffffffffu, n3, o);
     }
-    if ((lane & 3) == 0) {                                    // the same values from every warp that holds the octet
+    if ((lane & 3) == 0 && 8 * octet < (R.rows + 7) / 8 * 8) {
         n1_sm[8 * octet + (lane >> 2)] = n1 * 1.0001f;
         qe_sm[8 * octet + (lane >> 2)] = split_error(n1, n2, n3);
     }
     return ok;
+}
+
+// exp(s) of 16 keys against N octets of rows, added to z[octet][row pair's two]; `last`: the tile may hold keys that a row
+// does not see or that do not exist (qpos: the rows' positions). Returns the largest high word of |s|.
+template <int D, int N>
+__device__ __forceinline__ uint32_t pc_tile_sums(uint32_t arow, SplitGrid g, int lane, const uint4* f12, const uint2* f3, int j0, int k_end, bool last,
+                                                 const PcRows& R, int row0, double (*z)[2]) {
+    float hi[N][4], mid[N][4], lo[N][4];
+#pragma unroll
+    for (int o = 0; o < N; ++o)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) hi[o][x] = mid[o][x] = lo[o][x] = 0.f;
+#pragma unroll
+    for (int kk = 0; kk < D / 16; ++kk) {
+        uint32_t a[4], k1[4], k2[4], r2[4];
+        ldmatrix_x4(a, arow + (((kk * 2 + (lane >> 4)) ^ (lane & 7)) << 4));
+        split_key(a, g, k1, k2, r2);
+#pragma unroll
+        for (int o = 0; o < N; ++o) {
+            const uint4 b = f12[(o * (D / 16) + kk) * 32 + lane];
+            const uint2 b3 = f3[(o * (D / 16) + kk) * 32 + lane];
+            float t[4] = {0.f, 0.f, 0.f, 0.f};
+            mma16816(hi[o], k1, b.x, b.y);
+            mma16816(t, k2, b.z, b.w);
+            mma16816(mid[o], k1, b.z, b.w);
+            mma16816(t, r2, b.x, b.y);
+            mma16816(mid[o], k2, b.x, b.y);
+            mma16816(t, r2, b.z, b.w);
+            mma16816(t, k1, b3.x, b3.y);
+#pragma unroll
+            for (int x = 0; x < 4; ++x) lo[o][x] += t[x];
+        }
+    }
+    uint32_t top = 0u;
+    const double inv_root_d = inv_root_dim(D);
+#pragma unroll
+    for (int o = 0; o < N; ++o)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const double s = (((double)hi[o][x] + (double)mid[o][x]) + (double)lo[o][x]) * inv_root_d;
+            double e = exp_nonpos(s);
+            uint32_t h = (uint32_t)__double2hiint(s) & 0x7fffffffu;
+            if (last) {                                       // causal row: keys 1..position of the query
+                const int j = j0 + (lane >> 2) + (x >> 1) * 8;
+                if (j >= k_end || j >= R.pos(row0 + o * 8 + 2 * (lane & 3) + (x & 1))) { e = 0.0; h = 0u; }
+            }
+            top = max(top, h);
+            z[o][x & 1] += e;
+        }
+    return top;
+}
+
+// largest magnitude (bf16 bits) of a 16-key tile, by the warp that works on it
+template <int D>
+__device__ __forceinline__ uint32_t pc_tile_amax(const unsigned char* tile, int lane) {
+    uint32_t m = 0u;
+#pragma unroll
+    for (int x = 0; x < D / 16; ++x) {
+        const uint4 v = *reinterpret_cast<const uint4*>(tile + (x * 32 + lane) * 16);
+        m = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(m, v.x), v.y), v.z), v.w);
+    }
+    return __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16));
+}
+
+__device__ __forceinline__ void pc_leave_open(uint32_t* flags, PcMisc* misc, int row, int j) {
+    atomicOr(flags + (row >> 5), 1u << (row & 31));
+    const int at = atomicAdd(&misc->n_open, 1);
+    if (at < kPcOpenCap) misc->open[at] = make_int2(row, j);
+}
+
+// Verdicts that the bounds leave open, by a whole warp: bit x of `open` = key j0 + lane / 4 + 8 (x / 2) against row
+// row0 + 2 (lane % 4) + x % 2. Adds to the lane's marks what is sure; rows whose threshold is too close are flagged.
+template <typename T, int D>
+__device__ __noinline__ void pc_open_verdicts(const PromptParams& p, const PcRows& R, const T* Qu, const T* Ku, int j0, int row0, uint32_t open,
+                                              const double* thr_sm, const float* qe_sm, double eps_unit, uint32_t* flags, PcMisc* misc, uint32_t (&mark)[2]) {
+    const int lane = threadIdx.x & 31;
+    int n_near = 0;
+    for (int x = 0; x < 4; ++x) {
+        uint32_t who = __ballot_sync(0xffffffffu, (open >> x) & 1u);
+        n_near += __popc(who);
+        while (who) {
+            const int src = __ffs(who) - 1;
+            who &= who - 1u;
+            const int j = j0 + (src >> 2) + (x >> 1) * 8, row = row0 + 2 * (src & 3) + (x & 1);
+            const double s = warp_exact_dot<T, D>(R.q<T, D>(Qu, row), Ku + (size_t)j * D, lane) * inv_root_dim(D);
+            const double th = thr_sm[row], e = eps_unit * (double)qe_sm[row] + 1e-13 * (1.0 + fabs(th));
+            if (lane == src && s - th > e) mark[x >> 1] = pc_join(p.w, mark[x >> 1], pc_mark(p.w, R.rho(row), R.pos(row)));
+            if (lane == 0 && fabs(s - th) <= e) pc_leave_open(flags, misc, row, j);   // to the exact rows
+        }
+    }
+    if (lane == 0) atomicAdd(p.counters + CNT_NEAR, (unsigned long long)n_near);
 }
 
 template <typename T, int D>
@@ -228,10 +342,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     const PromptParams& p = pp.p;
     constexpr bool kBf16 = Elem<T>::kBytes == 2;
     constexpr int kRow = D * Elem<T>::kBytes, kChunks = kRow / 16;
-    constexpr int kRowUnit = kBf16 ? 8 : 4;                   // rows a warp works on at a time
-    constexpr int kKeyUnit = kBf16 ? 16 : 32;                 // keys
-    constexpr int kSubs = kPcKeys / kKeyUnit;                 // key units per buffer
-    constexpr int kBufs = pc_bufs<T, D>();
+    constexpr int kSubs = kPcKeys / 32;                       // fp32: units of 32 keys per buffer
     const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int cs = (int)cluster_size(), rank = (int)cluster_rank();
     asm volatile("griddepcontrol.wait;" ::: "memory");        // prompt_begin_kernel, and what precedes it on the stream
@@ -252,6 +363,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         return;
     }
     const PcSmem lay = pc_smem_layout<T, D>(pp.rows8);
+    const int n_buf = pc_bufs<T, D>(pp.rows8);
     double* zs = reinterpret_cast<double*>(smem + lay.zs);
     double* thr_sm = reinterpret_cast<double*>(smem + lay.thr);
     float* n1_sm = reinterpret_cast<float*>(smem + lay.n1);
@@ -266,7 +378,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     uint32_t* keep_g = p.keepmask + (size_t)u * keepmask_words(p.C) + w0;            // the block's keep bits
     const int k_begin = w0 * 32, k_end = min(P, w1 * 32), n_keys = max(0, k_end - k_begin);
     const int nc = (n_keys + kPcKeys - 1) / kPcKeys;
-    const bool resident = nc <= kBufs;
+    const bool resident = nc <= n_buf;                        // the block's keys stay on chip for all passes over them
     const T* Ku = reinterpret_cast<const T*>(p.k_prompt) + (size_t)u * p.p_max * D;
     const T* Vu = reinterpret_cast<const T*>(p.v_prompt) + (size_t)u * p.p_max * D;
     const T* Qu = reinterpret_cast<const T*>(p.q_last) + ((size_t)u << pp.log2g) * w * D;
@@ -274,9 +386,12 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     const double inv_root_d = inv_root_dim(D), root_d = D == 128 ? 11.313708498984760390 : 8.0;
     const uint32_t ring = smem_addr(smem + lay.ring);
 
-    auto issue = [&](int c) {                                 // chunk c of the block's keys -> its ring buffer
-        if (c < nc) {
-            const uint32_t dst = ring + (c % kBufs) * (kPcKeys * kRow);
+    // Passes over the block's keys take numbered steps, step s = chunk s % nc in ring buffer s % n_buf (a resident block
+    // loads every chunk once). Loads run n_buf - 1 steps ahead, `end` steps in all.
+    auto issue = [&](int step, int end) {
+        if (step < end) {
+            const int c = step % nc;
+            const uint32_t dst = ring + (step % n_buf) * (kPcKeys * kRow);
             const unsigned char* src = reinterpret_cast<const unsigned char*>(Ku + (size_t)(k_begin + c * kPcKeys) * D);
             const int valid = n_keys - c * kPcKeys;
 #pragma unroll 4
@@ -288,135 +403,135 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         }
         cp_async_commit();
     };
-    auto measure = [&](int c) {                               // largest magnitude of every 16-key tile of a buffer (warp = tile)
-        const unsigned char* buf = smem + lay.ring + (c % kBufs) * (kPcKeys * kRow);
-        uint32_t m = 0u;
-#pragma unroll
-        for (int x = 0; x < kChunks / 2; ++x) {
-            const uint4 v = *reinterpret_cast<const uint4*>(buf + warp * 16 * kRow + (x * 32 + lane) * 16);
-            m = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(m, v.x), v.y), v.z), v.w);
-        }
-        m = __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16));
-        if (lane == 0) { misc->tile_amax[(c % kBufs) * (kPcKeys / 16) + warp] = (uint16_t)m; atomicMax(&misc->amax, m); }
+    auto start = [&](int end) { for (int i = 0; i < n_buf - 1; ++i) issue(i, end); };
+    // waits for the step's chunk and starts the load n_buf - 1 steps on; returns the chunk's buffer
+    auto arrive = [&](int step, int end) -> const unsigned char* {
+        if (n_buf == 3) cp_async_wait<1>(); else cp_async_wait<0>();
+        __syncthreads();                                      // the chunk is in; everybody is done with the buffer that is filled next
+        issue(step + n_buf - 1, end);
+        return smem + lay.ring + (resident ? step % nc : step % n_buf) * (kPcKeys * kRow);
     };
-#pragma unroll
-    for (int i = 0; i < kBufs - 1; ++i) issue(i);
+    const int n_oct = pp.rows8 / 8;
+    const int n_grp = kBf16 ? (n_oct + kPcGroup - 1) / kPcGroup : 1;                 // passes of phase A
+    const int end_a = resident ? nc : n_grp * nc;
+    start(end_a);
     for (int i = tid; i < (pp.rows8 + 31) / 32; i += kPcThreads) flags[i] = 0u;
-    if (tid == 0) { misc->bad = 0; misc->amax = 0u; misc->fail = 0; }
+    if (tid == 0) { misc->bad = 0; misc->amax = 0u; misc->fail = 0; misc->n_open = 0; }
 
-    // who works on what: warps own row units where there are at least as many, otherwise they share them by key units
-    const int n_ru = (R.rows + kRowUnit - 1) / kRowUnit;
+    // ---- A. sums of exp(s) per row ----
+    bool bad = false;
+    // fp32: warps own units of four rows where there are at least as many, otherwise they share them by key units
+    const int n_ru = (R.rows + 3) / 4;
     int ru_slots = 1;                                         // warps side by side over the row units (a power of two)
     while (ru_slots < n_ru && ru_slots < kPcWarps) ru_slots *= 2;
     const int key_groups = min(kPcWarps / ru_slots, kSubs);
     const int my_ru = warp % ru_slots, my_kg = warp / ru_slots;
     const bool works = my_ru < n_ru && my_kg < key_groups;
-    const bool keep_rows = n_ru <= ru_slots;                  // a warp has one row unit at most: its pieces stay in registers
-
-    // ---- A. sums of exp(s) per row ----
-    bool bad = false;
-    {
-        PcFrag<kBf16 ? D : 16> f;
-        double z[4] = {0.0, 0.0, 0.0, 0.0};                   // bf16: rows 2 (lane % 4), + 1 of the octet; fp32: the four rows
-        double* qst = reinterpret_cast<double*>(smem + lay.stage) + warp * 4 * D;      // fp32: the rows as doubles
-        for (int i = tid; i < max(pp.rows8, 64); i += kPcThreads) zs[i] = 0.0;
-        auto fold = [&](int ru) {                             // the warp's lanes -> its slots of zs
-            if constexpr (kBf16) {
+    const bool keep_rows = n_ru <= ru_slots;                  // a warp has one row unit at most: it stays staged
+    double* qst = reinterpret_cast<double*>(smem + lay.stage) + warp * 4 * D;        // fp32: the rows as doubles
+    auto stage_rows = [&](int ru) {
+        __syncwarp();
+        for (int x = lane; x < 4 * D; x += 32) {
+            const int r = ru * 4 + x / D;
+            qst[x] = R.pos(r) ? (double)Elem<T>::load(R.q<T, D>(Qu, r) + x % D) : 0.0;
+        }
+        __syncwarp();
+    };
+    auto dot4 = [&](const unsigned char* buf, int kr, double (&acc)[4]) {           // the staged rows against key kr of the buffer
 #pragma unroll
-                for (int o = 4; o < 32; o <<= 1) { z[0] += __shfl_xor_sync(0xffffffffu, z[0], o); z[1] += __shfl_xor_sync(0xffffffffu, z[1], o); }
-                if (lane < 4) {
-                    double* dst = zs + my_kg * (n_ru * kRowUnit) + ru * kRowUnit + 2 * lane;
-                    dst[0] += z[0]; dst[1] += z[1];
-                }
-            } else {
+        for (int x = 0; x < 4; ++x) acc[x] = 0.0;
+#pragma unroll 4
+        for (int ch = 0; ch < kChunks; ++ch) {
+            const float4 kv = *reinterpret_cast<const float4*>(buf + pc_offset<T, D>(kr, ch));
+            const double k4[4] = {(double)kv.x, (double)kv.y, (double)kv.z, (double)kv.w};
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const double t = warp_sum(z[x]);
-                    if (lane == 0) zs[my_kg * (n_ru * kRowUnit) + ru * kRowUnit + x] += t;
+            for (int x = 0; x < 4; ++x) {
+                const double2 qa = *reinterpret_cast<const double2*>(qst + x * D + ch * 4);
+                const double2 qb = *reinterpret_cast<const double2*>(qst + x * D + ch * 4 + 2);
+                acc[x] = fma(qa.x, k4[0], acc[x]); acc[x] = fma(qa.y, k4[1], acc[x]);
+                acc[x] = fma(qb.x, k4[2], acc[x]); acc[x] = fma(qb.y, k4[3], acc[x]);
+            }
+        }
+    };
+    uint4* f12 = reinterpret_cast<uint4*>(smem + lay.frag);
+    if constexpr (kBf16) {
+        // A group of four octets of rows at a time: its pieces are made once and stay on chip while the block's keys pass;
+        // a warp takes one tile of every chunk, cuts it into pieces once per two octets and keeps its rows' sums in
+        // registers to the end of the pass.
+        uint32_t top = 0u;
+        for (int grp = 0; grp < n_grp; ++grp) {
+            const int oct0 = grp * kPcGroup, cnt = min(kPcGroup, n_oct - oct0), n_even = n_oct == 1 ? 1 : (cnt + 1) / 2 * 2;
+            uint2* f3 = reinterpret_cast<uint2*>(f12 + (n_oct == 1 ? 1 : min((n_oct + 1) / 2 * 2, kPcGroup)) * (D / 16) * 32);
+            if (grp) __syncthreads();                         // everybody is done with the group before
+            if (warp < n_even)
+                bad |= !pc_store_pieces<D>(R, Qu, oct0 + warp, lane, f12 + warp * (D / 16) * 32, f3 + warp * (D / 16) * 32, n1_sm, qe_sm);
+            double z[kPcGroup][2];
+#pragma unroll
+            for (int o = 0; o < kPcGroup; ++o) z[o][0] = z[o][1] = 0.0;
+            if (nc == 0) __syncthreads();
+            for (int c = 0; c < nc; ++c) {
+                const unsigned char* buf = arrive(grp * nc + c, end_a);
+                const int n_valid = min(kPcKeys, n_keys - c * kPcKeys), j0 = k_begin + c * kPcKeys + warp * 16;
+                if (warp * 16 >= n_valid) continue;
+                const uint32_t am = pc_tile_amax<D>(buf + warp * 16 * kRow, lane);
+                if (grp == 0 && lane == 0) atomicMax(&misc->amax, am);
+                const SplitGrid g = split_grid(am);
+                const uint32_t arow = smem_addr(buf) + (warp * 16 + (lane & 15)) * kRow;
+                const bool last = j0 + 16 > k_end || j0 + 16 > P - w + 1;
+                if (n_oct == 1) {
+                    top = max(top, pc_tile_sums<D, 1>(arow, g, lane, f12, f3, j0, k_end, last, R, 0, z));
+                } else {
+                    top = max(top, pc_tile_sums<D, 2>(arow, g, lane, f12, f3, j0, k_end, last, R, oct0 * 8, z));
+                    if (cnt > 2)
+                        top = max(top, pc_tile_sums<D, 2>(arow, g, lane, f12 + 2 * (D / 16) * 32, f3 + 2 * (D / 16) * 32, j0, k_end, last, R, oct0 * 8 + 16, z + 2));
                 }
             }
-            z[0] = z[1] = z[2] = z[3] = 0.0;
+#pragma unroll
+            for (int o = 0; o < kPcGroup; ++o) {
+#pragma unroll
+                for (int x = 4; x < 32; x <<= 1) { z[o][0] += __shfl_xor_sync(0xffffffffu, z[o][0], x); z[o][1] += __shfl_xor_sync(0xffffffffu, z[o][1], x); }
+                if (lane < 4) { misc->zw[warp][o * 8 + 2 * lane] = z[o][0]; misc->zw[warp][o * 8 + 2 * lane + 1] = z[o][1]; }
+            }
+            __syncthreads();
+            if (tid < cnt * 8) {
+                double t = 0.0;
+                for (int x = 0; x < kPcWarps; ++x) t += misc->zw[x][tid];
+                zs[oct0 * 8 + tid] = t;
+            }
+        }
+        bad |= top >= (uint32_t)__double2hiint(kPcLogitLimit);
+    } else {
+        double z[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int i = tid; i < max(pp.rows8, 64); i += kPcThreads) zs[i] = 0.0;
+        auto fold = [&](int ru) {                             // the warp's lanes -> its slots of zs
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const double t = warp_sum(z[x]);
+                if (lane == 0) zs[my_kg * (n_ru * 4) + ru * 4 + x] += t;
+                z[x] = 0.0;
+            }
         };
         bool have = false;
         for (int c = 0; c < nc; ++c) {
-            cp_async_wait<kBufs - 2>();
-            __syncthreads();                                  // chunk c is in; everybody is done with chunk c - 1
-            issue(c + kBufs - 1);
-            const unsigned char* buf = smem + lay.ring + (c % kBufs) * (kPcKeys * kRow);
-            if constexpr (kBf16) { measure(c); __syncthreads(); }
+            const unsigned char* buf = arrive(c, end_a);
             const int n_valid = min(kPcKeys, n_keys - c * kPcKeys);
             if (works)
                 for (int ru = my_ru; ru < n_ru; ru += ru_slots) {
-                    if (!keep_rows || !have) {
-                        if constexpr (kBf16) {
-                            bad |= !pc_load_frag<D>(R, Qu, ru, lane, f, n1_sm, qe_sm);
-                        } else {
-                            __syncwarp();
-                            for (int x = lane; x < 4 * D; x += 32) {
-                                const int r = ru * 4 + x / D;
-                                qst[x] = R.pos(r) ? (double)Elem<T>::load(R.q<T, D>(Qu, r) + x % D) : 0.0;
-                            }
-                            __syncwarp();
-                        }
-                        have = true;
-                    }
-                    const int r0 = ru * kRowUnit + (kBf16 ? 2 * (lane & 3) : 0);
-                    int qpos[kBf16 ? 2 : 4];
+                    if (!keep_rows || !have) stage_rows(ru);
+                    have = true;
+                    int qpos[4];
 #pragma unroll
-                    for (int x = 0; x < (kBf16 ? 2 : 4); ++x) qpos[x] = R.pos(r0 + x);
-                    for (int sub = my_kg; sub < kSubs && sub * kKeyUnit < n_valid; sub += key_groups) {
-                        const int j0 = k_begin + c * kPcKeys + sub * kKeyUnit;       // 0-based key index
-                        if constexpr (kBf16) {
-                            const SplitGrid g = split_grid(misc->tile_amax[(c % kBufs) * (kPcKeys / 16) + sub]);
-                            float hi[4] = {0.f, 0.f, 0.f, 0.f}, mid[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-                            const uint32_t arow = ring + (c % kBufs) * (kPcKeys * kRow) + (sub * 16 + (lane & 15)) * kRow;
+                    for (int x = 0; x < 4; ++x) qpos[x] = R.pos(ru * 4 + x);
+                    for (int sub = my_kg; sub < kSubs && sub * 32 < n_valid; sub += key_groups) {
+                        double acc[4];
+                        dot4(buf, sub * 32 + lane, acc);
+                        const int j = k_begin + c * kPcKeys + sub * 32 + lane;
 #pragma unroll
-                            for (int kk = 0; kk < D / 16; ++kk) {
-                                uint32_t a[4], k1[4], k2[4], r2[4];
-                                ldmatrix_x4(a, arow + (((kk * 2 + (lane >> 4)) ^ (lane & 7)) << 4));
-                                split_key(a, g, k1, k2, r2);
-                                float t[4] = {0.f, 0.f, 0.f, 0.f};
-                                mma16816(hi, k1, f.b1[kk][0], f.b1[kk][1]);
-                                mma16816(mid, k1, f.b2[kk][0], f.b2[kk][1]);
-                                mma16816(t, k2, f.b2[kk][0], f.b2[kk][1]);
-                                mma16816(mid, k2, f.b1[kk][0], f.b1[kk][1]);
-                                mma16816(t, r2, f.b1[kk][0], f.b1[kk][1]);
-                                mma16816(t, r2, f.b2[kk][0], f.b2[kk][1]);
-                                mma16816(t, k1, f.b3[kk][0], f.b3[kk][1]);
-#pragma unroll
-                                for (int x = 0; x < 4; ++x) lo[x] += t[x];
-                            }
-#pragma unroll
-                            for (int x = 0; x < 4; ++x) {
-                                const int j = j0 + (lane >> 2) + (x >> 1) * 8;
-                                const double s = (((double)hi[x] + (double)mid[x]) + (double)lo[x]) * inv_root_d;
-                                const bool on = j < k_end && j < qpos[x & 1];           // causal row: keys 1..position of the query
-                                bad |= on && !(fabs(s) < kPcLogitLimit);
-                                z[x & 1] += on ? exp_nonpos(s) : 0.0;
-                            }
-                        } else {
-                            double acc[4] = {0.0, 0.0, 0.0, 0.0};
-                            const int kr = sub * 32 + lane;
-#pragma unroll 4
-                            for (int ch = 0; ch < kChunks; ++ch) {
-                                const float4 kv = *reinterpret_cast<const float4*>(buf + pc_offset<T, D>(kr, ch));
-                                const double k4[4] = {(double)kv.x, (double)kv.y, (double)kv.z, (double)kv.w};
-#pragma unroll
-                                for (int x = 0; x < 4; ++x) {
-                                    const double2 qa = *reinterpret_cast<const double2*>(qst + x * D + ch * 4);
-                                    const double2 qb = *reinterpret_cast<const double2*>(qst + x * D + ch * 4 + 2);
-                                    acc[x] = fma(qa.x, k4[0], acc[x]); acc[x] = fma(qa.y, k4[1], acc[x]);
-                                    acc[x] = fma(qb.x, k4[2], acc[x]); acc[x] = fma(qb.y, k4[3], acc[x]);
-                                }
-                            }
-                            const int j = j0 + lane;
-#pragma unroll
-                            for (int x = 0; x < 4; ++x) {
-                                const double s = acc[x] * inv_root_d;
-                                const bool on = j < k_end && j < qpos[x];
-                                bad |= on && !(fabs(s) < kPcLogitLimit);
-                                z[x] += on ? exp_nonpos(s) : 0.0;
-                            }
+                        for (int x = 0; x < 4; ++x) {
+                            const double s = acc[x] * inv_root_d;
+                            const bool on = j < k_end && j < qpos[x];               // causal row: keys 1..position of the query
+                            bad |= on && !(fabs(s) < kPcLogitLimit);
+                            z[x] += on ? exp_nonpos(s) : 0.0;
                         }
                     }
                     if (!keep_rows) fold(ru);
@@ -424,14 +539,13 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         }
         __syncthreads();
         if (works && keep_rows) fold(my_ru);
-        if constexpr (kBf16)                                  // a block without keys has no pieces yet, but the norms are asked for
-            if (nc == 0 && works) for (int ru = my_ru; ru < n_ru; ru += ru_slots) pc_load_frag<D>(R, Qu, ru, lane, f, n1_sm, qe_sm);
     }
     if (bad) misc->bad = 1;
     __syncthreads();
     if (kBf16 && tid == 0 && misc->amax >= kSplitMaxBits) misc->bad = 1;
-    for (int i = tid; i < n_ru * kRowUnit; i += kPcThreads)   // key groups of this block, in a fixed order
-        for (int x = 1; x < key_groups; ++x) zs[i] += zs[x * (n_ru * kRowUnit) + i];
+    if (!kBf16)
+        for (int i = tid; i < n_ru * 4; i += kPcThreads)      // key groups of this block, in a fixed order
+            for (int x = 1; x < key_groups; ++x) zs[i] += zs[x * (n_ru * 4) + i];
     cluster_sync();
 
     // ---- thresholds of Definition 3.1 in log form: s >= lse + ln(alpha) - ln(position of the query) ----
@@ -441,7 +555,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         any_bad |= (int)ld_peer_u32(map_rank(smem_addr(&misc->bad), x));
         amax_unit = max(amax_unit, ld_peer_u32(map_rank(smem_addr(&misc->amax), x)));
     }
-    for (int r = tid; r < n_ru * kRowUnit; r += kPcThreads) {
+    for (int r = tid; r < R.rows; r += kPcThreads) {
         const int qpos = R.pos(r);
         double Z = 0.0;
         for (int x = 0; x < cs; ++x) Z += ld_peer_f64(map_rank(smem_addr(zs + r), x));
@@ -452,104 +566,84 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     const double eps_unit = kBf16 ? p.bound_scale * (double)split_amax(amax_unit) * inv_root_d : 0.0;
 
     // ---- B. verdicts -> registers ----
-    if (!resident) {
+    const int n_grp_b = kBf16 ? (n_oct + kPcGroupB - 1) / kPcGroupB : 1;
+    const int end_b = resident ? 0 : n_grp_b * nc;
+    if (!resident) start(end_b);
+    if constexpr (kBf16) {
+        uint2* fr = reinterpret_cast<uint2*>(f12);
+        for (int grp = 0; grp < n_grp_b; ++grp) {
+            const int oct0 = grp * kPcGroupB, cnt = min(kPcGroupB, n_oct - oct0);
+            __syncthreads();                                  // thresholds are there; everybody is done with the group before
+            if (warp < cnt) {
+                uint32_t raw[D / 16][2];
+                pc_load_raw<D>(R, Qu, oct0 + warp, lane, raw);
 #pragma unroll
-        for (int i = 0; i < kBufs - 1; ++i) issue(i);
-    }
-    for (int c = 0; c < nc; ++c) {
-        if (!resident) cp_async_wait<kBufs - 2>();
-        if (tid < kPcKeys) words_sm[tid] = 0u;
-        __syncthreads();
-        if (!resident) {
-            issue(c + kBufs - 1);
-            if constexpr (kBf16) { measure(c); __syncthreads(); }
-        }
-        const unsigned char* buf = smem + lay.ring + (c % kBufs) * (kPcKeys * kRow);
-        const int n_valid = min(kPcKeys, n_keys - c * kPcKeys);
-        if (works && !any_bad)
-            for (int ru = my_ru; ru < n_ru; ru += ru_slots) {
-                if constexpr (kBf16) {
-                    uint32_t q[D / 16][2];
-                    pc_load_raw<D>(R, Qu, ru, lane, q);
-                    const int r0 = ru * 8 + 2 * (lane & 3);
-                    float thr_f[2], err_f[2], slack[2];
-                    int qpos[2];
+                for (int kk = 0; kk < D / 16; ++kk) fr[(warp * (D / 16) + kk) * 32 + lane] = make_uint2(raw[kk][0], raw[kk][1]);
+            }
+            if (tid < cnt * 8) {
+                const int r = oct0 * 8 + tid;
+                const float tf = r < R.rows ? (float)(thr_sm[r] * root_d) : INFINITY;
+                misc->thr_f[tid] = tf;
+                // D roundings of 2^-23 on sums of at most A |q|_1 (a tenth of slack), the threshold's own rounding, and the
+                // threshold's error
+                misc->err_f[tid] = (float)p.bound_scale * ((float)D * 1.1f / 8388608.f * n1_sm[r]);
+                misc->slack[tid] = (tf < 3e38f ? fabsf(tf) : 0.f) * 2.4e-7f + (float)(eps_unit * qe_sm[r] * root_d) * 1.01f;
+            }
+            if (nc == 0) __syncthreads();
+            for (int c = 0; c < nc; ++c) {
+                const unsigned char* buf = arrive(grp * nc + c, end_b);
+                const int n_valid = min(kPcKeys, n_keys - c * kPcKeys), j0 = k_begin + c * kPcKeys + warp * 16;
+                if (warp * 16 >= n_valid) continue;
+                uint32_t mark[2] = {0u, 0u};                  // keys lane / 4 and lane / 4 + 8
+                if (!any_bad) {
+                    const float A = split_amax(pc_tile_amax<D>(buf + warp * 16 * kRow, lane));
+                    const uint32_t arow = smem_addr(buf) + (warp * 16 + (lane & 15)) * kRow;
+                    uint32_t a[D / 16][4];
 #pragma unroll
-                    for (int x = 0; x < 2; ++x) {
-                        qpos[x] = R.pos(r0 + x);
-                        thr_f[x] = (float)(thr_sm[r0 + x] * root_d);
-                        // D roundings of 2^-23 on sums of at most A |q|_1 (a tenth of slack), the threshold's own rounding,
-                        // and the threshold's error
-                        err_f[x] = (float)p.bound_scale * ((float)D * 1.1f / 8388608.f * n1_sm[r0 + x]);
-                        slack[x] = fabsf(thr_f[x]) * 2.4e-7f + (float)(eps_unit * qe_sm[r0 + x] * root_d) * 1.01f;
-                    }
-                    for (int sub = my_kg; sub < kSubs && sub * 16 < n_valid; sub += key_groups) {
-                        const int j0 = k_begin + c * kPcKeys + sub * 16;
-                        const float A = split_amax(misc->tile_amax[(c % kBufs) * (kPcKeys / 16) + sub]);
-                        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-                        const uint32_t arow = ring + (c % kBufs) * (kPcKeys * kRow) + (sub * 16 + (lane & 15)) * kRow;
+                    for (int kk = 0; kk < D / 16; ++kk) ldmatrix_x4(a[kk], arow + (((kk * 2 + (lane >> 4)) ^ (lane & 7)) << 4));
+                    for (int o = 0; o < cnt; ++o) {
+                        float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                         for (int kk = 0; kk < D / 16; ++kk) {
-                            uint32_t a[4];
-                            ldmatrix_x4(a, arow + (((kk * 2 + (lane >> 4)) ^ (lane & 7)) << 4));
-                            mma16816(acc, a, q[kk][0], q[kk][1]);
+                            const uint2 q = fr[(o * (D / 16) + kk) * 32 + lane];
+                            mma16816(kk & 1 ? acc2 : acc, a[kk], q.x, q.y);
                         }
-                        uint32_t mark[2] = {0u, 0u};          // keys lane / 4 and lane / 4 + 8
+                        const int r0 = o * 8 + 2 * (lane & 3);
+                        uint32_t open = 0u;
 #pragma unroll
                         for (int x = 0; x < 4; ++x) {
-                            const int j = j0 + (lane >> 2) + (x >> 1) * 8, row = r0 + (x & 1);
-                            const bool on = j < k_end && j < qpos[x & 1];
-                            const float margin = acc[x] - thr_f[x & 1], err = err_f[x & 1] * A + slack[x & 1];
-                            bool imp = on && margin >= err;
-                            uint32_t unsure = __ballot_sync(0xffffffffu, on && margin < err && margin > -err);
-                            if (unsure && lane == 0) atomicAdd(p.counters + CNT_NEAR, (unsigned long long)__popc(unsure));
-                            while (unsure) {                  // formed again in fp64, one after the other, by the whole warp
-                                const int src = __ffs(unsure) - 1;
-                                unsure &= unsure - 1u;
-                                const int js = __shfl_sync(0xffffffffu, j, src), rs = __shfl_sync(0xffffffffu, row, src);
-                                const double s = warp_exact_dot<T, D>(R.q<T, D>(Qu, rs), Ku + (size_t)js * D, lane) * inv_root_d;
-                                const double th = thr_sm[rs], e = eps_unit * (double)qe_sm[rs] + 1e-13 * (1.0 + fabs(th));
-                                if (lane == src) imp = s - th > e;                     // closer than that: left to the exact rows
-                                if (lane == 0 && fabs(s - th) <= e) atomicOr(flags + (rs >> 5), 1u << (rs & 31));
-                            }
-                            if (imp) mark[x >> 1] = pc_join(w, mark[x >> 1], pc_mark(w, R.rho(row), qpos[x & 1]));
+                            const int row = oct0 * 8 + r0 + (x & 1), qpos = R.pos(row), j = j0 + (lane >> 2) + (x >> 1) * 8;
+                            const float margin = (acc[x] + acc2[x]) - misc->thr_f[r0 + (x & 1)];
+                            const float err = misc->err_f[r0 + (x & 1)] * A + misc->slack[r0 + (x & 1)];
+                            const bool on = j < k_end && j < qpos;
+                            if (on && margin >= err) mark[x >> 1] = pc_join(w, mark[x >> 1], pc_mark(w, R.rho(row), qpos));
+                            else if (on && margin > -err) open |= 1u << x;
                         }
+                        if (__any_sync(0xffffffffu, open != 0u))
+                            pc_open_verdicts<T, D>(p, R, Qu, Ku, j0, oct0 * 8 + o * 8, open, thr_sm, qe_sm, eps_unit, flags, misc, mark);
+                    }
+                }
 #pragma unroll
-                        for (int y = 0; y < 2; ++y) {
-                            mark[y] = pc_join(w, mark[y], __shfl_xor_sync(0xffffffffu, mark[y], 1));
-                            mark[y] = pc_join(w, mark[y], __shfl_xor_sync(0xffffffffu, mark[y], 2));
-                            if ((lane & 3) == 0 && mark[y]) {
-                                uint32_t* dst = words_sm + sub * 16 + (lane >> 2) + y * 8;
-                                if (w <= 32) atomicOr(dst, mark[y]);
-                                else atomicMax(dst, mark[y]);
-                            }
-                        }
-                    }
-                } else {
-                    double* qst = reinterpret_cast<double*>(smem + lay.stage) + warp * 4 * D;
-                    if (!keep_rows) {
-                        __syncwarp();
-                        for (int x = lane; x < 4 * D; x += 32) {
-                            const int r = ru * 4 + x / D;
-                            qst[x] = R.pos(r) ? (double)Elem<T>::load(R.q<T, D>(Qu, r) + x % D) : 0.0;
-                        }
-                        __syncwarp();
-                    }
+                for (int y = 0; y < 2; ++y) {
+                    mark[y] = pc_join(w, mark[y], __shfl_xor_sync(0xffffffffu, mark[y], 1));
+                    mark[y] = pc_join(w, mark[y], __shfl_xor_sync(0xffffffffu, mark[y], 2));
+                    const int j = j0 + (lane >> 2) + y * 8;
+                    if ((lane & 3) == 0 && j < k_end) words_g[j] = grp ? pc_join(w, words_g[j], mark[y]) : mark[y];   // the same lane's
+                }
+            }
+        }
+    } else {
+        for (int c = 0; c < nc; ++c) {
+            if (tid < kPcKeys) words_sm[tid] = 0u;
+            const unsigned char* buf = arrive(c, end_b);
+            const int n_valid = min(kPcKeys, n_keys - c * kPcKeys);
+            if (works && !any_bad)
+                for (int ru = my_ru; ru < n_ru; ru += ru_slots) {
+                    if (!keep_rows) stage_rows(ru);
                     for (int sub = my_kg; sub < kSubs && sub * 32 < n_valid; sub += key_groups) {
-                        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                        double acc[4];
                         const int kr = sub * 32 + lane, j = k_begin + c * kPcKeys + kr;
-#pragma unroll 4
-                        for (int ch = 0; ch < kChunks; ++ch) {
-                            const float4 kv = *reinterpret_cast<const float4*>(buf + pc_offset<T, D>(kr, ch));
-                            const double k4[4] = {(double)kv.x, (double)kv.y, (double)kv.z, (double)kv.w};
-#pragma unroll
-                            for (int x = 0; x < 4; ++x) {
-                                const double2 qa = *reinterpret_cast<const double2*>(qst + x * D + ch * 4);
-                                const double2 qb = *reinterpret_cast<const double2*>(qst + x * D + ch * 4 + 2);
-                                acc[x] = fma(qa.x, k4[0], acc[x]); acc[x] = fma(qa.y, k4[1], acc[x]);
-                                acc[x] = fma(qb.x, k4[2], acc[x]); acc[x] = fma(qb.y, k4[3], acc[x]);
-                            }
-                        }
+                        dot4(buf, kr, acc);
                         uint32_t mark = 0u;
 #pragma unroll
                         for (int x = 0; x < 4; ++x) {
@@ -557,7 +651,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
                             if (j >= k_end || j >= qpos) continue;
                             const double margin = acc[x] * inv_root_d - thr_sm[row], e = 1e-13 * (1.0 + fabs(thr_sm[row]));
                             if (margin > e) mark = pc_join(w, mark, pc_mark(w, R.rho(row), qpos));
-                            else if (margin >= -e) atomicOr(flags + (row >> 5), 1u << (row & 31));   // a tie (a query at position 1): the exact rows
+                            else if (margin >= -e) pc_leave_open(flags, misc, row, j);               // a tie (a query at position 1)
                         }
                         if (mark) {
                             if (w <= 32) atomicOr(words_sm + kr, mark);
@@ -565,9 +659,9 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
                         }
                     }
                 }
-            }
-        __syncthreads();
-        if (tid < n_valid) words_g[k_begin + c * kPcKeys + tid] = words_sm[tid];
+            __syncthreads();
+            if (tid < n_valid) words_g[k_begin + c * kPcKeys + tid] = words_sm[tid];
+        }
     }
     __syncthreads();
 
@@ -605,7 +699,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         cluster_sync();
         for (int i = tid; i < (pp.rows8 + 31) / 32; i += kPcThreads) flags[i] = (uint32_t)__double_as_longlong(thr_sm[i]);
         __syncthreads();
-        pc_exact_rows<T, D>(p, R, Qu, Ku, k_begin, k_end, flags, words_g, misc, cs);
+        pc_exact_rows<T, D>(p, R, Qu, Ku, k_begin, k_end, any_bad != 0, flags, words_g, misc, cs);
         __syncthreads();
         keep_pass();
         cluster_sync();
