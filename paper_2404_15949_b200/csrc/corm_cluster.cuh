@@ -79,10 +79,13 @@ template <int NW> struct DcMisc {
     // largest key magnitude (bf16 bits), 1 << 16 if a magnitude is beyond the pieces' range, 1 << 17 if a wait expired,
     // 1 << 18 if the unit cannot take the token
     uint32_t state;
-    uint32_t flags;                               // heads to be formed exactly
+    struct alignas(16) Counts {                   // what the blocks tell one another after their verdicts
+        uint32_t flags;                           // heads to be formed exactly
+        int count, n_imp, pad;                    // kept slots and important keys of the block
+    } cnt;
     int n_open;                                   // open verdicts of marked heads: slot << 3 | head
     uint32_t open[kDcOpenCap];
-    int count, n_imp, n_moved;                    // kept slots and important keys of the block; row moves of the unit
+    int n_moved;                                  // row moves of the unit
     int scan[NW * 32];
 };
 constexpr uint32_t kDcBad = 1u << 16, kDcExpired = 1u << 17, kDcFull = 1u << 18;
@@ -102,6 +105,23 @@ __host__ __device__ inline DcSmem dc_smem_layout(int lcap) {
     s.logits = take(lcap * 4);
     s.total = off;
     return s;
+}
+
+// The GP (G of them, where an instance serves two group sizes) logits of one slot, stored side by side.
+template <int GP, bool kGlobal> __device__ __forceinline__ void load_logits(const float* src, int G, float (&out)[GP]) {
+    auto ld1 = [](const float* a) { if constexpr (kGlobal) return __ldcg(a); else return *a; };
+    if constexpr (GP % 4 == 0) {
+#pragma unroll
+        for (int h = 0; h < GP; h += 4) {
+            const float4* a = reinterpret_cast<const float4*>(src + h);
+            float4 v;
+            if constexpr (kGlobal) v = __ldcg(a); else v = *a;
+            out[h] = v.x; out[h + 1] = v.y; out[h + 2] = v.z; out[h + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int h = 0; h < GP; ++h) out[h] = h < G ? ld1(src + h) : 0.f;
+    }
 }
 
 // N contiguous elements of the cache past the L1 (rows move between launches that may overlap)
@@ -193,12 +213,12 @@ __device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G,
         }
         cluster_sync();                                       // everybody has read mz; the registers of this head are written
     }
-    if (added) atomicAdd(&misc->count, added);
-    if (added_imp) atomicAdd(&misc->n_imp, added_imp);
+    if (added) atomicAdd(&misc->cnt.count, added);
+    if (added_imp) atomicAdd(&misc->cnt.n_imp, added_imp);
 }
 
 // Verdicts that the error bounds leave open, by a whole warp: lane's slot j, heads `open`; true where a head is sure to
-// find the key important. Heads whose threshold is too close to tell are marked in misc->flags.
+// find the key important. Heads whose threshold is too close to tell are marked in misc->cnt.flags.
 template <typename T, int D, int NW>
 __device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int G, int j, uint32_t open, float eps_a, DcMisc<NW>* misc) {
     const int lane = threadIdx.x & 31;
@@ -220,7 +240,7 @@ __device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int 
             const double th = misc->thr[h], e = (double)(eps_a * misc->qe[h]) + 1e-13 * (1.0 + fabs(th));
             if (lane == src && s - th > e) imp = true;
             if (lane == 0 && fabs(s - th) <= e) {
-                atomicOr(&misc->flags, 1u << h);
+                atomicOr(&misc->cnt.flags, 1u << h);
                 const int at = atomicAdd(&misc->n_open, 1);
                 if (at < kDcOpenCap) misc->open[at] = ((uint32_t)js << 3) | (uint32_t)h;
             }
@@ -255,7 +275,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     if (tid == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&kmap)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&vmap)) : "memory");
-        misc->state = 0u; misc->flags = 0u; misc->count = 0; misc->n_imp = 0; misc->n_open = 0;
+        misc->state = 0u; misc->cnt.flags = 0u; misc->cnt.count = 0; misc->cnt.n_imp = 0; misc->n_open = 0;
     }
     if (lane == 0) {
 #pragma unroll
@@ -301,7 +321,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     if (tid == NT - 1) misc->log_t = log((double)t);
     // the block's slots: whole words, shared out evenly
     const int n_words = state ? 0 : (l + 31) >> 5;
-    const int w0 = (int)((long long)n_words * rank / cs), w1 = (int)((long long)n_words * (rank + 1) / cs);
+    auto word_begin = [&](int o) -> int { return (int)((uint32_t)(n_words * o) / (uint32_t)cs); };
+    const int w0 = word_begin(rank), w1 = word_begin(rank + 1);
     const int k_begin = w0 * 32, k_end = state ? 0 : min(l, w1 * 32), n_keys = max(0, k_end - k_begin);
     const int n_tiles = (n_keys + kDcKeys - 1) / kDcKeys;
     const int my_n = n_tiles > warp ? (n_tiles - warp + NW - 1) / NW : 0;       // tiles warp, warp + NW, ...
@@ -727,9 +748,15 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             const int i = base + k * NT + tid, j = k_begin + i;
             wv[k] = 0u; pv[k] = t;                            // the token appended by this step
             if (j < k_end && j < l_old) { wv[k] = __ldcg(wordu + j); pv[k] = __ldcg(posu + j); }
+        }
+        // (two branches: the addresses' space has to be known for one wide load per slot)
+        if (fits) {
+            const float* ls = reinterpret_cast<const float*>(smem + lay.logits);
 #pragma unroll
-            for (int h = 0; h < GP; ++h)
-                sv[k][h] = i < n_keys && h < G ? (fits ? lg[i * G + h] : __ldcg(lg + (size_t)i * G + h)) : 0.f;
+            for (int k = 0; k < kB; ++k) load_logits<GP, false>(ls + min(base + k * NT + tid, max(n_keys - 1, 0)) * G, G, sv[k]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < kB; ++k) load_logits<GP, true>(lg + (size_t)min(base + k * NT + tid, n_keys - 1) * G, G, sv[k]);
         }
     };
     __syncthreads();                                          // the appended slot's row, word and position are stored
@@ -737,7 +764,20 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     cluster_sync();                                           // every warp's record is complete (and the block's logits)
 
     // ---- thresholds of Definition 3.1 in log form, the same in every block: warp h reduces head h over the cluster's warps ----
-    const uint32_t unit_state = __reduce_max_sync(0xffffffffu, lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->state), lane)) : 0u);
+    constexpr int kEnt = kDcMaxCluster * NW / 32;             // (block, warp) entries per lane
+    float m[kEnt];
+    double z[kEnt];
+    auto load_entries = [&](int h) {
+#pragma unroll
+        for (int y = 0; y < kEnt; ++y) {
+            const int e = y * 32 + lane, blk = e / NW, w = e % NW;
+            m[y] = blk < cs ? __uint_as_float(ld_peer_u32(map_rank(smem_addr(&misc->wM[w][h]), blk))) : -INFINITY;
+            z[y] = blk < cs ? ld_peer_f64(map_rank(smem_addr(&misc->wZ[w][h]), blk)) : 0.0;
+        }
+    };
+    const uint32_t peer_state = lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->state), lane)) : 0u;
+    if (warp < G) load_entries(warp);                         // in one trip with the state
+    const uint32_t unit_state = __reduce_max_sync(0xffffffffu, peer_state);
     if (unit_state & (kDcExpired | kDcFull)) {                // the unit is left as it is
         cluster_sync();
         if (rank == 0 && tid == 0) {
@@ -752,15 +792,9 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     // error of a head's log-sum-exp per unit of qe (every logit of it is off by at most this much)
     const float eps_a = kBf16 ? split_amax(min(unit_state & 0xffffu, kSplitMaxBits)) * (float)inv_root_d * 1.0001f : 0.f;
     for (int h = warp; h < G; h += NW) {
-        constexpr int kEnt = kDcMaxCluster * NW / 32;         // (block, warp) entries per lane
-        float m[kEnt], M = -INFINITY;
-        double z[kEnt], Z = 0.0;
-#pragma unroll
-        for (int y = 0; y < kEnt; ++y) {
-            const int e = y * 32 + lane, blk = e / NW, w = e % NW;
-            m[y] = blk < cs ? __uint_as_float(ld_peer_u32(map_rank(smem_addr(&misc->wM[w][h]), blk))) : -INFINITY;
-            z[y] = blk < cs ? ld_peer_f64(map_rank(smem_addr(&misc->wZ[w][h]), blk)) : 0.0;
-        }
+        float M = -INFINITY;
+        double Z = 0.0;
+        if (h >= NW) load_entries(h);
 #pragma unroll
         for (int y = 0; y < kEnt; ++y) M = fmaxf(M, m[y]);
 #pragma unroll
@@ -797,6 +831,9 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         }
         __syncthreads();                                      // the other warps' records give way to the keep bits
         int n_imp = 0, n_keep = 0;
+        float tf[GP], sl[GP];
+#pragma unroll
+        for (int h = 0; h < GP; ++h) { tf[h] = h < G ? misc->thr_f[h] : INFINITY; sl[h] = h < G ? misc->slack[h] : 0.f; }
 #pragma unroll 1
         for (int base0 = 0; base0 < n_keys; base0 += kB * NT) {
             if (base0) load_regs(base0);
@@ -804,17 +841,16 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
 #pragma unroll
             for (int k = 0; k < kB; ++k) {
                 const int i = base0 + k * NT + tid;
-                open[k] = 0u;
-                if (i >= n_keys) continue;
+                bool sure = false;
+                uint32_t near = 0u;
 #pragma unroll
                 for (int h = 0; h < GP; ++h) {
-                    if (h >= G) continue;
-                    const float sf = sv[k][h], margin = sf - misc->thr_f[h];
-                    const float err = fabsf(sf) * 6.1e-8f + misc->slack[h];
-                    if (margin >= err) imp |= 1u << k;
-                    else if (margin > -err) open[k] |= 1u << h;
+                    const float sf = sv[k][h], margin = sf - tf[h], err = fmaf(fabsf(sf), 6.1e-8f, sl[h]);
+                    sure |= margin >= err;
+                    near |= margin > -err ? 1u << h : 0u;
                 }
-                if ((imp >> k) & 1u) open[k] = 0u;
+                open[k] = i < n_keys && !sure ? near : 0u;
+                imp |= i < n_keys && sure ? 1u << k : 0u;
             }
             uint32_t any_open = 0u;
 #pragma unroll
@@ -846,18 +882,31 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             }
         }
         if (lane == 0) {
-            atomicAdd(&misc->count, n_keep);
-            atomicAdd(&misc->n_imp, n_imp);
-            if (unit_state & kDcBad) atomicOr(&misc->flags, (1u << G) - 1u);    // magnitudes beyond the pieces' range: every head exactly
+            atomicAdd(&misc->cnt.count, n_keep);
+            atomicAdd(&misc->cnt.n_imp, n_imp);
+            if (unit_state & kDcBad) atomicOr(&misc->cnt.flags, (1u << G) - 1u);    // magnitudes beyond the pieces' range: every head exactly
         }
     }
     cluster_sync();
+    // the kept slots of the unit's word `wd`, from the block that owns it
+    auto peer_keep = [&](int wd) -> uint32_t {
+        const int o = (int)((uint32_t)((wd + 1) * cs - 1) / (uint32_t)n_words);    // the last o with word_begin(o) <= wd
+        return ld_peer_u32(map_rank(smem_addr(keep + (wd - word_begin(o))), o));
+    };
+    uint4 pc = make_uint4(0u, 0u, 0u, 0u);                    // a peer's counts
+    uint32_t last_keep = 0u;                                  // of the last 32 words, requested next to the counts
+    auto load_counts = [&]() {
+        if (lane < cs) pc = ld_peer_v4(map_rank(smem_addr(&misc->cnt), lane));
+        if (warp == 1 && n_words - 1 - lane >= 0) last_keep = peer_keep(n_words - 1 - lane);
+    };
+    load_counts();
     {
-        const uint32_t marks = __reduce_or_sync(0xffffffffu, lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->flags), lane)) : 0u);
+        const uint32_t marks = __reduce_or_sync(0xffffffffu, pc.x);
         if (marks) {                                          // uniform in the cluster
             cluster_sync();
             dc_exact_heads<T, D, NW>(p, u, G, t, k_begin, k_end, marks, (unit_state & kDcBad) != 0u, keep, misc, cs);
             cluster_sync();
+            load_counts();
         }
     }
     // outputs (Eq. 1): the unit's G x D values are shared out over the blocks, two channels per thread
@@ -882,21 +931,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     };
     // ---- 3. compaction: kept slots at or above the new length move into the holes below it ----
     // Hole number = evicted slots before it, mover number = kept slots behind it, so both follow from the blocks' counts.
-    // the kept slots of the unit's word `wd`, from the block that owns it
-    auto peer_keep = [&](int wd) -> uint32_t {
-        int o = 0;
-        while (o + 1 < cs && (int)((long long)n_words * (o + 1) / cs) <= wd) ++o;
-        return ld_peer_u32(map_rank(smem_addr(keep + (wd - (int)((long long)n_words * o / cs))), o));
-    };
-    uint32_t last_keep = 0u;                                  // of the last 32 words, requested next to the counts
-    if (warp == 1 && n_words - 1 - lane >= 0) last_keep = peer_keep(n_words - 1 - lane);
-    int before = 0, total = 0, imp_total = 0;
-    {
-        const int c = lane < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->count), lane)) : 0;
-        total = __reduce_add_sync(0xffffffffu, c);
-        before = __reduce_add_sync(0xffffffffu, lane < rank ? c : 0);
-        if (rank == 0) imp_total = __reduce_add_sync(0xffffffffu, lane < cs ? (int)ld_peer_u32(map_rank(smem_addr(&misc->n_imp), lane)) : 0);
-    }
+    const int total = __reduce_add_sync(0xffffffffu, (int)pc.y), before = __reduce_add_sync(0xffffffffu, lane < rank ? (int)pc.y : 0);
+    const int imp_total = rank == 0 && warp == 0 ? __reduce_add_sync(0xffffffffu, (int)pc.z) : 0;
     const int new_len = evict_on ? total : l;
     auto row_of = [&](int slot) -> size_t {
         return pt_u ? page_row(__ldcg(pt_u + (slot >> 5)), slot, p.pool_pages, p.status) : (size_t)u * p.C + (size_t)slot;
@@ -930,7 +966,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             }
         } else if (warp == 1) {
             const int first_w = new_len >> 5;                 // the unit's words that hold movers: [first_w, n_words), from the end
-            const int k_hi = k_begin < new_len ? k_lo + n_keys - misc->count : k_lo;
+            const int k_hi = k_begin < new_len ? k_lo + n_keys - misc->cnt.count : k_lo;
             int base = 0;
             for (int i0 = 0; n_words - 1 - i0 >= first_w; i0 += 32) {
                 const int wd = n_words - 1 - i0 - lane;
@@ -958,7 +994,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         }
         __syncthreads();
         const int n_moved = misc->n_moved;
-        const int mine = k_begin < new_len ? min(n_moved, k_lo + n_keys - misc->count) - k_lo : 0;
+        const int mine = k_begin < new_len ? min(n_moved, k_lo + n_keys - misc->cnt.count) - k_lo : 0;
         block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, movers, holes, mine, 0, 1, l, p.status);
     } else {
         write_outputs(tid, NT);
