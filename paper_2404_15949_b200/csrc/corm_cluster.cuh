@@ -469,6 +469,11 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         if (kmax >= kSplitMaxBits) { state |= kDcBad; kmax = kSplitMaxBits; }
         const SplitGrid g = split_grid(kmax);
         const int h0 = GP == 8 ? 2 * (lane & 3) : (lane & 3);                    // the thread's head(s)
+        // Lane offsets of the fragment loads inside a tile. Rows are 128 bytes and a tile starts on a multiple of 1024, so
+        // 16-byte chunk c of the lane's row (at c ^ row mod 8) is one exclusive-or away from chunk 0 or 1.
+        const uint32_t klane = (lane & 15) * 128 + (((lane >> 4) ^ (lane & 7)) << 4);
+        const uint32_t vlane = (((lane >> 4) << 3) + (lane & 7)) * 128 + ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
+        const uint32_t ring_a = smem_addr(ring);
         bool first = true;
         for (int it = 0; it < my_n; ++it) {
             const int j0 = k_begin + (warp + it * NW) * kDcKeys, n_valid = min(kDcKeys, k_end - j0);
@@ -480,9 +485,9 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             if (edge) patch_tile(ktile, j0, n_valid, 0, it);
             uint32_t a[KK][4];
             {
-                const uint32_t arow = smem_addr(ktile) + (lane & 15) * 128;
+                const uint32_t arow = ring_a + ks * S::kTile + klane;
 #pragma unroll
-                for (int kk = 0; kk < KK; ++kk) ldmatrix_x4(a[kk], arow + (kk >> 2) * S::kBox + ((((kk & 3) * 2 + (lane >> 4)) ^ (lane & 7)) << 4));
+                for (int kk = 0; kk < KK; ++kk) ldmatrix_x4(a[kk], (arow ^ ((kk & 3) << 5)) + (kk >> 2) * S::kBox);
             }
             __syncwarp();
             if (it + kKs < my_n) {                            // the whole tile is in registers: its stage is free
@@ -490,31 +495,33 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 if (lane == 0) { fence_async_smem(); issue(kmap, r0, ks); }
             }
             // sums of the products of pieces; see the head of the file
-            float x1[4] = {0.f, 0.f, 0.f, 0.f}, x2[4] = {0.f, 0.f, 0.f, 0.f}, x3[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-            float x4[4] = {0.f, 0.f, 0.f, 0.f};
+            float x1[4], x2[4], x3[4], x4[4], lo[4];
 #pragma unroll
             for (int kk = 0; kk < KK; ++kk) {
                 uint32_t k1[4], k2[4], r2[4];
                 split_key(a[kk], g, k1, k2, r2);
-                float tt[4] = {0.f, 0.f, 0.f, 0.f};
-                mma16816(x1, k1, b1[kk][0], b1[kk][1]);
-                mma16816(tt, r2, b1[kk][0], b1[kk][1]);
+                float tt[4];
+                auto mma = [&](float (&d)[4], const uint32_t (&x)[4], const uint32_t (&b)[2]) {   // the sum's first term, or one more
+                    if (kk == 0) mma16816_zero(d, x, b[0], b[1]); else mma16816(d, x, b[0], b[1]);
+                };
+                mma(x1, k1, b1[kk]);
+                mma16816_zero(tt, r2, b1[kk][0], b1[kk][1]);
                 if constexpr (GP == 8) {
-                    mma16816(x2, k1, b2[kk][0], b2[kk][1]);   // k1.q2 + k2.q1: exact together
+                    mma(x2, k1, b2[kk]);                      // k1.q2 + k2.q1: exact together
                     mma16816(x2, k2, b1[kk][0], b1[kk][1]);
-                    mma16816(x4, k2, b2[kk][0], b2[kk][1]);   // exact
+                    mma(x4, k2, b2[kk]);                      // exact
                     mma16816(tt, r2, b2[kk][0], b2[kk][1]);
-                    mma16816(x3, k1, b3[kk][0], b3[kk][1]);
+                    mma(x3, k1, b3[kk]);
                     mma16816(x3, k2, b3[kk][0], b3[kk][1]);
                 } else {
-                    mma16816(x2, k2, b1[kk][0], b1[kk][1]);
+                    mma(x2, k2, b1[kk]);
                     if constexpr (GP == 4) {
-                        mma16816(x3, k1, b2[kk][0], b2[kk][1]);
-                        mma16816(x4, k2, b2[kk][0], b2[kk][1]);
+                        mma(x3, k1, b2[kk]);
+                        mma(x4, k2, b2[kk]);
                     }
                 }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) lo[e] += tt[e];
+                for (int e = 0; e < 4; ++e) lo[e] = kk == 0 ? tt[e] : lo[e] + tt[e];
             }
             // Eq. 2's exponent, thread's keys lane / 4 and + 8
             double s[NK][NH];
@@ -568,12 +575,13 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 float hi_f[NH], lo_f[NH];
 #pragma unroll
                 for (int x = 0; x < NH; ++x) {
-                    const double ex = on[y][x] ? exp_nonpos(s[y][x] - (double)Mref[x]) : 0.0;
+                    const float sf = (float)s[y][x];
+                    const double ex = exp_nonpos_where(on[y][x] && sf - Mref[x] > -700.f, s[y][x] - (double)Mref[x]);
                     Zl[x] += ex;
                     const float pf = (float)ex;
                     hi_f[x] = __uint_as_float(pack_bf16x2(0.f, pf) << 16);
                     lo_f[x] = pf - hi_f[x];
-                    if (on[y][x]) lg[(j0 - k_begin + kq) * G + h0 + x] = (float)s[y][x];
+                    if (on[y][x]) lg[(j0 - k_begin + kq) * G + h0 + x] = sf;
                 }
                 if constexpr (GP == 8) {                      // [key][8 heads] high parts, then low parts
                     *reinterpret_cast<uint32_t*>(prob + kq * 16 + (lane & 3) * 4) = pack_bf16x2(hi_f[1 % NH], hi_f[0]);
@@ -588,12 +596,11 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             {
                 uint32_t bf[4];
                 ldmatrix_x4_trans(bf, smem_addr(prob) + (GP == 8 ? lane : lane & 15) * 16);       // keys 0-7 | 8-15 (| the low parts)
-                const int row = ((lane >> 4) << 3) + (lane & 7);
-                const uint32_t vrow = smem_addr(vtile) + row * 128;
+                const uint32_t vrow = ring_a + (kKs + vs) * S::kTile + vlane;
 #pragma unroll
                 for (int cb = 0; cb < D / 16; ++cb) {
                     uint32_t va[4];
-                    ldmatrix_x4_trans(va, vrow + (cb >> 2) * S::kBox + ((((cb & 3) * 2 + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
+                    ldmatrix_x4_trans(va, (vrow ^ ((cb & 3) << 5)) + (cb >> 2) * S::kBox);
                     mma16816(accd[cb], va, bf[0], bf[1]);     // Eq. 1
                     if constexpr (GP == 8) mma16816(accd[cb], va, bf[2], bf[3]);
                 }

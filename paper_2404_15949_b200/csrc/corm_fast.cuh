@@ -115,8 +115,7 @@ __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier
 // exp(x) for x <= ~0 (small positive arguments are fine), 0 below the normal range. Argument reduction by ln 2 in
 // two pieces, degree-11 Taylor polynomial on |r| <= ln2/2 (truncation ~6e-15 relative), scaling through the exponent.
 // Branch-free, so that several independent calls interleave.
-__device__ __forceinline__ double exp_nonpos(double x0) {
-    const double x = fmax(x0, -708.0);
+__device__ __forceinline__ double exp_reduced(double x) {
     const double t = fma(x, 1.4426950408889634074, 6755399441055744.0);   // round(x / ln 2) in the low word
     const int n = __double2loint(t);
     const double nf = t - 6755399441055744.0;
@@ -134,8 +133,16 @@ __device__ __forceinline__ double exp_nonpos(double x0) {
     p = fma(p, r, 0.5);
     p = fma(p, r, 1.0);
     p = fma(p, r, 1.0);
-    const double y = p * __hiloint2double((1023 + n) << 20, 0);
+    return p * __hiloint2double((1023 + n) << 20, 0);
+}
+__device__ __forceinline__ double exp_nonpos(double x0) {
+    const double y = exp_reduced(fmax(x0, -708.0));
     return x0 > -708.0 ? y : 0.0;
+}
+// the caller has seen to the range: exp(x) where `on` holds (which implies x > -708), else 0
+__device__ __forceinline__ double exp_nonpos_where(bool on, double x) {
+    const double y = exp_reduced(x);
+    return on ? y : 0.0;
 }
 
 __device__ __forceinline__ void unpack8_to_double(const uint4& raw, double (&kd)[8]) {
