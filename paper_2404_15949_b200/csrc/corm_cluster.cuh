@@ -17,12 +17,16 @@
 // fp32: a key per lane (its channels shared by two half-warps), fp64 products on the CUDA cores, P.V by fp32 FMAs.
 //
 // What bounds it: on units of a few hundred keys the chain of round trips (set-up 2 us, first tiles 2, exchange and
-// thresholds 3, verdicts 2, exchange 1, moves 2, launch 2); on long units HBM, shared out unevenly where units differ in
-// length. Measured, us per step from one call per step, before -> now:
-//   64 units x 970 keys, G 8, bf16          253 -> 32     128 units x 1090 keys, G 4, 64 channels   143 -> 30
-//   20 units x 250 keys, G 2, fp32           64 -> 16     8 units x 170 keys, G 1, fp32            37.7 -> 14
-//   128 units x 2800 keys, G 4, bf16         86 -> 68     32 units x 21400 keys, G 4, bf16          133 -> 103
-//   32 units x 8200 keys, G 4, no eviction   55 -> 47     32 units x 1160 keys, G 1, bf16            35 -> 24
+// thresholds 2.5, verdicts 1, exchange 1, moves 2, launch 2); on long units instruction issue in the streaming loop: about
+// 650 instructions per tile (192 of them the two-element additions that cut the keys), of 5000 cycles per tile and warp
+// with 16 warps on an SM only 270 are spent waiting for its copies. So one stage each for K and V is enough (with two for
+// K: 32 units x 8200 keys 43 us a step instead of 38), and what is smaller leaves more L1. Units differ in length and SMs
+// hold one block or two, which is what keeps the rest of HBM's rate away.
+// Measured, us per step from one call per step, before -> first version -> now:
+//   64 units x 970 keys, G 8, bf16          253 -> 32 -> 27     128 units x 1090 keys, G 4, 64 channels   143 -> 30 -> 26
+//   20 units x 250 keys, G 2, fp32           64 -> 16 -> 13     8 units x 170 keys, G 1, fp32            37.7 -> 14 -> 11
+//   128 units x 2800 keys, G 4, bf16         86 -> 68 -> 54     32 units x 21400 keys, G 4, bf16          133 -> 103 -> 80
+//   32 units x 8200 keys, G 4, no eviction   55 -> 47 -> 38     32 units x 1160 keys, G 1, bf16            35 -> 24 -> 20
 // (from one warp per key and the last-arriving split finishing the unit, from the balanced kernel and its verdict launch,
 // from the block-per-split kernel).
 //
@@ -55,9 +59,10 @@ template <typename T, int D, int GP> struct DcShape {
     static constexpr int kBoxes = kRow / 128;     // 128-byte wide boxes of the swizzled copies
     static constexpr int kBox = kDcKeys * 128;
     static constexpr int kTile = kDcKeys * kRow;
-    static constexpr int kKs = kTile >= 8192 ? 1 : kTile == 4096 ? 2 : 4;
+    static constexpr int kKs = kTile >= 4096 ? 1 : 2;
     static constexpr int kVs = kTile >= 4096 ? 1 : 2;
     static constexpr int kStages = kKs + kVs;
+    static constexpr int kPieces = GP == 8 ? 6 : GP == 4 ? 4 : 2;   // words per lane and 16 channels of the query pieces
     static constexpr int kWarpRing = kStages * kTile;
     static constexpr int kProb = kBf16 ? kDcKeys * (GP == 8 ? 32 : 16) : kDcKeys * GP * 4;   // a warp's probabilities
 };
@@ -76,6 +81,7 @@ template <int NW> struct DcMisc {
     double red[NW][2], mz[2];                     // exact heads
     float wM[NW][8];
     float sc[8][kDcMaxCluster * NW], qe[8], thr_f[8], slack[8];
+    float qe_part[NW][8];                         // the warps' shares of qe
     // largest key magnitude (bf16 bits), 1 << 16 if a magnitude is beyond the pieces' range, 1 << 17 if a wait expired,
     // 1 << 18 if the unit cannot take the token
     uint32_t state;
@@ -90,7 +96,7 @@ template <int NW> struct DcMisc {
 };
 constexpr uint32_t kDcBad = 1u << 16, kDcExpired = 1u << 17, kDcFull = 1u << 18;
 
-struct DcSmem { int prob, q, newrow, logits, bars, misc, total; };
+struct DcSmem { int prob, q, pieces, newrow, logits, bars, misc, total; };
 template <typename T, int D, int GP, int NW>
 __host__ __device__ inline DcSmem dc_smem_layout(int lcap) {
     using S = DcShape<T, D, GP>;
@@ -99,6 +105,7 @@ __host__ __device__ inline DcSmem dc_smem_layout(int lcap) {
     auto take = [&](int bytes) { int at = off; off = (off + bytes + 127) / 128 * 128; return at; };
     s.prob = take(NW * S::kProb);
     s.q = take(GP * D * (S::kBf16 ? 2 : 8));      // fp32: widened to fp64
+    s.pieces = take(S::kBf16 ? D / 16 * S::kPieces * 128 : 0);
     s.newrow = take(2 * S::kRow);
     s.bars = take(NW * S::kStages * 8);
     s.misc = take((int)sizeof(DcMisc<NW>));
@@ -390,9 +397,11 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     float* rec = reinterpret_cast<float*>(ring);              // the warp's record [G][D], once its tiles are done
 
     if constexpr (kBf16) {
-        // pieces of the queries, as B fragments: column n = lane / 4
-        constexpr int KK = D / 16;
+        // pieces of the queries, as B fragments (column n = lane / 4): every warp needs all of them, so a warp cuts the
+        // queries' channels 16 kk.. of kk = warp, warp + NW, ... and the others read them from shared memory
+        constexpr int KK = D / 16, kPieces = S::kPieces;
         uint32_t b1[KK][2], b2[GP == 2 ? 1 : KK][2], b3[GP == 8 ? KK : 1][2];
+        uint32_t* pieces = reinterpret_cast<uint32_t*>(smem + lay.pieces);      // [KK][kPieces / 2][32 lanes][2]
         {
             const int n = lane >> 2;
             const int hq = GP == 8 ? n : GP == 4 ? n >> 1 : (n & 3) >> 1;
@@ -400,23 +409,20 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             const uint32_t* src = reinterpret_cast<const uint32_t*>(smem + lay.q) + (on ? hq : 0) * (D / 2) + (lane & 3);
             uint32_t mx = 0u;
 #pragma unroll
-            for (int kk = 0; kk < KK; ++kk) {
-                b1[kk][0] = on ? src[kk * 8] : 0u;
-                b1[kk][1] = on ? src[kk * 8 + 4] : 0u;
-                mx = max_abs_bf16x2(max_abs_bf16x2(mx, b1[kk][0]), b1[kk][1]);
-            }
-            uint32_t m16 = max(mx & 0xffffu, mx >> 16);
+            for (int kk = 0; kk < KK; ++kk) mx = max_abs_bf16x2(max_abs_bf16x2(mx, src[kk * 8]), src[kk * 8 + 4]);
+            uint32_t m16 = on ? max(mx & 0xffffu, mx >> 16) : 0u;
             m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 1));
             m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 2));
             const bool ok = m16 < kSplitMaxBits;
             if (!ok) state |= kDcBad;
             const float c = split_query_const(ok ? __uint_as_float(m16 << 16) : 1.f);
             float n1 = 0.f, n2 = 0.f, n3 = 0.f;
-#pragma unroll
-            for (int kk = 0; kk < KK; ++kk)
+            for (int kk = warp; kk < KK; kk += NW) {
+                uint32_t w[kPieces];
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
-                    const float a[2] = {__uint_as_float(b1[kk][hf] << 16), __uint_as_float(b1[kk][hf] & 0xffff0000u)};
+                    const uint32_t raw = on ? src[kk * 8 + hf * 4] : 0u;
+                    const float a[2] = {__uint_as_float(raw << 16), __uint_as_float(raw & 0xffff0000u)};
                     uint32_t y1[2], y2[2], y3[2];
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
@@ -427,27 +433,46 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                     }
                     auto pack = [](const uint32_t (&y)[2]) { return (y[0] >> 16) | (y[1] & 0xffff0000u); };   // exact: bf16 numbers
                     if constexpr (GP == 8) {
-                        b1[kk][hf] = pack(y1); b2[kk][hf] = pack(y2); b3[kk][hf] = pack(y3);
+                        w[hf] = pack(y1); w[2 + hf] = pack(y2); w[4 + hf] = pack(y3);
                     } else if constexpr (GP == 4) {
-                        b1[kk][hf] = n & 1 ? pack(y2) : pack(y1);
-                        b2[kk][hf] = n & 1 ? 0u : pack(y3);
+                        w[hf] = n & 1 ? pack(y2) : pack(y1);
+                        w[2 + hf] = n & 1 ? 0u : pack(y3);
                     } else {
-                        b1[kk][hf] = n & 4 ? (n & 1 ? 0u : pack(y3)) : n & 1 ? pack(y2) : pack(y1);
+                        w[hf] = n & 4 ? (n & 1 ? 0u : pack(y3)) : n & 1 ? pack(y2) : pack(y1);
                     }
                 }
+#pragma unroll
+                for (int x = 0; x < kPieces; x += 2)
+                    *reinterpret_cast<uint2*>(pieces + ((kk * (kPieces / 2) + x / 2) * 32 + lane) * 2) = make_uint2(w[x], w[x + 1]);
+            }
 #pragma unroll
             for (int o = 1; o < 4; o <<= 1) {
                 n1 += __shfl_xor_sync(0xffffffffu, n1, o);
                 n2 += __shfl_xor_sync(0xffffffffu, n2, o);
                 n3 += __shfl_xor_sync(0xffffffffu, n3, o);
             }
-            // Error of a logit (before the 1/sqrt(d)) per unit of the unit's largest key magnitude A. r2.q: per 16 channels 17
-            // roundings of 2^-23 (a product of 16 terms and its accumulator; twice that for eight heads, whose two products
-            // share one) and 8 of 2^-24 in fp32, on terms of at most A/8192 |q|; k.q3: at most 2 * 8 * 17 roundings of 2^-23;
-            // r2.q3 <= A/8192 |q3| (left out for eight and four heads); the sum of the small parts (k2.q2 <= A/64 |q2|
-            // among them) rounds three times.
+            // Error of a logit (before the 1/sqrt(d)) per unit of the unit's largest key magnitude A, this warp's channels'
+            // share. r2.q: per 16 channels 17 roundings of 2^-23 (a product of 16 terms and its accumulator; twice that for
+            // eight heads, whose two products share one) and 8 of 2^-24 in fp32, on terms of at most A/8192 |q|; k.q3: at
+            // most 2 * 8 * 17 roundings of 2^-23; r2.q3 <= A/8192 |q3| (left out for eight and four heads); the sum of the
+            // small parts (k2.q2 <= A/64 |q2| among them) rounds three times.
             if (on && (lane & 3) == 0)
-                misc->qe[hq] = dp.bound_scale * 1.05f * ((GP == 8 ? 4.6e-6f : 2.6e-6f) * (n1 * 1.01f) * (1.f / 8192.f) + (3.3e-5f + 1.3e-4f) * n3 + 2.4e-7f * n2 * (1.f / 64.f));
+                misc->qe_part[warp][hq] = dp.bound_scale * 1.05f * ((GP == 8 ? 4.6e-6f : 2.6e-6f) * (n1 * 1.01f) * (1.f / 8192.f) + (3.3e-5f + 1.3e-4f) * n3 + 2.4e-7f * n2 * (1.f / 64.f));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < KK; ++kk) {
+            const uint2* src = reinterpret_cast<const uint2*>(pieces) + kk * (kPieces / 2) * 32 + lane;
+            const uint2 x = src[0];
+            b1[kk][0] = x.x; b1[kk][1] = x.y;
+            if constexpr (kPieces > 2) { const uint2 y = src[32]; b2[kk][0] = y.x; b2[kk][1] = y.y; }
+            if constexpr (kPieces > 4) { const uint2 z = src[64]; b3[kk][0] = z.x; b3[kk][1] = z.y; }
+        }
+        if (tid < G) {
+            float e = 0.f;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) e += misc->qe_part[w][tid];
+            misc->qe[tid] = e * 1.0001f;
         }
         float accd[D / 16][4];
 #pragma unroll
@@ -475,31 +500,36 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         const uint32_t vlane = (((lane >> 4) << 3) + (lane & 7)) * 128 + ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
         const uint32_t ring_a = smem_addr(ring);
         bool first = true;
-        for (int it = 0; it < my_n; ++it) {
-            const int j0 = k_begin + (warp + it * NW) * kDcKeys, n_valid = min(kDcKeys, k_end - j0);
+        // The tile that needs patching (keys past the block's end, or the appended slot, which is the unit's last) is the
+        // block's last one.
+        const int whole = k_end == l ? n_keys - 1 : n_keys;
+        float* lgp = lg + (warp * kDcKeys + (lane >> 2)) * G + h0;
+        int left = n_keys - warp * kDcKeys;                   // keys from the tile's first on
+        for (int it = 0; it < my_n; ++it, left -= NW * kDcKeys, lgp += NW * kDcKeys * G) {
+            const int n_valid = min(kDcKeys, left);
             const int ks = it % kKs, vs = it % kVs;
-            unsigned char* ktile = ring + ks * S::kTile;
-            unsigned char* vtile = ring + (kKs + vs) * S::kTile;
-            const bool edge = n_valid < kDcKeys || (l_old >= j0 && l_old < j0 + kDcKeys);
+            const bool edge = n_keys - left + kDcKeys > whole;
             if (!failed && !mbar_wait(bars + ks * 8, (it / kKs) & 1)) failed = true;   // once one wait has expired the rest are skipped
-            if (edge) patch_tile(ktile, j0, n_valid, 0, it);
-            uint32_t a[KK][4];
-            {
-                const uint32_t arow = ring_a + ks * S::kTile + klane;
-#pragma unroll
-                for (int kk = 0; kk < KK; ++kk) ldmatrix_x4(a[kk], (arow ^ ((kk & 3) << 5)) + (kk >> 2) * S::kBox);
-            }
-            __syncwarp();
-            if (it + kKs < my_n) {                            // the whole tile is in registers: its stage is free
-                const int r0 = tile_row0(it + kKs);
-                if (lane == 0) { fence_async_smem(); issue(kmap, r0, ks); }
-            }
+            if (edge) patch_tile(ring + ks * S::kTile, k_end - left, n_valid, 0, it);
+            const uint32_t arow = ring_a + ks * S::kTile + klane;
+            uint32_t a[4][4];                                 // 64 channels of the tile at a time
             // sums of the products of pieces; see the head of the file
             float x1[4], x2[4], x3[4], x4[4], lo[4];
 #pragma unroll
             for (int kk = 0; kk < KK; ++kk) {
+                if (kk % 4 == 0) {
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) ldmatrix_x4(a[x], (arow ^ (x << 5)) + (kk >> 2) * S::kBox);
+                    if (kk + 4 == KK) {                       // the rest of the tile is in registers: its stage is free
+                        __syncwarp();
+                        if (it + kKs < my_n) {
+                            const int r0 = tile_row0(it + kKs);
+                            if (lane == 0) issue(kmap, r0, ks);
+                        }
+                    }
+                }
                 uint32_t k1[4], k2[4], r2[4];
-                split_key(a[kk], g, k1, k2, r2);
+                split_key(a[kk % 4], g, k1, k2, r2);
                 float tt[4];
                 auto mma = [&](float (&d)[4], const uint32_t (&x)[4], const uint32_t (&b)[2]) {   // the sum's first term, or one more
                     if (kk == 0) mma16816_zero(d, x, b[0], b[1]); else mma16816(d, x, b[0], b[1]);
@@ -581,7 +611,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                     const float pf = (float)ex;
                     hi_f[x] = __uint_as_float(pack_bf16x2(0.f, pf) << 16);
                     lo_f[x] = pf - hi_f[x];
-                    if (on[y][x]) lg[(j0 - k_begin + kq) * G + h0 + x] = sf;
+                    if (on[y][x]) lgp[8 * y * G + x] = sf;
                 }
                 if constexpr (GP == 8) {                      // [key][8 heads] high parts, then low parts
                     *reinterpret_cast<uint32_t*>(prob + kq * 16 + (lane & 3) * 4) = pack_bf16x2(hi_f[1 % NH], hi_f[0]);
@@ -592,7 +622,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             }
             __syncwarp();
             if (!failed && !mbar_wait(bars + (kKs + vs) * 8, (it / kVs) & 1)) failed = true;
-            if (edge) patch_tile(vtile, j0, n_valid, 1, it);
+            if (edge) patch_tile(ring + (kKs + vs) * S::kTile, k_end - left, n_valid, 1, it);
             {
                 uint32_t bf[4];
                 ldmatrix_x4_trans(bf, smem_addr(prob) + (GP == 8 ? lane : lane & 15) * 16);       // keys 0-7 | 8-15 (| the low parts)
@@ -608,7 +638,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             __syncwarp();
             if (it + kVs < my_n) {
                 const int r0 = tile_row0(it + kVs);
-                if (lane == 0) { fence_async_smem(); issue(vmap, r0, kKs + vs); }
+                if (lane == 0) issue(vmap, r0, kKs + vs);
             }
         }
 #pragma unroll
@@ -754,16 +784,19 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         for (int k = 0; k < kB; ++k) {
             const int i = base + k * NT + tid, j = k_begin + i;
             wv[k] = 0u; pv[k] = t;                            // the token appended by this step
+            if (i - lane >= n_keys) continue;
             if (j < k_end && j < l_old) { wv[k] = __ldcg(wordu + j); pv[k] = __ldcg(posu + j); }
         }
         // (two branches: the addresses' space has to be known for one wide load per slot)
         if (fits) {
             const float* ls = reinterpret_cast<const float*>(smem + lay.logits);
 #pragma unroll
-            for (int k = 0; k < kB; ++k) load_logits<GP, false>(ls + min(base + k * NT + tid, max(n_keys - 1, 0)) * G, G, sv[k]);
+            for (int k = 0; k < kB; ++k)
+                if (base + k * NT + tid < n_keys) load_logits<GP, false>(ls + (base + k * NT + tid) * G, G, sv[k]);
         } else {
 #pragma unroll
-            for (int k = 0; k < kB; ++k) load_logits<GP, true>(lg + (size_t)min(base + k * NT + tid, n_keys - 1) * G, G, sv[k]);
+            for (int k = 0; k < kB; ++k)
+                if (base + k * NT + tid < n_keys) load_logits<GP, true>(lg + (size_t)(base + k * NT + tid) * G, G, sv[k]);
         }
     };
     __syncthreads();                                          // the appended slot's row, word and position are stored
@@ -848,6 +881,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
 #pragma unroll
             for (int k = 0; k < kB; ++k) {
                 const int i = base0 + k * NT + tid;
+                open[k] = 0u;
+                if (i - lane >= n_keys) continue;             // uniform in the warp
                 bool sure = false;
                 uint32_t near = 0u;
 #pragma unroll
@@ -1101,7 +1136,10 @@ inline corm_status_t launch_decode_cluster_as(DecodeClusterParams& dp, const CUt
     if (cs > kDcMaxCluster) cs = kDcMaxCluster;
     if (least > kDcMaxCluster) return CORM_ERR_UNSUPPORTED;
     const int base = dc_smem_layout<T, D, GP, NW>(0).total;
-    const int budget = (228 * 1024) / kBlocks - 1024;
+    // Room for logits: what is left of 164 KB per SM where that holds the rest, so that 92 KB of L1 stay for the logits that
+    // go through memory and for spilled registers (with 228 KB per SM taken: 128 units x 2800 keys, G 4, 58.7 us a step
+    // against 55.4, 32 units x 21400 keys 90.0 against 82.4), otherwise of everything.
+    const int budget = (base + 4096 <= 164 * 1024 / kBlocks - 1024 ? 164 : 228) * 1024 / kBlocks - 1024;
     const int need = (int)std::min<long long>(((upper + 31) / 32 + cs - 1) / cs * 32 * (long long)dp.G, 1 << 20);
     dp.lcap = std::max(0, std::min(need, (budget - base) / 128 * 32));
     const size_t smem = (size_t)dc_smem_layout<T, D, GP, NW>(dp.lcap).total;
