@@ -306,16 +306,17 @@ bool grids_follow_bound(const corm_cache* c) {
 }
 
 // Whether the cluster kernel takes a step of units of up to `upper` keys. Everything but one query head per KV head on
-// bf16 / head_dim 128, and that too when units are longer than a block of the block-per-split kernel finishes on chip and
-// eviction is at work (us per step, block-per-split -> cluster, 16000-key prompts: 32 units 61 -> 37, 128 units 130 -> 95,
-// 4000-key prompts: 32 units 26 -> 22, 256 units 61 -> 54; but 1000-key prompts: 32 units 17.7 -> 19.3, 512 units 32 -> 46;
-// 4000-key prompts: 512 units 87 -> 89).
-// Where nothing or little is evicted (alpha 0, windows beyond a register) its finish is cheap and its loop, which widens
-// keys to fp64 instead of cutting them into pieces, streams faster (128 units x 3400 keys 54 -> 62).
+// bf16 / head_dim 128. That too where there are few enough units for two blocks each (us per step, block-per-split ->
+// cluster, prompts of 1000 keys: 32 units 16.5 -> 14.9; of 3500 keys: 128 units, alpha 0 52.4 -> 47.6, windows of 64
+// 53.8 -> 47.4, of 256 53.0 -> 48.0); up to 512 units where they are longer than a block of the block-per-split kernel
+// finishes on chip and eviction is at work (prompts of 4000 keys: 256 units 61 -> 43, 512 units 79 -> 71). Otherwise its
+// loop, which widens keys to fp64 instead of cutting them into pieces, streams faster (prompts of 1000 keys: 256 units 21.0
+// against 22.0, 512 units 30 against 38; of 3000 keys: 1024 units 84 against 102, alpha 0 265 against 297).
 bool takes_cluster(const corm_cache* c, int upper, int n_units) {
     if (c->allow_fast != 1 || c->kmaps_row.empty()) return false;
     if (c->cfg.kv_dtype != CORM_BF16 || c->cfg.head_dim != 128 || c->G >= 2) return true;
-    return upper > 1024 && n_units <= 256 && c->cfg.window_w <= 32 && c->cfg.alpha > 0.f;
+    if (n_units <= c->sm_count) return true;
+    return upper > 1024 && n_units <= 512 && c->cfg.window_w <= 32 && c->cfg.alpha > 0.f;
 }
 
 // whether several layers from first_layer on may run as one launch as far as the kernels are concerned
