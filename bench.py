@@ -172,7 +172,7 @@ def measure_workload(cfg, args, local, world, rank, want_e2e, want_clocks):
     dev = lambda a: torch.from_numpy(a).cuda().to(tdt).contiguous()
     cache = CormCache(L, cfg.batch, cfg.n_q_heads, cfg.n_kv_heads, cfg.head_dim, cfg_r.max_tokens, cfg.window_w,
                       cfg.recent_r, cfg.alpha, cfg.dtype, local, pool_pages=args.pool_pages)
-    cache.corm_cache_set_tuning(args.split_len, 0 if args.no_fast else {"auto": 1, "inline": 2, "verdict": 3, "balanced": 4, "balanced-verdict": 5, "units": 6}[args.finish])
+    cache.corm_cache_set_tuning(args.split_len, 0 if args.no_fast else {"auto": 1, "inline": 2, "verdict": 3, "cluster": 4}[args.finish])
     ev = lambda: torch.cuda.Event(enable_timing=True)
     a, b = ev(), ev()
     prompts = [(dev(d.k_prompt), dev(d.v_prompt), dev(d.q_last), d.prompt_lens) for d in data]
@@ -320,7 +320,7 @@ def measure_workload(cfg, args, local, world, rank, want_e2e, want_clocks):
                      "frac_of_nominal_8TBs": achieved / 8000.0, "peak_source": peak_src, "traffic": traffic,
                      "traffic_note": None if traffic else "no ncu capture of the kernel as it stands at this launch shape",
                      "target": {"frac_of_nominal_8TBs": 0.60, "met": achieved / 8000.0 >= 0.60},
-                     "kernel": ("decode_balanced_kernel" if launches_per_step < 1.5 and cfg.group > 1 and args.finish in ("auto", "balanced")
+                     "kernel": ("decode_cluster_kernel" if not args.no_fast and (args.finish == "cluster" or (cfg.group > 1 and args.finish == "auto"))
                                 else "decode_fast_kernel") + f" ({launches_per_step:.2f} launches per layer per step, all counted in the time)",
                      "bytes_per_launch": abytes / (args.steps * L), "us_per_launch": 1e3 * med["ms"] / (args.steps * L)},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
@@ -375,9 +375,9 @@ def main():
     ap.add_argument("--ref-steps", type=int, default=512)
     ap.add_argument("--split-len", type=int, default=0)
     ap.add_argument("--no-fast", action="store_true")
-    ap.add_argument("--finish", default="auto", choices=["auto", "inline", "verdict", "balanced", "balanced-verdict", "units"],
+    ap.add_argument("--finish", default="auto", choices=["auto", "inline", "verdict", "cluster"],
                     help="which decode kernels: automatic, the block-per-split kernels finishing long units inside the "
-                         "decode launch / by the verdict launch, or the balanced single-launch kernel")
+                         "decode launch / by the verdict launch, or a cluster of blocks per unit")
     ap.add_argument("--alpha", type=float, default=None, help="override the threshold scale (0 keeps every key)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--window", type=int, default=None, help="override the verdict window w (1..256)")

@@ -142,7 +142,7 @@ corm_status_t corm_compress_prompt(corm_cache_t* cache, int32_t layer, const voi
  *   out    device [batch, n_q_heads, head_dim]
  * The call enqueues one or two launches and returns; it sizes them from the live lengths the kernels last reported (every
  * 8 steps, written to pinned host memory). Where the grid follows the longest unit (bf16 / head_dim 128 with one query head
- * per KV head, and tuning values other than 1), a host that has run 24 steps past a report that has not landed waits for
+ * per KV head, and tuning values 0, 2 and 3), a host that has run 24 steps past a report that has not landed waits for
  * it here, at most 20 ms (the GPU still has those steps queued). A layer's decode steps cannot be recorded into a CUDA
  * graph.
  * Errors: STATE if the layer has had no corm_compress_prompt since create/reset; INVALID_ARG. */
@@ -177,7 +177,7 @@ corm_status_t corm_decode_step_layers(corm_cache_t* cache, int32_t first_layer, 
  * once per step (registers, live lists and positions identical, outputs within rounding).
  * What the call adds: the units of a cache are independent (Algorithm 1 runs "on each head at every layer"), so
  * step s + 1 of a unit needs step s of that unit only. When a step's launch finishes every unit inside itself (all but
- * tuning values 3 and 5, and few long units of grouped heads), the next step's launch is chained to it: its blocks start
+ * tuning value 3, and few long units of grouped heads), the next step's launch is chained to it: its blocks start
  * as soon as a multiprocessor has room and each waits (bounded, like every wait here) for its own unit's previous
  * step instead of the whole previous launch, so consecutive steps fill one another's last waves. Steps that need the
  * verdict launch, and caches with the similarity monitor on, run as with the per-step calls.
@@ -246,9 +246,8 @@ corm_status_t corm_cache_import_state(corm_cache_t* cache, int32_t layer, int32_
  * head_dim 128 with one query head per KV head, where units fit one block, are many or lose nothing to eviction, the
  * block-per-split kernel, which finishes a unit of several splits inside the decode launch when the launch has many units
  * and by a second, verdict launch when it has few; 2 / 3 = the block-per-split
- * kernel with the first / the second way always; 4 / 5 = the balanced kernel for every group size it covers,
- * finishing inside its own launch / with the verdict launch; 6 = the balanced kernel's streaming loop with a block per
- * split, each unit finished by its last-arriving split. Errors: INVALID_ARG. */
+ * kernel with the first / the second way always; 4, 5, 6 = a cluster of blocks per unit for every shape (three values
+ * that once chose between forms of one kernel; they are the same now). Errors: INVALID_ARG. */
 corm_status_t corm_cache_set_tuning(corm_cache_t* cache, int32_t split_len, int32_t allow_fast_path);
 
 /* Opt-in monitor of the method's premise (Sections 3.2-3.3: the current query resembles recent ones, which is what

@@ -1,7 +1,6 @@
 // Host side of the C-ABI library: arena layout, argument checks, launch configuration. Every step of the hot
-// path runs in the kernels of corm_fast.cuh / corm_balanced.cuh / corm_verdict.cuh / corm_prompt.cuh /
-// corm_generic.cuh; nothing
-// here touches tensor data on the CPU.
+// path runs in the kernels of corm_cluster.cuh / corm_fast.cuh / corm_verdict.cuh / corm_prompt.cuh /
+// corm_generic.cuh; nothing here touches tensor data on the CPU.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -18,7 +17,6 @@
 #include "../../include/corm.h"
 #include "corm_common.cuh"
 #include "corm_fast.cuh"
-#include "corm_balanced.cuh"
 #include "corm_cluster.cuh"
 #include "corm_generic.cuh"
 #include "corm_prompt.cuh"
@@ -33,7 +31,7 @@ constexpr int kMinSplit = 64;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-    size_t K, V, word, pos, live, base_tokens, base_obs, ticket, ticket2, kmax, unit_stamp, counters, status, sim_acc, page_table, page_bits, page_room, q_prev, stash, partials, keepmask, unit_rec;
+    size_t K, V, word, pos, live, base_tokens, base_obs, ticket, kmax, unit_stamp, counters, status, sim_acc, page_table, page_bits, page_room, q_prev, stash, partials, keepmask, unit_rec;
     size_t stage_q, stage_k, stage_v, stage_out, total, bookkeeping_begin, bookkeeping_end;
 };
 
@@ -59,17 +57,14 @@ bool config_ok(const corm_config_t* c, corm_status_t* why) {
 
 int max_splits_of(const corm_config_t& c) { return (c.max_tokens + kMinSplit - 1) / kMinSplit; }
 
-// Split partial records the arena holds: one per (unit, split) of the block-per-split kernels, and enough for the
-// balanced kernel's one record per (block, unit) pair of its tile list at up to kMaxBalancedBlocks blocks.
-constexpr int kMaxBalancedBlocks = 1024;
 // layers whose units one launch may cover: all of a slab cache's layers if their units fit a grid dimension, else one
 size_t fused_layers_of(const corm_config_t& c, int pool_pages) {
     const long long U = (long long)c.batch * c.n_kv_heads;
     return (pool_pages == 0 && c.n_layers > 1 && U * c.n_layers <= 65535) ? (size_t)c.n_layers : 1;
 }
+// split partial records the arena holds: one per (unit, split) of the block-per-split kernels
 size_t partial_records_of(const corm_config_t& c, int pool_pages) {
-    const size_t U = (size_t)c.batch * c.n_kv_heads * fused_layers_of(c, pool_pages);
-    return std::max(U * (size_t)max_splits_of(c), bal_record_count(kMaxBalancedBlocks, (int)U));
+    return (size_t)c.batch * c.n_kv_heads * fused_layers_of(c, pool_pages) * (size_t)max_splits_of(c);
 }
 
 int pt_stride_of(const corm_config_t& c) { return (c.max_tokens + kPageKeys - 1) / kPageKeys; }
@@ -97,7 +92,6 @@ Layout make_layout(const corm_config_t& c, int pool_pages) {
     L.base_tokens = take(Ltot * c.batch * 4);
     L.base_obs = take(Ltot * c.batch * 4);
     L.ticket = take(Ltot * U * 4);
-    L.ticket2 = take(Ltot * U * 4);
     L.kmax = take(Ltot * U * 4);
     L.unit_stamp = take(Ltot * U * 8);
     L.counters = take(Ltot * CNT_COUNT * 8);
@@ -169,9 +163,6 @@ struct corm_cache {
     int sm_count = 148;
     long long launches = 0;
     int pool_pages = 0, pt_stride = 0;            // paged cache: pages per layer, page-table entries per unit
-    std::vector<CUtensorMap> vmaps;               // per layer: the V storage as a tiled tensor (balanced kernel); empty = unavailable
-    CUtensorMap vmap_all;                         // the V storage of all layers of a slab cache as one tensor (layers stepped together)
-    bool have_vmap_all = false;
     // per layer: K and V as tensors of 16-row boxes (cluster kernel; empty = unavailable); a slab layer's reach to the end
     // of the last layer, for layers stepped together
     std::vector<CUtensorMap> kmaps_row, vmaps_row;
@@ -300,9 +291,12 @@ corm_status_t monitor_similarity(corm_cache* c, int layer, const void* q, cudaSt
     return CORM_OK;
 }
 
+// Tuning values 1 (automatic) and 4..6 (always) admit the cluster kernel.
+bool may_cluster(const corm_cache* c) { return (c->allow_fast == 1 || c->allow_fast >= 4) && !c->kmaps_row.empty(); }
+
 // The cluster kernel works out its shares on the device; the other kernels' grids are sized from the host's bound.
 bool grids_follow_bound(const corm_cache* c) {
-    return c->allow_fast != 1 || c->kmaps_row.empty() || (c->cfg.kv_dtype == CORM_BF16 && c->cfg.head_dim == 128 && c->G == 1);
+    return !may_cluster(c) || (c->allow_fast == 1 && c->cfg.kv_dtype == CORM_BF16 && c->cfg.head_dim == 128 && c->G == 1);
 }
 
 // Whether the cluster kernel takes a step of units of up to `upper` keys. Everything but one query head per KV head on
@@ -313,8 +307,8 @@ bool grids_follow_bound(const corm_cache* c) {
 // loop, which widens keys to fp64 instead of cutting them into pieces, streams faster (prompts of 1000 keys: 256 units 21.0
 // against 22.0, 512 units 30 against 38; of 3000 keys: 1024 units 84 against 102, alpha 0 265 against 297).
 bool takes_cluster(const corm_cache* c, int upper, int n_units) {
-    if (c->allow_fast != 1 || c->kmaps_row.empty()) return false;
-    if (c->cfg.kv_dtype != CORM_BF16 || c->cfg.head_dim != 128 || c->G >= 2) return true;
+    if (!may_cluster(c)) return false;
+    if (c->allow_fast >= 4 || c->cfg.kv_dtype != CORM_BF16 || c->cfg.head_dim != 128 || c->G >= 2) return true;
     if (n_units <= c->sm_count) return true;
     return upper > 1024 && n_units <= 512 && c->cfg.window_w <= 32 && c->cfg.alpha > 0.f;
 }
@@ -323,9 +317,7 @@ bool takes_cluster(const corm_cache* c, int upper, int n_units) {
 bool can_fuse(const corm_cache* c, int first_layer) {
     const corm_config_t& cf = c->cfg;
     if (fused_layers_of(cf, c->pool_pages) <= 1 || !c->allow_fast || c->monitor_similarity) return false;
-    if (c->allow_fast == 1 && !c->kmaps_row.empty()) return true;
-    return cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4 &&
-           ((c->allow_fast != 6 && (c->G == 1 || c->allow_fast == 2 || c->allow_fast == 3)) || (c->have_vmap_all && first_layer == 0));
+    return may_cluster(c) || (cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4);
 }
 
 // One decode step of layers [layer, layer + n_fused) as ONE launch (pair): the layers' units are consecutive in every
@@ -350,7 +342,6 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     p.base_tokens = reinterpret_cast<int32_t*>(layer_ptr(c, c->lay.base_tokens, (size_t)cf.batch * 4, layer));
     p.base_obs = reinterpret_cast<int32_t*>(layer_ptr(c, c->lay.base_obs, (size_t)cf.batch * 4, layer));
     p.ticket = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.ticket, U * 4, layer));
-    p.ticket2 = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.ticket2, U * 4, layer));
     p.counters = reinterpret_cast<unsigned long long*>(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer));
     p.status = reinterpret_cast<int32_t*>(c->arena + c->lay.status);
     bool ask = true;                              // every 8 steps, all of the launch's layers together
@@ -380,14 +371,10 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     const bool fast = !cluster && c->allow_fast && cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4;
     corm_status_t rc;
     int n_launched = 1;
-    // Tuning values 4 / 5 / 6 force the balanced kernel's three forms.
-    const bool units = fast && !c->vmaps.empty() && c->allow_fast == 6;
-    const bool balanced = fast && !c->vmaps.empty() && (c->allow_fast == 4 || c->allow_fast == 5);
-    const bool balanced_verdict = c->allow_fast != 4;
     bool chain_ok_before = chain && !c->monitor_similarity;
     for (int i = 0; i < n_fused; ++i) chain_ok_before &= c->chain_ok[layer + i] != 0;
     bool self_finishing = false;
-    if (!(fast && !balanced) && !units && !cluster) p.unit_stamp = nullptr;    // only kernels that finish a unit in one launch keep stamps
+    if (!fast && !cluster) p.unit_stamp = nullptr;    // only kernels that finish a unit in one launch keep stamps
     if (cluster) {
         DecodeClusterParams dp{};
         dp.p = p;
@@ -400,15 +387,6 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
         rc = launch_decode_cluster(dp, cf.kv_dtype == CORM_BF16, cf.head_dim, c->kmaps_row[layer], c->vmaps_row[layer], upper, c->tune_split_len, c->sm_count, st);
         self_finishing = rc == CORM_OK && dp.p.unit_stamp;
         if (rc == CORM_OK && dp.p.chain_wait) c->chained_launches += 1;
-    } else if (units) {
-        const int typical = mean_known ? std::min(upper, mean_sum / n_fused + c->steps[layer] - c->last_report_step[layer] + 1) : 0;
-        rc = launch_decode_balanced_units(p, n_fused > 1 ? c->vmap_all : c->vmaps[layer], c->G, upper, typical, c->tune_split_len,
-                                          c->sm_count, partial_records_of(cf, c->pool_pages), st, &n_launched,
-                                          chain_ok_before, more && !c->monitor_similarity);
-        self_finishing = rc == CORM_OK;
-        if (rc == CORM_OK && p.chain_wait) c->chained_launches += 1;
-    } else if (balanced) {
-        rc = launch_decode_balanced(p, n_fused > 1 ? c->vmap_all : c->vmaps[layer], c->G, upper, c->sm_count, partial_records_of(cf, c->pool_pages), balanced_verdict, st, &n_launched);
     } else if (fast) {
         // the mean grows by at most one key per step, like the bound
         const int typical = mean_known ? std::min(upper, mean_sum / n_fused + c->steps[layer] - c->last_report_step[layer] + 1) : 0;
@@ -499,18 +477,6 @@ corm_status_t corm_cache_create_paged(const corm_config_t* cfg, int32_t pool_pag
     std::memset(c->report_host, 0, report_bytes);
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cfg->device) == cudaSuccess && sms > 0) c->sm_count = sms;
-    if (cfg->kv_dtype == CORM_BF16 && cfg->head_dim == 128 && c->G <= 4 && cfg->max_tokens <= kBalMaxTokens) {
-        const unsigned long long rows = pool_pages ? (unsigned long long)pool_pages * kPageKeys
-                                                   : (unsigned long long)c->U * cfg->max_tokens;
-        c->vmaps.resize(cfg->n_layers);
-        for (int l = 0; l < cfg->n_layers; ++l)
-            if (make_v_tensor_map(&c->vmaps[l], layer_ptr(c, lay.V, kv_layer_bytes(c), l), rows) != CORM_OK) {
-                c->vmaps.clear();                 // the block-per-split kernels serve the cache instead
-                break;
-            }
-        if (!c->vmaps.empty() && !pool_pages && cfg->n_layers > 1)
-            c->have_vmap_all = make_v_tensor_map(&c->vmap_all, layer_ptr(c, lay.V, kv_layer_bytes(c), 0), rows * cfg->n_layers) == CORM_OK;
-    }
     {
         const bool bf = cfg->kv_dtype == CORM_BF16;
         const unsigned long long rows = pool_pages ? (unsigned long long)pool_pages * kPageKeys : (unsigned long long)c->U * cfg->max_tokens;
@@ -590,7 +556,6 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     int n_clear = 0;
     auto clear = [&](void* ptr, size_t bytes) { bp.clear[n_clear++] = {static_cast<uint32_t*>(ptr), bytes / 4}; };
     clear(layer_ptr(c, c->lay.ticket, U * 4, layer), U * 4);
-    clear(layer_ptr(c, c->lay.ticket2, U * 4, layer), U * 4);
     clear(layer_ptr(c, c->lay.kmax, U * 4, layer), U * 4);
     clear(layer_ptr(c, c->lay.unit_stamp, U * 8, layer), U * 8);        // step counts restart
     clear(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer), CNT_COUNT * 8);   // a new prompt restarts the layer's statistics

@@ -27,8 +27,8 @@
 //   20 units x 250 keys, G 2, fp32           64 -> 16 -> 13     8 units x 170 keys, G 1, fp32            37.7 -> 14 -> 11
 //   128 units x 2800 keys, G 4, bf16         86 -> 68 -> 54     32 units x 21400 keys, G 4, bf16          133 -> 103 -> 80
 //   32 units x 8200 keys, G 4, no eviction   55 -> 47 -> 38     32 units x 1160 keys, G 1, bf16            35 -> 24 -> 20
-// (from one warp per key and the last-arriving split finishing the unit, from the balanced kernel and its verdict launch,
-// from the block-per-split kernel).
+// (from one warp per key and the last-arriving split finishing the unit, from fp64 logits on the CUDA cores with every
+// block an equal share of all tiles and a second launch for the verdicts, from the block-per-split kernel).
 //
 // Verdicts are the fp64 ones: a slot's logit is kept in fp32, and one that lies within the proven error of its threshold
 // is formed again in fp64. If it then lies within the error of the log-sum-exp itself, the head is marked and the
@@ -37,7 +37,7 @@
 
 #include <cuda.h>
 
-#include "corm_balanced.cuh"
+#include "corm_fast.cuh"
 #include "corm_mma.cuh"
 
 namespace corm {

@@ -53,7 +53,6 @@ struct DecodeParams {
     const int32_t* base_tokens;  // [B] tokens seen when the step counter was last rebased
     const int32_t* base_obs;     // [B] verdict rows recorded at that time
     uint32_t* ticket;         // [U] arrival counters of the splits of a unit (zero between steps)
-    uint32_t* ticket2;        // [U] second arrival counters (balanced kernel: blocks done with their verdicts)
     unsigned long long* counters;  // [CNT_COUNT]
     int32_t* status;          // sticky device status
     unsigned long long* report;   // [U] mapped host memory: units report their new lengths there (report_live); null = not asked for
@@ -62,7 +61,7 @@ struct DecodeParams {
     unsigned char* partials;  // [U][max_splits][G] records {double m, double Z, float acc[D]} (scratch)
     uint32_t* keepmask;       // [U][ceil(C/32)+2] keep bits of the verdict launch (scratch)
     uint32_t* kmax;           // [U] bf16 caches: bits of the largest key magnitude the unit has held since its prompt pass
-    int2* unit_rec;           // [U] balanced kernel -> verdict launch: a unit's first record and its record count (scratch)
+    int2* unit_rec;           // [U] cluster kernel: row moves of a unit that lists them in scratch
     unsigned long long* unit_stamp;  // [U] (decode steps the unit has finished << 32 | its live length after the last of them),
                                      // written by the block that finishes a unit inside the streaming launch; null = not kept
     int32_t chain_wait;       // fast kernel: a block waits for its own unit's stamp of the previous step, not for the previous launch
