@@ -27,11 +27,12 @@
 // out); for wide windows the tensor pipe's mma.sync rate in phase A (R P d multiply-adds, seven times).
 // Measured, us per pass: a two-launch pass (fp64 logits on the CUDA cores; one block per unit gathering; for fp32 or 64
 // channels one block per unit for everything) -> a first cluster pass (a warp per octet of rows, every warp cutting every
-// key; marked rows a key at a time) -> now:
-//   1024 units x 3250 keys, G 1, w 8    1597 -> 1036 ->  842    128 units x 3390 keys, G 1, w 256    5341 -> 1709 -> 1630
-//   128 units x 8192 keys, G 4, w 8     1821 ->  769 ->  607    32 units x 8192 keys, G 4, w 128     6736 -> 2206 -> 1747
-//   32 units x 32768 keys, G 4, w 16    4618 -> 2375 -> 1072    32 units x 4096 keys, G 1, w 8        259 ->   65 ->   61
-//   fp32: 20 units x 1300 keys, G 2     2787 ->  103            64 channels: 128 units x 2000, G 4  11037 ->  273 ->  247
+// key; marked rows a key at a time) -> now (of which products without a zeroed addend, fragment addresses from one lane
+// constant and exponentials without a range check, which the limit on the logits makes needless: 1755 -> 1699 at w 128):
+//   1024 units x 3250 keys, G 1, w 8    1597 -> 1036 ->  840    128 units x 3390 keys, G 1, w 256    5341 -> 1709 -> 1582
+//   128 units x 8192 keys, G 4, w 8     1821 ->  769 ->  598    32 units x 8192 keys, G 4, w 128     6736 -> 2206 -> 1699
+//   32 units x 32768 keys, G 4, w 16    4618 -> 2375 -> 1049    32 units x 4096 keys, G 1, w 8        259 ->   65 ->   60
+//   fp32: 20 units x 1300 keys, G 2     2787 ->  103            64 channels: 128 units x 2000, G 4  11037 ->  273 ->  238
 #pragma once
 
 #include "corm_fast.cuh"
@@ -247,32 +248,33 @@ __device__ __noinline__ bool pc_store_pieces(const PcRows& R, const bf16_t* Qu, 
 // exp(s) of 16 keys against N octets of rows, added to z[octet][row pair's two]; `last`: the tile may hold keys that a row
 // does not see or that do not exist (qpos: the rows' positions). Returns the largest high word of |s|.
 template <int D, int N>
-__device__ __forceinline__ uint32_t pc_tile_sums(uint32_t arow, SplitGrid g, int lane, const uint4* f12, const uint2* f3, int j0, int k_end, bool last,
+__device__ __forceinline__ uint32_t pc_tile_sums(uint32_t tile, uint32_t klane, SplitGrid g, int lane, const uint4* f12, const uint2* f3, int j0, int k_end, bool last,
                                                  const PcRows& R, int row0, double (*z)[2]) {
     float hi[N][4], mid[N][4], lo[N][4];
 #pragma unroll
-    for (int o = 0; o < N; ++o)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) hi[o][x] = mid[o][x] = lo[o][x] = 0.f;
-#pragma unroll
     for (int kk = 0; kk < D / 16; ++kk) {
         uint32_t a[4], k1[4], k2[4], r2[4];
-        ldmatrix_x4(a, arow + (((kk * 2 + (lane >> 4)) ^ (lane & 7)) << 4));
+        ldmatrix_x4(a, tile + (klane ^ (kk << 5)));
         split_key(a, g, k1, k2, r2);
 #pragma unroll
         for (int o = 0; o < N; ++o) {
             const uint4 b = f12[(o * (D / 16) + kk) * 32 + lane];
             const uint2 b3 = f3[(o * (D / 16) + kk) * 32 + lane];
-            float t[4] = {0.f, 0.f, 0.f, 0.f};
-            mma16816(hi[o], k1, b.x, b.y);
-            mma16816(t, k2, b.z, b.w);
-            mma16816(mid[o], k1, b.z, b.w);
+            float t[4];
+            if (kk == 0) {
+                mma16816_zero(hi[o], k1, b.x, b.y);
+                mma16816_zero(mid[o], k1, b.z, b.w);
+            } else {
+                mma16816(hi[o], k1, b.x, b.y);
+                mma16816(mid[o], k1, b.z, b.w);
+            }
+            mma16816_zero(t, k2, b.z, b.w);
             mma16816(t, r2, b.x, b.y);
             mma16816(mid[o], k2, b.x, b.y);
             mma16816(t, r2, b.z, b.w);
             mma16816(t, k1, b3.x, b3.y);
 #pragma unroll
-            for (int x = 0; x < 4; ++x) lo[o][x] += t[x];
+            for (int x = 0; x < 4; ++x) lo[o][x] = kk == 0 ? t[x] : lo[o][x] + t[x];
         }
     }
     uint32_t top = 0u;
@@ -282,7 +284,7 @@ __device__ __forceinline__ uint32_t pc_tile_sums(uint32_t arow, SplitGrid g, int
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const double s = (((double)hi[o][x] + (double)mid[o][x]) + (double)lo[o][x]) * inv_root_d;
-            double e = exp_nonpos(s);
+            double e = exp_reduced(s);                        // (any s beyond kPcLogitLimit sends the unit through the exact path)
             uint32_t h = (uint32_t)__double2hiint(s) & 0x7fffffffu;
             if (last) {                                       // causal row: keys 1..position of the query
                 const int j = j0 + (lane >> 2) + (x >> 1) * 8;
@@ -454,6 +456,8 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         }
     };
     uint4* f12 = reinterpret_cast<uint4*>(smem + lay.frag);
+    // a lane's offset for fragment loads inside a tile: chunk 2 kk of its row is one exclusive-or with kk << 5 away
+    const uint32_t klane = (lane & 15) * kRow + (((lane >> 4) ^ (lane & 7)) << 4);
     if constexpr (kBf16) {
         // A group of four octets of rows at a time: its pieces are made once and stay on chip while the block's keys pass;
         // a warp takes one tile of every chunk, cuts it into pieces once per two octets and keeps its rows' sums in
@@ -476,14 +480,14 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
                 const uint32_t am = pc_tile_amax<D>(buf + warp * 16 * kRow, lane);
                 if (grp == 0 && lane == 0) atomicMax(&misc->amax, am);
                 const SplitGrid g = split_grid(am);
-                const uint32_t arow = smem_addr(buf) + (warp * 16 + (lane & 15)) * kRow;
+                const uint32_t tile = smem_addr(buf) + warp * 16 * kRow;
                 const bool last = j0 + 16 > k_end || j0 + 16 > P - w + 1;
                 if (n_oct == 1) {
-                    top = max(top, pc_tile_sums<D, 1>(arow, g, lane, f12, f3, j0, k_end, last, R, 0, z));
+                    top = max(top, pc_tile_sums<D, 1>(tile, klane, g, lane, f12, f3, j0, k_end, last, R, 0, z));
                 } else {
-                    top = max(top, pc_tile_sums<D, 2>(arow, g, lane, f12, f3, j0, k_end, last, R, oct0 * 8, z));
+                    top = max(top, pc_tile_sums<D, 2>(tile, klane, g, lane, f12, f3, j0, k_end, last, R, oct0 * 8, z));
                     if (cnt > 2)
-                        top = max(top, pc_tile_sums<D, 2>(arow, g, lane, f12 + 2 * (D / 16) * 32, f3 + 2 * (D / 16) * 32, j0, k_end, last, R, oct0 * 8 + 16, z + 2));
+                        top = max(top, pc_tile_sums<D, 2>(tile, klane, g, lane, f12 + 2 * (D / 16) * 32, f3 + 2 * (D / 16) * 32, j0, k_end, last, R, oct0 * 8 + 16, z + 2));
                 }
             }
 #pragma unroll
@@ -531,7 +535,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
                             const double s = acc[x] * inv_root_d;
                             const bool on = j < k_end && j < qpos[x];               // causal row: keys 1..position of the query
                             bad |= on && !(fabs(s) < kPcLogitLimit);
-                            z[x] += on ? exp_nonpos(s) : 0.0;
+                            z[x] += on ? exp_reduced(s) : 0.0;
                         }
                     }
                     if (!keep_rows) fold(ru);
@@ -597,10 +601,10 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
                 uint32_t mark[2] = {0u, 0u};                  // keys lane / 4 and lane / 4 + 8
                 if (!any_bad) {
                     const float A = split_amax(pc_tile_amax<D>(buf + warp * 16 * kRow, lane));
-                    const uint32_t arow = smem_addr(buf) + (warp * 16 + (lane & 15)) * kRow;
+                    const uint32_t tile = smem_addr(buf) + warp * 16 * kRow;
                     uint32_t a[D / 16][4];
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) ldmatrix_x4(a[kk], arow + (((kk * 2 + (lane >> 4)) ^ (lane & 7)) << 4));
+                    for (int kk = 0; kk < D / 16; ++kk) ldmatrix_x4(a[kk], tile + (klane ^ (kk << 5)));
                     for (int o = 0; o < cnt; ++o) {
                         float acc[4] = {0.f, 0.f, 0.f, 0.f}, acc2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
