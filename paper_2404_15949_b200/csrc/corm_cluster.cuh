@@ -13,7 +13,10 @@
 // are (q1, q2) of each, and the accumulators of different columns are different numbers, so every product of pieces is
 // summed apart (exactly, where the pieces allow). Per 16 keys and 16 channels: 3 mma for one or two heads (the q3's take
 // the other columns), 5 for four, 8 for eight. P.V on the tensor cores as well: A = V^T (ldmatrix.trans), B = the
-// probabilities, each split into two bf16.
+// probabilities, each fp32 number as three bf16 whose sum it is (24 bits = 8 + 8 + 8): of one or two heads they fill the
+// eight columns of one mma, of four heads two, of eight three. Two parts leave 2^-18 of a probability out, which showed:
+// outputs that are not the exact ones rounded to bf16, of 10^4: two parts 9-12, three 1 (one to eight heads, 64 and 128
+// channels), as with fp32 products on the CUDA cores.
 // fp32: a key per lane (its channels shared by two half-warps), fp64 products on the CUDA cores, P.V by fp32 FMAs.
 //
 // What bounds it: on units of a few hundred keys the chain of round trips (set-up 2 us, first tiles 2, exchange and
@@ -64,7 +67,7 @@ template <typename T, int D, int GP> struct DcShape {
     static constexpr int kStages = kKs + kVs;
     static constexpr int kPieces = GP == 8 ? 6 : GP == 4 ? 4 : 2;   // words per lane and 16 channels of the query pieces
     static constexpr int kWarpRing = kStages * kTile;
-    static constexpr int kProb = kBf16 ? kDcKeys * (GP == 8 ? 32 : 16) : kDcKeys * GP * 4;   // a warp's probabilities
+    static constexpr int kProb = kBf16 ? kDcKeys * (GP == 8 ? 48 : GP == 4 ? 32 : 16) : kDcKeys * GP * 4;   // a warp's probabilities
 };
 // resident blocks per SM the register budget is set for
 template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int dc_blocks() {
@@ -593,6 +596,10 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                     scf[x] = (float)sc;
                     Mref[x] = mn;
                 }
+                if constexpr (GP == 2) {                      // lanes 2 and 3 of four accumulate the third parts of heads 0 and 1
+                    const float o = __shfl_xor_sync(0xffffffffu, scf[0], 2);
+                    if (lane & 2) scf[0] = o;
+                }
 #pragma unroll
                 for (int cb = 0; cb < D / 16; ++cb)           // the accumulators' columns are the thread's own heads
 #pragma unroll
@@ -602,22 +609,35 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
 #pragma unroll
             for (int y = 0; y < 2; ++y) {
                 const int kq = (lane >> 2) + 8 * y;
-                float hi_f[NH], lo_f[NH];
+                float pf[NH];
 #pragma unroll
                 for (int x = 0; x < NH; ++x) {
                     const float sf = (float)s[y][x];
                     const double ex = exp_nonpos_where(on[y][x] && sf - Mref[x] > -700.f, s[y][x] - (double)Mref[x]);
                     Zl[x] += ex;
-                    const float pf = (float)ex;
-                    hi_f[x] = __uint_as_float(pack_bf16x2(0.f, pf) << 16);
-                    lo_f[x] = pf - hi_f[x];
+                    pf[x] = (float)ex;
                     if (on[y][x]) lgp[8 * y * G + x] = sf;
                 }
-                if constexpr (GP == 8) {                      // [key][8 heads] high parts, then low parts
-                    *reinterpret_cast<uint32_t*>(prob + kq * 16 + (lane & 3) * 4) = pack_bf16x2(hi_f[1 % NH], hi_f[0]);
-                    *reinterpret_cast<uint32_t*>(prob + 256 + kq * 16 + (lane & 3) * 4) = pack_bf16x2(lo_f[1 % NH], lo_f[0]);
-                } else {
-                    *reinterpret_cast<uint32_t*>(prob + kq * 16 + (lane & 3) * 4) = pack_bf16x2(lo_f[0], hi_f[0]);   // [key][head x (high, low)]
+                uint32_t* const dst = reinterpret_cast<uint32_t*>(prob + kq * 16) + (lane & 3);
+                if constexpr (GP == 8) {                      // [key][8 heads] first parts, then second, then third
+#pragma unroll
+                    for (int part = 0; part < 3; ++part) {
+                        const uint32_t w = pack_bf16x2(pf[1 % NH], pf[0]);
+                        dst[part * 64] = w;
+                        pf[0] -= __uint_as_float(w << 16);
+                        pf[1 % NH] -= __uint_as_float(w & 0xffff0000u);
+                    }
+                } else {                                      // [key][head x (first, second)], and (third, 0) behind them
+                    const uint32_t a = pack_bf16x2(0.f, pf[0]) << 16;
+                    const float r = pf[0] - __uint_as_float(a);
+                    const uint32_t b = pack_bf16x2(r, 0.f) & 0xffff0000u, c = pack_bf16x2(0.f, r - __uint_as_float(b));
+                    if constexpr (GP == 4) {
+                        dst[0] = b | (a >> 16);
+                        dst[64] = c;
+                    } else if (h0 < 2) {
+                        dst[0] = b | (a >> 16);
+                        dst[2] = c;
+                    }
                 }
             }
             __syncwarp();
@@ -625,14 +645,17 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             if (edge) patch_tile(ring + (kKs + vs) * S::kTile, k_end - left, n_valid, 1, it);
             {
                 uint32_t bf[4];
-                ldmatrix_x4_trans(bf, smem_addr(prob) + (GP == 8 ? lane : lane & 15) * 16);       // keys 0-7 | 8-15 (| the low parts)
+                ldmatrix_x4_trans(bf, smem_addr(prob) + (GP > 2 ? lane : lane & 15) * 16);        // keys 0-7 | 8-15 (| the next parts)
+                uint32_t b3p[2];
+                if constexpr (GP == 8) ldmatrix_x2_trans(b3p, smem_addr(prob) + 512 + (lane & 15) * 16);
                 const uint32_t vrow = ring_a + (kKs + vs) * S::kTile + vlane;
 #pragma unroll
                 for (int cb = 0; cb < D / 16; ++cb) {
                     uint32_t va[4];
                     ldmatrix_x4_trans(va, (vrow ^ ((cb & 3) << 5)) + (cb >> 2) * S::kBox);
                     mma16816(accd[cb], va, bf[0], bf[1]);     // Eq. 1
-                    if constexpr (GP == 8) mma16816(accd[cb], va, bf[2], bf[3]);
+                    if constexpr (GP > 2) mma16816(accd[cb], va, bf[2], bf[3]);
+                    if constexpr (GP == 8) mma16816(accd[cb], va, b3p[0], b3p[1]);
                 }
             }
             __syncwarp();
@@ -654,9 +677,16 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 rec[(h0 + 1) * D + cb * 16 + (lane >> 2)] = accd[cb][1];
                 rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][2];
                 rec[(h0 + 1) * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][3];
-            } else if (h0 < G) {
-                rec[h0 * D + cb * 16 + (lane >> 2)] = accd[cb][0] + accd[cb][1];       // high + low parts
-                rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][2] + accd[cb][3];
+            } else {
+                float a0 = accd[cb][0] + accd[cb][1], a1 = accd[cb][2] + accd[cb][3];  // the parts' sums
+                if constexpr (GP == 2) {
+                    a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+                    a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
+                }
+                if (h0 < G) {
+                    rec[h0 * D + cb * 16 + (lane >> 2)] = a0;
+                    rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = a1;
+                }
             }
         }
         state = (state & ~0xffffu) | kmax;

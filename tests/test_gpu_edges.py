@@ -1,0 +1,40 @@
+"""Corners of the decode and prompt kernels: precision of the outputs, long units, magnitudes far outside the usual range,
+length reports. Against the CPU oracle unless a test says otherwise."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2404_15949_b200.workload import CONFIGS, generate
+from parity_util import OUT_TOL, assert_states_equal, make_gpu_cache, make_oracle, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _cfg(dtype, d, G, nkv, B, prange, steps, w, r, seed=50, **kw):
+    return CONFIGS[1].with_(name="edges", batch=B, n_q_heads=nkv * G, n_kv_heads=nkv, head_dim=d, dtype=dtype,
+                            prompt_min=prange[0], prompt_max=prange[1], steps=steps, window_w=w, recent_r=r,
+                            gqa_rho=0.7 if G > 1 else 0.0, hh_min=2, hh_max=6, seed=seed, **kw)
+
+
+@pytest.mark.parametrize("d,G", [(128, 1), (128, 2), (128, 4), (128, 8), (64, 1), (64, 4), (64, 8)])
+def test_bf16_outputs_are_the_exact_ones_rounded(d, G):
+    """Probabilities and products of fp32 precision leave an output off by about 2^-22 of its scale, so it rounds to
+    another bf16 than the exact one about once in 2^-22 / 2^-8 = 6 10^-5 (and a little more where outputs are small);
+    probabilities cut to two bf16 parts make that 10^-3. Bound: 3 10^-4, four standard deviations above 10^-4 for the
+    smallest number of outputs here (2 10^4)."""
+    nkv, B, steps = max(1, 8 // G), 4, 20
+    cfg = _cfg("bf16", d, G, nkv, B, (900, 1100), steps, 64, 256, alpha=1.0)
+    data = generate(cfg)
+    gpu, orc = make_gpu_cache(cfg, B, nkv), make_oracle(cfg, B, nkv)
+    gpu.corm_compress_prompt(0, to_dev(data.k_prompt, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(data.q_last, "bf16"),
+                             data.prompt_lens)
+    orc.compress_prompt(0, data.k_prompt, data.v_prompt, data.q_last, data.prompt_lens)
+    q, k, v = (to_dev(x, "bf16") for x in (data.q, data.k_new, data.v_new))
+    wrong = total = 0
+    for s in range(steps):
+        ref = torch.from_numpy(orc.decode_step(0, data.q[s], data.k_new[s], data.v_new[s])).to(torch.bfloat16)
+        out = gpu.corm_decode_step(0, q[s], k[s], v[s]).cpu()
+        wrong += int((out != ref).sum())
+        total += out.numel()
+    assert_states_equal(gpu, orc, 0, B, nkv, "end")
+    assert total >= 20000 and wrong <= 3e-4 * total, (wrong, total)
