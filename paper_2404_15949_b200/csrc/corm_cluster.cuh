@@ -47,7 +47,6 @@ namespace corm {
 
 constexpr int kDcMaxCluster = 8;
 constexpr int kDcKeys = 16;                       // keys per tile
-constexpr int kDcMaxWords = 4096;                 // 32-slot words a block may own (its keep bits and prefix sums lie in the ring: 41 KB)
 
 struct DecodeClusterParams {
     DecodeParams p;
@@ -75,6 +74,19 @@ template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int d
 }
 
 constexpr int kDcListCap = 1024;                  // slots a step may evict from a unit for its moves to be listed on chip
+
+// What the ring holds once the tiles are done: the block's record (the first 8 KB), the keep bits of its words and, behind
+// them, the lists of a step with few moves or the prefix sums (one more than words) of a step with many. So the words a
+// block may own follow from the instance's ring: 4096 for the rings of 64 KB, 3071 for the 32 KB of fp32 / 64 channels.
+constexpr int kDcRecBytes = 8192;
+template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int dc_max_words() {
+    constexpr int n = (NW * DcShape<T, D, GP>::kWarpRing - kDcRecBytes - 4) / 8;
+    return n < 4096 ? n : 4096;
+}
+template <typename T, int D, int GP, int NW> __host__ __device__ constexpr bool dc_ring_holds_lists() {
+    constexpr int words = dc_max_words<T, D, GP, NW>(), lists = 2 * kDcListCap * 4, sums = 4 * (words + 1);
+    return GP * D * 4 <= kDcRecBytes && kDcRecBytes + 4 * words + (lists > sums ? lists : sums) <= NW * DcShape<T, D, GP>::kWarpRing;
+}
 
 constexpr int kDcOpenCap = 32;
 template <int NW> struct DcMisc {
@@ -267,7 +279,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     extern __shared__ __align__(1024) unsigned char smem[];
     using S = DcShape<T, D, GP>;
     constexpr bool kBf16 = S::kBf16;
-    constexpr int NT = NW * 32, kKs = S::kKs, kVs = S::kVs;
+    constexpr int NT = NW * 32, kKs = S::kKs, kVs = S::kVs, kMaxWords = dc_max_words<T, D, GP, NW>();
+    static_assert(dc_ring_holds_lists<T, D, GP, NW>(), "keep bits, lists and prefix sums lie in the ring");
     constexpr int NH = kBf16 ? (GP == 8 ? 2 : 1) : GP;        // heads a thread handles logits of
     constexpr int NK = kBf16 ? 2 : 1;                         // keys of a tile a thread handles
     const DecodeParams& p = dp.p;
@@ -886,7 +899,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     __syncthreads();
 
     // ---- 2. verdicts, register update, keep bits ----
-    uint32_t* keep = reinterpret_cast<uint32_t*>(smem + 8192);                  // the ring is free behind the block's record
+    uint32_t* keep = reinterpret_cast<uint32_t*>(smem + kDcRecBytes);           // the ring is free behind the block's record
     {
         // first the block's record of the outputs' numerators (Eq. 1): its warps' merged, in place of the first warp's
         for (int x = tid; x < G * D; x += NT) {
@@ -950,7 +963,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 const uint32_t ballot = __ballot_sync(0xffffffffu, kp);
                 n_imp += __popc(__ballot_sync(0xffffffffu, im));
                 n_keep += __popc(ballot);
-                if (lane == 0 && CORM_IN_RANGE((base >> 5) + warp < kDcMaxWords, p.status)) keep[(base >> 5) + warp] = ballot;
+                if (lane == 0 && CORM_IN_RANGE((base >> 5) + warp < kMaxWords, p.status)) keep[(base >> 5) + warp] = ballot;
             }
         }
         if (lane == 0) {
@@ -1009,7 +1022,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     auto row_of = [&](int slot) -> size_t {
         return pt_u ? page_row(__ldcg(pt_u + (slot >> 5)), slot, p.pool_pages, p.status) : (size_t)u * p.C + (size_t)slot;
     };
-    int* holes = reinterpret_cast<int*>(smem + 8192) + kDcMaxWords;             // [kDcListCap] each, behind the keep bits
+    int* holes = reinterpret_cast<int*>(smem + kDcRecBytes) + kMaxWords;        // [kDcListCap] each, behind the keep bits
     int* movers = holes + kDcListCap;
     auto hole_words = [&](int i, uint32_t& m, uint32_t& hm) {                   // word i of the block: kept slots, holes
         m = keep[i];
@@ -1075,7 +1088,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         // many: the lists go to scratch and the moves are shared out evenly
         int* gholes = reinterpret_cast<int*>(p.stash + (size_t)u * G * p.C) + (size_t)G * p.C;   // behind the unit's logits
         int* gmovers = gholes + p.C / 2;
-        int* prefix = holes;                                  // [kDcMaxWords + 1]
+        int* prefix = holes;                                  // [kMaxWords + 1]
         const int nw = (n_keys + 31) >> 5;
         block_popc_scan<NT>(keep, prefix, nw, misc->scan);
         for (int i = tid; i < nw; i += NT) {
@@ -1161,7 +1174,8 @@ inline corm_status_t launch_decode_cluster_as(DecodeClusterParams& dp, const CUt
     if (tune_split_len) cs = (upper + tune_split_len - 1) / tune_split_len;
     if (cs > (upper + 63) / 64) cs = (upper + 63) / 64;
     // ... and no more words than a block can keep track of
-    const long long least = ((p.C + 31) / 32 + kDcMaxWords - 1) / kDcMaxWords;
+    constexpr int kMaxWords = dc_max_words<T, D, GP, NW>();
+    const long long least = ((p.C + 31) / 32 + kMaxWords - 1) / kMaxWords;
     cs = std::max(std::max(cs, least), 1ll);
     if (cs > kDcMaxCluster) cs = kDcMaxCluster;
     if (least > kDcMaxCluster) return CORM_ERR_UNSUPPORTED;

@@ -38,3 +38,43 @@ def test_bf16_outputs_are_the_exact_ones_rounded(d, G):
         total += out.numel()
     assert_states_equal(gpu, orc, 0, B, nkv, "end")
     assert total >= 20000 and wrong <= 3e-4 * total, (wrong, total)
+
+
+# one block per unit as long as its list space allows (a split length beyond the unit), so a block owns as many 32-slot
+# words as it can keep track of: 3071 for fp32 / 64 channels, 4096 otherwise; and one word more than that
+LONG_UNITS = [
+    # dtype, head_dim, group, live keys, max_tokens, paged
+    ("f32", 64, 1, 98250, 3071 * 32, False),
+    ("f32", 64, 8, 98270, 3071 * 32, True),
+    ("f32", 64, 2, 98290, 3072 * 32, False),
+    ("bf16", 64, 1, 100000, 4096 * 32, False),
+    ("bf16", 128, 4, 70000, 4097 * 32, True),
+]
+
+
+@pytest.mark.parametrize("case", LONG_UNITS, ids=lambda c: "-".join(str(x) for x in c))
+def test_long_unit_loses_thousands_of_keys_in_one_step(case):
+    """An imported unit whose keys are all up for eviction (window of one query): the first step removes thousands
+    of them, so the moves are listed in scratch, by blocks that own as many words as they may."""
+    dtype, d, G, n, C, paged = case
+    cfg = _cfg(dtype, d, G, 1, 1, (1, 1), 3, 1, 64)
+    rng = np.random.default_rng(17 + d + G)
+    to = (lambda x: to_dev(x, dtype).float().cpu().numpy())
+    k, v = (to(rng.standard_normal((n, d), dtype=np.float32)) for _ in range(2))
+    q = to(rng.standard_normal((3, 1, G, d), dtype=np.float32))
+    kn, vn = (to(rng.standard_normal((3, 1, 1, d), dtype=np.float32)) for _ in range(2))
+    word, pos = np.ones(n, np.uint32), np.arange(1, n + 1, dtype=np.int32)
+    gpu = make_gpu_cache(cfg, 1, 1, max_tokens=C, pool_pages=(C // 1024 + 2) * 32 if paged else 0)
+    orc = make_oracle(cfg, 1, 1, max_tokens=C)
+    orc.set_near_band(1e-10)           # 10^5 keys a step put one within the usual 10^-6; sums of fp64 terms differ by 10^-13
+    gpu.corm_cache_set_tuning(1 << 18, True)
+    gpu.corm_cache_import_state(0, 0, 0, k, v, word, pos, n, 1)
+    orc.import_unit(0, 0, 0, k, v, word, pos, n, 1)
+    for s in range(3):
+        out = gpu.corm_decode_step(0, to_dev(q[s], dtype), to_dev(kn[s], dtype), to_dev(vn[s], dtype))
+        ref = orc.decode_step(0, q[s], kn[s], vn[s])
+        assert np.abs(out.float().cpu().numpy() - ref).max() <= OUT_TOL[dtype]
+        assert_states_equal(gpu, orc, 0, 1, 1, f"step {s}")
+    assert orc.counters()["near_threshold"] == 0
+    st = gpu.corm_cache_stats()
+    assert st["device_status"] == 0 and st["evicted_keys"] > 8000
