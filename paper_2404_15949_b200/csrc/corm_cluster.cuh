@@ -505,7 +505,6 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 m = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(m, x.x), x.y), x.z), x.w);
             }
             kmax = max(kmax, __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16)));
-            if (tid == 0 && kmax > kmax_old && !state) p.kmax[u] = kmax;
         }
         if (kmax >= kSplitMaxBits) { state |= kDcBad; kmax = kSplitMaxBits; }
         const SplitGrid g = split_grid(kmax);
@@ -872,6 +871,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         }
         return;
     }
+    // the appended key enters the unit's magnitude whatever became of the queries (every block has read the old one)
+    if (kBf16 && rank == 0 && tid == 0) p.kmax[u] = unit_state & 0xffffu;
     // error of a head's log-sum-exp per unit of qe (every logit of it is off by at most this much)
     const float eps_a = kBf16 ? split_amax(min(unit_state & 0xffffu, kSplitMaxBits)) * (float)inv_root_d * 1.0001f : 0.f;
     for (int h = warp; h < G; h += NW) {

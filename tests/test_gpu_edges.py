@@ -78,3 +78,30 @@ def test_long_unit_loses_thousands_of_keys_in_one_step(case):
     assert orc.counters()["near_threshold"] == 0
     st = gpu.corm_cache_stats()
     assert st["device_status"] == 0 and st["evicted_keys"] > 8000
+
+
+def test_a_key_appended_next_to_an_overflowed_query_counts():
+    """Two steps whose queries leave the range of the exact pieces (an element of 2^60) append the largest keys a unit has
+    seen, 2^20 against 1, one bit of one channel apart. Later ordinary queries find their probabilities next to the
+    threshold often enough (128 units, 30 steps) to show logits formed on a grid that does not know these keys."""
+    B, nkv, d, steps = 8, 16, 128, 32
+    cfg = _cfg("bf16", d, 1, nkv, B, (40, 40), steps, 32, 256)
+    data = generate(cfg)
+    rng = np.random.default_rng(5)
+    big = (rng.standard_normal((B, nkv, d)) * 2.0 ** 20).astype(np.float32)
+    big = torch.from_numpy(big).to(torch.bfloat16).float().numpy()
+    big[..., 0] = 2.0 ** 12
+    q, kn, vn = data.q.copy(), data.k_new.copy(), data.v_new.copy()
+    kn[0], kn[1] = big, big
+    kn[1][..., 0] += 32.0                              # a bit of 2^12 in bf16: logits 2.8 q_0 apart
+    q[:2, ..., 1] = 2.0 ** 60
+    gpu, orc = make_gpu_cache(cfg, B, nkv), make_oracle(cfg, B, nkv)
+    orc.set_near_band(1e-10)
+    gpu.corm_compress_prompt(0, to_dev(data.k_prompt, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(data.q_last, "bf16"),
+                             data.prompt_lens)
+    orc.compress_prompt(0, data.k_prompt, data.v_prompt, data.q_last, data.prompt_lens)
+    for s in range(steps):
+        gpu.corm_decode_step(0, to_dev(q[s], "bf16"), to_dev(kn[s], "bf16"), to_dev(vn[s], "bf16"))
+        orc.decode_step(0, q[s], kn[s], vn[s])
+        assert_states_equal(gpu, orc, 0, B, nkv, f"step {s}")
+    assert gpu.corm_cache_stats()["device_status"] == 0
