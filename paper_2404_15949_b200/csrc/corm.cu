@@ -155,6 +155,7 @@ struct corm_cache {
     unsigned long long* report_host = nullptr;    // [n_layers][U], report_live's words
     std::vector<int> live_mean;                   // mean live length at the last report that landed (0 = unknown)
     std::vector<int> report_pending, last_report_step;
+    bool report_given = false;                    // some launch was given report_host's address; nothing clears this
     std::vector<unsigned> report_epoch;           // 1..4095: reports of before a prompt pass, an import or a reset do not count
     int tune_split_len = 0, allow_fast = 1;
     double bound_scale = 1.0;
@@ -348,6 +349,7 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     for (int i = 0; i < n_fused; ++i)
         ask &= !c->report_pending[layer + i] && c->steps[layer + i] + 1 - c->last_report_step[layer + i] >= 8 && c->report_epoch[layer + i] == c->report_epoch[layer];
     p.report = ask ? c->report_host + (size_t)layer * U : nullptr;
+    c->report_given |= ask;
     p.report_tag = c->report_epoch[layer];
     p.stash = reinterpret_cast<double*>(c->arena + c->lay.stash);
     p.partials = c->arena + c->lay.partials;
@@ -508,8 +510,7 @@ corm_status_t corm_cache_destroy(corm_cache_t* cache) {
     if (!cache) return CORM_ERR_INVALID_ARG;
     {
         DeviceGuard guard(cache->cfg.device);
-        for (int pending : cache->report_pending)
-            if (pending) { cudaDeviceSynchronize(); break; }      // a launch may still write its report
+        if (cache->report_given) cudaDeviceSynchronize();         // a launch may still write its report, wanted or not
         cudaFreeHost(cache->report_host);
     }
     delete cache;
@@ -580,6 +581,7 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     p.counters = reinterpret_cast<unsigned long long*>(layer_ptr(c, c->lay.counters, CNT_COUNT * 8, layer));
     p.status = reinterpret_cast<int32_t*>(c->arena + c->lay.status);
     p.report = c->report_host + (size_t)layer * U;
+    c->report_given = true;
     p.report_tag = c->report_epoch[layer];
     p.stash = reinterpret_cast<double*>(c->arena + c->lay.stash);
     p.U = (int)U; p.Hkv = cf.n_kv_heads; p.C = cf.max_tokens; p.p_max = p_max; p.w = cf.window_w; p.r = cf.recent_r;

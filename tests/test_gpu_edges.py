@@ -105,3 +105,24 @@ def test_a_key_appended_next_to_an_overflowed_query_counts():
         orc.decode_step(0, q[s], kn[s], vn[s])
         assert_states_equal(gpu, orc, 0, B, nkv, f"step {s}")
     assert gpu.corm_cache_stats()["device_status"] == 0
+
+
+def test_destroy_waits_for_launches_that_report_even_after_a_reset():
+    """Kernels write lengths to pinned host memory of the cache. A reset forgets the reports that are on their way, but the
+    launches behind them still run: the cache's memory must outlive them."""
+    cfg = _cfg("bf16", 128, 4, 8, 4, (2000, 2000), 64, 8, 64)
+    data = generate(cfg)
+    gpu = make_gpu_cache(cfg, 4, 8)
+    p = [to_dev(x, "bf16") for x in (data.k_prompt, data.v_prompt, data.q_last)]
+    q, k, v = (to_dev(x, "bf16") for x in (data.q, data.k_new, data.v_new))
+    out = torch.empty_like(q)
+    torch.cuda.synchronize()
+    for _ in range(8):
+        gpu.corm_compress_prompt(0, *p, data.prompt_lens)
+        for s in range(64):
+            gpu.corm_decode_step(0, q[s], k[s], v[s], out[s])
+    done = torch.cuda.Event()
+    done.record()
+    gpu.corm_cache_reset()
+    gpu.close()
+    assert done.query()
