@@ -156,7 +156,10 @@ struct corm_cache {
     std::vector<int> live_mean;                   // mean live length at the last report that landed (0 = unknown)
     std::vector<int> report_pending, last_report_step;
     bool report_given = false;                    // some launch was given report_host's address; nothing clears this
-    std::vector<unsigned> report_epoch;           // 1..4095: reports of before a prompt pass, an import or a reset do not count
+    // 1..65535, of the whole cache: moves with every prompt pass, import and reset of any layer, so that reports of before
+    // it do not count. A launch over several layers writes one tag; each layer remembers the one it was asked under.
+    unsigned report_epoch = 1;
+    std::vector<unsigned> asked_epoch;
     int tune_split_len = 0, allow_fast = 1;
     double bound_scale = 1.0;
     int monitor_similarity = 0;
@@ -243,7 +246,7 @@ bool take_report(corm_cache* c, int layer) {
     for (int u = 0; u < c->U; ++u) {
         const unsigned long long v = r[u];
         const int steps = (int)((v >> kReportLenBits) & ((1ull << kReportStepBits) - 1)), len = (int)(v & ((1ull << kReportLenBits) - 1));
-        if ((unsigned)(v >> (kReportLenBits + kReportStepBits)) != c->report_epoch[layer] || steps < c->last_report_step[layer]) return false;
+        if ((unsigned)(v >> (kReportLenBits + kReportStepBits)) != c->asked_epoch[layer] || steps < c->last_report_step[layer]) return false;
         bound = std::max(bound, len + c->steps[layer] - steps);
         sum += len;
     }
@@ -265,7 +268,7 @@ void poll_live_bound(corm_cache* c, int layer, bool sized) {
 // Reports of launches before this call do not count any more.
 void forget_reports(corm_cache* c, int layer) {
     c->report_pending[layer] = 0;
-    c->report_epoch[layer] = c->report_epoch[layer] % 4095 + 1;
+    c->report_epoch = c->report_epoch % ((1u << kReportTagBits) - 1u) + 1;
 }
 
 // Eq. 3 between this step's queries and the layer's previous decode queries (opt-in; one small launch), after any
@@ -347,10 +350,10 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     p.status = reinterpret_cast<int32_t*>(c->arena + c->lay.status);
     bool ask = true;                              // every 8 steps, all of the launch's layers together
     for (int i = 0; i < n_fused; ++i)
-        ask &= !c->report_pending[layer + i] && c->steps[layer + i] + 1 - c->last_report_step[layer + i] >= 8 && c->report_epoch[layer + i] == c->report_epoch[layer];
+        ask &= !c->report_pending[layer + i] && c->steps[layer + i] + 1 - c->last_report_step[layer + i] >= 8;
     p.report = ask ? c->report_host + (size_t)layer * U : nullptr;
     c->report_given |= ask;
-    p.report_tag = c->report_epoch[layer];
+    p.report_tag = c->report_epoch;
     p.stash = reinterpret_cast<double*>(c->arena + c->lay.stash);
     p.partials = c->arena + c->lay.partials;
     p.keepmask = reinterpret_cast<uint32_t*>(c->arena + c->lay.keepmask);
@@ -417,7 +420,7 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
         c->parity[l] ^= 1;
         c->steps[l] += 1;
         c->live_upper[l] = std::min(cf.max_tokens, c->live_upper[l] + 1);
-        if (ask) { c->report_pending[l] = 1; c->last_report_step[l] = c->steps[l]; }
+        if (ask) { c->report_pending[l] = 1; c->last_report_step[l] = c->steps[l]; c->asked_epoch[l] = c->report_epoch; }
     }
     return n_fused == 1 ? monitor_similarity(c, layer, q, st) : CORM_OK;
 }
@@ -469,7 +472,7 @@ corm_status_t corm_cache_create_paged(const corm_config_t* cfg, int32_t pool_pag
     c->chain_ok.assign(cfg->n_layers, 0);
     c->report_pending.assign(cfg->n_layers, 0);
     c->last_report_step.assign(cfg->n_layers, 0);
-    c->report_epoch.assign(cfg->n_layers, 1);
+    c->asked_epoch.assign(cfg->n_layers, 0);
     const size_t report_bytes = sizeof(unsigned long long) * (size_t)cfg->n_layers * c->U;
     if (cudaHostAlloc(reinterpret_cast<void**>(&c->report_host), report_bytes, cudaHostAllocMapped) != cudaSuccess) {   // pinned HOST memory
         std::fprintf(stderr, "corm: could not set up the host-side report buffer\n");
@@ -582,7 +585,7 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     p.status = reinterpret_cast<int32_t*>(c->arena + c->lay.status);
     p.report = c->report_host + (size_t)layer * U;
     c->report_given = true;
-    p.report_tag = c->report_epoch[layer];
+    p.report_tag = c->report_epoch;
     p.stash = reinterpret_cast<double*>(c->arena + c->lay.stash);
     p.U = (int)U; p.Hkv = cf.n_kv_heads; p.C = cf.max_tokens; p.p_max = p_max; p.w = cf.window_w; p.r = cf.recent_r;
     p.log_alpha = log_alpha_of(c);
@@ -599,6 +602,7 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     c->have_q_prev[layer] = 0;                    // the previous decode query belonged to the old text
     c->last_report_step[layer] = 0;
     c->report_pending[layer] = 1;
+    c->asked_epoch[layer] = c->report_epoch;
     return CORM_OK;
 }
 

@@ -205,9 +205,9 @@ __device__ __forceinline__ void note_key_magnitude(uint32_t* kmax_u, uint4 x) {
 }
 
 // A unit's new live length for the host's launch sizing: one word written straight to mapped host memory (tag in the top
-// 12 bits, steps done, length), so that neither a copy nor an event stands between two launches (two copies and an event
-// every 8 steps cost 1.2 us per step and broke the overlap of consecutive launches).
-constexpr int kReportLenBits = 24, kReportStepBits = 28;
+// bits, steps done, length, which is at most 2^19), so that neither a copy nor an event stands between two launches (two
+// copies and an event every 8 steps cost 1.2 us per step and broke the overlap of consecutive launches).
+constexpr int kReportLenBits = 20, kReportStepBits = 28, kReportTagBits = 16;
 template <typename P> __device__ __forceinline__ void report_live(const P& p, int u, int steps_done, int live) {
     if (p.report)
         *reinterpret_cast<volatile unsigned long long*>(p.report + u) =

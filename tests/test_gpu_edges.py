@@ -126,3 +126,24 @@ def test_destroy_waits_for_launches_that_report_even_after_a_reset():
     gpu.corm_cache_reset()
     gpu.close()
     assert done.query()
+
+
+def test_layers_of_different_history_stepped_together_still_report_their_lengths():
+    """One layer has had a prompt pass more than the other. Launches over both must go on reporting lengths: the grids of
+    the block-per-split kernel follow them, and once the units are known to fit one split (1024 keys) a step is one launch
+    instead of two."""
+    cfg = _cfg("bf16", 128, 1, 4, 2, (3000, 3000), 40, 8, 64)                    # 1900 keys of a unit survive the prompt, 900 the steps
+    data = [generate(cfg, layer=l) for l in range(2)]
+    gpu = make_gpu_cache(cfg, 2, 4, n_layers=2)
+    gpu.corm_cache_set_tuning(1024, 3)
+    for l in (0, 0, 1):
+        gpu.corm_compress_prompt(l, *(to_dev(getattr(data[l], n), "bf16") for n in ("k_prompt", "v_prompt", "q_last")),
+                                 data[l].prompt_lens)
+    q, k, v = (torch.stack([to_dev(getattr(x, n), "bf16") for x in data], dim=1).contiguous() for n in ("q", "k_new", "v_new"))
+    out = torch.empty_like(q)
+    for s in range(40):
+        torch.cuda.synchronize()                       # whatever was asked for has been reported
+        before = gpu.corm_cache_kernel_launches()
+        gpu.corm_decode_step_layers(0, *([t[s, l] for l in range(2)] for t in (q, k, v, out)))
+    assert max(int(gpu.corm_cache_live_lens(l).max()) for l in range(2)) < 1000
+    assert gpu.corm_cache_kernel_launches() - before == 1
