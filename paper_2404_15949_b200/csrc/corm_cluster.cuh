@@ -17,7 +17,9 @@
 // eight columns of one mma, of four heads two, of eight three. Two parts leave 2^-18 of a probability out, which showed:
 // outputs that are not the exact ones rounded to bf16, of 10^4: two parts 9-12, three 1 (one to eight heads, 64 and 128
 // channels), as with fp32 products on the CUDA cores.
-// fp32: a key per lane (its channels shared by two half-warps), fp64 products on the CUDA cores, P.V by fp32 FMAs.
+// fp32: a key per lane (its channels shared by two half-warps), fp64 products on the CUDA cores, P.V by fp32 FMAs. A bf16
+// unit with a key or query element the pieces cannot hold (2^56 and more, infinity, NaN) takes that loop too: its products
+// have no bounds on the tensor cores.
 //
 // What bounds it: on units of a few hundred keys the chain of round trips (set-up 2 us, first tiles 2, exchange and
 // thresholds 2.5, verdicts 1, exchange 1, moves 2, launch 2); on long units instruction issue in the streaming loop: about
@@ -91,15 +93,15 @@ template <typename T, int D, int GP, int NW> __host__ __device__ constexpr bool 
 constexpr int kDcOpenCap = 32;
 template <int NW> struct DcMisc {
     unsigned long long stamp;
-    double wZ[NW][8];                             // per warp and head, read by the cluster
+    double wM[NW][8], wZ[NW][8];                  // per warp and head, read by the cluster
     double thr[8], Zt[8], log_t;
     double red[NW][2], mz[2];                     // exact heads
-    float wM[NW][8];
     float sc[8][kDcMaxCluster * NW], qe[8], thr_f[8], slack[8];
     float qe_part[NW][8];                         // the warps' shares of qe
-    // largest key magnitude (bf16 bits), 1 << 16 if a magnitude is beyond the pieces' range, 1 << 17 if a wait expired,
-    // 1 << 18 if the unit cannot take the token
+    // largest key magnitude (bf16 bits), 1 << 16 if the block took the fp64 loop for it, 1 << 17 if a wait expired, 1 << 18
+    // if the unit cannot take the token
     uint32_t state;
+    uint32_t cut_for;                             // bf16: the unit's magnitude before the appended key; 0 if that asks for the fp64 loop
     struct alignas(16) Counts {                   // what the blocks tell one another after their verdicts
         uint32_t flags;                           // heads to be formed exactly
         int count, n_imp, pad;                    // kept slots and important keys of the block
@@ -109,7 +111,7 @@ template <int NW> struct DcMisc {
     int n_moved;                                  // row moves of the unit
     int scan[NW * 32];
 };
-constexpr uint32_t kDcBad = 1u << 16, kDcExpired = 1u << 17, kDcFull = 1u << 18;
+constexpr uint32_t kDcWide = 1u << 16, kDcExpired = 1u << 17, kDcFull = 1u << 18;
 
 struct DcSmem { int prob, q, pieces, newrow, logits, bars, misc, total; };
 template <typename T, int D, int GP, int NW>
@@ -120,7 +122,8 @@ __host__ __device__ inline DcSmem dc_smem_layout(int lcap) {
     auto take = [&](int bytes) { int at = off; off = (off + bytes + 127) / 128 * 128; return at; };
     s.prob = take(NW * S::kProb);
     s.q = take(GP * D * (S::kBf16 ? 2 : 8));      // fp32: widened to fp64
-    s.pieces = take(S::kBf16 ? D / 16 * S::kPieces * 128 : 0);
+    // (or the queries widened to fp64)
+    s.pieces = take(S::kBf16 ? (D / 16 * S::kPieces * 128 > GP * D * 8 ? D / 16 * S::kPieces * 128 : GP * D * 8) : 0);
     s.newrow = take(2 * S::kRow);
     s.bars = take(NW * S::kStages * 8);
     s.misc = take((int)sizeof(DcMisc<NW>));
@@ -163,6 +166,16 @@ template <typename T, int N> __device__ __forceinline__ void load_slice_cg(const
     }
 }
 
+// the largest of the lanes' numbers (none NaN): of the high words, then of the low words that go with it
+__device__ __forceinline__ double warp_max(double x) {
+    const long long b = __double_as_longlong(x);
+    const unsigned long long o = (unsigned long long)(b ^ ((b >> 63) | (long long)0x8000000000000000ull));
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(o >> 32));
+    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(o >> 32) == hi ? (uint32_t)o : 0u);
+    const unsigned long long m = ((unsigned long long)hi << 32) | lo;
+    return __longlong_as_double((long long)(m >> 63 ? m ^ 0x8000000000000000ull : ~m));
+}
+
 // exact q.k of a slot by a whole warp: fp64, before the 1/sqrt(d)
 template <typename T, int D>
 __device__ __forceinline__ double warp_exact_dot_cg(const T* q, const T* k, int lane) {
@@ -177,12 +190,11 @@ __device__ __forceinline__ double warp_exact_dot_cg(const T* q, const T* k, int 
 }
 
 // The marked heads, exactly, by the whole cluster: their log-sum-exp in fp64 with a running maximum, then the verdicts
-// that were left open (misc->open, or every slot of the block where those did not fit or magnitudes are beyond the pieces'
-// range). A verdict that was sure before holds for the exact threshold too, so adding importance is enough: the register
+// that were left open (misc->open, or every slot of the block where those did not fit). A verdict that was sure before holds for the exact threshold too, so adding importance is enough: the register
 // gets its newest bit (or stamp), the keep bit is set. About one step in ten of 32 units x 21000 keys comes here: 16 keys
 // per warp at a time instead of 8, and no second pass over the keys, took 100 us of such a step to 20.
 template <typename T, int D, int NW>
-__device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G, int t, int k_begin, int k_end, uint32_t heads, bool all_slots,
+__device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G, int t, int k_begin, int k_end, uint32_t heads,
                                             uint32_t* keep, DcMisc<NW>* misc, int cs) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & 3;
     const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
@@ -198,7 +210,7 @@ __device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G,
         added_imp += 1;
         if (!(atomicOr(keep + ((j - k_begin) >> 5), bit) & bit)) added += 1;
     };
-    const int n_open = all_slots || misc->n_open > kDcOpenCap ? -1 : misc->n_open;
+    const int n_open = misc->n_open > kDcOpenCap ? -1 : misc->n_open;
     for (int h = 0; h < G; ++h) {
         if (!((heads >> h) & 1u)) continue;
         const T* q = reinterpret_cast<const T*>(p.q) + ((size_t)u * G + h) * D;
@@ -259,7 +271,7 @@ __device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int 
             os &= os - 1u;
             const double s = warp_exact_dot_cg<T, D>(reinterpret_cast<const T*>(p.q) + ((size_t)u * G + h) * D,
                                                      reinterpret_cast<const T*>(p.K) + row * D, lane) * inv_root_dim(D);
-            const double th = misc->thr[h], e = (double)(eps_a * misc->qe[h]) + 1e-13 * (1.0 + fabs(th));
+            const double th = misc->thr[h], e = (eps_a > 0.f ? (double)(eps_a * misc->qe[h]) : 0.0) + 1e-13 * (1.0 + fabs(th));
             if (lane == src && s - th > e) imp = true;
             if (lane == 0 && fabs(s - th) <= e) {
                 atomicOr(&misc->cnt.flags, 1u << h);
@@ -271,6 +283,172 @@ __device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int 
     }
     if (lane == 0) atomicAdd(p.counters + CNT_NEAR, (unsigned long long)n_near);
     return imp;
+}
+
+// The tiles of a warp: where they lie, the copies that fetch them, and the repair of the one that holds the appended token
+// or the unit's end.
+template <typename T, int D, int GP, int NW> struct DcTiles {
+    using S = DcShape<T, D, GP>;
+    const DecodeParams& p;
+    const CUtensorMap &kmap, &vmap;
+    const int32_t* pt_u;
+    unsigned char *ring, *newrow;
+    uint32_t bars;
+    int u, l_old, t, k_begin, k_end, my_n, my_page;           // lane i keeps the page entry of the warp's tile i
+
+    __device__ __forceinline__ int first_key(int it) const { return k_begin + ((int)(threadIdx.x >> 5) + it * NW) * kDcKeys; }
+    __device__ __forceinline__ int row0(int it) const {       // first row of a tile in the layer's K / V storage (all lanes call)
+        const int j = first_key(it);
+        if (!pt_u) return (int)((size_t)u * p.C) + j;
+        const int pg = it < 32 ? __shfl_sync(0xffffffffu, my_page, it) : __ldcg(pt_u + (j >> 5));
+        return (int)page_row(pg, j, p.pool_pages, p.status);
+    }
+    __device__ __forceinline__ void issue(const CUtensorMap& map, int row, int stage) const {             // lane 0
+        const uint32_t bar = bars + stage * 8, dst = smem_addr(ring + stage * S::kTile);
+        mbar_expect_tx(bar, S::kTile);
+#pragma unroll
+        for (int x = 0; x < S::kBoxes; ++x) tma_load_2d(dst + x * S::kBox, &map, x * (128 / Elem<T>::kBytes), row, bar);
+    }
+    // the appended token's row replaces whatever the copy fetched for its slot; rows past the unit's end become zero
+    __device__ __forceinline__ void patch(unsigned char* tile, int j0, int n_valid, int which, int it) const {
+        const int lane = threadIdx.x & 31;
+        auto chunk_at = [&](int r, int c) { return tile + (c >> 3) * S::kBox + r * 128 + ((((c & 7) ^ r) & 7) << 4); };
+        if (l_old >= j0 && l_old < j0 + kDcKeys) {
+            const int row = row0(it);
+            if (lane < S::kRow / 16) {
+                const uint4 x = *reinterpret_cast<const uint4*>(newrow + which * S::kRow + lane * 16);
+                *reinterpret_cast<uint4*>(chunk_at(l_old - j0, lane)) = x;
+                unsigned char* storage = reinterpret_cast<unsigned char*>(which ? p.V : p.K);
+                reinterpret_cast<uint4*>(storage + (size_t)(row + (l_old - j0)) * S::kRow)[lane] = x;
+            }
+            if (which == 0 && lane == 0) { p.word[(size_t)u * p.C + l_old] = 0u; p.pos[(size_t)u * p.C + l_old] = t; }
+        }
+        if (n_valid < kDcKeys)
+            for (int x = lane; x < (kDcKeys - n_valid) * (S::kRow / 16); x += 32)
+                *reinterpret_cast<uint4*>(chunk_at(n_valid + x / (S::kRow / 16), x % (S::kRow / 16))) = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+    }
+};
+
+// The streaming loop in fp64 on the CUDA cores for NG heads: a key per lane, its channels shared by two half-warps; P.V by
+// fp32 FMAs. qd: the queries as doubles [NG][D], pr: room for 16 x NG probabilities, lg: the block's logits [slot][NG].
+// Magnitudes are whatever the inputs are: references and sums stay in fp64, a logit beyond fp32 is kept as an infinity (its
+// verdict is formed again). A logit of +infinity makes its head's output NaN and no key important; so does NaN, but for bf16
+// with 128 channels and up to four heads, where it counts for nothing: what the kernels for these shapes have always done
+// (the block-per-split kernel there, the generic one elsewhere). Returns false if a wait expired.
+template <typename T, int D, int GP, int NW, int NG>
+__device__ __forceinline__ bool dc_stream_fp64(const DcTiles<T, D, GP, NW>& c, const double* qd, float* pr, float* lg, float* rec, DcMisc<NW>* misc) {
+    using S = DcShape<T, D, GP>;
+    constexpr int kKs = S::kKs, kVs = S::kVs, NC = D / 32;    // channels a lane accumulates
+    constexpr int kHalf = S::kRow / 32, kEl = 16 / Elem<T>::kBytes;             // 16-byte chunks of half a row, elements of one
+    // bf16: twice only, next to the tensor-core loop (a call costs that loop 2 %, all eight chunks unrolled 0.7 %, two nothing)
+    constexpr int kUnroll = S::kBf16 ? 2 : kHalf;
+    constexpr bool kNanPasses = !(S::kBf16 && D == 128 && GP <= 4);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, key = lane & 15, half = lane >> 4;
+    bool failed = false, first = true;
+    float acc[NG][NC];
+    double Zl[NG], Mref[NG];
+#pragma unroll
+    for (int x = 0; x < NG; ++x) {
+        Zl[x] = 0.0; Mref[x] = -INFINITY;
+#pragma unroll
+        for (int e = 0; e < NC; ++e) acc[x][e] = 0.f;
+    }
+    for (int it = 0; it < c.my_n; ++it) {
+        const int j0 = c.first_key(it), n_valid = min(kDcKeys, c.k_end - j0);
+        const int ks = it % kKs, vs = it % kVs;
+        unsigned char* ktile = c.ring + ks * S::kTile;
+        unsigned char* vtile = c.ring + (kKs + vs) * S::kTile;
+        const bool edge = n_valid < kDcKeys || (c.l_old >= j0 && c.l_old < j0 + kDcKeys);
+        if (!failed && !mbar_wait(c.bars + ks * 8, (it / kKs) & 1)) failed = true;
+        if (edge) c.patch(ktile, j0, n_valid, 0, it);
+        double s[NG];
+#pragma unroll
+        for (int x = 0; x < NG; ++x) s[x] = 0.0;
+#pragma unroll kUnroll
+        for (int i = 0; i < kHalf; ++i) {
+            const int ch = half * kHalf + i;
+            const uint4 raw = *reinterpret_cast<const uint4*>(ktile + (ch >> 3) * S::kBox + key * 128 + (((ch ^ key) & 7) << 4));
+            double kd[kEl];
+            if constexpr (S::kBf16) {
+                unpack8_to_double(raw, kd);
+            } else {
+                kd[0] = (double)__uint_as_float(raw.x); kd[1] = (double)__uint_as_float(raw.y);
+                kd[2] = (double)__uint_as_float(raw.z); kd[3] = (double)__uint_as_float(raw.w);
+            }
+#pragma unroll
+            for (int x = 0; x < NG; ++x)
+#pragma unroll
+                for (int e = 0; e < kEl; e += 2) {
+                    const double2 q = *reinterpret_cast<const double2*>(qd + x * D + ch * kEl + e);
+                    s[x] = fma(q.x, kd[e], s[x]); s[x] = fma(q.y, kd[e + 1], s[x]);
+                }
+        }
+        __syncwarp();
+        if (it + kKs < c.my_n) {
+            const int r0 = c.row0(it + kKs);
+            if (lane == 0) { fence_async_smem(); c.issue(c.kmap, r0, ks); }
+        }
+        const bool on = key < n_valid;
+        bool over = first;
+#pragma unroll
+        for (int x = 0; x < NG; ++x) {
+            s[x] = (s[x] + __shfl_xor_sync(0xffffffffu, s[x], 16)) * inv_root_dim(D);
+            over |= on && s[x] > Mref[x] + 16.0;
+        }
+        if (__any_sync(0xffffffffu, over)) {
+#pragma unroll
+            for (int x = 0; x < NG; ++x) {
+                const double mn = fmax(Mref[x], warp_max(on && s[x] == s[x] ? s[x] : -INFINITY));
+                const double sc = first || mn == -INFINITY ? 0.0 : exp_nonpos(Mref[x] - mn);
+                Zl[x] *= sc;
+                Mref[x] = mn;
+#pragma unroll
+                for (int e = 0; e < NC; ++e) acc[x][e] *= (float)sc;
+            }
+            first = false;
+        }
+#pragma unroll
+        for (int x = 0; x < NG; ++x) {
+            if (NG > 1 && (x & 1) != half) continue;          // the half-warps share the heads
+            double ex = on ? exp_nonpos(s[x] - Mref[x]) : 0.0;
+            if (on && (s[x] == INFINITY || (kNanPasses && s[x] != s[x]))) ex = NAN;
+            if (NG > 1 || half == 0) {
+                Zl[x] += ex;
+                pr[key * NG + x] = (float)ex;
+                if (on) lg[(j0 - c.k_begin + key) * NG + x] = s[x] == s[x] ? (float)s[x] : -INFINITY;
+            }
+        }
+        __syncwarp();
+        if (!failed && !mbar_wait(c.bars + (kKs + vs) * 8, (it / kVs) & 1)) failed = true;
+        if (edge) c.patch(vtile, j0, n_valid, 1, it);
+#pragma unroll 4
+        for (int r = 0; r < kDcKeys; ++r) {
+            const int at = lane * NC * Elem<T>::kBytes, ch = at >> 4;           // the lane's channels
+            const unsigned char* src = vtile + (ch >> 3) * S::kBox + r * 128 + (((ch ^ r) & 7) << 4) + (at & 15);
+            float v[NC];
+            load_slice<T, NC>(reinterpret_cast<const T*>(src), v);
+#pragma unroll
+            for (int x = 0; x < NG; ++x) {
+                const float pj = pr[r * NG + x];
+#pragma unroll
+                for (int e = 0; e < NC; ++e) acc[x][e] = fmaf(pj, v[e], acc[x][e]);
+            }
+        }
+        __syncwarp();
+        if (it + kVs < c.my_n) {
+            const int r0 = c.row0(it + kVs);
+            if (lane == 0) { fence_async_smem(); c.issue(c.vmap, r0, kKs + vs); }
+        }
+    }
+#pragma unroll
+    for (int x = 0; x < NG; ++x) {
+        Zl[x] = warp_sum(Zl[x]);
+        if (lane == 0) { misc->wM[warp][x] = Mref[x]; misc->wZ[warp][x] = Zl[x]; }
+#pragma unroll
+        for (int e = 0; e < NC; ++e) rec[x * D + lane * NC + e] = acc[x][e];
+    }
+    return !failed;
 }
 
 template <typename T, int D, int GP, int NW>
@@ -353,27 +531,16 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     float* lg = fits ? reinterpret_cast<float*>(smem + lay.logits)
                      : reinterpret_cast<float*>(p.stash + (size_t)u * G * p.C) + (size_t)k_begin * G;   // the unit's own scratch: launches overlap
     int my_page = 0;
-    if (pt_u) {                                               // lane i keeps the page entry of the warp's tile i
+    if (pt_u) {
         const int j = k_begin + (warp + lane * NW) * kDcKeys;
         if (j < k_end) my_page = __ldcg(pt_u + (j >> 5));
     }
-    auto tile_row0 = [&](int it) -> int {                     // first row of a tile in the layer's K / V storage (all lanes call)
-        const int j = k_begin + (warp + it * NW) * kDcKeys;
-        if (!pt_u) return (int)((size_t)u * p.C) + j;
-        const int pg = it < 32 ? __shfl_sync(0xffffffffu, my_page, it) : __ldcg(pt_u + (j >> 5));
-        return (int)page_row(pg, j, p.pool_pages, p.status);
-    };
-    auto issue = [&](const CUtensorMap& map, int row0, int stage) {             // lane 0
-        const uint32_t bar = bars + stage * 8, dst = smem_addr(ring + stage * S::kTile);
-        mbar_expect_tx(bar, S::kTile);
-#pragma unroll
-        for (int x = 0; x < S::kBoxes; ++x) tma_load_2d(dst + x * S::kBox, &map, x * (128 / Elem<T>::kBytes), row0, bar);
-    };
+    const DcTiles<T, D, GP, NW> tiles{p, kmap, vmap, pt_u, ring, newrow, bars, u, l_old, t, k_begin, k_end, my_n, my_page};
 #pragma unroll
     for (int it = 0; it < (kKs > kVs ? kKs : kVs); ++it)
         if (it < my_n) {
-            const int r0 = tile_row0(it);
-            if (lane == 0) { if (it < kKs) issue(kmap, r0, it); if (it < kVs) issue(vmap, r0, kKs + it); }
+            const int r0 = tiles.row0(it);
+            if (lane == 0) { if (it < kKs) tiles.issue(kmap, r0, it); if (it < kVs) tiles.issue(vmap, r0, kKs + it); }
         }
     cp_async_wait_all();
     if (!kBf16) {
@@ -384,39 +551,15 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
 
     // ---- 1. streaming ----
     const double inv_root_d = inv_root_dim(D);
-    unsigned char* Kl = reinterpret_cast<unsigned char*>(p.K);
-    unsigned char* Vl = reinterpret_cast<unsigned char*>(p.V);
     uint32_t* wordu = p.word + (size_t)u * p.C;
     int32_t* posu = p.pos + (size_t)u * p.C;
     bool failed = false;
-    double Zl[NH];
-    float Mref[NH];
-#pragma unroll
-    for (int x = 0; x < NH; ++x) { Zl[x] = 0.0; Mref[x] = -INFINITY; }
-    // the appended token's row replaces whatever the copy fetched for its slot; rows past the unit's end become zero
-    auto patch_tile = [&](unsigned char* tile, int j0, int n_valid, int which, int it) {
-        auto chunk_at = [&](int r, int c) { return tile + (c >> 3) * S::kBox + r * 128 + ((((c & 7) ^ r) & 7) << 4); };
-        if (l_old >= j0 && l_old < j0 + kDcKeys) {
-            const int row0 = tile_row0(it);
-            if (lane < S::kRow / 16) {
-                const uint4 x = *reinterpret_cast<const uint4*>(newrow + which * S::kRow + lane * 16);
-                *reinterpret_cast<uint4*>(chunk_at(l_old - j0, lane)) = x;
-                reinterpret_cast<uint4*>((which ? Vl : Kl) + (size_t)(row0 + (l_old - j0)) * S::kRow)[lane] = x;
-            }
-            if (which == 0 && lane == 0) { wordu[l_old] = 0u; posu[l_old] = t; }
-        }
-        if (n_valid < kDcKeys)
-            for (int x = lane; x < (kDcKeys - n_valid) * (S::kRow / 16); x += 32)
-                *reinterpret_cast<uint4*>(chunk_at(n_valid + x / (S::kRow / 16), x % (S::kRow / 16))) = make_uint4(0, 0, 0, 0);
-        __syncwarp();
-    };
     float* rec = reinterpret_cast<float*>(ring);              // the warp's record [G][D], once its tiles are done
 
     if constexpr (kBf16) {
         // pieces of the queries, as B fragments (column n = lane / 4): every warp needs all of them, so a warp cuts the
         // queries' channels 16 kk.. of kk = warp, warp + NW, ... and the others read them from shared memory
         constexpr int KK = D / 16, kPieces = S::kPieces;
-        uint32_t b1[KK][2], b2[GP == 2 ? 1 : KK][2], b3[GP == 8 ? KK : 1][2];
         uint32_t* pieces = reinterpret_cast<uint32_t*>(smem + lay.pieces);      // [KK][kPieces / 2][32 lanes][2]
         {
             const int n = lane >> 2;
@@ -430,7 +573,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 1));
             m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 2));
             const bool ok = m16 < kSplitMaxBits;
-            if (!ok) state |= kDcBad;
+            if (__any_sync(0xffffffffu, !ok) || kmax_old >= kSplitMaxBits) state |= kDcWide;
+            if (tid == 0) misc->cut_for = state & kDcWide ? 0u : kmax_old;
             const float c = split_query_const(ok ? __uint_as_float(m16 << 16) : 1.f);
             float n1 = 0.f, n2 = 0.f, n3 = 0.f;
             for (int kk = warp; kk < KK; kk += NW) {
@@ -476,25 +620,6 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 misc->qe_part[warp][hq] = dp.bound_scale * 1.05f * ((GP == 8 ? 4.6e-6f : 2.6e-6f) * (n1 * 1.01f) * (1.f / 8192.f) + (3.3e-5f + 1.3e-4f) * n3 + 2.4e-7f * n2 * (1.f / 64.f));
         }
         __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < KK; ++kk) {
-            const uint2* src = reinterpret_cast<const uint2*>(pieces) + kk * (kPieces / 2) * 32 + lane;
-            const uint2 x = src[0];
-            b1[kk][0] = x.x; b1[kk][1] = x.y;
-            if constexpr (kPieces > 2) { const uint2 y = src[32]; b2[kk][0] = y.x; b2[kk][1] = y.y; }
-            if constexpr (kPieces > 4) { const uint2 z = src[64]; b3[kk][0] = z.x; b3[kk][1] = z.y; }
-        }
-        if (tid < G) {
-            float e = 0.f;
-#pragma unroll
-            for (int w = 0; w < NW; ++w) e += misc->qe_part[w][tid];
-            misc->qe[tid] = e * 1.0001f;
-        }
-        float accd[D / 16][4];
-#pragma unroll
-        for (int cb = 0; cb < D / 16; ++cb)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) accd[cb][e] = 0.f;
         // The keys are cut on a grid of the unit's, kept in p.kmax: the largest magnitude it has ever held (scanning every
         // tile for its own cost 96 instructions of 550 per tile and a chain of 32 dependent ones).
         uint32_t kmax = kmax_old;
@@ -506,306 +631,241 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             }
             kmax = max(kmax, __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16)));
         }
-        if (kmax >= kSplitMaxBits) { state |= kDcBad; kmax = kSplitMaxBits; }
-        const SplitGrid g = split_grid(kmax);
-        const int h0 = GP == 8 ? 2 * (lane & 3) : (lane & 3);                    // the thread's head(s)
-        // Lane offsets of the fragment loads inside a tile. Rows are 128 bytes and a tile starts on a multiple of 1024, so
-        // 16-byte chunk c of the lane's row (at c ^ row mod 8) is one exclusive-or away from chunk 0 or 1.
-        const uint32_t klane = (lane & 15) * 128 + (((lane >> 4) ^ (lane & 7)) << 4);
-        const uint32_t vlane = (((lane >> 4) << 3) + (lane & 7)) * 128 + ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
-        const uint32_t ring_a = smem_addr(ring);
-        bool first = true;
-        // The tile that needs patching (keys past the block's end, or the appended slot, which is the unit's last) is the
-        // block's last one.
-        const int whole = k_end == l ? n_keys - 1 : n_keys;
-        float* lgp = lg + (warp * kDcKeys + (lane >> 2)) * G + h0;
-        int left = n_keys - warp * kDcKeys;                   // keys from the tile's first on
-        for (int it = 0; it < my_n; ++it, left -= NW * kDcKeys, lgp += NW * kDcKeys * G) {
-            const int n_valid = min(kDcKeys, left);
-            const int ks = it % kKs, vs = it % kVs;
-            const bool edge = n_keys - left + kDcKeys > whole;
-            if (!failed && !mbar_wait(bars + ks * 8, (it / kKs) & 1)) failed = true;   // once one wait has expired the rest are skipped
-            if (edge) patch_tile(ring + ks * S::kTile, k_end - left, n_valid, 0, it);
-            const uint32_t arow = ring_a + ks * S::kTile + klane;
-            uint32_t a[4][4];                                 // 64 channels of the tile at a time
-            // sums of the products of pieces; see the head of the file
-            float x1[4], x2[4], x3[4], x4[4], lo[4];
+        if (kmax >= kSplitMaxBits) state |= kDcWide;
+        if (tid < G) {
+            float e = 0.f;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) e += misc->qe_part[w][tid];
+            misc->qe[tid] = e * 1.0001f;
+        }
+        if (state & kDcWide) {
+            double* qd = reinterpret_cast<double*>(pieces);
+            for (int x = tid; x < G * D; x += NT) qd[x] = (double)Elem<bf16_t>::load(reinterpret_cast<const bf16_t*>(smem + lay.q) + x);
+            __syncthreads();
+            float* pr = reinterpret_cast<float*>(prob);
+            if constexpr (GP == 2) {
+                if (G == 1) failed = !dc_stream_fp64<T, D, GP, NW, 1>(tiles, qd, pr, lg, rec, misc);
+                else failed = !dc_stream_fp64<T, D, GP, NW, 2>(tiles, qd, pr, lg, rec, misc);
+            } else {
+                failed = !dc_stream_fp64<T, D, GP, NW, GP>(tiles, qd, pr, lg, rec, misc);
+            }
+        } else {
+            uint32_t b1[KK][2], b2[GP == 2 ? 1 : KK][2], b3[GP == 8 ? KK : 1][2];
 #pragma unroll
             for (int kk = 0; kk < KK; ++kk) {
-                if (kk % 4 == 0) {
+                const uint2* src = reinterpret_cast<const uint2*>(pieces) + kk * (kPieces / 2) * 32 + lane;
+                const uint2 x = src[0];
+                b1[kk][0] = x.x; b1[kk][1] = x.y;
+                if constexpr (kPieces > 2) { const uint2 y = src[32]; b2[kk][0] = y.x; b2[kk][1] = y.y; }
+                if constexpr (kPieces > 4) { const uint2 z = src[64]; b3[kk][0] = z.x; b3[kk][1] = z.y; }
+            }
+            double Zl[NH];
+            float Mref[NH];
 #pragma unroll
-                    for (int x = 0; x < 4; ++x) ldmatrix_x4(a[x], (arow ^ (x << 5)) + (kk >> 2) * S::kBox);
-                    if (kk + 4 == KK) {                       // the rest of the tile is in registers: its stage is free
-                        __syncwarp();
-                        if (it + kKs < my_n) {
-                            const int r0 = tile_row0(it + kKs);
-                            if (lane == 0) issue(kmap, r0, ks);
+            for (int x = 0; x < NH; ++x) { Zl[x] = 0.0; Mref[x] = -INFINITY; }
+            float accd[D / 16][4];
+#pragma unroll
+            for (int cb = 0; cb < D / 16; ++cb)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) accd[cb][e] = 0.f;
+            const SplitGrid g = split_grid(kmax);
+            const int h0 = GP == 8 ? 2 * (lane & 3) : (lane & 3);                    // the thread's head(s)
+            // Lane offsets of the fragment loads inside a tile. Rows are 128 bytes and a tile starts on a multiple of 1024, so
+            // 16-byte chunk c of the lane's row (at c ^ row mod 8) is one exclusive-or away from chunk 0 or 1.
+            const uint32_t klane = (lane & 15) * 128 + (((lane >> 4) ^ (lane & 7)) << 4);
+            const uint32_t vlane = (((lane >> 4) << 3) + (lane & 7)) * 128 + ((((lane >> 3) & 1) ^ (lane & 7)) << 4);
+            const uint32_t ring_a = smem_addr(ring);
+            bool first = true;
+            // The tile that needs patching (keys past the block's end, or the appended slot, which is the unit's last) is the
+            // block's last one.
+            const int whole = k_end == l ? n_keys - 1 : n_keys;
+            float* lgp = lg + (warp * kDcKeys + (lane >> 2)) * G + h0;
+            int left = n_keys - warp * kDcKeys;                   // keys from the tile's first on
+            for (int it = 0; it < my_n; ++it, left -= NW * kDcKeys, lgp += NW * kDcKeys * G) {
+                const int n_valid = min(kDcKeys, left);
+                const int ks = it % kKs, vs = it % kVs;
+                const bool edge = n_keys - left + kDcKeys > whole;
+                if (!failed && !mbar_wait(bars + ks * 8, (it / kKs) & 1)) failed = true;   // once one wait has expired the rest are skipped
+                if (edge) tiles.patch(ring + ks * S::kTile, k_end - left, n_valid, 0, it);
+                const uint32_t arow = ring_a + ks * S::kTile + klane;
+                uint32_t a[4][4];                                 // 64 channels of the tile at a time
+                // sums of the products of pieces; see the head of the file
+                float x1[4], x2[4], x3[4], x4[4], lo[4];
+#pragma unroll
+                for (int kk = 0; kk < KK; ++kk) {
+                    if (kk % 4 == 0) {
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) ldmatrix_x4(a[x], (arow ^ (x << 5)) + (kk >> 2) * S::kBox);
+                        if (kk + 4 == KK) {                       // the rest of the tile is in registers: its stage is free
+                            __syncwarp();
+                            if (it + kKs < my_n) {
+                                const int r0 = tiles.row0(it + kKs);
+                                if (lane == 0) tiles.issue(kmap, r0, ks);
+                            }
+                        }
+                    }
+                    uint32_t k1[4], k2[4], r2[4];
+                    split_key(a[kk % 4], g, k1, k2, r2);
+                    float tt[4];
+                    auto mma = [&](float (&d)[4], const uint32_t (&x)[4], const uint32_t (&b)[2]) {   // the sum's first term, or one more
+                        if (kk == 0) mma16816_zero(d, x, b[0], b[1]); else mma16816(d, x, b[0], b[1]);
+                    };
+                    mma(x1, k1, b1[kk]);
+                    mma16816_zero(tt, r2, b1[kk][0], b1[kk][1]);
+                    if constexpr (GP == 8) {
+                        mma(x2, k1, b2[kk]);                      // k1.q2 + k2.q1: exact together
+                        mma16816(x2, k2, b1[kk][0], b1[kk][1]);
+                        mma(x4, k2, b2[kk]);                      // exact
+                        mma16816(tt, r2, b2[kk][0], b2[kk][1]);
+                        mma(x3, k1, b3[kk]);
+                        mma16816(x3, k2, b3[kk][0], b3[kk][1]);
+                    } else {
+                        mma(x2, k2, b1[kk]);
+                        if constexpr (GP == 4) {
+                            mma(x3, k1, b2[kk]);
+                            mma(x4, k2, b2[kk]);
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) lo[e] = kk == 0 ? tt[e] : lo[e] + tt[e];
+                }
+                // Eq. 2's exponent, thread's keys lane / 4 and + 8
+                double s[NK][NH];
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    if constexpr (GP == 8) {
+#pragma unroll
+                        for (int x = 0; x < 2; ++x) {
+                            const int e = 2 * y + x;
+                            s[y][x] = (((double)x1[e] + (double)x2[e]) + (double)(x4[e] + (lo[e] + x3[e]))) * inv_root_d;
+                        }
+                    } else {
+                        // columns: (.q1, .q2) of the thread's head; two heads: the q3 products two lanes further on
+                        float small = x2[2 * y + 1] + (lo[2 * y] + lo[2 * y + 1]);
+                        if constexpr (GP == 4) small += x3[2 * y] + x4[2 * y];
+                        else small += __shfl_xor_sync(0xffffffffu, x1[2 * y] + (x2[2 * y] + lo[2 * y]), 2);
+                        s[y][0] = (((double)x1[2 * y] + (double)(x1[2 * y + 1] + x2[2 * y])) + (double)small) * inv_root_d;
+                    }
+                }
+                bool on[NK][NH];
+                bool over = first;
+#pragma unroll
+                for (int y = 0; y < 2; ++y)
+#pragma unroll
+                    for (int x = 0; x < NH; ++x) {
+                        on[y][x] = (lane >> 2) + 8 * y < n_valid && h0 + x < G;
+                        over |= on[y][x] && (float)s[y][x] > Mref[x] + 16.f;
+                    }
+                if (__any_sync(0xffffffffu, over)) {              // the reference moves: first tile, or a logit far above it (rare)
+                    float scf[NH];
+#pragma unroll
+                    for (int x = 0; x < NH; ++x) {
+                        float mt = fmaxf(on[0][x] ? (float)s[0][x] : -INFINITY, on[1][x] ? (float)s[1][x] : -INFINITY);
+#pragma unroll
+                        for (int o = 4; o < 32; o <<= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+                        const float mn = fmaxf(Mref[x], mt);
+                        const double sc = first || mn == -INFINITY ? 0.0 : exp_nonpos((double)Mref[x] - (double)mn);
+                        Zl[x] *= sc;
+                        scf[x] = (float)sc;
+                        Mref[x] = mn;
+                    }
+                    if constexpr (GP == 2) {                      // lanes 2 and 3 of four accumulate the third parts of heads 0 and 1
+                        const float o = __shfl_xor_sync(0xffffffffu, scf[0], 2);
+                        if (lane & 2) scf[0] = o;
+                    }
+#pragma unroll
+                    for (int cb = 0; cb < D / 16; ++cb)           // the accumulators' columns are the thread's own heads
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) accd[cb][e] *= GP == 8 ? scf[(e & 1) % NH] : scf[0];
+                    first = false;
+                }
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    const int kq = (lane >> 2) + 8 * y;
+                    float pf[NH];
+#pragma unroll
+                    for (int x = 0; x < NH; ++x) {
+                        const float sf = (float)s[y][x];
+                        const double ex = exp_nonpos_where(on[y][x] && sf - Mref[x] > -700.f, s[y][x] - (double)Mref[x]);
+                        Zl[x] += ex;
+                        pf[x] = (float)ex;
+                        if (on[y][x]) lgp[8 * y * G + x] = sf;
+                    }
+                    uint32_t* const dst = reinterpret_cast<uint32_t*>(prob + kq * 16) + (lane & 3);
+                    if constexpr (GP == 8) {                      // [key][8 heads] first parts, then second, then third
+#pragma unroll
+                        for (int part = 0; part < 3; ++part) {
+                            const uint32_t w = pack_bf16x2(pf[1 % NH], pf[0]);
+                            dst[part * 64] = w;
+                            pf[0] -= __uint_as_float(w << 16);
+                            pf[1 % NH] -= __uint_as_float(w & 0xffff0000u);
+                        }
+                    } else {                                      // [key][head x (first, second)], and (third, 0) behind them
+                        const uint32_t a = pack_bf16x2(0.f, pf[0]) << 16;
+                        const float r = pf[0] - __uint_as_float(a);
+                        const uint32_t b = pack_bf16x2(r, 0.f) & 0xffff0000u, c = pack_bf16x2(0.f, r - __uint_as_float(b));
+                        if constexpr (GP == 4) {
+                            dst[0] = b | (a >> 16);
+                            dst[64] = c;
+                        } else if (h0 < 2) {
+                            dst[0] = b | (a >> 16);
+                            dst[2] = c;
                         }
                     }
                 }
-                uint32_t k1[4], k2[4], r2[4];
-                split_key(a[kk % 4], g, k1, k2, r2);
-                float tt[4];
-                auto mma = [&](float (&d)[4], const uint32_t (&x)[4], const uint32_t (&b)[2]) {   // the sum's first term, or one more
-                    if (kk == 0) mma16816_zero(d, x, b[0], b[1]); else mma16816(d, x, b[0], b[1]);
-                };
-                mma(x1, k1, b1[kk]);
-                mma16816_zero(tt, r2, b1[kk][0], b1[kk][1]);
+                __syncwarp();
+                if (!failed && !mbar_wait(bars + (kKs + vs) * 8, (it / kVs) & 1)) failed = true;
+                if (edge) tiles.patch(ring + (kKs + vs) * S::kTile, k_end - left, n_valid, 1, it);
+                {
+                    uint32_t bf[4];
+                    ldmatrix_x4_trans(bf, smem_addr(prob) + (GP > 2 ? lane : lane & 15) * 16);        // keys 0-7 | 8-15 (| the next parts)
+                    uint32_t b3p[2];
+                    if constexpr (GP == 8) ldmatrix_x2_trans(b3p, smem_addr(prob) + 512 + (lane & 15) * 16);
+                    const uint32_t vrow = ring_a + (kKs + vs) * S::kTile + vlane;
+#pragma unroll
+                    for (int cb = 0; cb < D / 16; ++cb) {
+                        uint32_t va[4];
+                        ldmatrix_x4_trans(va, (vrow ^ ((cb & 3) << 5)) + (cb >> 2) * S::kBox);
+                        mma16816(accd[cb], va, bf[0], bf[1]);     // Eq. 1
+                        if constexpr (GP > 2) mma16816(accd[cb], va, bf[2], bf[3]);
+                        if constexpr (GP == 8) mma16816(accd[cb], va, b3p[0], b3p[1]);
+                    }
+                }
+                __syncwarp();
+                if (it + kVs < my_n) {
+                    const int r0 = tiles.row0(it + kVs);
+                    if (lane == 0) tiles.issue(vmap, r0, kKs + vs);
+                }
+            }
+#pragma unroll
+            for (int x = 0; x < NH; ++x) {
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) Zl[x] += __shfl_xor_sync(0xffffffffu, Zl[x], o);
+                if ((lane >> 2) == 0 && h0 + x < G) { misc->wM[warp][h0 + x] = (double)Mref[x]; misc->wZ[warp][h0 + x] = Zl[x]; }
+            }
+#pragma unroll
+            for (int cb = 0; cb < D / 16; ++cb) {
                 if constexpr (GP == 8) {
-                    mma(x2, k1, b2[kk]);                      // k1.q2 + k2.q1: exact together
-                    mma16816(x2, k2, b1[kk][0], b1[kk][1]);
-                    mma(x4, k2, b2[kk]);                      // exact
-                    mma16816(tt, r2, b2[kk][0], b2[kk][1]);
-                    mma(x3, k1, b3[kk]);
-                    mma16816(x3, k2, b3[kk][0], b3[kk][1]);
+                    rec[h0 * D + cb * 16 + (lane >> 2)] = accd[cb][0];
+                    rec[(h0 + 1) * D + cb * 16 + (lane >> 2)] = accd[cb][1];
+                    rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][2];
+                    rec[(h0 + 1) * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][3];
                 } else {
-                    mma(x2, k2, b1[kk]);
-                    if constexpr (GP == 4) {
-                        mma(x3, k1, b2[kk]);
-                        mma(x4, k2, b2[kk]);
+                    float a0 = accd[cb][0] + accd[cb][1], a1 = accd[cb][2] + accd[cb][3];  // the parts' sums
+                    if constexpr (GP == 2) {
+                        a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+                        a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
                     }
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) lo[e] = kk == 0 ? tt[e] : lo[e] + tt[e];
-            }
-            // Eq. 2's exponent, thread's keys lane / 4 and + 8
-            double s[NK][NH];
-#pragma unroll
-            for (int y = 0; y < 2; ++y) {
-                if constexpr (GP == 8) {
-#pragma unroll
-                    for (int x = 0; x < 2; ++x) {
-                        const int e = 2 * y + x;
-                        s[y][x] = (((double)x1[e] + (double)x2[e]) + (double)(x4[e] + (lo[e] + x3[e]))) * inv_root_d;
+                    if (h0 < G) {
+                        rec[h0 * D + cb * 16 + (lane >> 2)] = a0;
+                        rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = a1;
                     }
-                } else {
-                    // columns: (.q1, .q2) of the thread's head; two heads: the q3 products two lanes further on
-                    float small = x2[2 * y + 1] + (lo[2 * y] + lo[2 * y + 1]);
-                    if constexpr (GP == 4) small += x3[2 * y] + x4[2 * y];
-                    else small += __shfl_xor_sync(0xffffffffu, x1[2 * y] + (x2[2 * y] + lo[2 * y]), 2);
-                    s[y][0] = (((double)x1[2 * y] + (double)(x1[2 * y + 1] + x2[2 * y])) + (double)small) * inv_root_d;
-                }
-            }
-            bool on[NK][NH];
-            bool over = first;
-#pragma unroll
-            for (int y = 0; y < 2; ++y)
-#pragma unroll
-                for (int x = 0; x < NH; ++x) {
-                    on[y][x] = (lane >> 2) + 8 * y < n_valid && h0 + x < G;
-                    over |= on[y][x] && (float)s[y][x] > Mref[x] + 16.f;
-                }
-            if (__any_sync(0xffffffffu, over)) {              // the reference moves: first tile, or a logit far above it (rare)
-                float scf[NH];
-#pragma unroll
-                for (int x = 0; x < NH; ++x) {
-                    float mt = fmaxf(on[0][x] ? (float)s[0][x] : -INFINITY, on[1][x] ? (float)s[1][x] : -INFINITY);
-#pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
-                    const float mn = fmaxf(Mref[x], mt);
-                    const double sc = first || mn == -INFINITY ? 0.0 : exp_nonpos((double)Mref[x] - (double)mn);
-                    Zl[x] *= sc;
-                    scf[x] = (float)sc;
-                    Mref[x] = mn;
-                }
-                if constexpr (GP == 2) {                      // lanes 2 and 3 of four accumulate the third parts of heads 0 and 1
-                    const float o = __shfl_xor_sync(0xffffffffu, scf[0], 2);
-                    if (lane & 2) scf[0] = o;
-                }
-#pragma unroll
-                for (int cb = 0; cb < D / 16; ++cb)           // the accumulators' columns are the thread's own heads
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) accd[cb][e] *= GP == 8 ? scf[(e & 1) % NH] : scf[0];
-                first = false;
-            }
-#pragma unroll
-            for (int y = 0; y < 2; ++y) {
-                const int kq = (lane >> 2) + 8 * y;
-                float pf[NH];
-#pragma unroll
-                for (int x = 0; x < NH; ++x) {
-                    const float sf = (float)s[y][x];
-                    const double ex = exp_nonpos_where(on[y][x] && sf - Mref[x] > -700.f, s[y][x] - (double)Mref[x]);
-                    Zl[x] += ex;
-                    pf[x] = (float)ex;
-                    if (on[y][x]) lgp[8 * y * G + x] = sf;
-                }
-                uint32_t* const dst = reinterpret_cast<uint32_t*>(prob + kq * 16) + (lane & 3);
-                if constexpr (GP == 8) {                      // [key][8 heads] first parts, then second, then third
-#pragma unroll
-                    for (int part = 0; part < 3; ++part) {
-                        const uint32_t w = pack_bf16x2(pf[1 % NH], pf[0]);
-                        dst[part * 64] = w;
-                        pf[0] -= __uint_as_float(w << 16);
-                        pf[1 % NH] -= __uint_as_float(w & 0xffff0000u);
-                    }
-                } else {                                      // [key][head x (first, second)], and (third, 0) behind them
-                    const uint32_t a = pack_bf16x2(0.f, pf[0]) << 16;
-                    const float r = pf[0] - __uint_as_float(a);
-                    const uint32_t b = pack_bf16x2(r, 0.f) & 0xffff0000u, c = pack_bf16x2(0.f, r - __uint_as_float(b));
-                    if constexpr (GP == 4) {
-                        dst[0] = b | (a >> 16);
-                        dst[64] = c;
-                    } else if (h0 < 2) {
-                        dst[0] = b | (a >> 16);
-                        dst[2] = c;
-                    }
-                }
-            }
-            __syncwarp();
-            if (!failed && !mbar_wait(bars + (kKs + vs) * 8, (it / kVs) & 1)) failed = true;
-            if (edge) patch_tile(ring + (kKs + vs) * S::kTile, k_end - left, n_valid, 1, it);
-            {
-                uint32_t bf[4];
-                ldmatrix_x4_trans(bf, smem_addr(prob) + (GP > 2 ? lane : lane & 15) * 16);        // keys 0-7 | 8-15 (| the next parts)
-                uint32_t b3p[2];
-                if constexpr (GP == 8) ldmatrix_x2_trans(b3p, smem_addr(prob) + 512 + (lane & 15) * 16);
-                const uint32_t vrow = ring_a + (kKs + vs) * S::kTile + vlane;
-#pragma unroll
-                for (int cb = 0; cb < D / 16; ++cb) {
-                    uint32_t va[4];
-                    ldmatrix_x4_trans(va, (vrow ^ ((cb & 3) << 5)) + (cb >> 2) * S::kBox);
-                    mma16816(accd[cb], va, bf[0], bf[1]);     // Eq. 1
-                    if constexpr (GP > 2) mma16816(accd[cb], va, bf[2], bf[3]);
-                    if constexpr (GP == 8) mma16816(accd[cb], va, b3p[0], b3p[1]);
-                }
-            }
-            __syncwarp();
-            if (it + kVs < my_n) {
-                const int r0 = tile_row0(it + kVs);
-                if (lane == 0) issue(vmap, r0, kKs + vs);
-            }
-        }
-#pragma unroll
-        for (int x = 0; x < NH; ++x) {
-#pragma unroll
-            for (int o = 4; o < 32; o <<= 1) Zl[x] += __shfl_xor_sync(0xffffffffu, Zl[x], o);
-            if ((lane >> 2) == 0 && h0 + x < G) { misc->wM[warp][h0 + x] = Mref[x]; misc->wZ[warp][h0 + x] = Zl[x]; }
-        }
-#pragma unroll
-        for (int cb = 0; cb < D / 16; ++cb) {
-            if constexpr (GP == 8) {
-                rec[h0 * D + cb * 16 + (lane >> 2)] = accd[cb][0];
-                rec[(h0 + 1) * D + cb * 16 + (lane >> 2)] = accd[cb][1];
-                rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][2];
-                rec[(h0 + 1) * D + cb * 16 + 8 + (lane >> 2)] = accd[cb][3];
-            } else {
-                float a0 = accd[cb][0] + accd[cb][1], a1 = accd[cb][2] + accd[cb][3];  // the parts' sums
-                if constexpr (GP == 2) {
-                    a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
-                    a1 += __shfl_xor_sync(0xffffffffu, a1, 2);
-                }
-                if (h0 < G) {
-                    rec[h0 * D + cb * 16 + (lane >> 2)] = a0;
-                    rec[h0 * D + cb * 16 + 8 + (lane >> 2)] = a1;
                 }
             }
         }
         state = (state & ~0xffffu) | kmax;
     } else {
-        const double* qd = reinterpret_cast<const double*>(smem + lay.q);
-        float* pr = reinterpret_cast<float*>(prob);           // [key][GP]
-        constexpr int NC = D / 32;                            // channels a lane accumulates
-        float acc[GP][NC];
-#pragma unroll
-        for (int x = 0; x < GP; ++x)
-#pragma unroll
-            for (int e = 0; e < NC; ++e) acc[x][e] = 0.f;
-        const int key = lane & 15, half = lane >> 4;
-        bool first = true;
-        for (int it = 0; it < my_n; ++it) {
-            const int j0 = k_begin + (warp + it * NW) * kDcKeys, n_valid = min(kDcKeys, k_end - j0);
-            const int ks = it % kKs, vs = it % kVs;
-            unsigned char* ktile = ring + ks * S::kTile;
-            unsigned char* vtile = ring + (kKs + vs) * S::kTile;
-            const bool edge = n_valid < kDcKeys || (l_old >= j0 && l_old < j0 + kDcKeys);
-            if (!failed && !mbar_wait(bars + ks * 8, (it / kKs) & 1)) failed = true;
-            if (edge) patch_tile(ktile, j0, n_valid, 0, it);
-            double s[GP];
-#pragma unroll
-            for (int x = 0; x < GP; ++x) s[x] = 0.0;
-#pragma unroll
-            for (int bx = 0; bx < S::kBoxes / 2; ++bx) {
-                const int box = half * (S::kBoxes / 2) + bx;
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float4 kv = *reinterpret_cast<const float4*>(ktile + box * S::kBox + key * 128 + ((c ^ (key & 7)) << 4));
-                    const double k4[4] = {(double)kv.x, (double)kv.y, (double)kv.z, (double)kv.w};
-#pragma unroll
-                    for (int x = 0; x < GP; ++x) {
-                        const double2 qa = *reinterpret_cast<const double2*>(qd + x * D + box * 32 + c * 4);
-                        const double2 qb = *reinterpret_cast<const double2*>(qd + x * D + box * 32 + c * 4 + 2);
-                        s[x] = fma(qa.x, k4[0], s[x]); s[x] = fma(qa.y, k4[1], s[x]);
-                        s[x] = fma(qb.x, k4[2], s[x]); s[x] = fma(qb.y, k4[3], s[x]);
-                    }
-                }
-            }
-            __syncwarp();
-            if (it + kKs < my_n) {
-                const int r0 = tile_row0(it + kKs);
-                if (lane == 0) { fence_async_smem(); issue(kmap, r0, ks); }
-            }
-            const bool on = key < n_valid;
-            bool over = first;
-#pragma unroll
-            for (int x = 0; x < GP; ++x) {
-                s[x] = (s[x] + __shfl_xor_sync(0xffffffffu, s[x], 16)) * inv_root_d;
-                over |= on && (float)s[x] > Mref[x] + 16.f;
-            }
-            if (__any_sync(0xffffffffu, over)) {
-#pragma unroll
-                for (int x = 0; x < GP; ++x) {
-                    float mt = on ? (float)s[x] : -INFINITY;
-#pragma unroll
-                    for (int o = 1; o < 16; o <<= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o));
-                    const float mn = fmaxf(Mref[x], mt);
-                    const double sc = first || mn == -INFINITY ? 0.0 : exp_nonpos((double)Mref[x] - (double)mn);
-                    Zl[x] *= sc;
-                    Mref[x] = mn;
-#pragma unroll
-                    for (int e = 0; e < NC; ++e) acc[x][e] *= (float)sc;
-                }
-                first = false;
-            }
-#pragma unroll
-            for (int x = 0; x < GP; ++x) {
-                if (GP > 1 && (x & 1) != half) continue;      // the half-warps share the heads
-                const double ex = on ? exp_nonpos(s[x] - (double)Mref[x]) : 0.0;
-                if (GP > 1 || half == 0) {
-                    Zl[x] += ex;
-                    pr[key * GP + x] = (float)ex;
-                    if (on) lg[(j0 - k_begin + key) * GP + x] = (float)s[x];
-                }
-            }
-            __syncwarp();
-            if (!failed && !mbar_wait(bars + (kKs + vs) * 8, (it / kVs) & 1)) failed = true;
-            if (edge) patch_tile(vtile, j0, n_valid, 1, it);
-#pragma unroll 4
-            for (int r = 0; r < kDcKeys; ++r) {
-                const int c = NC == 4 ? lane : lane >> 1;     // 16-byte chunk of the lane's channels
-                const unsigned char* src = vtile + (c >> 3) * S::kBox + r * 128 + ((((c & 7) ^ r) & 7) << 4) + (NC == 2 ? (lane & 1) * 8 : 0);
-                float v[NC];
-                load_slice<float, NC>(reinterpret_cast<const float*>(src), v);
-#pragma unroll
-                for (int x = 0; x < GP; ++x) {
-                    const float pj = pr[r * GP + x];
-#pragma unroll
-                    for (int e = 0; e < NC; ++e) acc[x][e] = fmaf(pj, v[e], acc[x][e]);
-                }
-            }
-            __syncwarp();
-            if (it + kVs < my_n) {
-                const int r0 = tile_row0(it + kVs);
-                if (lane == 0) { fence_async_smem(); issue(vmap, r0, kKs + vs); }
-            }
-        }
-#pragma unroll
-        for (int x = 0; x < GP; ++x) {
-            Zl[x] = warp_sum(Zl[x]);
-            if (lane == 0) { misc->wM[warp][x] = Mref[x]; misc->wZ[warp][x] = Zl[x]; }
-#pragma unroll
-            for (int e = 0; e < NC; ++e) rec[x * D + lane * NC + e] = acc[x][e];
-        }
+        failed = !dc_stream_fp64<T, D, GP, NW, GP>(tiles, reinterpret_cast<const double*>(smem + lay.q), reinterpret_cast<float*>(prob), lg, rec, misc);
         if (warp == 0 && lane < GP) misc->qe[lane] = 0.f;
     }
     if (failed) state |= kDcExpired;
@@ -847,13 +907,12 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
 
     // ---- thresholds of Definition 3.1 in log form, the same in every block: warp h reduces head h over the cluster's warps ----
     constexpr int kEnt = kDcMaxCluster * NW / 32;             // (block, warp) entries per lane
-    float m[kEnt];
-    double z[kEnt];
+    double m[kEnt], z[kEnt];
     auto load_entries = [&](int h) {
 #pragma unroll
         for (int y = 0; y < kEnt; ++y) {
             const int e = y * 32 + lane, blk = e / NW, w = e % NW;
-            m[y] = blk < cs ? __uint_as_float(ld_peer_u32(map_rank(smem_addr(&misc->wM[w][h]), blk))) : -INFINITY;
+            m[y] = blk < cs ? ld_peer_f64(map_rank(smem_addr(&misc->wM[w][h]), blk)) : -INFINITY;
             z[y] = blk < cs ? ld_peer_f64(map_rank(smem_addr(&misc->wZ[w][h]), blk)) : 0.0;
         }
     };
@@ -873,28 +932,28 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     }
     // the appended key enters the unit's magnitude whatever became of the queries (every block has read the old one)
     if (kBf16 && rank == 0 && tid == 0) p.kmax[u] = unit_state & 0xffffu;
-    // error of a head's log-sum-exp per unit of qe (every logit of it is off by at most this much)
-    const float eps_a = kBf16 ? split_amax(min(unit_state & 0xffffu, kSplitMaxBits)) * (float)inv_root_d * 1.0001f : 0.f;
+    // error of a head's log-sum-exp per unit of qe (every logit of it is off by at most this much): from the magnitude the
+    // keys were cut for. Where the appended key sent its block to the fp64 loop the others cut for the one before it.
+    const uint32_t cut_for = unit_state & kDcWide ? misc->cut_for : unit_state & 0xffffu;
+    const float eps_a = kBf16 && (cut_for || !(unit_state & kDcWide)) ? split_amax(cut_for) * (float)inv_root_d * 1.0001f : 0.f;
     for (int h = warp; h < G; h += NW) {
-        float M = -INFINITY;
-        double Z = 0.0;
+        double M = -INFINITY, Z = 0.0;
         if (h >= NW) load_entries(h);
 #pragma unroll
-        for (int y = 0; y < kEnt; ++y) M = fmaxf(M, m[y]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        for (int y = 0; y < kEnt; ++y) M = fmax(M, m[y]);
+        M = warp_max(M);
 #pragma unroll
         for (int y = 0; y < kEnt; ++y) {
-            const double sc = m[y] == -INFINITY ? 0.0 : exp_nonpos((double)m[y] - (double)M);
+            const double sc = m[y] == -INFINITY ? 0.0 : exp_nonpos(m[y] - M);
             Z = fma(z[y], sc, Z);
             misc->sc[h][y * 32 + lane] = (float)sc;
         }
         Z = warp_sum(Z);                                      // a fixed tree: every block gets the same bits
         if (lane == 0) {
-            const double thr = (double)M + log(Z) + p.log_alpha - misc->log_t;
-            const float tf = (float)thr, ta = fabsf(tf);
+            const double thr = M + log(Z) + p.log_alpha - misc->log_t;
+            const float tf = thr == thr ? (float)thr : INFINITY, ta = fabsf(tf);     // behind a NaN no key is important
             misc->thr[h] = thr; misc->Zt[h] = Z; misc->thr_f[h] = tf;
-            misc->slack[h] = 2.f * eps_a * misc->qe[h] + (ta < 3e38f ? ta : 0.f) * 1.3e-7f + 1e-12f;
+            misc->slack[h] = (eps_a > 0.f ? 2.f * eps_a * misc->qe[h] : 0.f) + (ta < 3e38f ? ta : 0.f) * 1.3e-7f + 1e-12f;
         }
     }
     __syncthreads();
@@ -933,7 +992,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 for (int h = 0; h < GP; ++h) {
                     const float sf = sv[k][h], margin = sf - tf[h], err = fmaf(fabsf(sf), 6.1e-8f, sl[h]);
                     sure |= margin >= err;
-                    near |= margin > -err ? 1u << h : 0u;
+                    near |= !(margin <= -err) ? 1u << h : 0u; // (two infinities: to be formed again)
                 }
                 open[k] = i < n_keys && !sure ? near : 0u;
                 imp |= i < n_keys && sure ? 1u << k : 0u;
@@ -970,7 +1029,6 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         if (lane == 0) {
             atomicAdd(&misc->cnt.count, n_keep);
             atomicAdd(&misc->cnt.n_imp, n_imp);
-            if (unit_state & kDcBad) atomicOr(&misc->cnt.flags, (1u << G) - 1u);    // magnitudes beyond the pieces' range: every head exactly
         }
     }
     cluster_sync();
@@ -990,7 +1048,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         const uint32_t marks = __reduce_or_sync(0xffffffffu, pc.x);
         if (marks) {                                          // uniform in the cluster
             cluster_sync();
-            dc_exact_heads<T, D, NW>(p, u, G, t, k_begin, k_end, marks, (unit_state & kDcBad) != 0u, keep, misc, cs);
+            dc_exact_heads<T, D, NW>(p, u, G, t, k_begin, k_end, marks, keep, misc, cs);
             cluster_sync();
             load_counts();
         }

@@ -147,3 +147,84 @@ def test_layers_of_different_history_stepped_together_still_report_their_lengths
         gpu.corm_decode_step_layers(0, *([t[s, l] for l in range(2)] for t in (q, k, v, out)))
     assert max(int(gpu.corm_cache_live_lens(l).max()) for l in range(2)) < 1000
     assert gpu.corm_cache_kernel_launches() - before == 1
+
+
+# magnitudes that the pieces of the tensor-core logits do not hold (2^56 and more), and logits beyond fp32
+OUT_OF_RANGE = [
+    # dtype, head_dim, group, kv heads, batch, prompt range, steps, paged, what
+    ("bf16", 128, 1, 2, 2, (300, 420), 12, False, "keys"),
+    ("bf16", 128, 2, 2, 1, (31, 33), 40, True, "late key"),
+    ("bf16", 128, 4, 2, 2, (700, 900), 12, True, "queries"),
+    ("bf16", 128, 8, 1, 2, (500, 600), 12, False, "late key"),
+    ("bf16", 64, 1, 3, 1, (1, 17), 40, True, "late key"),
+    ("bf16", 64, 4, 2, 1, (900, 1000), 12, False, "keys"),
+    ("bf16", 64, 8, 1, 1, (600, 600), 12, False, "both"),
+    ("bf16", 128, 4, 1, 1, (3000, 3000), 6, False, "both"),
+    ("f32", 128, 2, 2, 1, (400, 500), 12, False, "both"),
+    ("f32", 64, 1, 1, 2, (100, 130), 24, True, "late key"),
+]
+
+
+@pytest.mark.parametrize("case", OUT_OF_RANGE, ids=lambda c: "-".join(str(x) for x in c))
+def test_decode_of_magnitudes_out_of_the_pieces_range(case):
+    """Prompts of ordinary keys, then keys and queries scaled by powers of two (so that logits are spread over 2^60 and
+    the top key has all the weight, or, between one key and its double, exactly known weights): the oracle's registers,
+    rows and outputs through per-step and chained calls."""
+    dtype, d, G, nkv, B, prange, steps, paged, what = case
+    cfg = _cfg(dtype, d, G, nkv, B, prange, steps, 8, 16)
+    data = generate(cfg)
+    q, kn = data.q.copy(), data.k_new.copy()
+    big = 2.0 ** 60 if dtype == "bf16" else 2.0 ** 70
+    if what == "keys":
+        kn[2:] *= big
+    elif what == "late key":
+        kn[steps // 2] *= big
+    elif what == "queries":
+        q[3:6] *= big
+    else:
+        kn[1] *= big
+        q[2:] *= big if dtype == "bf16" else 2.0 ** 60
+    pages = -(-B * nkv * (cfg.max_tokens // 32 + 2) // 32) * 32 if paged else 0
+    one, many = (make_gpu_cache(cfg, B, nkv, pool_pages=pages) for _ in range(2))
+    orc = make_oracle(cfg, B, nkv)
+    orc.set_near_band(1e-12)
+    p = [to_dev(x, dtype) for x in (data.k_prompt, data.v_prompt, data.q_last)]
+    for g in (one, many):
+        g.corm_cache_set_tuning(0, 4)                  # the cluster kernel for every shape
+        g.corm_compress_prompt(0, *p, data.prompt_lens)
+    orc.compress_prompt(0, data.k_prompt, data.v_prompt, data.q_last, data.prompt_lens)
+    qd, kd, vd = (to_dev(x, dtype) for x in (q, kn, data.v_new))
+    outs = many.corm_decode_steps(0, 1, qd[:, None], kd[:, None], vd[:, None])
+    for s in range(steps):
+        ref = orc.decode_step(0, q[s], kn[s], data.v_new[s])
+        out = one.corm_decode_step(0, qd[s], kd[s], vd[s])
+        assert np.abs(out.float().cpu().numpy() - ref).max() <= OUT_TOL[dtype], s
+        assert np.abs(outs[s, 0].float().cpu().numpy() - ref).max() <= OUT_TOL[dtype], s
+        assert_states_equal(one, orc, 0, B, nkv, f"step {s}")
+    assert_states_equal(many, orc, 0, B, nkv, "multi-step")
+    assert one.corm_cache_stats()["device_status"] == many.corm_cache_stats()["device_status"] == 0
+
+
+@pytest.mark.parametrize("dtype,d,G", [("bf16", 128, 8), ("bf16", 64, 2), ("f32", 128, 1), ("f32", 64, 4)])
+@pytest.mark.parametrize("what", ["nan", "inf"])
+def test_a_key_that_is_not_a_number(dtype, d, G, what):
+    """One NaN or infinite channel of one key, against the generic kernel (tuning value 0): the same outputs are NaN, the
+    others agree, and so do the registers."""
+    cfg = _cfg(dtype, d, G, 2, 1, (200, 260), 12, 8, 16)
+    data = generate(cfg)
+    kn = data.k_new.copy()
+    kn[3, 0, 1, 7] = np.nan if what == "nan" else np.inf
+    caches = [make_gpu_cache(cfg, 1, 2) for _ in range(2)]
+    caches[1].corm_cache_set_tuning(0, False)
+    p = [to_dev(x, dtype) for x in (data.k_prompt, data.v_prompt, data.q_last)]
+    for g in caches:
+        g.corm_compress_prompt(0, *p, data.prompt_lens)
+    for s in range(12):
+        a, b = (g.corm_decode_step(0, to_dev(data.q[s], dtype), to_dev(kn[s], dtype), to_dev(data.v_new[s], dtype)).float().cpu()
+                for g in caches)
+        assert torch.equal(torch.isnan(a), torch.isnan(b)), s
+        assert (a - b).nan_to_num().abs().max() <= OUT_TOL[dtype], s
+        for h in range(2):
+            x, y = (g.corm_cache_export_state(0, 0, h) for g in caches)
+            i, j = np.argsort(x["pos"]), np.argsort(y["pos"])
+            assert np.array_equal(x["pos"][i], y["pos"][j]) and np.array_equal(x["word"][i], y["word"][j]), (s, h)
