@@ -19,7 +19,7 @@
 // channels), as with fp32 products on the CUDA cores.
 // fp32: a key per lane (its channels shared by two half-warps), fp64 products on the CUDA cores, P.V by fp32 FMAs. A bf16
 // unit with a key or query element the pieces cannot hold (2^56 and more, infinity, NaN) takes that loop too: its products
-// have no bounds on the tensor cores.
+// have no bounds on the tensor cores. So does one whose bounds are too wide to be of use (kDcReach).
 //
 // What bounds it: on units of a few hundred keys the chain of round trips (set-up 2 us, first tiles 2, exchange and
 // thresholds 2.5, verdicts 1, exchange 1, moves 2, launch 2); on long units instruction issue in the streaming loop: about
@@ -111,6 +111,17 @@ template <int NW> struct DcMisc {
     int n_moved;                                  // row moves of the unit
     int scan[NW * 32];
 };
+
+// When a bf16 unit takes the fp64 loop. Errors of the tensor-core logits grow with A Aq, the product of the unit's largest key
+// and query magnitudes, while its logits need not (one large key channel next to small query channels). Where the bounds
+// leave verdicts open in most steps (about A Aq times the unit's keys, per head), forming heads again costs more than fp64
+// does: us per step never / always / a multi-pass fp64 kernel, one key channel 256 times the others: 32 units x 20000 keys,
+// G 4, 146 / 126 / 131; 32 units x 8200 keys, G 4, 66 / 57 / 55; 128 units x 3400 keys, G 1, 82 / 54 / 54 (ordinary keys 55 /
+// 54 / 54); but 128 units x 2800 keys, G 4, 78 / 82 / 84 and 64 units x 700 keys, G 8, 31 / 51. One and two heads switch
+// earlier: their fp64 loop costs 0-5 and 12 % of ordinary steps, that of four 20-55 %. And beyond A Aq = 16384 logits would
+// be less exact than fp32 probabilities.
+constexpr float kDcReach = 16384.f;
+template <int GP> __device__ __forceinline__ float dc_reach_keys(int G) { return GP > 2 ? 6e7f : G == 2 ? 4e6f : 5e5f; }
 constexpr uint32_t kDcWide = 1u << 16, kDcExpired = 1u << 17, kDcFull = 1u << 18;
 
 struct DcSmem { int prob, q, pieces, newrow, logits, bars, misc, total; };
@@ -561,6 +572,11 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         // queries' channels 16 kk.. of kk = warp, warp + NW, ... and the others read them from shared memory
         constexpr int KK = D / 16, kPieces = S::kPieces;
         uint32_t* pieces = reinterpret_cast<uint32_t*>(smem + lay.pieces);      // [KK][kPieces / 2][32 lanes][2]
+        uint32_t qmax = 0u;                                   // largest magnitude of the unit's queries, as kmax
+        auto too_wide = [&](uint32_t k) {                     // of keys of up to this magnitude
+            const float reach = __uint_as_float(k << 16) * __uint_as_float(qmax << 16);
+            return max(k, qmax) >= kSplitMaxBits || reach > kDcReach || reach * (float)l > dc_reach_keys<GP>(G);
+        };
         {
             const int n = lane >> 2;
             const int hq = GP == 8 ? n : GP == 4 ? n >> 1 : (n & 3) >> 1;
@@ -573,7 +589,8 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 1));
             m16 = max(m16, __shfl_xor_sync(0xffffffffu, m16, 2));
             const bool ok = m16 < kSplitMaxBits;
-            if (__any_sync(0xffffffffu, !ok) || kmax_old >= kSplitMaxBits) state |= kDcWide;
+            qmax = __reduce_max_sync(0xffffffffu, m16);
+            if (too_wide(kmax_old)) state |= kDcWide;
             if (tid == 0) misc->cut_for = state & kDcWide ? 0u : kmax_old;
             const float c = split_query_const(ok ? __uint_as_float(m16 << 16) : 1.f);
             float n1 = 0.f, n2 = 0.f, n3 = 0.f;
@@ -631,7 +648,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             }
             kmax = max(kmax, __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16)));
         }
-        if (kmax >= kSplitMaxBits) state |= kDcWide;
+        if (too_wide(kmax)) state |= kDcWide;
         if (tid < G) {
             float e = 0.f;
 #pragma unroll

@@ -228,3 +228,33 @@ def test_a_key_that_is_not_a_number(dtype, d, G, what):
             x, y = (g.corm_cache_export_state(0, 0, h) for g in caches)
             i, j = np.argsort(x["pos"]), np.argsort(y["pos"])
             assert np.array_equal(x["pos"][i], y["pos"][j]) and np.array_equal(x["word"][i], y["word"][j]), (s, h)
+
+
+# one key channel f times the others, its query channel 1 / f: logits stay as they are, bounds on the tensor cores grow by f.
+# f = 64 is on this side of the switch to the fp64 loop for groups and beyond it for single heads, 4096 beyond it for all
+@pytest.mark.parametrize("f", [64.0, 4096.0])
+@pytest.mark.parametrize("d,G", [(128, 1), (128, 2), (128, 4), (128, 8), (64, 1), (64, 4)])
+def test_one_large_key_channel(d, G, f):
+    """Outputs stay the exact ones rounded (the bound of the test of that name) and registers the oracle's, also where some
+    of a unit's keys, from the middle of the run on, are the first large ones."""
+    nkv, B, steps = max(1, 8 // G), 2, 24
+    cfg = _cfg("bf16", d, G, nkv, B, (900, 1100), steps, 8, 64)
+    data = generate(cfg)
+    rnd = (lambda a: torch.from_numpy(a).to(torch.bfloat16).float().numpy())
+    q, kn, kp, ql = (rnd(x.copy()) for x in (data.q, data.k_new, data.k_prompt, data.q_last))
+    q[..., 3] /= f
+    kn[..., 3] *= f
+    kp[0, ..., 3] *= f                                 # the second sequence meets its first large key in a decode step
+    ql[0, ..., 3] /= f
+    gpu, orc = make_gpu_cache(cfg, B, nkv), make_oracle(cfg, B, nkv)
+    orc.set_near_band(1e-11)
+    gpu.corm_compress_prompt(0, to_dev(kp, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(ql, "bf16"), data.prompt_lens)
+    orc.compress_prompt(0, kp, data.v_prompt, ql, data.prompt_lens)
+    wrong = total = 0
+    for s in range(steps):
+        ref = torch.from_numpy(orc.decode_step(0, q[s], kn[s], data.v_new[s])).to(torch.bfloat16)
+        out = gpu.corm_decode_step(0, to_dev(q[s], "bf16"), to_dev(kn[s], "bf16"), to_dev(data.v_new[s], "bf16")).cpu()
+        wrong += int((out != ref).sum())
+        total += out.numel()
+        assert_states_equal(gpu, orc, 0, B, nkv, f"step {s}")
+    assert wrong <= 3e-4 * total + 6, (wrong, total)
