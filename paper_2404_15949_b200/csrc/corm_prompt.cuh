@@ -653,7 +653,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
                         for (int x = 0; x < 4; ++x) {
                             const int row = ru * 4 + x, qpos = R.pos(row);
                             if (j >= k_end || j >= qpos) continue;
-                            const double margin = acc[x] * inv_root_d - thr_sm[row], e = 1e-13 * (1.0 + fabs(thr_sm[row]));
+                            const double th = thr_sm[row], margin = acc[x] * inv_root_d - th, e = th > -INFINITY ? 1e-13 * (1.0 + fabs(th)) : 0.0;   // (alpha = 0: all important)
                             if (margin > e) mark = pc_join(w, mark, pc_mark(w, R.rho(row), qpos));
                             else if (margin >= -e) pc_leave_open(flags, misc, row, j);               // a tie (a query at position 1)
                         }

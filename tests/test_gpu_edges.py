@@ -258,3 +258,33 @@ def test_one_large_key_channel(d, G, f):
         total += out.numel()
         assert_states_equal(gpu, orc, 0, B, nkv, f"step {s}")
     assert wrong <= 3e-4 * total + 6, (wrong, total)
+
+
+def _prompt_time(cfg, data, dtype):
+    """median time of five prompt passes (ms), after two"""
+    gpu = make_gpu_cache(cfg, len(data.seqs), len(data.kv_heads))
+    p = [to_dev(x, dtype) for x in (data.k_prompt, data.v_prompt, data.q_last)]
+    times = []
+    for _ in range(7):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        torch.cuda.synchronize()
+        a.record()
+        gpu.corm_compress_prompt(0, *p, data.prompt_lens)
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    return sorted(times[2:])[2], gpu
+
+
+@pytest.mark.parametrize("d,G", [(128, 1), (64, 4)])
+def test_fp32_prompt_without_eviction_leaves_nothing_open(d, G):
+    """alpha = 0 puts every threshold at minus infinity: no verdict is near it, so the pass takes no longer than with
+    thresholds that evict (it took ten times as long while every key went through the exact rows)."""
+    t, cache = {}, None
+    for alpha in (1.0, 0.0):
+        cfg = _cfg("f32", d, G, 8, 8, (300, 300), 1, 8, 16, alpha=alpha)
+        t[alpha], cache = _prompt_time(cfg, generate(cfg), "f32")
+    assert (cache.corm_cache_live_lens(0) == 300).all()
+    word = cache.corm_cache_export_state(0, 0, 0)["word"]
+    assert (word[:293] == 0xff).all()
+    assert t[0.0] < 3 * t[1.0], t
