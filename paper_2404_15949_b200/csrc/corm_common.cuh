@@ -21,7 +21,7 @@ inline cudaError_t ensure_dynamic_smem(const void* kernel, size_t bytes) {
     static std::mutex mu;
     static Entry seen[kSlots];
     static int n_seen = 0;
-    if (bytes <= 48 * 1024) return cudaSuccess;
+    if (bytes <= 32 * 1024) return cudaSuccess;       // with the kernels' static shared memory (under 8 KB) below the default limit
     int device = 0;
     cudaError_t e = cudaGetDevice(&device);
     if (e != cudaSuccess) return e;

@@ -288,3 +288,21 @@ def test_fp32_prompt_without_eviction_leaves_nothing_open(d, G):
     word = cache.corm_cache_export_state(0, 0, 0)["word"]
     assert (word[:293] == 0xff).all()
     assert t[0.0] < 3 * t[1.0], t
+
+
+@pytest.mark.parametrize("C", [150000, 176000])
+def test_verdict_launch_next_to_the_default_shared_memory_limit(C):
+    """The verdict launch of long slabs takes 38-46 KB of dynamic shared memory next to its static lists: together they are
+    beyond what a kernel gets unasked."""
+    cfg = _cfg("bf16", 128, 1, 1, 1, (3000, 3000), 3, 8, 64)
+    data = generate(cfg)
+    gpu, orc = make_gpu_cache(cfg, 1, 1, max_tokens=C), make_oracle(cfg, 1, 1, max_tokens=C)
+    gpu.corm_cache_set_tuning(512, 3)
+    gpu.corm_compress_prompt(0, to_dev(data.k_prompt, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(data.q_last, "bf16"),
+                             data.prompt_lens)
+    orc.compress_prompt(0, data.k_prompt, data.v_prompt, data.q_last, data.prompt_lens)
+    for s in range(3):
+        gpu.corm_decode_step(0, to_dev(data.q[s], "bf16"), to_dev(data.k_new[s], "bf16"), to_dev(data.v_new[s], "bf16"))
+        orc.decode_step(0, data.q[s], data.k_new[s], data.v_new[s])
+    assert gpu.corm_cache_kernel_launches() == 2 + 6           # prompt pass; streaming and verdict launch per step
+    assert_states_equal(gpu, orc, 0, 1, 1, "end")
