@@ -298,22 +298,42 @@ corm_status_t monitor_similarity(corm_cache* c, int layer, const void* q, cudaSt
 // Tuning values 1 (automatic) and 4..6 (always) admit the cluster kernel.
 bool may_cluster(const corm_cache* c) { return (c->allow_fast == 1 || c->allow_fast >= 4) && !c->kmaps_row.empty(); }
 
-// The cluster kernel works out its shares on the device; the other kernels' grids are sized from the host's bound.
-bool grids_follow_bound(const corm_cache* c) {
-    return !may_cluster(c) || (c->allow_fast == 1 && c->cfg.kv_dtype == CORM_BF16 && c->cfg.head_dim == 128 && c->G == 1);
+// Few long units that lose next to nothing to eviction (alpha 0 or windows of more than 32 queries, or a small alpha on longer
+// ones still): a cluster has eight blocks at most, so they would leave multiprocessors idle, while the block-per-split kernel
+// cuts a unit into as many splits as there is room for and the verdict launch that follows has little to move. us per step,
+// cluster -> block-per-split with the verdict launch, alpha 0, keys per unit: G 1, 4000 / 16000 / 64000, 1 unit 16.3 -> 14.4 /
+// 36.8 -> 17.6 / 121 -> 30, 16 units 20 -> 16 / 53 -> 36 / 177 -> 116; G 2, 4000 / 8000 / 64000, 1 unit 16.5 -> 16.4 / 23.6 ->
+// 16.7 / 121 -> 34; G 4, 4000 / 8000 / 64000, 1 unit 17 -> 20 / 24 -> 20 / 126 -> 43, 16 units 22 -> 24 / 34 -> 32 / 193 -> 153.
+// With eviction at work its last block has many rows to move: alpha 1, 8 units, prompts of 16000, G 1, 26 -> 36.
+bool few_long_units(const corm_cache* c, int upper, int n_units) {
+    const corm_config_t& cf = c->cfg;
+    if (cf.kv_dtype != CORM_BF16 || cf.head_dim != 128 || c->G > 4 || (long long)n_units * kDcMaxCluster > c->sm_count) return false;
+    const bool stays = cf.alpha == 0.f || cf.window_w > 32 || (cf.alpha <= 0.25f && upper > 12288);
+    return stays && upper > (c->G == 1 ? 3072 : 6144);
 }
 
-// Whether the cluster kernel takes a step of units of up to `upper` keys. Everything but one query head per KV head on
-// bf16 / head_dim 128. That too where there are few enough units for two blocks each (us per step, block-per-split ->
-// cluster, prompts of 1000 keys: 32 units 16.5 -> 14.9; of 3500 keys: 128 units, alpha 0 52.4 -> 47.6, windows of 64
-// 53.8 -> 47.4, of 256 53.0 -> 48.0); up to 512 units where they are longer than a block of the block-per-split kernel
-// finishes on chip and eviction is at work (prompts of 4000 keys: 256 units 61 -> 43, 512 units 79 -> 71). Otherwise its
-// loop, which widens keys to fp64 instead of cutting them into pieces, streams faster (prompts of 1000 keys: 256 units 21.0
-// against 22.0, 512 units 30 against 38; of 3000 keys: 1024 units 84 against 102, alpha 0 265 against 297).
+// The cluster kernel works out its shares on the device; the other kernels' grids are sized from the host's bound.
+bool grids_follow_bound(const corm_cache* c) {
+    const corm_config_t& cf = c->cfg;
+    return !may_cluster(c) || (c->allow_fast == 1 && cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 &&
+                               (c->G == 1 || (c->G <= 4 && (long long)c->U * kDcMaxCluster <= c->sm_count)));
+}
+
+// Whether the cluster kernel takes a step of units of up to `upper` keys. Everything but few long units (above) and one query
+// head per KV head on bf16 / head_dim 128. That too where there are few enough units for two blocks each (us per step,
+// block-per-split -> cluster, prompts of 1000 keys: 32 units 16.5 -> 14.9; of 3500 keys: 128 units, alpha 0 52.4 -> 47.6, windows
+// of 64 53.8 -> 47.4, of 256 53.0 -> 48.0) and they are longer than two of the block-per-split kernel's shortest splits (1-128
+// units of 224 keys 10.8-12.2 against 10.2-12.8, of 324 keys 14.3-17.1 against 10.0-14.3; of 60 keys 10.4-12.6 against
+// 11.3-14.3, and in one call of several steps 8.3-8.8 against 10.9-11.5); up to 512 units where they are longer than a block of
+// the block-per-split kernel finishes on chip and eviction is at work (prompts of 4000 keys: 256 units 61 -> 43, 512 units 79 ->
+// 71). Otherwise its loop, which widens keys to fp64 instead of cutting them into pieces, streams faster (prompts of 1000 keys:
+// 256 units 21.0 against 22.0, 512 units 30 against 38; of 3000 keys: 1024 units 84 against 102, alpha 0 265 against 297).
 bool takes_cluster(const corm_cache* c, int upper, int n_units) {
     if (!may_cluster(c)) return false;
-    if (c->allow_fast >= 4 || c->cfg.kv_dtype != CORM_BF16 || c->cfg.head_dim != 128 || c->G >= 2) return true;
-    if (n_units <= c->sm_count) return true;
+    if (c->allow_fast >= 4) return true;
+    if (few_long_units(c, upper, n_units)) return false;
+    if (c->cfg.kv_dtype != CORM_BF16 || c->cfg.head_dim != 128 || c->G >= 2) return true;
+    if (n_units <= c->sm_count) return upper > 256;
     return upper > 1024 && n_units <= 512 && c->cfg.window_w <= 32 && c->cfg.alpha > 0.f;
 }
 
@@ -395,7 +415,9 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
     } else if (fast) {
         // the mean grows by at most one key per step, like the bound
         const int typical = mean_known ? std::min(upper, mean_sum / n_fused + c->steps[layer] - c->last_report_step[layer] + 1) : 0;
-        rc = launch_decode_fast(p, c->G, upper, typical, c->tune_split_len, c->sm_count, st, &n_launched, c->allow_fast,
+        // (few long units: the last split would walk its unit alone)
+        const int finish = c->allow_fast == 1 && few_long_units(c, upper, p.U) ? 3 : c->allow_fast;
+        rc = launch_decode_fast(p, c->G, upper, typical, c->tune_split_len, c->sm_count, st, &n_launched, finish,
                                 chain_ok_before, more && !c->monitor_similarity, &self_finishing);
         if (rc == CORM_OK && p.chain_wait) c->chained_launches += 1;
     } else {

@@ -96,6 +96,7 @@ def test_a_key_appended_next_to_an_overflowed_query_counts():
     kn[1][..., 0] += 32.0                              # a bit of 2^12 in bf16: logits 2.8 q_0 apart
     q[:2, ..., 1] = 2.0 ** 60
     gpu, orc = make_gpu_cache(cfg, B, nkv), make_oracle(cfg, B, nkv)
+    gpu.corm_cache_set_tuning(0, 4)                    # the cluster kernel
     orc.set_near_band(1e-10)
     gpu.corm_compress_prompt(0, to_dev(data.k_prompt, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(data.q_last, "bf16"),
                              data.prompt_lens)
@@ -306,3 +307,46 @@ def test_verdict_launch_next_to_the_default_shared_memory_limit(C):
         orc.decode_step(0, data.q[s], data.k_new[s], data.v_new[s])
     assert gpu.corm_cache_kernel_launches() == 2 + 6           # prompt pass; streaming and verdict launch per step
     assert_states_equal(gpu, orc, 0, 1, 1, "end")
+
+
+# the lines between the cluster and the block-per-split kernel: few long units that keep their keys take the latter and the
+# verdict launch (two launches a step), on either side of the length at which they do; short units of single heads it alone
+FEW_UNITS = [
+    # group, kv heads, batch, prompt, steps, w, alpha, paged, launches per step
+    (1, 1, 1, 3600, 6, 8, 0.0, False, 2),
+    (1, 2, 3, 3600, 6, 100, 1.0, True, 2),
+    (1, 1, 1, 3000, 6, 8, 0.0, False, 1),
+    (2, 1, 2, 6200, 4, 8, 0.0, True, 2),
+    (4, 2, 1, 6300, 4, 40, 1.0, False, 2),
+    (4, 2, 1, 6000, 4, 8, 0.0, True, 1),
+    (4, 1, 1, 12500, 3, 8, 0.25, False, 2),
+    (1, 2, 2, 240, 40, 8, 0.0, False, 1),               # 256 keys are reached on the way
+    (1, 2, 2, 120, 40, 4, 1.0, True, 1),
+]
+
+
+@pytest.mark.parametrize("case", FEW_UNITS, ids=lambda c: "-".join(str(x) for x in c))
+def test_few_units_on_either_side_of_the_kernels_lines(case):
+    G, nkv, B, P, steps, w, alpha, paged, launches = case
+    cfg = _cfg("bf16", 128, G, nkv, B, (P, P), steps, w, 32, alpha=alpha)
+    data = generate(cfg)
+    pages = -(-B * nkv * (cfg.max_tokens // 32 + 2) // 32) * 32 if paged else 0
+    one, many = (make_gpu_cache(cfg, B, nkv, pool_pages=pages) for _ in range(2))
+    orc = make_oracle(cfg, B, nkv)
+    orc.set_near_band(1e-11)
+    for g in (one, many):
+        g.corm_compress_prompt(0, to_dev(data.k_prompt, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(data.q_last, "bf16"),
+                               data.prompt_lens)
+    orc.compress_prompt(0, data.k_prompt, data.v_prompt, data.q_last, data.prompt_lens)
+    q, k, v = (to_dev(x, "bf16") for x in (data.q, data.k_new, data.v_new))
+    outs = many.corm_decode_steps(0, 1, q[:, None], k[:, None], v[:, None])
+    before = one.corm_cache_kernel_launches()
+    for s in range(steps):
+        ref = orc.decode_step(0, data.q[s], data.k_new[s], data.v_new[s])
+        out = one.corm_decode_step(0, q[s], k[s], v[s])
+        assert np.abs(out.float().cpu().numpy() - ref).max() <= OUT_TOL["bf16"], s
+        assert np.abs(outs[s, 0].float().cpu().numpy() - ref).max() <= OUT_TOL["bf16"], s
+    assert_states_equal(one, orc, 0, B, nkv, "per step")
+    assert_states_equal(many, orc, 0, B, nkv, "multi-step")
+    assert one.corm_cache_stats()["device_status"] == many.corm_cache_stats()["device_status"] == 0
+    assert one.corm_cache_kernel_launches() - before == launches * steps
