@@ -4,8 +4,9 @@
 // attention row (Eq. 2) before any verdict (Definition 3.1) can be taken. The cluster's blocks share the unit's keys
 // (whole 32-key words each) and go through
 //   A. logits of every row against the block's keys, summed as exp(s) per row (fp64, no running maximum: |s| below 650
-//      cannot overflow; anything larger sends the unit through the exact path below);
+//      cannot overflow);
 //   -- the blocks exchange their sums through distributed shared memory: one threshold per row
+//      (a unit with larger logits, or with bounds too wide to be of use, does A and B over in fp64: pc_fp64_rows)
 //   B. verdicts of the block's keys for every row -> verdict registers;
 //   -- the blocks exchange their counts of surviving keys
 //   C. every block gathers its own survivors (K, V rows, registers, positions) to their place in token order.
@@ -51,6 +52,11 @@ constexpr int kPcGroup = 4;                     // octets of rows (bf16) whose p
 constexpr int kPcGroupB = 8;                    // ... whose raw values do in phase B
 constexpr int kPcMaxCluster = 8;
 constexpr double kPcLogitLimit = 650.0;         // exp of anything below stays finite in fp64, also summed over 2^19 keys
+// Bound of a logit's error, times the prompt's keys, beyond which a unit does both phases in fp64: so many verdicts would be
+// left open that most rows are formed apart. us per pass, tensor cores / fp64, one key channel 256 and 1024 times the others:
+// 32 units x 32768 keys, G 4, w 16, 6240 / 4210 and 13440 / 4210; 32 x 8192, G 4, w 128, 8190 / 8080 and 25440 / 8080; 1024 x
+// 3250, w 8, 1570 / 3100 and 3070 / 3180; 128 x 3390, w 256, 5420 / 6510 and 14230 / 6510.
+constexpr double kPcReachKeys = 1.2;
 
 struct PromptClusterParams {
     PromptParams p;
@@ -135,16 +141,16 @@ __device__ __forceinline__ uint32_t pc_mark(int w, int rho, int qpos) { return w
 __device__ __forceinline__ uint32_t pc_join(int w, uint32_t a, uint32_t b) { return w <= 32 ? (a | b) : max(a, b); }
 
 // The marked rows, exactly, by all blocks of the cluster: log-sum-exp in fp64 with a running maximum, then the verdicts that
-// phase B left open (misc->open, or every key where those did not fit or `all_keys`). Verdicts that phase B was sure of hold
+// phase B left open (misc->open, or every key where those did not fit). Verdicts that phase B was sure of hold
 // for the exact threshold too, so adding marks is enough. Rare, but a launch is as long as its longest unit: with a key at a
 // time per warp and a second pass over the keys for the verdicts this took 714 us of 1592 on 32768-key prompts.
 template <typename T, int D>
-__device__ __noinline__ void pc_exact_rows(const PromptParams& p, const PcRows& R, const T* Qu, const T* Ku, int k_begin, int k_end, bool all_keys,
+__device__ __noinline__ void pc_exact_rows(const PromptParams& p, const PcRows& R, const T* Qu, const T* Ku, int k_begin, int k_end,
                                            const uint32_t* flags, uint32_t* words_g, PcMisc* misc, int cs) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & 3;
     const uint32_t mz_addr = smem_addr(misc->mz);
     auto row_of = [&](int j) -> const T* { return Ku + (size_t)j * D; };
-    const int n_open = all_keys || misc->n_open > kPcOpenCap ? -1 : misc->n_open;
+    const int n_open = misc->n_open > kPcOpenCap ? -1 : misc->n_open;
     for (int r = 0; r < R.rows; ++r) {
         if (!((flags[r >> 5] >> (r & 31)) & 1u)) continue;
         const int qpos = R.pos(r);
@@ -184,6 +190,183 @@ __device__ __noinline__ void pc_exact_rows(const PromptParams& p, const PcRows& 
         }
         cluster_sync();                                       // everybody has read mz; the marks of this row are written
     }
+}
+
+__device__ __forceinline__ void pc_leave_open(uint32_t* flags, PcMisc* misc, int row, int j) {
+    atomicOr(flags + (row >> 5), 1u << (row & 31));
+    const int at = atomicAdd(&misc->n_open, 1);
+    if (at < kPcOpenCap) misc->open[at] = make_int2(row, j);
+}
+
+// Units whose logits are too large for plain sums of exponentials (650 and more), whose elements the pieces cannot hold, or
+// whose error bounds are too wide to be of use: both phases in fp64 on the CUDA cores, with running maxima. A warp owns units
+// of four rows (the queries widened in shared memory), a lane one or two keys; warps share rows by groups of 32 keys where
+// there are fewer than eight row units. On return the thresholds and the scratch registers are there; rows are marked, and
+// their keys listed, for ties only. key_buf: 128 rows of keys, q_stage: 4 rows of doubles per warp, words: 128 registers.
+template <typename T, int D>
+__device__ __noinline__ void pc_fp64_rows(const PromptParams& p, const PcRows& R, const T* Qu, const T* Ku, int k_begin, int n_keys, unsigned char* key_buf,
+                                          double* q_stage, double* zs, double* thr_sm, uint32_t* words, uint32_t* words_g, uint32_t* flags, PcMisc* misc, int cs) {
+    constexpr int kRow = D * Elem<T>::kBytes, kChunks = kRow / 16, kEl = 16 / Elem<T>::kBytes, kSubs = kPcKeys / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nc = (n_keys + kPcKeys - 1) / kPcKeys;
+    const int n_ru = (R.rows + 3) / 4;
+    int slots = 1;                                            // warps side by side over the row units (a power of two)
+    while (slots < n_ru && slots < kPcWarps) slots *= 2;
+    const int groups = min(kPcWarps / slots, kSubs), my_ru = warp % slots, my_kg = warp / slots;
+    const bool works = my_ru < n_ru && my_kg < groups;
+    double* const q = q_stage + warp * 4 * D;
+    double* const ms = groups > 1 ? zs + 32 : thr_sm;         // running maxima next to the sums (fewer than 32 rows x groups)
+    auto load = [&](int c) {
+        __syncthreads();                                      // everybody is done with the chunk before
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(Ku + (size_t)(k_begin + c * kPcKeys) * D);
+        const int valid = n_keys - c * kPcKeys;
+#pragma unroll 8
+        for (int x = tid; x < kPcKeys * kChunks; x += kPcThreads) {
+            const int r = x / kChunks;
+            *reinterpret_cast<uint4*>(key_buf + pc_offset<T, D>(r, x % kChunks)) = r < valid ? __ldg(reinterpret_cast<const uint4*>(src) + x) : make_uint4(0, 0, 0, 0);
+        }
+        __syncthreads();
+    };
+    auto stage = [&](int ru) {
+        __syncwarp();
+        for (int x = lane; x < 4 * D; x += 32) {
+            const int r = ru * 4 + x / D;
+            q[x] = R.pos(r) ? (double)Elem<T>::load(R.template q<T, D>(Qu, r) + x % D) : 0.0;
+        }
+        __syncwarp();
+    };
+    // logits of the staged rows against the lane's keys of one group of 32, or of two
+    auto logits = [&](int sub, bool two, double (&s)[2][4]) {
+        const int r0 = sub * 32 + lane, r1 = two ? r0 + groups * 32 : r0;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) s[0][x] = s[1][x] = 0.0;
+#pragma unroll 2
+        for (int ch = 0; ch < kChunks; ++ch) {
+            double k[2][kEl];
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const uint4 raw = *reinterpret_cast<const uint4*>(key_buf + pc_offset<T, D>(y ? r1 : r0, ch));
+                if constexpr (kEl == 8) {
+                    unpack8_to_double(raw, k[y]);
+                } else {
+                    k[y][0] = (double)__uint_as_float(raw.x); k[y][1] = (double)__uint_as_float(raw.y);
+                    k[y][2] = (double)__uint_as_float(raw.z); k[y][3] = (double)__uint_as_float(raw.w);
+                }
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+                for (int e = 0; e < kEl; e += 2) {
+                    const double2 a = *reinterpret_cast<const double2*>(q + x * D + ch * kEl + e);
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) { s[y][x] = fma(a.x, k[y][e], s[y][x]); s[y][x] = fma(a.y, k[y][e + 1], s[y][x]); }
+                }
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x) { s[0][x] *= inv_root_dim(D); s[1][x] *= inv_root_dim(D); }
+    };
+    auto join = [](double& m, double& z, double mo, double zo) {          // (log-)sums of exponentials
+        const double mn = fmax(m, mo);
+        z = z * exp_nonpos(m - mn) + zo * exp_nonpos(mo - mn);
+        m = mn;
+    };
+
+    // A. per row: largest logit and sum of exponentials below it
+    for (int i = tid; i < (groups > 1 ? 32 : n_ru * 4); i += kPcThreads) { zs[i] = 0.0; ms[i] = -INFINITY; }
+    for (int c = 0; c < nc; ++c) {
+        load(c);
+        const int n_valid = min(kPcKeys, n_keys - c * kPcKeys);
+        if (!works) continue;
+        for (int ru = my_ru; ru < n_ru; ru += slots) {
+            if (c == 0 || n_ru > slots) stage(ru);            // a warp with one row unit keeps it staged
+            double m[4], z[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) { m[x] = -INFINITY; z[x] = 0.0; }
+            for (int sub = my_kg; sub < kSubs && sub * 32 < n_valid; sub += 2 * groups) {
+                const bool two = sub + groups < kSubs && (sub + groups) * 32 < n_valid;
+                double s[2][4];
+                logits(sub, two, s);
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    const int at = (sub + y * groups) * 32 + lane, j = k_begin + c * kPcKeys + at;
+                    if (y && !two) continue;
+#pragma unroll
+                    for (int x = 0; x < 4; ++x)
+                        if (at < n_valid && j < R.pos(ru * 4 + x)) join(m[x], z[x], s[y][x], 1.0);      // causal row
+                }
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) join(m[x], z[x], __shfl_xor_sync(0xffffffffu, m[x], o), __shfl_xor_sync(0xffffffffu, z[x], o));
+                if (lane == 0) {                              // the warp's own place
+                    const int at = my_kg * (n_ru * 4) + ru * 4 + x;
+                    join(m[x], z[x], ms[at], zs[at]);
+                    ms[at] = m[x]; zs[at] = z[x];
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (groups > 1) {                                         // the groups of this block
+        double m = -INFINITY, z = 0.0;
+        if (tid < n_ru * 4)
+            for (int x = 0; x < groups; ++x) join(m, z, ms[x * (n_ru * 4) + tid], zs[x * (n_ru * 4) + tid]);
+        __syncthreads();
+        if (tid < n_ru * 4) { zs[tid] = z; thr_sm[tid] = m; }
+    }
+    cluster_sync();
+    constexpr int kPer = 2048 / kPcThreads;                   // rows per thread (256 queries of eight heads at most)
+    double t[kPer];
+#pragma unroll
+    for (int y = 0; y < kPer; ++y) {
+        const int r = tid + y * kPcThreads;
+        double m = -INFINITY, z = 0.0;
+        if (r < R.rows)
+            for (int x = 0; x < cs; ++x) join(m, z, ld_peer_f64(map_rank(smem_addr(thr_sm + r), x)), ld_peer_f64(map_rank(smem_addr(zs + r), x)));
+        t[y] = r < R.rows && R.pos(r) ? m + log(z) + p.log_alpha - log((double)R.pos(r)) : INFINITY;
+    }
+    cluster_sync();                                           // everybody has read everybody's sums
+#pragma unroll
+    for (int y = 0; y < kPer; ++y)
+        if (tid + y * kPcThreads < R.rows) thr_sm[tid + y * kPcThreads] = t[y];
+
+    // B. verdicts
+    for (int c = 0; c < nc; ++c) {
+        load(c);                                              // (the thresholds are there behind its barriers)
+        if (tid < kPcKeys) words[tid] = 0u;
+        __syncthreads();
+        const int n_valid = min(kPcKeys, n_keys - c * kPcKeys);
+        if (works)
+            for (int ru = my_ru; ru < n_ru; ru += slots) {
+                if (n_ru > slots) stage(ru);
+                for (int sub = my_kg; sub < kSubs && sub * 32 < n_valid; sub += 2 * groups) {
+                    const bool two = sub + groups < kSubs && (sub + groups) * 32 < n_valid;
+                    double s[2][4];
+                    logits(sub, two, s);
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) {
+                        const int at = (sub + y * groups) * 32 + lane, j = k_begin + c * kPcKeys + at;
+                        if ((y && !two) || at >= n_valid) continue;
+                        uint32_t mark = 0u;
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) {
+                            const int row = ru * 4 + x, qpos = R.pos(row);
+                            if (j >= qpos) continue;
+                            const double th = thr_sm[row], margin = s[y][x] - th, e = th > -INFINITY ? 1e-13 * (1.0 + fabs(th)) : 0.0;
+                            if (margin > e) mark = pc_join(p.w, mark, pc_mark(p.w, R.rho(row), qpos));
+                            else if (margin >= -e) pc_leave_open(flags, misc, row, j);
+                        }
+                        if (mark) {
+                            if (p.w <= 32) atomicOr(words + at, mark);
+                            else atomicMax(words + at, mark);
+                        }
+                    }
+                }
+            }
+        __syncthreads();
+        if (tid < n_valid) words_g[k_begin + c * kPcKeys + tid] = words[tid];
+    }
+    __syncthreads();
 }
 
 // Raw values of 8 rows in the B operand's layout (row n = lane / 4); zeros for rows that do not exist.
@@ -306,12 +489,6 @@ __device__ __forceinline__ uint32_t pc_tile_amax(const unsigned char* tile, int 
         m = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(m, v.x), v.y), v.z), v.w);
     }
     return __reduce_max_sync(0xffffffffu, max(m & 0xffffu, m >> 16));
-}
-
-__device__ __forceinline__ void pc_leave_open(uint32_t* flags, PcMisc* misc, int row, int j) {
-    atomicOr(flags + (row >> 5), 1u << (row & 31));
-    const int at = atomicAdd(&misc->n_open, 1);
-    if (at < kPcOpenCap) misc->open[at] = make_int2(row, j);
 }
 
 // Verdicts that the bounds leave open, by a whole warp: bit x of `open` = key j0 + lane / 4 + 8 (x / 2) against row
@@ -564,16 +741,26 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         double Z = 0.0;
         for (int x = 0; x < cs; ++x) Z += ld_peer_f64(map_rank(smem_addr(zs + r), x));
         thr_sm[r] = qpos ? log(Z) + p.log_alpha - log((double)qpos) : INFINITY;
-        if (any_bad && qpos) atomicOr(flags + (r >> 5), 1u << (r & 31));      // every row of the unit goes through the exact path
     }
     // error of a threshold per unit of qe (every logit of the row is off by at most this much, so its log-sum-exp is too)
     const double eps_unit = kBf16 ? p.bound_scale * (double)split_amax(amax_unit) * inv_root_d : 0.0;
+    bool wide = any_bad != 0;                                 // the same in every block: unit and rows are
+    if constexpr (kBf16)
+        if (!wide)
+            for (int r = tid; r < R.rows; r += kPcThreads) wide |= eps_unit * qe_sm[r] * (double)P > kPcReachKeys * p.bound_scale;
+    wide = __syncthreads_or(wide);
 
     // ---- B. verdicts -> registers ----
     const int n_grp_b = kBf16 ? (n_oct + kPcGroupB - 1) / kPcGroupB : 1;
-    const int end_b = resident ? 0 : n_grp_b * nc;
-    if (!resident) start(end_b);
-    if constexpr (kBf16) {
+    const int end_b = resident || wide ? 0 : n_grp_b * nc;
+    if (!resident && !wide) start(end_b);
+    if (wide) {
+        cluster_sync();                                       // everybody has read everybody's sums of phase A
+        constexpr int kBuf = kPcKeys * kRow;
+        static_assert(kPcWarps * 4 * D * 8 <= kBuf, "the widened rows fit a ring buffer");
+        pc_fp64_rows<T, D>(p, R, Qu, Ku, k_begin, n_keys, smem + lay.ring, reinterpret_cast<double*>(smem + lay.ring + kBuf), zs, thr_sm,
+                           kBf16 ? reinterpret_cast<uint32_t*>(f12) : words_sm, words_g, flags, misc, cs);
+    } else if constexpr (kBf16) {
         uint2* fr = reinterpret_cast<uint2*>(f12);
         for (int grp = 0; grp < n_grp_b; ++grp) {
             const int oct0 = grp * kPcGroupB, cnt = min(kPcGroupB, n_oct - oct0);
@@ -599,7 +786,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
                 const int n_valid = min(kPcKeys, n_keys - c * kPcKeys), j0 = k_begin + c * kPcKeys + warp * 16;
                 if (warp * 16 >= n_valid) continue;
                 uint32_t mark[2] = {0u, 0u};                  // keys lane / 4 and lane / 4 + 8
-                if (!any_bad) {
+                {
                     const float A = split_amax(pc_tile_amax<D>(buf + warp * 16 * kRow, lane));
                     const uint32_t tile = smem_addr(buf) + warp * 16 * kRow;
                     uint32_t a[D / 16][4];
@@ -641,7 +828,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
             if (tid < kPcKeys) words_sm[tid] = 0u;
             const unsigned char* buf = arrive(c, end_b);
             const int n_valid = min(kPcKeys, n_keys - c * kPcKeys);
-            if (works && !any_bad)
+            if (works)
                 for (int ru = my_ru; ru < n_ru; ru += ru_slots) {
                     if (!keep_rows) stage_rows(ru);
                     for (int sub = my_kg; sub < kSubs && sub * 32 < n_valid; sub += key_groups) {
@@ -703,7 +890,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         cluster_sync();
         for (int i = tid; i < (pp.rows8 + 31) / 32; i += kPcThreads) flags[i] = (uint32_t)__double_as_longlong(thr_sm[i]);
         __syncthreads();
-        pc_exact_rows<T, D>(p, R, Qu, Ku, k_begin, k_end, any_bad != 0, flags, words_g, misc, cs);
+        pc_exact_rows<T, D>(p, R, Qu, Ku, k_begin, k_end, flags, words_g, misc, cs);
         __syncthreads();
         keep_pass();
         cluster_sync();

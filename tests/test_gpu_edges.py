@@ -350,3 +350,59 @@ def test_few_units_on_either_side_of_the_kernels_lines(case):
     assert_states_equal(many, orc, 0, B, nkv, "multi-step")
     assert one.corm_cache_stats()["device_status"] == many.corm_cache_stats()["device_status"] == 0
     assert one.corm_cache_kernel_launches() - before == launches * steps
+
+
+# prompts whose logits overflow plain sums of exponentials, whose elements leave the pieces' range, or whose bounds are too
+# wide to be of use: row counts below, at and beyond one unit of four rows per warp, windows below and beyond a register
+WIDE_PROMPTS = [
+    # dtype, head_dim, group, prompt range, w, what
+    ("bf16", 128, 1, (300, 340), 3, "large logits"),
+    ("bf16", 128, 4, (1000, 1100), 8, "large logits"),
+    ("bf16", 128, 8, (250, 420), 33, "one channel"),
+    ("bf16", 64, 1, (600, 700), 256, "one channel"),
+    ("bf16", 64, 2, (2040, 2060), 16, "out of range"),
+    ("bf16", 128, 1, (1, 40), 5, "out of range"),
+    ("f32", 128, 2, (900, 1000), 40, "large logits"),
+    ("f32", 64, 8, (255, 300), 64, "large logits"),
+]
+
+
+def _widen(data, what, dtype):
+    rnd = (lambda a: torch.from_numpy(a).to(torch.bfloat16).float().numpy()) if dtype == "bf16" else (lambda a: a)
+    kp, ql = rnd(data.k_prompt.copy()), rnd(data.q_last.copy())
+    if what == "large logits":
+        kp *= 128.0
+    elif what == "out of range":
+        kp *= 2.0 ** 58
+    else:
+        kp[..., 3] *= 4096.0
+        ql[..., 3] /= 4096.0
+    return kp, ql
+
+
+@pytest.mark.parametrize("case", WIDE_PROMPTS, ids=lambda c: "-".join(str(x) for x in c))
+def test_prompts_of_wide_range(case):
+    dtype, d, G, prange, w, what = case
+    cfg = _cfg(dtype, d, G, 2, 3, prange, 2, w, 16)
+    data = generate(cfg)
+    kp, ql = _widen(data, what, dtype)
+    orc = make_oracle(cfg, 3, 2)
+    orc.set_near_band(1e-11)
+    orc.compress_prompt(0, kp, data.v_prompt, ql, data.prompt_lens)
+    for pool in (0, -(-6 * (cfg.max_tokens // 32 + 2) // 32) * 32):
+        gpu = make_gpu_cache(cfg, 3, 2, pool_pages=pool)
+        gpu.corm_compress_prompt(0, to_dev(kp, dtype), to_dev(data.v_prompt, dtype), to_dev(ql, dtype), data.prompt_lens)
+        assert_states_equal(gpu, orc, 0, 3, 2, f"pool {pool}")
+        assert gpu.corm_cache_stats()["device_status"] == 0
+
+
+@pytest.mark.parametrize("what", ["large logits", "one channel"])
+def test_prompts_of_wide_range_take_fp64_time_not_a_pass_per_row(what):
+    """256 rows of 32 units: both phases in fp64 take about four times the ordinary pass; forming each row apart, with two
+    passes over its keys, took more than ten times."""
+    cfg = _cfg("bf16", 128, 1, 8, 4, (2000, 2000), 1, 256, 64)
+    data = generate(cfg)
+    plain, _ = _prompt_time(cfg, data, "bf16")
+    data.k_prompt, data.q_last = _widen(data, what, "bf16")
+    wide, _ = _prompt_time(cfg, data, "bf16")
+    assert wide < 7 * plain, (plain, wide)
