@@ -152,6 +152,17 @@ def workload_config(cfg, args, which=None):
             "l2": "live K/V read per step exceeds the 126 MB L2 (no flush needed)"}
 
 
+def decode_kernel_name(cfg, args, layers):
+    """The kernel that the library's rule picks for the bulk of the workload's steps."""
+    if args.no_fast:
+        return "decode_generic_kernel"
+    block_per_split = cfg.dtype == "bf16" and cfg.head_dim == 128 and cfg.group <= 4
+    if args.finish == "cluster" or not block_per_split:
+        return "decode_cluster_kernel"
+    units = cfg.batch * cfg.n_kv_heads * layers
+    return "decode_cluster_kernel" if args.finish == "auto" and (cfg.group > 1 or units <= 148) else "decode_fast_kernel"
+
+
 def measure_workload(cfg, args, local, world, rank, want_e2e, want_clocks):
     """Prompt pass, then `repeats` timed passes over the same decode steps, each from the restored post-prompt state
     (the prompt pass is run again and the warm-up replayed), and an end-to-end pass over the same steps through the
@@ -320,8 +331,7 @@ def measure_workload(cfg, args, local, world, rank, want_e2e, want_clocks):
                      "frac_of_nominal_8TBs": achieved / 8000.0, "peak_source": peak_src, "traffic": traffic,
                      "traffic_note": None if traffic else "no ncu capture of the kernel as it stands at this launch shape",
                      "target": {"frac_of_nominal_8TBs": 0.60, "met": achieved / 8000.0 >= 0.60},
-                     "kernel": ("decode_cluster_kernel" if not args.no_fast and (args.finish == "cluster" or (cfg.group > 1 and args.finish == "auto"))
-                                else "decode_fast_kernel") + f" ({launches_per_step:.2f} launches per layer per step, all counted in the time)",
+                     "kernel": (decode_kernel_name(cfg, args, L)) + f" ({launches_per_step:.2f} launches per layer per step, all counted in the time)",
                      "bytes_per_launch": abytes / (args.steps * L), "us_per_launch": 1e3 * med["ms"] / (args.steps * L)},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "steps": "the same decode steps as `value`, from the same restored state",

@@ -142,7 +142,7 @@ corm_status_t corm_compress_prompt(corm_cache_t* cache, int32_t layer, const voi
  *   out    device [batch, n_q_heads, head_dim]
  * The call enqueues one or two launches and returns; it sizes them from the live lengths the kernels last reported (every
  * 8 steps, written to pinned host memory). Where the grid follows the longest unit (bf16 / head_dim 128 with one query head
- * per KV head, and tuning values 0, 2 and 3), a host that has run 24 steps past a report that has not landed waits for
+ * per KV head or few units of up to four, and tuning values 0, 2 and 3), a host that has run 24 steps past a report that has not landed waits for
  * it here, at most 20 ms (the GPU still has those steps queued). A layer's decode steps cannot be recorded into a CUDA
  * graph.
  * Errors: STATE if the layer has had no corm_compress_prompt since create/reset; INVALID_ARG. */
@@ -156,7 +156,7 @@ corm_status_t corm_decode_step(corm_cache_t* cache, int32_t layer, const void* q
  * layer order on `stream` (outputs within rounding: blocks may be cut differently). It exists because one launch per
  * layer of a single-sequence model is a few microseconds of GPU work behind a chain of launch and memory latencies:
  * when the layers' buffers are contiguous in layer order (q[i + 1] directly behind q[i], likewise k_new, v_new, out),
- * the cache is a slab cache on the bf16 / head_dim-128 kernels, and all the layers are at the same step, ALL layers
+ * the cache is a slab cache, and all the layers are at the same step, ALL layers
  * run as one launch (the layers' units are one array to the kernels); otherwise the per-layer launches are enqueued
  * one after the other. The step's counters are then added to the first layer's (totals in corm_cache_stats are
  * the same). In a model the layers' inputs depend on each other's outputs; use this where they are all known
@@ -177,7 +177,7 @@ corm_status_t corm_decode_step_layers(corm_cache_t* cache, int32_t first_layer, 
  * once per step (registers, live lists and positions identical, outputs within rounding).
  * What the call adds: the units of a cache are independent (Algorithm 1 runs "on each head at every layer"), so
  * step s + 1 of a unit needs step s of that unit only. When a step's launch finishes every unit inside itself (all but
- * tuning value 3, and few long units of grouped heads), the next step's launch is chained to it: its blocks start
+ * tuning value 3, and few long units), the next step's launch is chained to it: its blocks start
  * as soon as a multiprocessor has room and each waits (bounded, like every wait here) for its own unit's previous
  * step instead of the whole previous launch, so consecutive steps fill one another's last waves. Steps that need the
  * verdict launch, and caches with the similarity monitor on, run as with the per-step calls.
@@ -243,8 +243,8 @@ corm_status_t corm_cache_import_state(corm_cache_t* cache, int32_t layer, int32_
 /* Tuning knobs (performance only; live lists and registers do not depend on them, outputs only within rounding):
  * keys per split of the block-per-split decode kernel (multiple of 32, 0 = automatic) and which kernels may be used:
  * allow_fast_path 0 = the generic kernel only; 1 = automatic (default): a cluster of blocks per unit, and for bf16 /
- * head_dim 128 with one query head per KV head, where units fit one block, are many or lose nothing to eviction, the
- * block-per-split kernel, which finishes a unit of several splits inside the decode launch when the launch has many units
+ * head_dim 128 with one query head per KV head, where units are short, or many and fit one block or lose nothing to
+ * eviction, and with up to four, where units are few and long and lose nothing to eviction, the block-per-split kernel, which finishes a unit of several splits inside the decode launch when the launch has many units
  * and by a second, verdict launch when it has few; 2 / 3 = the block-per-split
  * kernel with the first / the second way always; 4, 5, 6 = a cluster of blocks per unit for every shape (three values
  * that once chose between forms of one kernel; they are the same now). Errors: INVALID_ARG. */
@@ -260,7 +260,7 @@ corm_status_t corm_cache_set_similarity_monitor(corm_cache_t* cache, int32_t ena
 corm_status_t corm_cache_similarity(corm_cache_t* cache, double* sum_host, int64_t* count_host, void* stream);
 
 /* The prompt pass of bf16 caches forms its logits on the tensor cores with proven bounds on their errors; a verdict
- * that a bound leaves open is decided in fp64, so results never depend on it. `scale` >= 1 multiplies the bounds
+ * that a bound leaves open is decided in fp64, so results never depend on it; decode does the same. `scale` >= 1 multiplies the bounds
  * (default 1): larger values send more logits and rows through the exact path, which is how the tests exercise it.
  * Errors: INVALID_ARG. */
 corm_status_t corm_cache_set_bound_scale(corm_cache_t* cache, double scale);

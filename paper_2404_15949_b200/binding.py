@@ -325,8 +325,8 @@ class CormCache:
         return total.value, n.value
 
     def corm_cache_set_bound_scale(self, scale):
-        """Multiplies the proven fp32 error bound of the tiled prompt pass (>= 1; results never change, only how many
-        logits are formed again in fp64)."""
+        """Multiplies the proven error bounds of bf16 logits on the tensor cores (>= 1; results never change, only how many
+        verdicts are formed again in fp64)."""
         _check("corm_cache_set_bound_scale", self.lib.corm_cache_set_bound_scale(self.handle, float(scale)))
 
     def corm_cache_kernel_launches(self):

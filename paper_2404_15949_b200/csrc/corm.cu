@@ -338,7 +338,7 @@ bool takes_cluster(const corm_cache* c, int upper, int n_units) {
 }
 
 // whether several layers from first_layer on may run as one launch as far as the kernels are concerned
-bool can_fuse(const corm_cache* c, int first_layer) {
+bool can_fuse(const corm_cache* c) {
     const corm_config_t& cf = c->cfg;
     if (fused_layers_of(cf, c->pool_pages) <= 1 || !c->allow_fast || c->monitor_similarity) return false;
     return may_cluster(c) || (cf.kv_dtype == CORM_BF16 && cf.head_dim == 128 && c->G <= 4);
@@ -354,7 +354,7 @@ corm_status_t launch_decode(corm_cache* c, int layer, const void* q, const void*
                             cudaStream_t st, int n_fused = 1, bool chain = false, bool more = false) {
     for (int i = 0; i < n_fused; ++i) poll_live_bound(c, layer + i, grids_follow_bound(c));
     const corm_config_t& cf = c->cfg;
-    const size_t C = cf.max_tokens, D = cf.head_dim, U = c->U;
+    const size_t C = cf.max_tokens, U = c->U;
     DecodeParams p{};
     p.K = layer_ptr(c, c->lay.K, kv_layer_bytes(c), layer);
     p.V = layer_ptr(c, c->lay.V, kv_layer_bytes(c), layer);
@@ -654,13 +654,11 @@ corm_status_t corm_decode_step_layers(corm_cache_t* c, int32_t first_layer, int3
     }
     DeviceGuard guard(c->cfg.device);
     if (!guard.ok) return CORM_ERR_CUDA;
-    // One launch for all the layers when the kernels can see them as one array of units: a slab cache on the
-    // bf16 / head_dim-128 kernels, every layer at the same step with the same buffer parity, and the layers' q,
-    // k_new, v_new and out contiguous in layer order. (Grouped heads also need the tensor map over all layers, which
-    // starts at layer 0.)
+    // One launch for all the layers when the kernels can see them as one array of units: a slab cache, every layer at
+    // the same step with the same buffer parity, and the layers' q, k_new, v_new and out contiguous in layer order.
     const corm_config_t& cf = c->cfg;
     const size_t qb = (size_t)cf.batch * cf.n_q_heads * cf.head_dim * c->e, kb = (size_t)c->U * cf.head_dim * c->e;
-    bool fuse = n_layers > 1 && can_fuse(c, first_layer);
+    bool fuse = n_layers > 1 && can_fuse(c);
     for (int i = 1; fuse && i < n_layers; ++i) {
         const auto at = [](const void* ptr, size_t off) { return static_cast<const unsigned char*>(ptr) + off; };
         fuse = c->steps[first_layer + i] == c->steps[first_layer] && c->parity[first_layer + i] == c->parity[first_layer] &&
@@ -695,7 +693,7 @@ corm_status_t decode_steps_impl(corm_cache_t* c, int32_t first_layer, int32_t n_
     const size_t qb = (size_t)cf.batch * cf.n_q_heads * cf.head_dim * c->e, kb = (size_t)c->U * cf.head_dim * c->e;
     // all layers of a step as one launch under the same conditions as corm_decode_step_layers (the buffers are
     // contiguous by this call's layout)
-    bool fuse = n_layers > 1 && can_fuse(c, first_layer);
+    bool fuse = n_layers > 1 && can_fuse(c);
     for (int i = 1; fuse && i < n_layers; ++i)
         fuse = c->steps[first_layer + i] == c->steps[first_layer] && c->parity[first_layer + i] == c->parity[first_layer];
     const auto at = [](const void* ptr, size_t off) { return static_cast<const unsigned char*>(ptr) + off; };

@@ -170,12 +170,6 @@ __device__ __forceinline__ void mul_f32x2(unsigned long long& acc, unsigned long
 __device__ __forceinline__ unsigned long long bf16x2_to_f32x2(uint32_t w) {
     return pack_f32x2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
-__device__ __forceinline__ void unpack8_to_float(const uint4& raw, float (&v)[8]) {
-    v[0] = __uint_as_float(raw.x << 16); v[1] = __uint_as_float(raw.x & 0xffff0000u);
-    v[2] = __uint_as_float(raw.y << 16); v[3] = __uint_as_float(raw.y & 0xffff0000u);
-    v[4] = __uint_as_float(raw.z << 16); v[5] = __uint_as_float(raw.z & 0xffff0000u);
-    v[6] = __uint_as_float(raw.w << 16); v[7] = __uint_as_float(raw.w & 0xffff0000u);
-}
 
 // Unscaled q.k sums of one 32-key tile. Lane (h = lane>>4, i = lane&15) reads channel chunk i of the keys of half h;
 // on return the lane holds, per query head, the full sum of tile key  16h + 8(i&1) + (i>>1).

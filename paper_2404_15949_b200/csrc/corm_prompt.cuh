@@ -467,7 +467,7 @@ __device__ __forceinline__ uint32_t pc_tile_sums(uint32_t tile, uint32_t klane, 
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const double s = (((double)hi[o][x] + (double)mid[o][x]) + (double)lo[o][x]) * inv_root_d;
-            double e = exp_reduced(s);                        // (any s beyond kPcLogitLimit sends the unit through the exact path)
+            double e = exp_reduced(s);                        // (any s beyond kPcLogitLimit sends the unit through pc_fp64_rows)
             uint32_t h = (uint32_t)__double2hiint(s) & 0x7fffffffu;
             if (last) {                                       // causal row: keys 1..position of the query
                 const int j = j0 + (lane >> 2) + (x >> 1) * 8;
@@ -1028,7 +1028,8 @@ inline corm_status_t launch_prompt_cluster(const PromptParams& p, int G, int max
     pp.rows8 = (p.w * G + 7) / 8 * 8;
     const int n_words = std::max(1, (max_p + 31) / 32);
     // As many blocks per unit as make the launch at least five waves of resident blocks: fewer leave the machine
-    // to the longest units, more pay each block's fixed chain of round trips more often. us per pass with 1 / 2 / 4 / 8:
+    // to the longest units, more pay each block's fixed chain of round trips more often. us per pass with 1 / 2 / 4 / 8, on the
+    // first version of the kernel (the shapes take 840, 598 and 60 us now, with 2, 8 and 8):
     // 1024 units x 3250 keys 969-1353 (with the slab's stride) / 956-1033 / 1073 / 1365, 128 units x 8192 keys (G 4) 2152 / 1281 / 811 / 752, 32 units x
     // 4096 keys 350 / 192 / 120 / 93.
     int cs = 1;
