@@ -35,6 +35,11 @@
 // (from one warp per key and the last-arriving split finishing the unit, from fp64 logits on the CUDA cores with every
 // block an equal share of all tiles and a second launch for the verdicts, from the block-per-split kernel).
 //
+// What the blocks tell one another is pushed (st.async: value and byte count travel together, one way), each block waiting on
+// its own barriers, instead of cluster barriers and loads from the peers behind them (two round trips and a flush each):
+// 8 units x 170 keys, fp32, 11.0 -> 9.4 us a step, 32 units x 1160 keys, G 1, 19.6 -> 17.0, 128 units x 1090 keys, 64
+// channels, 27.2 -> 25.5, 128 units x 1800 keys, G 4, 54 -> 52 (of which 1-3 us are the lists of row moves).
+//
 // Verdicts are the fp64 ones: a slot's logit is kept in fp32, and one that lies within the proven error of its threshold
 // is formed again in fp64. If it then lies within the error of the log-sum-exp itself, the head is marked and the
 // cluster forms that head's log-sum-exp and verdicts in fp64 once more before anything is evicted (rare).
@@ -75,12 +80,14 @@ template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int d
     return Elem<T>::kBytes == 4 ? (D == 128 ? 12 : 16) / NW : (GP == 8 ? 12 : 16) / NW;
 }
 
-constexpr int kDcListCap = 1024;                  // slots a step may evict from a unit for its moves to be listed on chip
+// Slots a step may evict from a unit for its moves to be listed on chip: what moves lies in the unit's last 32 words then.
+constexpr int kDcListCap = 992;
 
-// What the ring holds once the tiles are done: the block's record (the first 8 KB), the keep bits of its words and, behind
-// them, the lists of a step with few moves or the prefix sums (one more than words) of a step with many. So the words a
-// block may own follow from the instance's ring: 4096 for the rings of 64 KB, 3071 for the 32 KB of fp32 / 64 channels.
-constexpr int kDcRecBytes = 8192;
+// What the ring holds once the tiles are done: the warps' records at the start of their parts, and from 4 KB on the keep bits
+// of the block's words and, behind them, the lists of a step with few moves or the prefix sums (one more than words) of a
+// step with many. So the words a block may own follow from the instance's ring: 4096 for the rings of 64 KB, 3583 for the
+// 32 KB of fp32 / 64 channels.
+constexpr int kDcRecBytes = 4096;
 template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int dc_max_words() {
     constexpr int n = (NW * DcShape<T, D, GP>::kWarpRing - kDcRecBytes - 4) / 8;
     return n < 4096 ? n : 4096;
@@ -91,26 +98,39 @@ template <typename T, int D, int GP, int NW> __host__ __device__ constexpr bool 
 }
 
 constexpr int kDcOpenCap = 32;
-template <int NW> struct DcMisc {
-    unsigned long long stamp;
-    double wM[NW][8], wZ[NW][8];                  // per warp and head, read by the cluster
-    double thr[8], Zt[8], log_t;
-    double red[NW][2], mz[2];                     // exact heads
-    float sc[8][kDcMaxCluster * NW], qe[8], thr_f[8], slack[8];
-    float qe_part[NW][8];                         // the warps' shares of qe
+// A block's barriers: what every warp of the unit's blocks found (kDcRecords), the block's share of the outputs' numerators
+// from every block (kDcOutputs), the warps' verdicts in numbers and the unit's last keep bits (kDcCounts), all blocks
+// (kDcMeet) and, at the first block, the others being done with the unit (kDcDone).
+enum { kDcRecords = 0, kDcOutputs = 1, kDcCounts = 2, kDcMeet = 3, kDcDone = 4, kDcBars = 5 };
+template <int NW, int GP> struct DcMisc {
+    unsigned long long bar[kDcBars], stamp;
+    // pushed by the unit's blocks, block by block and warp by warp: {m, Z} of each head, state words, verdicts (kept slots |
+    // heads to be formed exactly << 24, important keys), and the keep bits of the unit's last 32 words, the last one first
+    struct alignas(16) Entry { double m, z; };
+    union { Entry rec[GP][kDcMaxCluster * NW]; int scan[NW * 32]; };    // (the scan: of steps with many moves)
+    uint2 verdicts[kDcMaxCluster * NW];
+    uint32_t tail[32];
     // largest key magnitude (bf16 bits), 1 << 16 if the block took the fp64 loop for it, 1 << 17 if a wait expired, 1 << 18
     // if the unit cannot take the token
-    uint32_t state;
+    uint32_t state[kDcMaxCluster * NW];
+    double thr[GP], Zt[GP], log_t;
+    double red[NW][2], mz[2];                     // exact heads
+    float sc[GP][NW], qe[GP], thr_f[GP], slack[GP];
+    float qe_part[NW][GP];                        // the warps' shares of qe
     uint32_t cut_for;                             // bf16: the unit's magnitude before the appended key; 0 if that asks for the fp64 loop
-    struct alignas(16) Counts {                   // what the blocks tell one another after their verdicts
-        uint32_t flags;                           // heads to be formed exactly
-        int count, n_imp, pad;                    // kept slots and important keys of the block
-    } cnt;
+    uint32_t flags[NW];                           // per warp: heads to be formed exactly
+    struct alignas(16) Counts { int count, n_imp, pad[2]; } cnt;      // kept slots and important keys of the block (exact heads)
     int n_open;                                   // open verdicts of marked heads: slot << 3 | head
     uint32_t open[kDcOpenCap];
     int n_moved;                                  // row moves of the unit
-    int scan[NW * 32];
 };
+
+// All blocks of the unit meet: what they wrote before is there for the others behind. Returns false if the wait expired.
+__device__ __forceinline__ bool dc_meet(uint32_t bar, int cs, uint32_t& phase) {
+    __syncthreads();
+    if ((int)threadIdx.x < cs) mbar_arrive_peer(map_rank(bar, threadIdx.x));
+    return mbar_wait_cluster(bar, phase++ & 1u);
+}
 
 // When a bf16 unit takes the fp64 loop. Errors of the tensor-core logits grow with A Aq, the product of the unit's largest key
 // and query magnitudes, while its logits need not (one large key channel next to small query channels). Where the bounds
@@ -137,7 +157,7 @@ __host__ __device__ inline DcSmem dc_smem_layout(int lcap) {
     s.pieces = take(S::kBf16 ? (D / 16 * S::kPieces * 128 > GP * D * 8 ? D / 16 * S::kPieces * 128 : GP * D * 8) : 0);
     s.newrow = take(2 * S::kRow);
     s.bars = take(NW * S::kStages * 8);
-    s.misc = take((int)sizeof(DcMisc<NW>));
+    s.misc = take((int)sizeof(DcMisc<NW, GP>));
     s.logits = take(lcap * 4);
     s.total = off;
     return s;
@@ -204,9 +224,11 @@ __device__ __forceinline__ double warp_exact_dot_cg(const T* q, const T* k, int 
 // that were left open (misc->open, or every slot of the block where those did not fit). A verdict that was sure before holds for the exact threshold too, so adding importance is enough: the register
 // gets its newest bit (or stamp), the keep bit is set. About one step in ten of 32 units x 21000 keys comes here: 16 keys
 // per warp at a time instead of 8, and no second pass over the keys, took 100 us of such a step to 20.
-template <typename T, int D, int NW>
-__device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G, int t, int k_begin, int k_end, uint32_t heads,
-                                            uint32_t* keep, DcMisc<NW>* misc, int cs) {
+template <typename T, int D, int NW, int GP>
+__device__ __noinline__ bool dc_exact_heads(const DecodeParams& p, int u, int G, int t, int k_begin, int k_end, uint32_t heads,
+                                            uint32_t* keep, DcMisc<NW, GP>* misc, int cs, uint32_t phase) {
+    const uint32_t meet = smem_addr(&misc->bar[kDcMeet]);
+    bool ok = true;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & 3;
     const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
     const T* Kl = reinterpret_cast<const T*>(p.K);
@@ -236,7 +258,7 @@ __device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G,
                 if (misc->red[x][1] > 0.0) Zb += misc->red[x][1] * exp(misc->red[x][0] - mb);
             misc->mz[0] = mb; misc->mz[1] = Zb;
         }
-        cluster_sync();
+        ok &= dc_meet(meet, cs, phase);
         double M = -INFINITY, Zt = 0.0;
         for (int x = 0; x < cs; ++x) M = fmax(M, ld_peer_f64(map_rank(mz_addr, x)));
         for (int x = 0; x < cs; ++x) {
@@ -256,16 +278,17 @@ __device__ __noinline__ void dc_exact_heads(const DecodeParams& p, int u, int G,
             quad_exact_dots<T, D, 1>(qr, rows, sub, s);
             if (on && sub == 0 && s[0] * inv_root_dim(D) >= thr) add_importance(j);
         }
-        cluster_sync();                                       // everybody has read mz; the registers of this head are written
+        ok &= dc_meet(meet, cs, phase);                       // everybody has read mz; the registers of this head are written
     }
     if (added) atomicAdd(&misc->cnt.count, added);
     if (added_imp) atomicAdd(&misc->cnt.n_imp, added_imp);
+    return ok;
 }
 
 // Verdicts that the error bounds leave open, by a whole warp: lane's slot j, heads `open`; true where a head is sure to
-// find the key important. Heads whose threshold is too close to tell are marked in misc->cnt.flags.
-template <typename T, int D, int NW>
-__device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int G, int j, uint32_t open, float eps_a, DcMisc<NW>* misc) {
+// find the key important. Heads whose threshold is too close to tell are marked in the warp's misc->flags.
+template <typename T, int D, int NW, int GP>
+__device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int G, int j, uint32_t open, float eps_a, DcMisc<NW, GP>* misc) {
     const int lane = threadIdx.x & 31;
     const int32_t* pt_u = p.page_table ? p.page_table + (size_t)u * p.pt_stride : nullptr;
     bool imp = false;
@@ -285,7 +308,7 @@ __device__ __noinline__ bool dc_open_verdicts(const DecodeParams& p, int u, int 
             const double th = misc->thr[h], e = (eps_a > 0.f ? (double)(eps_a * misc->qe[h]) : 0.0) + 1e-13 * (1.0 + fabs(th));
             if (lane == src && s - th > e) imp = true;
             if (lane == 0 && fabs(s - th) <= e) {
-                atomicOr(&misc->cnt.flags, 1u << h);
+                misc->flags[threadIdx.x >> 5] |= 1u << h;
                 const int at = atomicAdd(&misc->n_open, 1);
                 if (at < kDcOpenCap) misc->open[at] = ((uint32_t)js << 3) | (uint32_t)h;
             }
@@ -344,18 +367,18 @@ template <typename T, int D, int GP, int NW> struct DcTiles {
 // The streaming loop in fp64 on the CUDA cores for NG heads: a key per lane, its channels shared by two half-warps; P.V by
 // fp32 FMAs. qd: the queries as doubles [NG][D], pr: room for 16 x NG probabilities, lg: the block's logits [slot][NG].
 // Magnitudes are whatever the inputs are: references and sums stay in fp64, a logit beyond fp32 is kept as an infinity (its
-// verdict is formed again). A logit of +infinity makes its head's output NaN and no key important; so does NaN, but for bf16
+// verdict is formed again). push(h, m, Z): a head's sums go to the unit's blocks (the whole warp calls). A logit of +infinity makes its head's output NaN and no key important; so does NaN, but for bf16
 // with 128 channels and up to four heads, where it counts for nothing: what the kernels for these shapes have always done
 // (the block-per-split kernel there, the generic one elsewhere). Returns false if a wait expired.
-template <typename T, int D, int GP, int NW, int NG>
-__device__ __forceinline__ bool dc_stream_fp64(const DcTiles<T, D, GP, NW>& c, const double* qd, float* pr, float* lg, float* rec, DcMisc<NW>* misc) {
+template <typename T, int D, int GP, int NW, int NG, typename Push>
+__device__ __forceinline__ bool dc_stream_fp64(const DcTiles<T, D, GP, NW>& c, const double* qd, float* pr, float* lg, float* rec, Push push) {
     using S = DcShape<T, D, GP>;
     constexpr int kKs = S::kKs, kVs = S::kVs, NC = D / 32;    // channels a lane accumulates
     constexpr int kHalf = S::kRow / 32, kEl = 16 / Elem<T>::kBytes;             // 16-byte chunks of half a row, elements of one
     // bf16: twice only, next to the tensor-core loop (a call costs that loop 2 %, all eight chunks unrolled 0.7 %, two nothing)
     constexpr int kUnroll = S::kBf16 ? 2 : kHalf;
     constexpr bool kNanPasses = !(S::kBf16 && D == 128 && GP <= 4);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, key = lane & 15, half = lane >> 4;
+    const int lane = threadIdx.x & 31, key = lane & 15, half = lane >> 4;
     bool failed = false, first = true;
     float acc[NG][NC];
     double Zl[NG], Mref[NG];
@@ -455,7 +478,7 @@ __device__ __forceinline__ bool dc_stream_fp64(const DcTiles<T, D, GP, NW>& c, c
 #pragma unroll
     for (int x = 0; x < NG; ++x) {
         Zl[x] = warp_sum(Zl[x]);
-        if (lane == 0) { misc->wM[warp][x] = Mref[x]; misc->wZ[warp][x] = Zl[x]; }
+        push(x, Mref[x], Zl[x]);
 #pragma unroll
         for (int e = 0; e < NC; ++e) rec[x * D + lane * NC + e] = acc[x][e];
     }
@@ -475,19 +498,24 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     const DecodeParams& p = dp.p;
     const int G = kBf16 && GP == 2 ? dp.G : GP;               // one or two heads share an instance
     const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int cs = (int)cluster_size(), rank = (int)cluster_rank();
+    const int cs0 = (int)cluster_size(), rank0 = (int)cluster_rank();            // (read again behind the loop, which has no registers to spare)
     const DcSmem lay = dc_smem_layout<T, D, GP, NW>(0);       // the logits come last: every other offset is a constant
     unsigned char* ring = smem + warp * S::kWarpRing;
     unsigned char* prob = smem + lay.prob + warp * S::kProb;
     unsigned char* newrow = smem + lay.newrow;
     const uint32_t bars = smem_addr(smem + lay.bars) + warp * S::kStages * 8;
-    DcMisc<NW>* misc = reinterpret_cast<DcMisc<NW>*>(smem + lay.misc);
+    DcMisc<NW, GP>* misc = reinterpret_cast<DcMisc<NW, GP>*>(smem + lay.misc);
+    const uint32_t xbar = smem_addr(misc->bar);
 
     // ---- set-up that reads nothing of the previous launch ----
     if (tid == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&kmap)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&vmap)) : "memory");
-        misc->state = 0u; misc->cnt.flags = 0u; misc->cnt.count = 0; misc->cnt.n_imp = 0; misc->n_open = 0;
+        misc->n_open = 0;
+#pragma unroll
+        for (int x = 0; x < NW; ++x) misc->flags[x] = 0u;
+#pragma unroll
+        for (int x = 0; x < kDcBars; ++x) mbar_init(xbar + x * 8, x < kDcMeet ? 1 : cs0);
     }
     if (lane == 0) {
 #pragma unroll
@@ -495,6 +523,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         fence_mbar_init();
         fence_async_smem();
     }
+    cluster_arrive();                                         // the barriers are there before anybody's first push (cluster_wait below)
     int l_old;
     uint32_t state = smem_addr(smem) & 1023u ? kDcExpired : 0u;          // swizzled tiles need the alignment; never expected
     if (p.chain_wait) {                                       // this unit's previous step, not the whole previous launch
@@ -516,7 +545,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     if constexpr (kBf16)
         for (int x = tid; x < G * (S::kRow / 16); x += NT)
             cp_async16(smem_addr(smem + lay.q + x * 16), reinterpret_cast<const unsigned char*>(p.q) + ((size_t)u * G * (S::kRow / 16) + x) * 16);
-    if (rank == cs - 1)
+    if (rank0 == cs0 - 1)
         for (int x = tid; x < 2 * (S::kRow / 16); x += NT) {
             const int c = x % (S::kRow / 16);
             cp_async16(smem_addr(newrow + x * 16), reinterpret_cast<const unsigned char*>(x < S::kRow / 16 ? p.k_new : p.v_new) + (size_t)u * S::kRow + c * 16);
@@ -533,8 +562,16 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     if (tid == NT - 1) misc->log_t = log((double)t);
     // the block's slots: whole words, shared out evenly
     const int n_words = state ? 0 : (l + 31) >> 5;
-    auto word_begin = [&](int o) -> int { return (int)((uint32_t)(n_words * o) / (uint32_t)cs); };
-    const int w0 = word_begin(rank), w1 = word_begin(rank + 1);
+    auto word_begin = [&](int o, int cs) -> int { return (int)((uint32_t)(n_words * o) / (uint32_t)cs); };
+    const int w0 = word_begin(rank0, cs0), w1 = word_begin(rank0 + 1, cs0);
+    // the outputs are shared out over the blocks, two channels at a time
+    constexpr int kHalfD = D / 2;
+    auto first_pair = [&](int o, int cs) { return G * kHalfD * o / cs; };
+    if (tid == 0) {                                           // what will be pushed into this block
+        mbar_expect_tx(xbar + kDcRecords * 8, cs0 * NW * (G * 16 + 4));
+        mbar_expect_tx(xbar + kDcOutputs * 8, cs0 * (first_pair(rank0 + 1, cs0) - first_pair(rank0, cs0)) * 8);
+        mbar_expect_tx(xbar + kDcCounts * 8, cs0 * NW * 8 + min(32, n_words) * 4);
+    }
     const int k_begin = w0 * 32, k_end = state ? 0 : min(l, w1 * 32), n_keys = max(0, k_end - k_begin);
     const int n_tiles = (n_keys + kDcKeys - 1) / kDcKeys;
     const int my_n = n_tiles > warp ? (n_tiles - warp + NW - 1) / NW : 0;       // tiles warp, warp + NW, ...
@@ -559,6 +596,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         for (int x = tid; x < G * D; x += NT) qd[x] = q_raw[x];
     }
     __syncthreads();
+    cluster_wait();
 
     // ---- 1. streaming ----
     const double inv_root_d = inv_root_dim(D);
@@ -566,6 +604,11 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     int32_t* posu = p.pos + (size_t)u * p.C;
     bool failed = false;
     float* rec = reinterpret_cast<float*>(ring);              // the warp's record [G][D], once its tiles are done
+    auto push_sums = [&](int h, double m, double z, int peer) {                // a head's {m, Z} of this warp, to one block
+        const uint32_t at = smem_addr(&misc->rec[h][cluster_rank() * NW + warp]);
+        push_2f64(map_rank(at, peer), m, z, map_rank(xbar + kDcRecords * 8, peer));
+    };
+    auto push_all = [&](int h, double m, double z) { if (lane < (int)cluster_size()) push_sums(h, m, z, lane); };
 
     if constexpr (kBf16) {
         // pieces of the queries, as B fragments (column n = lane / 4): every warp needs all of them, so a warp cuts the
@@ -640,7 +683,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         // The keys are cut on a grid of the unit's, kept in p.kmax: the largest magnitude it has ever held (scanning every
         // tile for its own cost 96 instructions of 550 per tile and a chain of 32 dependent ones).
         uint32_t kmax = kmax_old;
-        if (rank == cs - 1) {
+        if (cluster_rank() == cluster_size() - 1) {
             uint32_t m = 0u;
             if (lane < S::kRow / 16) {
                 const uint4 x = *reinterpret_cast<const uint4*>(newrow + lane * 16);
@@ -661,10 +704,10 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             __syncthreads();
             float* pr = reinterpret_cast<float*>(prob);
             if constexpr (GP == 2) {
-                if (G == 1) failed = !dc_stream_fp64<T, D, GP, NW, 1>(tiles, qd, pr, lg, rec, misc);
-                else failed = !dc_stream_fp64<T, D, GP, NW, 2>(tiles, qd, pr, lg, rec, misc);
+                if (G == 1) failed = !dc_stream_fp64<T, D, GP, NW, 1>(tiles, qd, pr, lg, rec, push_all);
+                else failed = !dc_stream_fp64<T, D, GP, NW, 2>(tiles, qd, pr, lg, rec, push_all);
             } else {
-                failed = !dc_stream_fp64<T, D, GP, NW, GP>(tiles, qd, pr, lg, rec, misc);
+                failed = !dc_stream_fp64<T, D, GP, NW, GP>(tiles, qd, pr, lg, rec, push_all);
             }
         } else {
             uint32_t b1[KK][2], b2[GP == 2 ? 1 : KK][2], b3[GP == 8 ? KK : 1][2];
@@ -858,7 +901,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             for (int x = 0; x < NH; ++x) {
 #pragma unroll
                 for (int o = 4; o < 32; o <<= 1) Zl[x] += __shfl_xor_sync(0xffffffffu, Zl[x], o);
-                if ((lane >> 2) == 0 && h0 + x < G) { misc->wM[warp][h0 + x] = (double)Mref[x]; misc->wZ[warp][h0 + x] = Zl[x]; }
+                if ((lane >> 2) < (int)cluster_size() && h0 + x < G) push_sums(h0 + x, (double)Mref[x], Zl[x], lane >> 2);
             }
 #pragma unroll
             for (int cb = 0; cb < D / 16; ++cb) {
@@ -882,15 +925,14 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         }
         state = (state & ~0xffffu) | kmax;
     } else {
-        failed = !dc_stream_fp64<T, D, GP, NW, GP>(tiles, reinterpret_cast<const double*>(smem + lay.q), reinterpret_cast<float*>(prob), lg, rec, misc);
+        failed = !dc_stream_fp64<T, D, GP, NW, GP>(tiles, reinterpret_cast<const double*>(smem + lay.q), reinterpret_cast<float*>(prob), lg, rec, push_all);
         if (warp == 0 && lane < GP) misc->qe[lane] = 0.f;
     }
+    const int cs = (int)cluster_size(), rank = (int)cluster_rank();
     if (failed) state |= kDcExpired;
     state = __reduce_or_sync(0xffffffffu, state);             // the magnitude is the same in every lane
-    if (lane == 0) {
-        if (state & kDcExpired) report_status(p.status, CORM_ERR_TIMEOUT);
-        atomicMax(&misc->state, state);
-    }
+    if (lane == 0 && (state & kDcExpired)) report_status(p.status, CORM_ERR_TIMEOUT);
+    if (lane < cs) push_u32(map_rank(smem_addr(&misc->state[rank * NW + warp]), lane), state, map_rank(xbar + kDcRecords * 8, lane));
     // the next launch may become resident while this one judges and compacts (it waits for this one to complete)
     if (!p.early_trigger) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // registers and positions of the first slots this thread judges are requested before the blocks meet
@@ -920,31 +962,30 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     };
     __syncthreads();                                          // the appended slot's row, word and position are stored
     load_regs(0);
-    cluster_sync();                                           // every warp's record is complete (and the block's logits)
-
-    // ---- thresholds of Definition 3.1 in log form, the same in every block: warp h reduces head h over the cluster's warps ----
-    constexpr int kEnt = kDcMaxCluster * NW / 32;             // (block, warp) entries per lane
-    double m[kEnt], z[kEnt];
-    auto load_entries = [&](int h) {
-#pragma unroll
-        for (int y = 0; y < kEnt; ++y) {
-            const int e = y * 32 + lane, blk = e / NW, w = e % NW;
-            m[y] = blk < cs ? ld_peer_f64(map_rank(smem_addr(&misc->wM[w][h]), blk)) : -INFINITY;
-            z[y] = blk < cs ? ld_peer_f64(map_rank(smem_addr(&misc->wZ[w][h]), blk)) : 0.0;
-        }
-    };
-    const uint32_t peer_state = lane < cs ? ld_peer_u32(map_rank(smem_addr(&misc->state), lane)) : 0u;
-    if (warp < G) load_entries(warp);                         // in one trip with the state
-    const uint32_t unit_state = __reduce_max_sync(0xffffffffu, peer_state);
-    if (unit_state & (kDcExpired | kDcFull)) {                // the unit is left as it is
-        cluster_sync();
-        if (rank == 0 && tid == 0) {
-            const bool full = !(unit_state & kDcExpired) || l > p.C || !room;
+    bool late = !mbar_wait_cluster(xbar + kDcRecords * 8, 0);                   // a push that should have been here
+    // A block that misses pushes stays until its peers are done: the cluster's barrier counts blocks that have ended as there.
+    auto leave = [&](bool full) {
+        if (late) report_status(p.status, CORM_ERR_TIMEOUT);
+        if (rank == 0 && tid == 0) {                          // the unit is left as it is
             if (full) report_status(p.status, CORM_ERR_CAPACITY);
             p.live_out[u] = l_old;
             if (full) publish_unit_stamp(p, u, l_old);
             report_live(p, u, p.step + 1, l_old);
         }
+        if (late) cluster_sync();
+    };
+
+    // ---- thresholds of Definition 3.1 in log form, the same in every block: warp h reduces head h over the unit's warps ----
+    constexpr int kEnt = kDcMaxCluster * NW / 32;             // (block, warp) entries per lane
+    uint32_t unit_state = 0u;
+#pragma unroll
+    for (int y = 0; y < kEnt; ++y)
+        if (y * 32 + lane < cs * NW) unit_state = max(unit_state, misc->state[y * 32 + lane]);
+    unit_state = __reduce_max_sync(0xffffffffu, unit_state);
+    late = __syncthreads_or(late);
+    if (late) unit_state |= kDcExpired;
+    if (unit_state & (kDcExpired | kDcFull)) {
+        leave(!(unit_state & kDcExpired) || l > p.C || !room);
         return;
     }
     // the appended key enters the unit's magnitude whatever became of the queries (every block has read the old one)
@@ -954,16 +995,20 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     const uint32_t cut_for = unit_state & kDcWide ? misc->cut_for : unit_state & 0xffffu;
     const float eps_a = kBf16 && (cut_for || !(unit_state & kDcWide)) ? split_amax(cut_for) * (float)inv_root_d * 1.0001f : 0.f;
     for (int h = warp; h < G; h += NW) {
-        double M = -INFINITY, Z = 0.0;
-        if (h >= NW) load_entries(h);
+        double m[kEnt], z[kEnt], M = -INFINITY, Z = 0.0;
 #pragma unroll
-        for (int y = 0; y < kEnt; ++y) M = fmax(M, m[y]);
+        for (int y = 0; y < kEnt; ++y) {
+            const bool on = y * 32 + lane < cs * NW;
+            m[y] = on ? misc->rec[h][y * 32 + lane].m : -INFINITY;
+            z[y] = on ? misc->rec[h][y * 32 + lane].z : 0.0;
+            M = fmax(M, m[y]);
+        }
         M = warp_max(M);
 #pragma unroll
         for (int y = 0; y < kEnt; ++y) {
             const double sc = m[y] == -INFINITY ? 0.0 : exp_nonpos(m[y] - M);
             Z = fma(z[y], sc, Z);
-            misc->sc[h][y * 32 + lane] = (float)sc;
+            if ((y * 32 + lane) / NW == rank) misc->sc[h][(y * 32 + lane) % NW] = (float)sc;
         }
         Z = warp_sum(Z);                                      // a fixed tree: every block gets the same bits
         if (lane == 0) {
@@ -976,21 +1021,29 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     __syncthreads();
 
     // ---- 2. verdicts, register update, keep bits ----
-    uint32_t* keep = reinterpret_cast<uint32_t*>(smem + kDcRecBytes);           // the ring is free behind the block's record
+    uint32_t* keep = reinterpret_cast<uint32_t*>(smem + kDcRecBytes);           // the ring is free behind the warps' records
+    // the block's share of the unit's output numerators, as the blocks push it: [block][pair]
+    const int np = G * kHalfD, pair0 = first_pair(rank, cs), pair1 = first_pair(rank + 1, cs), pair_cap = (np + cs - 1) / cs;
+    float2* outputs = reinterpret_cast<float2*>(smem + (kBf16 ? lay.pieces : lay.q));           // (every warp is done with the queries)
+    int n_imp = 0, n_keep = 0;
     {
-        // first the block's record of the outputs' numerators (Eq. 1): its warps' merged, in place of the first warp's
-        for (int x = tid; x < G * D; x += NT) {
-            const int h = x / D;
-            float acc = 0.f;
+        // first the numerators (Eq. 1) of the block's slots, its warps' records merged, each to the block that writes it
+        const int shift = 31 - __clz(kHalfD) + __popc(G - 1);
+        for (int x = tid; x < np; x += NT) {
+            const int h = x / kHalfD;
+            float a0 = 0.f, a1 = 0.f;
 #pragma unroll
             for (int w = 0; w < NW; ++w) {
-                const float sc = misc->sc[h][rank * NW + w];
-                acc += sc != 0.f ? reinterpret_cast<const float*>(smem + w * S::kWarpRing)[x] * sc : 0.f;
+                const float sc = misc->sc[h][w];
+                const float2 v = reinterpret_cast<const float2*>(smem + w * S::kWarpRing)[x];
+                a0 += sc != 0.f ? v.x * sc : 0.f;
+                a1 += sc != 0.f ? v.y * sc : 0.f;
             }
-            reinterpret_cast<float*>(smem)[x] = acc;
+            const int owner = ((x + 1) * cs - 1) >> shift, first = first_pair(owner, cs);        // the last one with first <= x
+            push_2u32(map_rank(smem_addr(outputs + rank * pair_cap + (x - first)), owner), __float_as_uint(a0), __float_as_uint(a1),
+                      map_rank(xbar + kDcOutputs * 8, owner));
         }
-        __syncthreads();                                      // the other warps' records give way to the keep bits
-        int n_imp = 0, n_keep = 0;
+        if (n_keys > (S::kWarpRing - kDcRecBytes) * 8) __syncthreads();          // so many keep bits reach the second warp's record
         float tf[GP], sl[GP];
 #pragma unroll
         for (int h = 0; h < GP; ++h) { tf[h] = h < G ? misc->thr_f[h] : INFINITY; sl[h] = h < G ? misc->slack[h] : 0.f; }
@@ -1023,7 +1076,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                     uint32_t ok = 0u;
 #pragma unroll
                     for (int x = 0; x < kB; ++x) ok = x == k ? open[x] : ok;
-                    if (dc_open_verdicts<T, D, NW>(p, u, G, k_begin + base0 + k * NT + tid, ok, eps_a, misc)) imp |= 1u << k;
+                    if (dc_open_verdicts<T, D, NW, GP>(p, u, G, k_begin + base0 + k * NT + tid, ok, eps_a, misc)) imp |= 1u << k;
                 }
             }
 #pragma unroll
@@ -1040,60 +1093,85 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 const uint32_t ballot = __ballot_sync(0xffffffffu, kp);
                 n_imp += __popc(__ballot_sync(0xffffffffu, im));
                 n_keep += __popc(ballot);
-                if (lane == 0 && CORM_IN_RANGE((base >> 5) + warp < kMaxWords, p.status)) keep[(base >> 5) + warp] = ballot;
+                const int wd = (base >> 5) + warp, from_end = n_words - 1 - ((k_begin >> 5) + wd);
+                if (lane == 0 && CORM_IN_RANGE(wd < kMaxWords, p.status)) keep[wd] = ballot;
+                if (from_end < 32 && lane < cs) push_u32(map_rank(smem_addr(misc->tail + from_end), lane), ballot, map_rank(xbar + kDcCounts * 8, lane));
             }
         }
-        if (lane == 0) {
-            atomicAdd(&misc->cnt.count, n_keep);
-            atomicAdd(&misc->cnt.n_imp, n_imp);
-        }
+        __syncwarp();
+        if (lane < cs)
+            push_2u32(map_rank(smem_addr(&misc->verdicts[rank * NW + warp]), lane), (uint32_t)n_keep | (misc->flags[warp] << 24), (uint32_t)n_imp,
+                      map_rank(xbar + kDcCounts * 8, lane));
     }
-    cluster_sync();
-    // the kept slots of the unit's word `wd`, from the block that owns it
-    auto peer_keep = [&](int wd) -> uint32_t {
-        const int o = (int)((uint32_t)((wd + 1) * cs - 1) / (uint32_t)n_words);    // the last o with word_begin(o) <= wd
-        return ld_peer_u32(map_rank(smem_addr(keep + (wd - word_begin(o))), o));
-    };
-    uint4 pc = make_uint4(0u, 0u, 0u, 0u);                    // a peer's counts
-    uint32_t last_keep = 0u;                                  // of the last 32 words, requested next to the counts
-    auto load_counts = [&]() {
+    // outputs (Eq. 1), while the counts travel
+    late |= !mbar_wait_cluster(xbar + kDcOutputs * 8, 0);
+    for (int x = pair0 + tid; x < pair1; x += NT) {
+        float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+        for (int y = 0; y < kDcMaxCluster; ++y) {
+            if (y >= cs) break;
+            const float2 v = outputs[y * pair_cap + (x - pair0)];
+            a0 += v.x;
+            a1 += v.y;
+        }
+        const double Z = misc->Zt[x / kHalfD];
+        const float o0 = (float)((double)a0 / Z), o1 = (float)((double)a1 / Z);
+        if constexpr (kBf16) reinterpret_cast<uint32_t*>(p.out)[(size_t)u * np + x] = (uint32_t)float_to_bf16_bits(o0) | ((uint32_t)float_to_bf16_bits(o1) << 16);
+        else reinterpret_cast<float2*>(p.out)[(size_t)u * np + x] = make_float2(o0, o1);
+    }
+    late |= !mbar_wait_cluster(xbar + kDcCounts * 8, 0);
+    if (__syncthreads_or(late)) {                             // (and the block's keep bits are there)
+        late = true;
+        leave(false);
+        return;
+    }
+    int total = 0, before = 0, mine = 0, imp_total = 0;       // kept slots of the unit, of the blocks before this one, of this one
+    uint32_t marks = 0u;
+#pragma unroll
+    for (int y = 0; y < kEnt; ++y) {
+        const int e = y * 32 + lane;
+        if (e >= cs * NW) break;
+        const uint2 v = misc->verdicts[e];
+        const int n = (int)(v.x & 0xffffffu);
+        total += n;
+        before += e / NW < rank ? n : 0;
+        mine += e / NW == rank ? n : 0;
+        imp_total += (int)v.y;
+        marks |= v.x >> 24;
+    }
+    total = __reduce_add_sync(0xffffffffu, total);
+    before = __reduce_add_sync(0xffffffffu, before);
+    marks = __reduce_or_sync(0xffffffffu, marks);
+    uint32_t tail = lane < n_words ? misc->tail[lane] : 0u;   // kept slots of the unit's last words, the last one first
+    if (marks) {                                              // the same in every block
+        const uint32_t meet = xbar + kDcMeet * 8;
+        mine = __reduce_add_sync(0xffffffffu, mine);
+        const int mine_imp = __reduce_add_sync(0xffffffffu, lane < NW ? (int)misc->verdicts[rank * NW + lane].y : 0);
+        if (tid == 0) { misc->cnt.count = mine; misc->cnt.n_imp = mine_imp; }
+        uint32_t phase = 0u;
+        late |= !dc_meet(meet, cs, phase);
+        late |= !dc_exact_heads<T, D, NW, GP>(p, u, G, t, k_begin, k_end, marks, keep, misc, cs, phase);
+        phase += 2u * __popc(marks);
+        late |= !dc_meet(meet, cs, phase);
+        uint4 pc = make_uint4(0u, 0u, 0u, 0u);
         if (lane < cs) pc = ld_peer_v4(map_rank(smem_addr(&misc->cnt), lane));
-        if (warp == 1 && n_words - 1 - lane >= 0) last_keep = peer_keep(n_words - 1 - lane);
-    };
-    load_counts();
-    {
-        const uint32_t marks = __reduce_or_sync(0xffffffffu, pc.x);
-        if (marks) {                                          // uniform in the cluster
-            cluster_sync();
-            dc_exact_heads<T, D, NW>(p, u, G, t, k_begin, k_end, marks, keep, misc, cs);
-            cluster_sync();
-            load_counts();
+        total = __reduce_add_sync(0xffffffffu, (int)pc.x);
+        before = __reduce_add_sync(0xffffffffu, lane < rank ? (int)pc.x : 0);
+        imp_total = (int)pc.y;
+        const int wd = n_words - 1 - lane;
+        if (wd >= 0) {                                        // from the block that owns the word: the last one with word_begin <= wd
+            const int o = (int)((uint32_t)((wd + 1) * cs - 1) / (uint32_t)n_words);
+            tail = ld_peer_u32(map_rank(smem_addr(keep + (wd - word_begin(o, cs))), o));
+        }
+        late |= !dc_meet(meet, cs, phase);                    // a block's shared memory stays until its peers have read it
+        if (__syncthreads_or(late)) {
+            late = true;
+            leave(false);
+            return;
         }
     }
-    // outputs (Eq. 1): the unit's G x D values are shared out over the blocks, two channels per thread
-    auto write_outputs = [&](int first, int step) {
-        const int np = G * D / 2, x0 = np * rank / cs, x1 = np * (rank + 1) / cs;
-        for (int x = x0 + first; x < x1; x += step) {
-            const uint32_t at = smem_addr(smem) + x * 8;
-            double v[kDcMaxCluster];
-#pragma unroll
-            for (int y = 0; y < kDcMaxCluster; ++y) v[y] = y < cs ? ld_peer_f64(map_rank(at, y)) : 0.0;
-            float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-            for (int y = 0; y < kDcMaxCluster; ++y) {
-                a0 += __uint_as_float((uint32_t)__double2loint(v[y]));
-                a1 += __uint_as_float((uint32_t)__double2hiint(v[y]));
-            }
-            const double Z = misc->Zt[x / (D / 2)];
-            const float o0 = (float)((double)a0 / Z), o1 = (float)((double)a1 / Z);
-            if constexpr (kBf16) reinterpret_cast<uint32_t*>(p.out)[(size_t)u * np + x] = (uint32_t)float_to_bf16_bits(o0) | ((uint32_t)float_to_bf16_bits(o1) << 16);
-            else reinterpret_cast<float2*>(p.out)[(size_t)u * np + x] = make_float2(o0, o1);
-        }
-    };
     // ---- 3. compaction: kept slots at or above the new length move into the holes below it ----
     // Hole number = evicted slots before it, mover number = kept slots behind it, so both follow from the blocks' counts.
-    const int total = __reduce_add_sync(0xffffffffu, (int)pc.y), before = __reduce_add_sync(0xffffffffu, lane < rank ? (int)pc.y : 0);
-    const int imp_total = rank == 0 && warp == 0 ? __reduce_add_sync(0xffffffffu, (int)pc.z) : 0;
     const int new_len = evict_on ? total : l;
     auto row_of = [&](int slot) -> size_t {
         return pt_u ? page_row(__ldcg(pt_u + (slot >> 5)), slot, p.pool_pages, p.status) : (size_t)u * p.C + (size_t)slot;
@@ -1108,59 +1186,46 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         hm = ~m & valid & below;
         m &= ~below;                                          // kept slots at or above the new length
     };
+    int n_moved = 0;                                          // row moves of the unit
+    auto inclusive_scan = [&](int x) -> int {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += up; }
+        return x;
+    };
     if (new_len < l && l - new_len <= kDcListCap) {
-        // The usual step: every block fills its own holes; the last words of the unit, where the movers are, are read from
-        // the blocks that own them. Warp 0 lists the block's holes, warp 1 the movers that go there.
+        // The usual step: every block fills its own holes; what moves is in the last words of the unit. A word's bits are
+        // listed by a warp at once, a bit per lane (one lane walking through a word's bits took 1-2 us of a step).
         const int nw = (n_keys + 31) >> 5, k_lo = max(0, k_begin - before);     // number of the block's first hole
-        if (warp == 0) {
-            int base = 0;
-            for (int i0 = 0; i0 < nw && k_begin + i0 * 32 < new_len; i0 += 32) {
-                uint32_t m = 0u, hm = 0u;
-                if (i0 + lane < nw) hole_words(i0 + lane, m, hm);
-                int at = __popc(hm);
+        int n_holes = 0;
+        for (int i0 = 0; i0 < nw && k_begin + i0 * 32 < new_len; i0 += 32) {
+            uint32_t m = 0u, hm = 0u;
+            if (i0 + lane < nw) hole_words(i0 + lane, m, hm);
+            const int upto = inclusive_scan(__popc(hm));
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xffffffffu, at, o); if (lane >= o) at += up; }
-                const int all = __shfl_sync(0xffffffffu, at, 31);
-                at += base - __popc(hm);
-                base += all;
-                for (; hm; hm &= hm - 1u) holes[at++] = k_begin + (i0 + lane) * 32 + __ffs(hm) - 1;
+            for (int y = 0; y < 32; y += NW) {
+                const uint32_t bits = __shfl_sync(0xffffffffu, hm, y + warp);
+                const int end = __shfl_sync(0xffffffffu, upto, y + warp);
+                if ((bits >> lane) & 1u) holes[n_holes + end - __popc(bits >> lane)] = k_begin + (i0 + y + warp) * 32 + lane;
             }
-        } else if (warp == 1) {
-            const int first_w = new_len >> 5;                 // the unit's words that hold movers: [first_w, n_words), from the end
-            const int k_hi = k_begin < new_len ? k_lo + n_keys - misc->cnt.count : k_lo;
-            int base = 0;
-            for (int i0 = 0; n_words - 1 - i0 >= first_w; i0 += 32) {
-                const int wd = n_words - 1 - i0 - lane;
-                uint32_t km = 0u;
-                if (wd >= first_w) {
-                    km = i0 == 0 ? last_keep : peer_keep(wd);
-                    if (wd == first_w) km &= ~((1u << (new_len & 31)) - 1u);
-                }
-                int at = __popc(km);
+            n_holes += __shfl_sync(0xffffffffu, upto, 31);
+        }
+        {
+            const int first_w = new_len >> 5, my_w = n_words - 1 - lane;         // the unit's words that hold movers: [first_w, n_words)
+            uint32_t km = my_w >= first_w ? tail : 0u;
+            if (my_w == first_w) km &= ~((1u << (new_len & 31)) - 1u);
+            const int upto = inclusive_scan(__popc(km));
+            n_moved = __shfl_sync(0xffffffffu, upto, 31);
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xffffffffu, at, o); if (lane >= o) at += up; }
-                const int all = __shfl_sync(0xffffffffu, at, 31);
-                at += base - __popc(km);
-                base += all;
-                while (km) {                                  // from the last slot down
-                    const int bit = 31 - __clz(km);
-                    km &= ~(1u << bit);
-                    if (at >= k_lo && at < k_hi) movers[at - k_lo] = wd * 32 + bit;
-                    ++at;
-                }
+            for (int y = 0; y < 32; y += NW) {                // movers are numbered from the last slot down
+                const uint32_t bits = __shfl_sync(0xffffffffu, km, y + warp);
+                const int at = __shfl_sync(0xffffffffu, upto, y + warp) - __popc(bits & ((2u << lane) - 1u)) - k_lo;
+                if (((bits >> lane) & 1u) && at >= 0 && at < n_holes) movers[at] = (n_words - 1 - y - warp) * 32 + lane;
             }
-            if (lane == 0) misc->n_moved = base;
-        } else {
-            write_outputs(tid - 64, NT - 64);
         }
         __syncthreads();
-        const int n_moved = misc->n_moved;
-        const int mine = k_begin < new_len ? min(n_moved, k_lo + n_keys - misc->cnt.count) - k_lo : 0;
-        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, movers, holes, mine, 0, 1, l, p.status);
-    } else {
-        write_outputs(tid, NT);
-    }
-    if (new_len < l && l - new_len > kDcListCap) {
+        const int n = min(n_holes, n_moved - k_lo);
+        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, movers, holes, n, 0, 1, l, p.status);
+    } else if (new_len < l) {
         // many: the lists go to scratch and the moves are shared out evenly
         int* gholes = reinterpret_cast<int*>(p.stash + (size_t)u * G * p.C) + (size_t)G * p.C;   // behind the unit's logits
         int* gmovers = gholes + p.C / 2;
@@ -1183,17 +1248,29 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
                 if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) gmovers[x] = s0 + bit;
             }
         }
-        cluster_sync();
+        uint32_t phase = marks ? 3u + 2u * __popc(marks) : 0u;
+        late = !dc_meet(xbar + kDcMeet * 8, cs, phase);
+        if (__syncthreads_or(late)) {
+            late = true;
+            leave(false);
+            return;
+        }
         if (tid == 0) misc->n_moved = __ldcg(&p.unit_rec[u].x);
         __syncthreads();
-        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, gmovers, gholes, misc->n_moved, rank, cs, l, p.status);
+        n_moved = misc->n_moved;
+        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, gmovers, gholes, n_moved, rank, cs, l, p.status);
     }
-    // every block's row moves come before released pages and the stamp; and a block's shared memory stays until its peers
-    // have read it
-    cluster_sync();
+    // every block's row moves come before released pages and the stamp
+    if (pt_u || p.unit_stamp) {
+        __syncthreads();
+        if (tid == 0) mbar_arrive_peer(map_rank(xbar + kDcDone * 8, 0));
+        if (rank == 0) late = !mbar_wait_cluster(xbar + kDcDone * 8, 0);
+    }
     if (rank != 0) return;
+    if (late) report_status(p.status, CORM_ERR_TIMEOUT);
     if (pt_u) settle_pages<NT>(p.page_table, p.page_bits, p.page_room, p.pool_pages, p.pt_stride, p.U, u, l_old, new_len);
     if (pt_u && p.unit_stamp) __syncthreads();
+    if (warp == 0) imp_total = __reduce_add_sync(0xffffffffu, imp_total);
     if (tid == 0) {
         p.live_out[u] = new_len;
         publish_unit_stamp(p, u, new_len);
@@ -1202,8 +1279,9 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         atomicAdd(p.counters + CNT_ATTENDED, (unsigned long long)l);
         if (imp_total) atomicAdd(p.counters + CNT_IMPORTANT, (unsigned long long)imp_total);
         if (new_len < l) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(l - new_len));
-        if (new_len < l && misc->n_moved) atomicAdd(p.counters + CNT_MOVED, (unsigned long long)misc->n_moved);
+        if (n_moved) atomicAdd(p.counters + CNT_MOVED, (unsigned long long)n_moved);
     }
+    if (late) cluster_sync();
 }
 
 // One layer's (or, from it on, all layers') K or V storage as a 2-D tensor [rows][D] with boxes of 16 rows x 128 bytes and

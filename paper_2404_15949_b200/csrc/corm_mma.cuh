@@ -20,7 +20,7 @@
 // again in fp64 by the callers, so results never depend on it.
 #pragma once
 
-#include "corm_common.cuh"
+#include "corm_fast.cuh"
 
 namespace corm {
 
@@ -220,6 +220,36 @@ __device__ __forceinline__ double ld_peer_f64(uint32_t addr) {
     double v;
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
     return v;
+}
+
+// Pushes into the shared memory of a block of the cluster: value and byte count (on that block's barrier) arrive together.
+__device__ __forceinline__ void push_u32(uint32_t addr, uint32_t v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void push_2u32(uint32_t addr, uint32_t x, uint32_t y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void push_2f64(uint32_t addr, double x, double y, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];"
+                 ::"r"(addr), "l"(__double_as_longlong(x)), "l"(__double_as_longlong(y)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_peer(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// mbar_wait for what other blocks of the cluster wrote
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
+    auto try_wait = [&]() -> bool {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        return ok != 0;
+    };
+    if (try_wait()) return true;
+    const long long start = clock64();
+    while (!try_wait())
+        if (clock64() - start > kWaitLimitCycles) return false;
+    return true;
 }
 
 }  // namespace corm
