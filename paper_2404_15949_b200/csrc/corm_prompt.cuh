@@ -14,7 +14,7 @@
 // reads K once, otherwise later passes find it in L2 (a unit's K is a few MB and only as many units are in flight as fit the
 // machine).
 //
-// bf16: both contractions run on the tensor cores. Phase A needs fp64-grade logits: operands cut into exact pieces
+// bf16: both contractions run on the tensor cores (units of many rows: on tcgen05, corm_prompt_tc.cuh). Phase A needs fp64-grade logits: operands cut into exact pieces
 // (corm_mma.cuh), 7 mma.m16n8k16 per 16 channels for 16 keys x 8 rows; the rows' pieces lie on chip for 32 rows at a time,
 // and a warp's tile of keys is cut once for 16 of them. Phase B only has to place a logit on one side of its threshold: one
 // plain mma per 16 channels, whose rounding is at most 2^-23 per term; the few logits inside that bound are formed again in
@@ -51,6 +51,7 @@ template <typename T, int D> __host__ __device__ constexpr int pc_bufs(int rows8
 constexpr int kPcGroup = 4;                     // octets of rows (bf16) whose pieces lie on chip at a time in phase A
 constexpr int kPcGroupB = 8;                    // ... whose raw values do in phase B
 constexpr int kPcMaxCluster = 8;
+constexpr int kTcMinRows = 96;                  // rows of a unit from which phases A and B may run on tcgen05
 constexpr double kPcLogitLimit = 650.0;         // exp of anything below stays finite in fp64, also summed over 2^19 keys
 // Bound of a logit's error, times the prompt's keys, beyond which a unit does both phases in fp64: so many verdicts would be
 // left open that most rows are formed apart. us per pass, tensor cores / fp64, one key channel 256 and 1024 times the others:
@@ -64,7 +65,7 @@ struct PromptClusterParams {
     int32_t rows8;           // w G rounded up to a multiple of 8
 };
 
-struct PcSmem { int ring, zs, thr, n1, qe, flags, words, list, stage, frag, misc, total; };
+struct PcSmem { int ring, zs, thr, n1, qe, flags, words, list, stage, frag, misc, tc, total; };
 constexpr int kPcOpenCap = 64;
 struct PcMisc {
     double red[kPcWarps][2];
@@ -514,8 +515,15 @@ __device__ __noinline__ void pc_open_verdicts(const PromptParams& p, const PcRow
     if (lane == 0) atomicAdd(p.counters + CNT_NEAR, (unsigned long long)n_near);
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kPcThreads, (D * Elem<T>::kBytes <= 256) ? 2 : 1)
+}  // namespace corm
+
+#include "corm_prompt_tc.cuh"
+
+namespace corm {
+
+// kTc: phases A and B on tcgen05 (corm_prompt_tc.cuh)
+template <typename T, int D, bool kTc>
+__global__ void __launch_bounds__(kTc ? kTcThreads : kPcThreads, !kTc && D * Elem<T>::kBytes <= 256 ? 2 : 1)
 prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     extern __shared__ __align__(128) unsigned char smem[];
     const PromptParams& p = pp.p;
@@ -541,7 +549,8 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         }
         return;
     }
-    const PcSmem lay = pc_smem_layout<T, D>(pp.rows8);
+    PcSmem lay;
+    if constexpr (kTc) lay = tc_smem_layout<D>(pp.rows8); else lay = pc_smem_layout<T, D>(pp.rows8);
     const int n_buf = pc_bufs<T, D>(pp.rows8);
     double* zs = reinterpret_cast<double*>(smem + lay.zs);
     double* thr_sm = reinterpret_cast<double*>(smem + lay.thr);
@@ -593,7 +602,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     const int n_oct = pp.rows8 / 8;
     const int n_grp = kBf16 ? (n_oct + kPcGroup - 1) / kPcGroup : 1;                 // passes of phase A
     const int end_a = resident ? nc : n_grp * nc;
-    start(end_a);
+    if (!kTc) start(end_a);
     for (int i = tid; i < (pp.rows8 + 31) / 32; i += kPcThreads) flags[i] = 0u;
     if (tid == 0) { misc->bad = 0; misc->amax = 0u; misc->fail = 0; misc->n_open = 0; }
 
@@ -635,7 +644,28 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     uint4* f12 = reinterpret_cast<uint4*>(smem + lay.frag);
     // a lane's offset for fragment loads inside a tile: chunk 2 kk of its row is one exclusive-or with kk << 5 away
     const uint32_t klane = (lane & 15) * kRow + (((lane >> 4) ^ (lane & 7)) << 4);
-    if constexpr (kBf16) {
+    TcMisc* tc = reinterpret_cast<TcMisc*>(smem + lay.tc);
+    TcBlock block{R, reinterpret_cast<const bf16_t*>(Qu), reinterpret_cast<const bf16_t*>(Ku), k_begin, k_end, n_keys, smem + lay.ring, tc, 0u, 0, false};
+    if constexpr (kTc) {
+        if (tid == 0) {
+            mbar_init(smem_addr(tc->bar), 1);
+            mbar_init(smem_addr(tc->bar + 1), 1);
+            mbar_init(smem_addr(tc->full), kPcWarps);
+            mbar_init(smem_addr(tc->full + 1), kPcWarps);
+            fence_mbar_init();
+        }
+        if (tid < 16) tc->exp16[tid] = TcExp<D>::entry(tid);
+        if (warp == 0) tc_alloc(smem_addr(&tc->tmem));
+        tc_before_sync();
+        __syncthreads();
+        tc_after_sync();
+        block.tmem = tc->tmem;
+        if (warp == kPcWarps) {                               // its work is done with phase A's products (barriers don't count it then)
+            tc_issue_a<D>(block);
+            return;
+        }
+        bad = !tc_phase_a<D>(block, zs, n1_sm, qe_sm, &misc->amax) || (smem_addr(smem) & 1023u);     // (the swizzle's alignment; never expected)
+    } else if constexpr (kBf16) {
         // A group of four octets of rows at a time: its pieces are made once and stay on chip while the block's keys pass;
         // a warp takes one tile of every chunk, cuts it into pieces once per two octets and keeps its rows' sums in
         // registers to the end of the pass.
@@ -753,13 +783,15 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
     // ---- B. verdicts -> registers ----
     const int n_grp_b = kBf16 ? (n_oct + kPcGroupB - 1) / kPcGroupB : 1;
     const int end_b = resident || wide ? 0 : n_grp_b * nc;
-    if (!resident && !wide) start(end_b);
+    if (!kTc && !resident && !wide) start(end_b);
     if (wide) {
         cluster_sync();                                       // everybody has read everybody's sums of phase A
         constexpr int kBuf = kPcKeys * kRow;
         static_assert(kPcWarps * 4 * D * 8 <= kBuf, "the widened rows fit a ring buffer");
         pc_fp64_rows<T, D>(p, R, Qu, Ku, k_begin, n_keys, smem + lay.ring, reinterpret_cast<double*>(smem + lay.ring + kBuf), zs, thr_sm,
                            kBf16 ? reinterpret_cast<uint32_t*>(f12) : words_sm, words_g, flags, misc, cs);
+    } else if constexpr (kTc) {
+        tc_phase_b<D>(p, block, thr_sm, n1_sm, qe_sm, eps_unit, words_g, flags, misc);
     } else if constexpr (kBf16) {
         uint2* fr = reinterpret_cast<uint2*>(f12);
         for (int grp = 0; grp < n_grp_b; ++grp) {
@@ -855,6 +887,10 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         }
     }
     __syncthreads();
+    if constexpr (kTc) {
+        if (warp == 0) tc_free(block.tmem);
+        if (block.late) report_status(p.status, CORM_ERR_TIMEOUT);
+    }
 
     // ---- keep rule of Algorithm 1 for the block's keys; counts and marked rows are exchanged together ----
     const bool evict_on = wp >= w;
@@ -1019,9 +1055,22 @@ inline cudaError_t launch_prompt_begin(PromptBeginParams& bp, const int32_t* len
     return cudaSuccess;
 }
 
+// Whether phases A and B of a bf16 pass run on tcgen05. A block has an SM to itself there, so it takes rows enough to fill the
+// 128 lanes, and either few units (whose clusters of eight fit the machine at once) or much work. us per pass, mma.sync ->
+// tcgen05, 128 channels: 32 units x 1000 keys, 96 / 128 / 256 rows, 68 -> 118 / 96 -> 119 / 144 -> 93; 32 x 1500, 128 rows, 127 -> 142;
+// 128 x 3000, 96 / 128 rows, 569 -> 566 / 703 -> 556; 1024 x 3000, 100 rows, 3760 -> 3070; 8 x 256, 96 rows, 46 -> 39; 8 x 4096, 128
+// rows, 160 -> 89; 32 x 300, 192 rows, 85 -> 65; 64 channels: 64 x 2000, 128 rows, 178 -> 192; 32 x 1000, 256 rows, 98 -> 69.
+inline bool tc_takes(int n_units, int rows, int max_p, int sm_count) {
+    if (rows < kTcMinRows || rows > kTcMaxRows || max_p < 256) return false;
+    if (rows >= 192 || n_units * kPcMaxCluster <= sm_count) return true;
+    return (double)n_units * max_p * rows >= (rows >= 128 ? 2e7 : 2e8);
+}
+
 // Host side. Returns CORM_ERR_UNSUPPORTED when the launch does not fit.
-template <typename T, int D>
+template <typename T, int D, bool kTc = false>
 inline corm_status_t launch_prompt_cluster(const PromptParams& p, int G, int max_p, int sm_count, cudaStream_t st) {
+    if constexpr (!kTc && Elem<T>::kBytes == 2)
+        if (tc_takes(p.U, p.w * G, max_p, sm_count)) return launch_prompt_cluster<T, D, true>(p, G, max_p, sm_count, st);
     PromptClusterParams pp{};
     pp.p = p;
     while ((1 << pp.log2g) < G) ++pp.log2g;
@@ -1032,16 +1081,21 @@ inline corm_status_t launch_prompt_cluster(const PromptParams& p, int G, int max
     // first version of the kernel (the shapes take 840, 598 and 60 us now, with 2, 8 and 8):
     // 1024 units x 3250 keys 969-1353 (with the slab's stride) / 956-1033 / 1073 / 1365, 128 units x 8192 keys (G 4) 2152 / 1281 / 811 / 752, 32 units x
     // 4096 keys 350 / 192 / 120 / 93.
+    // On tcgen05, one block per SM: one wave where clusters of two or more fit it, else three waves and more (128 units of 2048..
+    // 4096 keys, w 256, with 1 / 2 / 4 / 8: 985 / 967 / 907 / 1197).
     int cs = 1;
-    while (cs < kPcMaxCluster && cs * 2 <= n_words && (long long)p.U * cs < 1500ll * sm_count / 148) cs *= 2;
-    const PcSmem lay = pc_smem_layout<T, D>(pp.rows8);
+    const bool one_wave = kTc && p.U * 2 <= sm_count;
+    const long long blocks = one_wave ? sm_count / 2 + 1 : (kTc ? 500ll : 1500ll) * sm_count / 148;
+    while (cs < kPcMaxCluster && cs * 2 <= n_words && (long long)p.U * cs < blocks) cs *= 2;
+    PcSmem lay;
+    if constexpr (kTc) lay = tc_smem_layout<D>(pp.rows8); else lay = pc_smem_layout<T, D>(pp.rows8);
     if (lay.total > 227 * 1024) return CORM_ERR_UNSUPPORTED;
-    auto kern = prompt_cluster_kernel<T, D>;
+    auto kern = prompt_cluster_kernel<T, D, kTc>;
     cudaError_t e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), (size_t)lay.total);
     if (e == cudaSuccess) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)p.U, (unsigned)cs);
-        cfg.blockDim = dim3(kPcThreads);
+        cfg.blockDim = dim3(kTc ? kTcThreads : kPcThreads);
         cfg.dynamicSmemBytes = (size_t)lay.total;
         cfg.stream = st;
         cudaLaunchAttribute attr[2];

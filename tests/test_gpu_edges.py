@@ -406,3 +406,84 @@ def test_prompts_of_wide_range_take_fp64_time_not_a_pass_per_row(what):
     data.k_prompt, data.q_last = _widen(data, what, "bf16")
     wide, _ = _prompt_time(cfg, data, "bf16")
     assert wide < 7 * plain, (plain, wide)
+
+
+# a step lists its row moves on chip up to 992 evicted slots (what moves lies in the unit's last 32 words then), and in scratch
+# beyond; holes spread out, all at the front, all in the last words; the most words a block of fp32 / 64 channels may own
+EVICTED = [
+    # dtype, head_dim, group, live keys, max_tokens, evicted, where, one block
+    ("bf16", 128, 4, 3000, 3100, 1, "anywhere", False),
+    ("bf16", 128, 1, 3000, 3100, 991, "anywhere", False),
+    ("bf16", 128, 4, 3007, 3100, 992, "front", False),
+    ("bf16", 64, 8, 3040, 3100, 992, "back", False),
+    ("f32", 128, 2, 2999, 3100, 993, "anywhere", False),
+    ("f32", 64, 1, 1500, 1600, 992, "anywhere", True),
+    ("bf16", 128, 2, 1055, 1100, 992, "front", True),
+    ("f32", 64, 1, 114000, 3583 * 32, 1500, "anywhere", True),
+    ("f32", 64, 2, 114600, 3584 * 32, 700, "back", True),
+]
+
+
+@pytest.mark.parametrize("case", EVICTED, ids=lambda c: "-".join(str(x) for x in c))
+def test_steps_around_the_lists_of_row_moves(case):
+    dtype, d, G, n, C, evicted, where, one_block = case
+    cfg = _cfg(dtype, d, G, 1, 1, (1, 1), 2, 4, 8, alpha=1e9)         # no key is important: what goes is what has no bit set
+    rng = np.random.default_rng(evicted + d)
+    to = (lambda x: to_dev(x, dtype).float().cpu().numpy())
+    k, v = (to(rng.standard_normal((n, d), dtype=np.float32)) for _ in range(2))
+    q = to(rng.standard_normal((2, 1, G, d), dtype=np.float32))
+    kn, vn = (to(rng.standard_normal((2, 1, 1, d), dtype=np.float32)) for _ in range(2))
+    word, pos = np.ones(n, np.uint32), np.arange(1, n + 1, dtype=np.int32)
+    old = n - 16                                                      # (the last eight tokens stay in any case)
+    word[{"anywhere": rng.choice(old, evicted, replace=False), "front": np.arange(evicted), "back": np.arange(old - evicted, old)}[where]] = 0
+    gpu, orc = make_gpu_cache(cfg, 1, 1, max_tokens=C), make_oracle(cfg, 1, 1, max_tokens=C)
+    gpu.corm_cache_set_tuning(1 << 18 if one_block else 0, 4)
+    gpu.corm_cache_import_state(0, 0, 0, k, v, word, pos, n, 4)
+    orc.import_unit(0, 0, 0, k, v, word, pos, n, 4)
+    for s in range(2):
+        out = gpu.corm_decode_step(0, to_dev(q[s], dtype), to_dev(kn[s], dtype), to_dev(vn[s], dtype))
+        ref = orc.decode_step(0, q[s], kn[s], vn[s])
+        assert np.abs(out.float().cpu().numpy() - ref).max() <= OUT_TOL[dtype]
+        assert_states_equal(gpu, orc, 0, 1, 1, f"step {s}")
+        if s == 0:
+            assert gpu.corm_cache_stats()["evicted_keys"] == evicted
+    assert gpu.corm_cache_stats()["device_status"] == 0
+
+
+# windows and groups of 96 to 1024 rows on prompts from 256 keys on go through tcgen05, 128 rows and 64 keys at a time: the
+# rows just enough, a full and a nearly empty last group, the most; tiles full, one key over, one short; ragged prompts
+# shorter than the window and than a tile
+MANY_ROWS = [
+    # head_dim, group, kv heads, batch, prompt range, w
+    (128, 1, 2, 3, (256, 256), 96),
+    (128, 8, 1, 3, (257, 330), 12),
+    (128, 8, 1, 2, (1000, 1100), 16),
+    (128, 1, 2, 3, (319, 321), 128),
+    (128, 1, 3, 4, (3, 700), 129),
+    (128, 2, 2, 2, (640, 640), 100),
+    (128, 4, 2, 2, (500, 2100), 256),
+    (64, 1, 2, 3, (40, 600), 97),
+    (64, 4, 1, 3, (255, 449), 32),
+    (64, 8, 1, 2, (1023, 1025), 128),
+]
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e6], ids=["", "all-open"])
+@pytest.mark.parametrize("case", MANY_ROWS, ids=lambda c: "-".join(str(x) for x in c))
+def test_prompts_of_many_rows(case, scale):
+    """Verdicts are the oracle's; with the bounds a million times as wide every one is left open and formed again."""
+    d, G, nkv, B, prange, w = case
+    if scale > 1.0 and w * G * prange[1] > 150000:
+        pytest.skip("a pass per row: long")
+    cfg = _cfg("bf16", d, G, nkv, B, prange, 2, w, 16)
+    data = generate(cfg)
+    orc = make_oracle(cfg, B, nkv)
+    orc.set_near_band(1e-11)
+    orc.compress_prompt(0, data.k_prompt, data.v_prompt, data.q_last, data.prompt_lens)
+    for pool in (0, -(-B * nkv * (cfg.max_tokens // 32 + 2) // 32) * 32):
+        gpu = make_gpu_cache(cfg, B, nkv, pool_pages=pool)
+        gpu.corm_cache_set_bound_scale(scale)
+        gpu.corm_compress_prompt(0, to_dev(data.k_prompt, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(data.q_last, "bf16"),
+                                 data.prompt_lens)
+        assert_states_equal(gpu, orc, 0, B, nkv, f"pool {pool}")
+        assert gpu.corm_cache_stats()["device_status"] == 0
