@@ -100,7 +100,8 @@ __device__ __forceinline__ float tc_split_error(float n1, float n2, float n3) {
 }
 
 // exp(s / sqrt(D)) is added to z: 2^(n / 16) from a table, a Taylor polynomial of degree 6 on what is left (at most ln2 / 32:
-// truncation 5e-16), the 1/sqrt(D) inside the constants. Any s beyond the limit gives some number.
+// truncation 5e-16), the 1/sqrt(D) inside the constants. An s beyond the limit gives any number or none; a logit that is not
+// `on` may lie there and adds nothing: its power of two is that of n = 0 (0 x infinity would be no number).
 template <int D> struct TcExp {
     static constexpr double kScale = D == 128 ? 2.040278893193579 : 2.8853900817779268;
     static constexpr double kC1 = D == 128 ? 0.49012907172436826 : 0.3465735902718734;              // sqrt(D) ln2 / 16, its first 35 bits
@@ -113,7 +114,7 @@ template <int D> struct TcExp {
     static __device__ __forceinline__ void add(double& z, double s, const double* exp16, bool on) {
         constexpr double kMagic = 6755399441055744.0;
         const double t = fma(s, kScale, kMagic), nf = t - kMagic;
-        const int n = __double2loint(t);
+        const int n = on ? __double2loint(t) : 0;
         const double r = fma(nf, -kC2, fma(nf, -kC1, s));
         double p = c1 * c1 * c1 * c1 * c1 * c1 / 720.0;
         p = fma(p, r, c1 * c1 * c1 * c1 * c1 / 120.0);

@@ -487,3 +487,34 @@ def test_prompts_of_many_rows(case, scale):
                                  data.prompt_lens)
         assert_states_equal(gpu, orc, 0, B, nkv, f"pool {pool}")
         assert gpu.corm_cache_stats()["device_status"] == 0
+
+
+# logits that the causal mask hides, where 2^(logit / ln 2) leaves the exponents of fp64 for infinity and NaN: 709.8..710.4 and
+# -709.8..-709.1, every 1419.6 from there on
+HIDDEN_LOGITS = (710.1, -709.45, 2129.7, -2129.0)
+
+
+@pytest.mark.parametrize("target", HIDDEN_LOGITS)
+@pytest.mark.parametrize("d,G,w", [(128, 1, 128), (64, 1, 128), (128, 4, 32), (64, 2, 64)])
+def test_hidden_logits_of_any_size(d, G, w, target):
+    """Every query but the last has the target logit with the prompt's last key, which none of them sees; the last query,
+    which does, is orthogonal to it. All visible logits are ordinary. Elements are multiples of 1/16, so that the unit's
+    bounds stay narrow next to so large a key."""
+    cfg = _cfg("bf16", d, G, 2, 3, (256, 330), 2, w, 16)
+    data = generate(cfg)
+    kp, ql = (np.round(x * 16.0) / 16.0 for x in (data.k_prompt, data.q_last))
+    grid = torch.arange(64, 160) / 16.0                                         # the query's channel; the key's follows from it
+    key = (abs(target) * np.sqrt(d) / grid).to(torch.bfloat16).float()
+    best = (grid * key / np.sqrt(d) - abs(target)).abs().argmin()
+    assert abs(float(grid[best] * key[best]) / np.sqrt(d) - abs(target)) < 0.3
+    kp[..., 0] = 0.0
+    ql[:, :, :w - 1, 0], ql[:, :, w - 1, 0] = float(grid[best]), 0.0
+    for b, P in enumerate(data.prompt_lens):
+        kp[b, :, P - 1, 0] = float(key[best]) * np.sign(target)
+    kp, ql = kp.astype(np.float32), ql.astype(np.float32)
+    orc, gpu = make_oracle(cfg, 3, 2), make_gpu_cache(cfg, 3, 2)
+    orc.set_near_band(1e-11)
+    orc.compress_prompt(0, kp, data.v_prompt, ql, data.prompt_lens)
+    gpu.corm_compress_prompt(0, to_dev(kp, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(ql, "bf16"), data.prompt_lens)
+    assert_states_equal(gpu, orc, 0, 3, 2, "")
+    assert gpu.corm_cache_stats()["device_status"] == 0
