@@ -86,21 +86,23 @@ constexpr int kDcListCap = 992;
 // What the ring holds once the tiles are done: the warps' records at the start of their parts, and from 4 KB on the keep bits
 // of the block's words and, behind them, the lists of a step with few moves or the prefix sums (one more than words) of a
 // step with many. So the words a block may own follow from the instance's ring: 4096 for the rings of 64 KB, 3583 for the
-// 32 KB of fp32 / 64 channels.
-constexpr int kDcRecBytes = 4096;
+// 32 KB of fp32 / 64 channels. The ring's last 4 KB hold the registers of the unit's last 32 words.
+constexpr int kDcRecBytes = 4096, kDcRegBytes = 32 * 32 * 4;
 template <typename T, int D, int GP, int NW> __host__ __device__ constexpr int dc_max_words() {
     constexpr int n = (NW * DcShape<T, D, GP>::kWarpRing - kDcRecBytes - 4) / 8;
     return n < 4096 ? n : 4096;
 }
 template <typename T, int D, int GP, int NW> __host__ __device__ constexpr bool dc_ring_holds_lists() {
     constexpr int words = dc_max_words<T, D, GP, NW>(), lists = 2 * kDcListCap * 4, sums = 4 * (words + 1);
-    return GP * D * 4 <= kDcRecBytes && kDcRecBytes + 4 * words + (lists > sums ? lists : sums) <= NW * DcShape<T, D, GP>::kWarpRing;
+    constexpr int ring = DcShape<T, D, GP>::kWarpRing;
+    return GP * D * 4 <= kDcRecBytes && kDcRecBytes + kDcRegBytes <= ring && kDcRecBytes + 4 * words + sums <= NW * ring &&
+           kDcRecBytes + 4 * words + lists + kDcRegBytes <= NW * ring;
 }
 
 constexpr int kDcOpenCap = 32;
 // A block's barriers: what every warp of the unit's blocks found (kDcRecords), the block's share of the outputs' numerators
-// from every block (kDcOutputs), the warps' verdicts in numbers and the unit's last keep bits (kDcCounts), all blocks
-// (kDcMeet) and, at the first block, the others being done with the unit (kDcDone).
+// from every block (kDcOutputs), the warps' verdicts in numbers, the unit's last keep bits and registers and the appended row
+// (kDcCounts), all blocks (kDcMeet) and, at the first block, the others being done with the unit (kDcDone).
 enum { kDcRecords = 0, kDcOutputs = 1, kDcCounts = 2, kDcMeet = 3, kDcDone = 4, kDcBars = 5 };
 template <int NW, int GP> struct DcMisc {
     unsigned long long bar[kDcBars], stamp;
@@ -570,7 +572,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     if (tid == 0) {                                           // what will be pushed into this block
         mbar_expect_tx(xbar + kDcRecords * 8, cs0 * NW * (G * 16 + 4));
         mbar_expect_tx(xbar + kDcOutputs * 8, cs0 * (first_pair(rank0 + 1, cs0) - first_pair(rank0, cs0)) * 8);
-        mbar_expect_tx(xbar + kDcCounts * 8, cs0 * NW * 8 + min(32, n_words) * 4);
+        mbar_expect_tx(xbar + kDcCounts * 8, cs0 * NW * 8 + min(32, n_words) * (4 + 128) + (rank0 < cs0 - 1 ? 2 * S::kRow : 0));
     }
     const int k_begin = w0 * 32, k_end = state ? 0 : min(l, w1 * 32), n_keys = max(0, k_end - k_begin);
     const int n_tiles = (n_keys + kDcKeys - 1) / kDcKeys;
@@ -994,6 +996,14 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     // keys were cut for. Where the appended key sent its block to the fp64 loop the others cut for the one before it.
     const uint32_t cut_for = unit_state & kDcWide ? misc->cut_for : unit_state & 0xffffu;
     const float eps_a = kBf16 && (cut_for || !(unit_state & kDcWide)) ? split_amax(cut_for) * (float)inv_root_d * 1.0001f : 0.f;
+    // The appended row goes to the blocks, one of which may move it into a hole: by the warps that have no head here.
+    if (rank == cs - 1 && (G >= NW || warp >= G)) {
+        constexpr int kNew = 2 * S::kRow / 16;
+        const int first = G >= NW ? 0 : G * 32;
+        for (int x = tid - first; x < (cs - 1) * kNew; x += NT - first)
+            push_v4(map_rank(smem_addr(newrow + x % kNew * 16), x / kNew), *reinterpret_cast<const uint4*>(newrow + x % kNew * 16),
+                    map_rank(xbar + kDcCounts * 8, x / kNew));
+    }
     for (int h = warp; h < G; h += NW) {
         double m[kEnt], z[kEnt], M = -INFINITY, Z = 0.0;
 #pragma unroll
@@ -1022,6 +1032,12 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
 
     // ---- 2. verdicts, register update, keep bits ----
     uint32_t* keep = reinterpret_cast<uint32_t*>(smem + kDcRecBytes);           // the ring is free behind the warps' records
+    // Pushes don't order a block's ordinary stores for the others, so what a row move needs of this step, the registers of the
+    // unit's last 32 words and the appended row, is pushed too. us per request with a release (an arrival on a barrier of its own)
+    // instead / with these pushes: tiny fp32 721 / 682, 32 layers 11004 / 10705, G 8 1255 / 1223, 64 channels 1293 / 1232, fp32
+    // 728 / 699, but G 4 5846 / 5880 and 6042 / 6137 (more registers than there are behind the loop of that instance).
+    uint32_t* tail_regs = reinterpret_cast<uint32_t*>(smem + NW * S::kWarpRing - kDcRegBytes);
+    const int tail_slot = (n_words - 32) * 32;                // the first of them (negative in short units)
     // the block's share of the unit's output numerators, as the blocks push it: [block][pair]
     const int np = G * kHalfD, pair0 = first_pair(rank, cs), pair1 = first_pair(rank + 1, cs), pair_cap = (np + cs - 1) / cs;
     float2* outputs = reinterpret_cast<float2*>(smem + (kBf16 ? lay.pieces : lay.q));           // (every warp is done with the queries)
@@ -1083,19 +1099,29 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             for (int k = 0; k < kB; ++k) {
                 const int base = base0 + k * NT, i = base + tid;
                 if (base + warp * 32 >= n_keys) break;        // uniform in the warp
+                const int word = (base >> 5) + warp, from_end = n_words - 1 - ((k_begin >> 5) + word);
                 const bool on = i < n_keys, im = (imp >> k) & 1u;
                 bool kp = false;
+                uint32_t wd = 0u;
                 if (on) {
-                    const uint32_t wd = update_register(wv[k], im, p.w, t);
+                    wd = update_register(wv[k], im, p.w, t);
                     if (CORM_IN_RANGE(k_begin + i < p.C, p.status)) wordu[k_begin + i] = wd;
                     kp = !evict_on || register_needed(wd, p.w, t) || pv[k] > t - p.r;
                 }
                 const uint32_t ballot = __ballot_sync(0xffffffffu, kp);
                 n_imp += __popc(__ballot_sync(0xffffffffu, im));
                 n_keep += __popc(ballot);
-                const int wd = (base >> 5) + warp, from_end = n_words - 1 - ((k_begin >> 5) + wd);
-                if (lane == 0 && CORM_IN_RANGE(wd < kMaxWords, p.status)) keep[wd] = ballot;
-                if (from_end < 32 && lane < cs) push_u32(map_rank(smem_addr(misc->tail + from_end), lane), ballot, map_rank(xbar + kDcCounts * 8, lane));
+                if (lane == 0 && CORM_IN_RANGE(word < kMaxWords, p.status)) keep[word] = ballot;
+                if (from_end < 32) {
+                    if (lane < cs) push_u32(map_rank(smem_addr(misc->tail + from_end), lane), ballot, map_rank(xbar + kDcCounts * 8, lane));
+                    const int s0 = (lane & 7) * 4;            // four registers a lane, four blocks at a time
+                    uint4 four;
+                    four.x = __shfl_sync(0xffffffffu, wd, s0); four.y = __shfl_sync(0xffffffffu, wd, s0 + 1);
+                    four.z = __shfl_sync(0xffffffffu, wd, s0 + 2); four.w = __shfl_sync(0xffffffffu, wd, s0 + 3);
+                    const uint32_t at = smem_addr(tail_regs + (31 - from_end) * 32 + s0);
+#pragma unroll 1
+                    for (int o = lane >> 3; o < cs; o += 4) push_v4(map_rank(at, o), four, map_rank(xbar + kDcCounts * 8, o));
+                }
             }
         }
         __syncwarp();
@@ -1120,145 +1146,158 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         else reinterpret_cast<float2*>(p.out)[(size_t)u * np + x] = make_float2(o0, o1);
     }
     late |= !mbar_wait_cluster(xbar + kDcCounts * 8, 0);
-    if (__syncthreads_or(late)) {                             // (and the block's keep bits are there)
+    int new_len = l, imp_total = 0, n_moved = 0;              // n_moved: row moves of the unit
+    // Counts, exact heads, moves. Returns false if a wait expired.
+    auto compact = [&]() -> bool {
+        if (__syncthreads_or(late)) return false;             // (and the block's keep bits are there)
+        int total = 0, before = 0, mine = 0;                  // kept slots of the unit, of the blocks before this one, of this one
+        uint32_t marks = 0u;
+#pragma unroll
+        for (int y = 0; y < kEnt; ++y) {
+            const int e = y * 32 + lane;
+            if (e >= cs * NW) break;
+            const uint2 v = misc->verdicts[e];
+            const int n = (int)(v.x & 0xffffffu);
+            total += n;
+            before += e / NW < rank ? n : 0;
+            mine += e / NW == rank ? n : 0;
+            imp_total += (int)v.y;
+            marks |= v.x >> 24;
+        }
+        total = __reduce_add_sync(0xffffffffu, total);
+        before = __reduce_add_sync(0xffffffffu, before);
+        marks = __reduce_or_sync(0xffffffffu, marks);
+        uint32_t tail = lane < n_words ? misc->tail[lane] : 0u; // kept slots of the unit's last words, the last one first
+        if (marks) {                                          // the same in every block
+            const uint32_t meet = xbar + kDcMeet * 8;
+            mine = __reduce_add_sync(0xffffffffu, mine);
+            const int mine_imp = __reduce_add_sync(0xffffffffu, lane < NW ? (int)misc->verdicts[rank * NW + lane].y : 0);
+            if (tid == 0) { misc->cnt.count = mine; misc->cnt.n_imp = mine_imp; }
+            uint32_t phase = 0u;
+            late |= !dc_meet(meet, cs, phase);
+            late |= !dc_exact_heads<T, D, NW, GP>(p, u, G, t, k_begin, k_end, marks, keep, misc, cs, phase);
+            phase += 2u * __popc(marks);
+            late |= !dc_meet(meet, cs, phase);
+            uint4 pc = make_uint4(0u, 0u, 0u, 0u);
+            if (lane < cs) pc = ld_peer_v4(map_rank(smem_addr(&misc->cnt), lane));
+            total = __reduce_add_sync(0xffffffffu, (int)pc.x);
+            before = __reduce_add_sync(0xffffffffu, lane < rank ? (int)pc.x : 0);
+            imp_total = (int)pc.y;
+            const int wd = n_words - 1 - lane;
+            if (wd >= 0) {                                    // from the block that owns the word: the last one with word_begin <= wd
+                const int o = (int)((uint32_t)((wd + 1) * cs - 1) / (uint32_t)n_words);
+                tail = ld_peer_u32(map_rank(smem_addr(keep + (wd - word_begin(o, cs))), o));
+            }
+            late |= !dc_meet(meet, cs, phase);                // a block's shared memory stays until its peers have read it
+            if (__syncthreads_or(late)) return false;
+        }
+        // ---- 3. compaction: kept slots at or above the new length move into the holes below it ----
+        // Hole number = evicted slots before it, mover number = kept slots behind it, so both follow from the blocks' counts.
+        if (evict_on) new_len = total;
+        auto row_of = [&](int slot) -> size_t {
+            return pt_u ? page_row(__ldcg(pt_u + (slot >> 5)), slot, p.pool_pages, p.status) : (size_t)u * p.C + (size_t)slot;
+        };
+        int* holes = reinterpret_cast<int*>(smem + kDcRecBytes) + kMaxWords;    // [kDcListCap] each, behind the keep bits
+        int* movers = holes + kDcListCap;
+        auto hole_words = [&](int i, uint32_t& m, uint32_t& hm) {               // word i of the block: kept slots, holes
+            m = keep[i];
+            const int s0 = k_begin + i * 32;
+            const uint32_t valid = k_end - s0 >= 32 ? 0xffffffffu : (1u << (k_end - s0)) - 1u;
+            const uint32_t below = new_len - s0 >= 32 ? 0xffffffffu : (new_len > s0 ? (1u << (new_len - s0)) - 1u : 0u);
+            hm = ~m & valid & below;
+            m &= ~below;                                      // kept slots at or above the new length
+        };
+        auto inclusive_scan = [&](int x) -> int {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += up; }
+            return x;
+        };
+        if (new_len < l && l - new_len <= kDcListCap) {
+            // The usual step: every block fills its own holes; what moves is in the last words of the unit. A word's bits are
+            // listed by a warp at once, a bit per lane (one lane walking through a word's bits took 1-2 us of a step).
+            const int nw = (n_keys + 31) >> 5, k_lo = max(0, k_begin - before); // number of the block's first hole
+            int n_holes = 0;
+            for (int i0 = 0; i0 < nw && k_begin + i0 * 32 < new_len; i0 += 32) {
+                uint32_t m = 0u, hm = 0u;
+                if (i0 + lane < nw) hole_words(i0 + lane, m, hm);
+                const int upto = inclusive_scan(__popc(hm));
+#pragma unroll
+                for (int y = 0; y < 32; y += NW) {
+                    const uint32_t bits = __shfl_sync(0xffffffffu, hm, y + warp);
+                    const int end = __shfl_sync(0xffffffffu, upto, y + warp);
+                    if ((bits >> lane) & 1u) holes[n_holes + end - __popc(bits >> lane)] = k_begin + (i0 + y + warp) * 32 + lane;
+                }
+                n_holes += __shfl_sync(0xffffffffu, upto, 31);
+            }
+            {
+                const int first_w = new_len >> 5, my_w = n_words - 1 - lane;     // the unit's words that hold movers: [first_w, n_words)
+                uint32_t km = my_w >= first_w ? tail : 0u;
+                if (my_w == first_w) km &= ~((1u << (new_len & 31)) - 1u);
+                const int upto = inclusive_scan(__popc(km));
+                n_moved = __shfl_sync(0xffffffffu, upto, 31);
+#pragma unroll
+                for (int y = 0; y < 32; y += NW) {            // movers are numbered from the last slot down
+                    const uint32_t bits = __shfl_sync(0xffffffffu, km, y + warp);
+                    const int at = __shfl_sync(0xffffffffu, upto, y + warp) - __popc(bits & ((2u << lane) - 1u)) - k_lo;
+                    if (((bits >> lane) & 1u) && at >= 0 && at < n_holes) movers[at] = (n_words - 1 - y - warp) * 32 + lane;
+                }
+            }
+            __syncthreads();
+            const int n = min(n_holes, n_moved - k_lo);
+            // mover 0 is the unit's last slot, if it stays: the row that was appended
+            const int fresh = n > 0 && movers[0] == l_old ? 1 : 0;
+            if (fresh && warp == NW - 1 && CORM_IN_RANGE(holes[0] >= 0 && holes[0] < l, p.status)) {
+                constexpr int kChunks = S::kRow / 16;
+                const size_t at = row_of(holes[0]) * kChunks;
+                for (int c = lane; c < 2 * kChunks; c += 32)
+                    (c < kChunks ? reinterpret_cast<uint4*>(p.K) + at + c : reinterpret_cast<uint4*>(p.V) + at + c - kChunks)[0] =
+                        *reinterpret_cast<const uint4*>(newrow + c * 16);
+            }
+            block_move_rows<T, D, NT, 4, false>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, movers + fresh, holes + fresh, n - fresh, 0, 1, l, p.status);
+            for (int i = tid; i < n; i += NT) {               // registers and positions, a mover per thread
+                const int from = movers[i], to = holes[i];
+                if (!CORM_IN_RANGE(from >= 0 && from < l && to >= 0 && to < l, p.status)) continue;
+                const int32_t pos = from == l_old ? t : __ldcg(posu + from);
+                wordu[to] = marks ? __ldcg(wordu + from) : tail_regs[from - tail_slot];        // (exact heads change registers)
+                posu[to] = pos;
+            }
+        } else if (new_len < l) {
+            // many: the lists go to scratch and the moves are shared out evenly
+            int* gholes = reinterpret_cast<int*>(p.stash + (size_t)u * G * p.C) + (size_t)G * p.C;   // behind the unit's logits
+            int* gmovers = gholes + p.C / 2;
+            int* prefix = holes;                              // [kMaxWords + 1]
+            const int nw = (n_keys + 31) >> 5;
+            block_popc_scan<NT>(keep, prefix, nw, misc->scan);
+            for (int i = tid; i < nw; i += NT) {
+                uint32_t km, hm;
+                hole_words(i, km, hm);
+                const uint32_t m = keep[i];
+                const int s0 = k_begin + i * 32, kb = before + prefix[i];        // kept slots before this word
+                if (new_len >= s0 && new_len < s0 + 32 && new_len < k_end)       // how many: evicted slots below the new length
+                    p.unit_rec[u] = make_int2(new_len - kb - __popc(m & ~km), 0);
+                for (; hm; hm &= hm - 1u) {
+                    const int bit = __ffs(hm) - 1, x = s0 + bit - kb - __popc(m & ((1u << bit) - 1u));
+                    if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) gholes[x] = s0 + bit;
+                }
+                for (; km; km &= km - 1u) {
+                    const int bit = __ffs(km) - 1, x = total - 1 - kb - __popc(m & ((1u << bit) - 1u));
+                    if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) gmovers[x] = s0 + bit;
+                }
+            }
+            uint32_t phase = marks ? 3u + 2u * __popc(marks) : 0u;
+            late = !dc_meet(xbar + kDcMeet * 8, cs, phase);
+            if (__syncthreads_or(late)) return false;
+            if (tid == 0) misc->n_moved = __ldcg(&p.unit_rec[u].x);
+            __syncthreads();
+            n_moved = misc->n_moved;
+            block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, gmovers, gholes, n_moved, rank, cs, l, p.status);
+        }
+        return true;
+    };
+    if (!compact()) {
         late = true;
         leave(false);
         return;
-    }
-    int total = 0, before = 0, mine = 0, imp_total = 0;       // kept slots of the unit, of the blocks before this one, of this one
-    uint32_t marks = 0u;
-#pragma unroll
-    for (int y = 0; y < kEnt; ++y) {
-        const int e = y * 32 + lane;
-        if (e >= cs * NW) break;
-        const uint2 v = misc->verdicts[e];
-        const int n = (int)(v.x & 0xffffffu);
-        total += n;
-        before += e / NW < rank ? n : 0;
-        mine += e / NW == rank ? n : 0;
-        imp_total += (int)v.y;
-        marks |= v.x >> 24;
-    }
-    total = __reduce_add_sync(0xffffffffu, total);
-    before = __reduce_add_sync(0xffffffffu, before);
-    marks = __reduce_or_sync(0xffffffffu, marks);
-    uint32_t tail = lane < n_words ? misc->tail[lane] : 0u;   // kept slots of the unit's last words, the last one first
-    if (marks) {                                              // the same in every block
-        const uint32_t meet = xbar + kDcMeet * 8;
-        mine = __reduce_add_sync(0xffffffffu, mine);
-        const int mine_imp = __reduce_add_sync(0xffffffffu, lane < NW ? (int)misc->verdicts[rank * NW + lane].y : 0);
-        if (tid == 0) { misc->cnt.count = mine; misc->cnt.n_imp = mine_imp; }
-        uint32_t phase = 0u;
-        late |= !dc_meet(meet, cs, phase);
-        late |= !dc_exact_heads<T, D, NW, GP>(p, u, G, t, k_begin, k_end, marks, keep, misc, cs, phase);
-        phase += 2u * __popc(marks);
-        late |= !dc_meet(meet, cs, phase);
-        uint4 pc = make_uint4(0u, 0u, 0u, 0u);
-        if (lane < cs) pc = ld_peer_v4(map_rank(smem_addr(&misc->cnt), lane));
-        total = __reduce_add_sync(0xffffffffu, (int)pc.x);
-        before = __reduce_add_sync(0xffffffffu, lane < rank ? (int)pc.x : 0);
-        imp_total = (int)pc.y;
-        const int wd = n_words - 1 - lane;
-        if (wd >= 0) {                                        // from the block that owns the word: the last one with word_begin <= wd
-            const int o = (int)((uint32_t)((wd + 1) * cs - 1) / (uint32_t)n_words);
-            tail = ld_peer_u32(map_rank(smem_addr(keep + (wd - word_begin(o, cs))), o));
-        }
-        late |= !dc_meet(meet, cs, phase);                    // a block's shared memory stays until its peers have read it
-        if (__syncthreads_or(late)) {
-            late = true;
-            leave(false);
-            return;
-        }
-    }
-    // ---- 3. compaction: kept slots at or above the new length move into the holes below it ----
-    // Hole number = evicted slots before it, mover number = kept slots behind it, so both follow from the blocks' counts.
-    const int new_len = evict_on ? total : l;
-    auto row_of = [&](int slot) -> size_t {
-        return pt_u ? page_row(__ldcg(pt_u + (slot >> 5)), slot, p.pool_pages, p.status) : (size_t)u * p.C + (size_t)slot;
-    };
-    int* holes = reinterpret_cast<int*>(smem + kDcRecBytes) + kMaxWords;        // [kDcListCap] each, behind the keep bits
-    int* movers = holes + kDcListCap;
-    auto hole_words = [&](int i, uint32_t& m, uint32_t& hm) {                   // word i of the block: kept slots, holes
-        m = keep[i];
-        const int s0 = k_begin + i * 32;
-        const uint32_t valid = k_end - s0 >= 32 ? 0xffffffffu : (1u << (k_end - s0)) - 1u;
-        const uint32_t below = new_len - s0 >= 32 ? 0xffffffffu : (new_len > s0 ? (1u << (new_len - s0)) - 1u : 0u);
-        hm = ~m & valid & below;
-        m &= ~below;                                          // kept slots at or above the new length
-    };
-    int n_moved = 0;                                          // row moves of the unit
-    auto inclusive_scan = [&](int x) -> int {
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const int up = __shfl_up_sync(0xffffffffu, x, o); if (lane >= o) x += up; }
-        return x;
-    };
-    if (new_len < l && l - new_len <= kDcListCap) {
-        // The usual step: every block fills its own holes; what moves is in the last words of the unit. A word's bits are
-        // listed by a warp at once, a bit per lane (one lane walking through a word's bits took 1-2 us of a step).
-        const int nw = (n_keys + 31) >> 5, k_lo = max(0, k_begin - before);     // number of the block's first hole
-        int n_holes = 0;
-        for (int i0 = 0; i0 < nw && k_begin + i0 * 32 < new_len; i0 += 32) {
-            uint32_t m = 0u, hm = 0u;
-            if (i0 + lane < nw) hole_words(i0 + lane, m, hm);
-            const int upto = inclusive_scan(__popc(hm));
-#pragma unroll
-            for (int y = 0; y < 32; y += NW) {
-                const uint32_t bits = __shfl_sync(0xffffffffu, hm, y + warp);
-                const int end = __shfl_sync(0xffffffffu, upto, y + warp);
-                if ((bits >> lane) & 1u) holes[n_holes + end - __popc(bits >> lane)] = k_begin + (i0 + y + warp) * 32 + lane;
-            }
-            n_holes += __shfl_sync(0xffffffffu, upto, 31);
-        }
-        {
-            const int first_w = new_len >> 5, my_w = n_words - 1 - lane;         // the unit's words that hold movers: [first_w, n_words)
-            uint32_t km = my_w >= first_w ? tail : 0u;
-            if (my_w == first_w) km &= ~((1u << (new_len & 31)) - 1u);
-            const int upto = inclusive_scan(__popc(km));
-            n_moved = __shfl_sync(0xffffffffu, upto, 31);
-#pragma unroll
-            for (int y = 0; y < 32; y += NW) {                // movers are numbered from the last slot down
-                const uint32_t bits = __shfl_sync(0xffffffffu, km, y + warp);
-                const int at = __shfl_sync(0xffffffffu, upto, y + warp) - __popc(bits & ((2u << lane) - 1u)) - k_lo;
-                if (((bits >> lane) & 1u) && at >= 0 && at < n_holes) movers[at] = (n_words - 1 - y - warp) * 32 + lane;
-            }
-        }
-        __syncthreads();
-        const int n = min(n_holes, n_moved - k_lo);
-        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, movers, holes, n, 0, 1, l, p.status);
-    } else if (new_len < l) {
-        // many: the lists go to scratch and the moves are shared out evenly
-        int* gholes = reinterpret_cast<int*>(p.stash + (size_t)u * G * p.C) + (size_t)G * p.C;   // behind the unit's logits
-        int* gmovers = gholes + p.C / 2;
-        int* prefix = holes;                                  // [kMaxWords + 1]
-        const int nw = (n_keys + 31) >> 5;
-        block_popc_scan<NT>(keep, prefix, nw, misc->scan);
-        for (int i = tid; i < nw; i += NT) {
-            uint32_t km, hm;
-            hole_words(i, km, hm);
-            const uint32_t m = keep[i];
-            const int s0 = k_begin + i * 32, kb = before + prefix[i];            // kept slots before this word
-            if (new_len >= s0 && new_len < s0 + 32 && new_len < k_end)           // how many: evicted slots below the new length
-                p.unit_rec[u] = make_int2(new_len - kb - __popc(m & ~km), 0);
-            for (; hm; hm &= hm - 1u) {
-                const int bit = __ffs(hm) - 1, x = s0 + bit - kb - __popc(m & ((1u << bit) - 1u));
-                if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) gholes[x] = s0 + bit;
-            }
-            for (; km; km &= km - 1u) {
-                const int bit = __ffs(km) - 1, x = total - 1 - kb - __popc(m & ((1u << bit) - 1u));
-                if (CORM_IN_RANGE(x >= 0 && x < p.C / 2, p.status)) gmovers[x] = s0 + bit;
-            }
-        }
-        uint32_t phase = marks ? 3u + 2u * __popc(marks) : 0u;
-        late = !dc_meet(xbar + kDcMeet * 8, cs, phase);
-        if (__syncthreads_or(late)) {
-            late = true;
-            leave(false);
-            return;
-        }
-        if (tid == 0) misc->n_moved = __ldcg(&p.unit_rec[u].x);
-        __syncthreads();
-        n_moved = misc->n_moved;
-        block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, gmovers, gholes, n_moved, rank, cs, l, p.status);
     }
     // every block's row moves come before released pages and the stamp
     if (pt_u || p.unit_stamp) {

@@ -347,8 +347,8 @@ __device__ __forceinline__ int kept_before(const uint32_t* mask, const int* pref
 // bandwidth-limited). Rows are D*sizeof(T) bytes = a multiple of 16.
 // row_of(slot) gives the slot's row in the layer's K / V storage (Kl, Vl).
 // part / n_parts: this block takes the chunks of NT / 8 rows numbered part, part + n_parts, ... (several blocks
-// sharing one unit's moves); the default is every chunk.
-template <typename T, int D, int NT, int KROWS = 4, typename RowOf>
+// sharing one unit's moves); the default is every chunk. kRegisters: registers and positions too.
+template <typename T, int D, int NT, int KROWS = 4, bool kRegisters = true, typename RowOf>
 __device__ __forceinline__ void block_move_rows(T* Kl, T* Vl, RowOf row_of, uint32_t* wordu, int32_t* posu,
                                                 const int* movers, const int* holes, int n_moved, int part = 0,
                                                 int n_parts = 1, int slot_limit = 0x7fffffff, int32_t* status = nullptr) {
@@ -379,7 +379,7 @@ __device__ __forceinline__ void block_move_rows(T* Kl, T* Vl, RowOf row_of, uint
                 if (c < kChunks) buf[r][x] = __ldcg(reinterpret_cast<const uint4*>(Kl + srow[r] * D) + c);
                 else if (c < 2 * kChunks) buf[r][x] = __ldcg(reinterpret_cast<const uint4*>(Vl + srow[r] * D) + (c - kChunks));
             }
-            if (lane == r) { wd = __ldcg(wordu + src[r]); ps = __ldcg(posu + src[r]); }
+            if (kRegisters && lane == r) { wd = __ldcg(wordu + src[r]); ps = __ldcg(posu + src[r]); }
         }
 #pragma unroll
         for (int r = 0; r < kRows; ++r) {
@@ -390,7 +390,7 @@ __device__ __forceinline__ void block_move_rows(T* Kl, T* Vl, RowOf row_of, uint
                 if (c < kChunks) reinterpret_cast<uint4*>(Kl + drow[r] * D)[c] = buf[r][x];
                 else if (c < 2 * kChunks) reinterpret_cast<uint4*>(Vl + drow[r] * D)[c - kChunks] = buf[r][x];
             }
-            if (lane == r) { wordu[dst[r]] = wd; posu[dst[r]] = ps; }
+            if (kRegisters && lane == r) { wordu[dst[r]] = wd; posu[dst[r]] = ps; }
         }
     }
 }

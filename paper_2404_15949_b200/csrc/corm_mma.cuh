@@ -229,6 +229,10 @@ __device__ __forceinline__ void push_u32(uint32_t addr, uint32_t v, uint32_t bar
 __device__ __forceinline__ void push_2u32(uint32_t addr, uint32_t x, uint32_t y, uint32_t bar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(x), "r"(y), "r"(bar) : "memory");
 }
+__device__ __forceinline__ void push_v4(uint32_t addr, uint4 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
+}
 __device__ __forceinline__ void push_2f64(uint32_t addr, double x, double y, uint32_t bar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];"
                  ::"r"(addr), "l"(__double_as_longlong(x)), "l"(__double_as_longlong(y)), "r"(bar) : "memory");

@@ -518,3 +518,30 @@ def test_hidden_logits_of_any_size(d, G, w, target):
     gpu.corm_compress_prompt(0, to_dev(kp, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(ql, "bf16"), data.prompt_lens)
     assert_states_equal(gpu, orc, 0, 3, 2, "")
     assert gpu.corm_cache_stats()["device_status"] == 0
+
+
+@pytest.mark.parametrize("dtype,d,G", [("bf16", 128, 1), ("bf16", 128, 4), ("bf16", 64, 8), ("f32", 64, 1), ("f32", 128, 2)])
+def test_rows_that_move_in_the_step_that_wrote_them(dtype, d, G):
+    """Every step evicts, so the row it appends, and the registers it has just updated in the unit's last words, move into
+    holes that other blocks of the unit fill (blocks of two words each): newest bits, rows and positions travel."""
+    nkv, B, steps = 8, 8, 72
+    cfg = _cfg(dtype, d, G, nkv, B, (600, 700), steps, 4, 2)
+    data = generate(cfg)
+    orc = make_oracle(cfg, B, nkv)
+    orc.set_near_band(1e-11)
+    one, many = (make_gpu_cache(cfg, B, nkv) for _ in range(2))
+    for g in (one, many):
+        g.corm_cache_set_tuning(64, 4)
+        g.corm_compress_prompt(0, to_dev(data.k_prompt, dtype), to_dev(data.v_prompt, dtype), to_dev(data.q_last, dtype),
+                               data.prompt_lens)
+    orc.compress_prompt(0, data.k_prompt, data.v_prompt, data.q_last, data.prompt_lens)
+    q, k, v = (to_dev(x, dtype) for x in (data.q, data.k_new, data.v_new))
+    for s0 in range(0, steps, 12):
+        many.corm_decode_steps(0, 1, *(x[s0:s0 + 12, None] for x in (q, k, v)))
+        for s in range(s0, s0 + 12):
+            one.corm_decode_step(0, q[s], k[s], v[s])
+            orc.decode_step(0, data.q[s], data.k_new[s], data.v_new[s])
+        assert_states_equal(one, orc, 0, B, nkv, f"per step, {s0 + 12}")
+        assert_states_equal(many, orc, 0, B, nkv, f"chained, {s0 + 12}")
+    st = one.corm_cache_stats()
+    assert st["device_status"] == 0 and st["moved_rows"] > steps * B * nkv // 4, st
