@@ -1147,7 +1147,7 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
     }
     late |= !mbar_wait_cluster(xbar + kDcCounts * 8, 0);
     int new_len = l, imp_total = 0, n_moved = 0;              // n_moved: row moves of the unit
-    // Counts, exact heads, moves. Returns false if a wait expired.
+    // Counts, exact heads, moves; the first block waits for the others'. Returns false if a wait expired.
     auto compact = [&]() -> bool {
         if (__syncthreads_or(late)) return false;             // (and the block's keep bits are there)
         int total = 0, before = 0, mine = 0;                  // kept slots of the unit, of the blocks before this one, of this one
@@ -1292,21 +1292,23 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
             n_moved = misc->n_moved;
             block_move_rows<T, D, NT>(reinterpret_cast<T*>(p.K), reinterpret_cast<T*>(p.V), row_of, wordu, posu, gmovers, gholes, n_moved, rank, cs, l, p.status);
         }
+        // every block's row moves come before released pages and the stamp
+        if (pt_u || p.unit_stamp) {
+            __syncthreads();
+            if (tid == 0) mbar_arrive_peer(map_rank(xbar + kDcDone * 8, 0));
+            if (rank == 0) {
+                late = !mbar_wait_cluster(xbar + kDcDone * 8, 0);
+                if (__syncthreads_or(late)) return false;
+            }
+        }
         return true;
     };
-    if (!compact()) {
+    if (!compact()) {                                         // (no stamp: the unit's next step must not start on rows that may still move)
         late = true;
         leave(false);
         return;
     }
-    // every block's row moves come before released pages and the stamp
-    if (pt_u || p.unit_stamp) {
-        __syncthreads();
-        if (tid == 0) mbar_arrive_peer(map_rank(xbar + kDcDone * 8, 0));
-        if (rank == 0) late = !mbar_wait_cluster(xbar + kDcDone * 8, 0);
-    }
     if (rank != 0) return;
-    if (late) report_status(p.status, CORM_ERR_TIMEOUT);
     if (pt_u) settle_pages<NT>(p.page_table, p.page_bits, p.page_room, p.pool_pages, p.pt_stride, p.U, u, l_old, new_len);
     if (pt_u && p.unit_stamp) __syncthreads();
     if (warp == 0) imp_total = __reduce_add_sync(0xffffffffu, imp_total);
@@ -1320,7 +1322,6 @@ decode_cluster_kernel(const __grid_constant__ DecodeClusterParams dp, const __gr
         if (new_len < l) atomicAdd(p.counters + CNT_EVICTED, (unsigned long long)(l - new_len));
         if (n_moved) atomicAdd(p.counters + CNT_MOVED, (unsigned long long)n_moved);
     }
-    if (late) cluster_sync();
 }
 
 // One layer's (or, from it on, all layers') K or V storage as a 2-D tensor [rows][D] with boxes of 16 rows x 128 bytes and
