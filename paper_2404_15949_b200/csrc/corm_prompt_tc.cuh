@@ -30,6 +30,11 @@ constexpr int kTcMaxRows = 1024;                 // rows of a unit whose sums an
 constexpr int kTcNearFlush = 2048, kTcNearCap = kTcNearFlush + kTcRows * kTcKeys;      // listed logits: a tile's always fit
 constexpr int kTcThreads = kPcThreads + 32;      // a ninth warp issues phase A's products
 constexpr int kTcStagesB = 4;
+// A block takes all of an SM's tensor memory and keeps it while it meets its cluster. A second one on the SM would wait for
+// columns that the first gives back only after meeting peers that may wait in the same way, without end: so a block asks for
+// more than half of the SM's shared memory (228 KB, of which the system takes 1 KB per block), whatever its operands need.
+constexpr int kTcMinSmem = 114 * 1024;
+static_assert(2 * (kTcMinSmem + 1024) > 228 * 1024, "two blocks must not fit an SM");
 
 template <int D> struct TcShape {
     static constexpr int kSteps = D / 16, kBlocks = D / 64;               // 16-channel steps, 128-byte wide blocks of an operand
@@ -84,7 +89,7 @@ __device__ __forceinline__ void tc_arrive(uint32_t bar) { asm volatile("mbarrier
 __device__ __forceinline__ void tc_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// all 512 columns, by one warp (a block of this kernel has an SM to itself)
+// all 512 columns, by one warp (a block of this kernel has an SM to itself: kTcMinSmem)
 __device__ __forceinline__ void tc_alloc(uint32_t dst) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(dst) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -545,7 +550,7 @@ __host__ __device__ inline PcSmem tc_smem_layout(int rows8) {
     s.list = take(kPcWarps * 32);
     s.misc = take((int)sizeof(PcMisc));
     s.tc = take((int)sizeof(TcMisc));
-    s.total = off;
+    s.total = off > kTcMinSmem ? off : kTcMinSmem;
     return s;
 }
 

@@ -465,6 +465,7 @@ MANY_ROWS = [
     (64, 1, 2, 3, (40, 600), 97),
     (64, 4, 1, 3, (255, 449), 32),
     (64, 8, 1, 2, (1023, 1025), 128),
+    (64, 1, 8, 12, (256, 320), 192),                    # more blocks of 64 channels (clusters of four and eight) than SMs
 ]
 
 
