@@ -562,12 +562,15 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     if (!layer_ok(c, layer) || !prompt_lens_host || p_max < 0) return CORM_ERR_INVALID_ARG;
     const corm_config_t& cf = c->cfg;
     int max_p = 0;
+    long long sum_p = 0;
     for (int b = 0; b < cf.batch; ++b) {
         const int P = prompt_lens_host[b];
         if (P < 0 || P > p_max) return CORM_ERR_INVALID_ARG;
         if (P > cf.max_tokens) return CORM_ERR_CAPACITY;
         max_p = std::max(max_p, P);
+        sum_p += P;
     }
+    const int mean_p = (int)(sum_p / cf.batch);
     if (max_p > 0 && (!k_prompt || !v_prompt || !q_last)) return CORM_ERR_INVALID_ARG;
     if (max_p > 0 && ((reinterpret_cast<uintptr_t>(k_prompt) | reinterpret_cast<uintptr_t>(v_prompt) |
                        reinterpret_cast<uintptr_t>(q_last)) % 16)) return CORM_ERR_INVALID_ARG;
@@ -616,8 +619,8 @@ corm_status_t corm_compress_prompt(corm_cache_t* c, int32_t layer, const void* k
     p.kmax = reinterpret_cast<uint32_t*>(layer_ptr(c, c->lay.kmax, U * 4, layer));
     const bool bf = cf.kv_dtype == CORM_BF16;
     const corm_status_t rc =
-        cf.head_dim == 128 ? (bf ? launch_prompt_cluster<bf16_t, 128>(p, c->G, max_p, c->sm_count, st) : launch_prompt_cluster<float, 128>(p, c->G, max_p, c->sm_count, st))
-                           : (bf ? launch_prompt_cluster<bf16_t, 64>(p, c->G, max_p, c->sm_count, st) : launch_prompt_cluster<float, 64>(p, c->G, max_p, c->sm_count, st));
+        cf.head_dim == 128 ? (bf ? launch_prompt_cluster<bf16_t, 128>(p, c->G, mean_p, max_p, c->sm_count, st) : launch_prompt_cluster<float, 128>(p, c->G, mean_p, max_p, c->sm_count, st))
+                           : (bf ? launch_prompt_cluster<bf16_t, 64>(p, c->G, mean_p, max_p, c->sm_count, st) : launch_prompt_cluster<float, 64>(p, c->G, mean_p, max_p, c->sm_count, st));
     if (rc != CORM_OK) return rc;
     c->launches += n_begin + 1;
     c->parity[layer] = 0; c->steps[layer] = 0; c->ready[layer] = 1; c->live_upper[layer] = max_p; c->live_mean[layer] = 0;

@@ -55,8 +55,10 @@ constexpr int kTcMinRows = 96;                  // rows of a unit from which pha
 constexpr double kPcLogitLimit = 650.0;         // exp of anything below stays finite in fp64, also summed over 2^19 keys
 // Bound of a logit's error, times the prompt's keys, beyond which a unit does both phases in fp64: so many verdicts would be
 // left open that most rows are formed apart. us per pass, tensor cores / fp64, one key channel 256 and 1024 times the others:
-// 32 units x 32768 keys, G 4, w 16, 6240 / 4210 and 13440 / 4210; 32 x 8192, G 4, w 128, 8190 / 8080 and 25440 / 8080; 1024 x
-// 3250, w 8, 1570 / 3100 and 3070 / 3180; 128 x 3390, w 256, 5420 / 6510 and 14230 / 6510.
+// mma.sync 32 units x 32768 keys, G 4, w 16, 6240 / 4210 and 13440 / 4210; 1024 x 3250, w 8, 1570 / 3100 and 3070 / 3180; tcgen05
+// 32 x 8192, G 4, w 128, 10500 / 7360 and 24650 / 7360; 128 x 3390, w 256, 3520 / 6650 and 10360 / 6650; 32 x 2000, w 256, 650 /
+// 950 and 1750 / 950; 16 x 8192, w 128, 1450 / 2010 and 3860 / 2010 (fp64 inside the mma.sync launch, which has twice the blocks
+// per SM or more L1: 8140, 6770, 1060 and 1810).
 constexpr double kPcReachKeys = 1.2;
 
 struct PromptClusterParams {
@@ -1056,7 +1058,9 @@ inline cudaError_t launch_prompt_begin(PromptBeginParams& bp, const int32_t* len
 }
 
 // Whether phases A and B of a bf16 pass run on tcgen05. A block has an SM to itself there, so it takes rows enough to fill the
-// 128 lanes, and either few units (whose clusters of eight fit the machine at once) or much work. us per pass, mma.sync ->
+// 128 lanes, and either few units (whose clusters of eight fit the machine at once) or much work. From 192 rows on it is the
+// faster one for any number of units and keys (32 to 1024 units of 256 to 1000 keys, both head sizes: 1.0 to 6.6 times; the least
+// with 192 rows and 1024 units of 512 keys, 1168 -> 1169 us, 256 keys 693 -> 635, with 256 rows 1570 -> 1184). us per pass, mma.sync ->
 // tcgen05, 128 channels: 32 units x 1000 keys, 96 / 128 / 256 rows, 68 -> 118 / 96 -> 119 / 144 -> 93; 32 x 1500, 128 rows, 127 -> 142;
 // 128 x 3000, 96 / 128 rows, 569 -> 566 / 703 -> 556; 1024 x 3000, 100 rows, 3760 -> 3070; 8 x 256, 96 rows, 46 -> 39; 8 x 4096, 128
 // rows, 160 -> 89; 32 x 300, 192 rows, 85 -> 65; 64 channels: 64 x 2000, 128 rows, 178 -> 192; 32 x 1000, 256 rows, 98 -> 69.
@@ -1066,11 +1070,33 @@ inline bool tc_takes(int n_units, int rows, int max_p, int sm_count) {
     return (double)n_units * max_p * rows >= (rows >= 128 ? 2e7 : 2e8);
 }
 
-// Host side. Returns CORM_ERR_UNSUPPORTED when the launch does not fit.
+// Blocks per unit on tcgen05 (one per SM; 33 clusters of four and 15 of eight are resident at once): those that let the pass
+// end first, a block costing 160 keys beside its own. Equal prompts take whole waves; of ragged ones the last wave is half full
+// in the mean. us per pass with 1 / 2 / 4 / 8 blocks, 128 channels unless said otherwise:
+//   256 rows, 3000 keys, 40 units 774 / 443 / 470 / 393, 64 units 784 / 453 / 489 / 599, 72 units 785 / 456 / 656 / 628; 2048..4096
+//   keys, 75 units 942 / 741 / 649 / 691, 96 units 958 / 800 / 705 / 898, 124 units 1014 / 895 / 905 / 1084, 128 units 994 / 908
+//   / 932 / 1174; 1500..3000 keys, 200 units 1192 / 978 / 1097 / 1437, 320 units 1581 / 1407 / 1653 / 2235; 128 units x 256 keys 115
+//   / 169 / 281, 80 x 500 172 / 174 / 179 / 277, 120 x 1000 329 / 340 / 388 / 519; 800..1600 keys, 496 units 1299 / 1255 / 1656
+//   100 rows, 512 x 3000 1767 / 1706 / 2212 / 2566; 512 rows, 80 x 4096 1981 / 1948 / 1554 / 1678; 64 channels, 80 x 3000 583 /
+//   570 / 475 / 515. Off by the most: 16 units x 8192 keys, 128 rows, 1134 / 603 / 344 / 330 (four).
+inline int tc_blocks_per_unit(int n_units, int mean_p, int max_p, int n_words, int sm_count) {
+    const double sms = sm_count > 0 ? sm_count : 148, resident[4] = {sms, sms / 2, sms * 33 / 148, sms * 15 / 148};
+    const double ragged = std::min(1.0, 4.0 * (max_p - mean_p) / std::max(1, max_p));
+    int best = 1;
+    double least = 0.0;
+    for (int i = 0, cs = 1; cs <= kPcMaxCluster && cs <= n_words; ++i, cs *= 2) {
+        const double waves = n_units / resident[i], longest = 160.0 + (double)max_p / cs, last = std::ceil(waves) - waves;
+        const double cost = waves <= 1.0 ? longest : waves * (160.0 + (double)mean_p / cs) + (last + ragged * (0.5 - last)) * longest;
+        if (cs == 1 || cost < least) { best = cs; least = cost; }
+    }
+    return best;
+}
+
+// Host side. Returns CORM_ERR_UNSUPPORTED when the launch does not fit. mean_p: tokens of a prompt in the mean.
 template <typename T, int D, bool kTc = false>
-inline corm_status_t launch_prompt_cluster(const PromptParams& p, int G, int max_p, int sm_count, cudaStream_t st) {
+inline corm_status_t launch_prompt_cluster(const PromptParams& p, int G, int mean_p, int max_p, int sm_count, cudaStream_t st) {
     if constexpr (!kTc && Elem<T>::kBytes == 2)
-        if (tc_takes(p.U, p.w * G, max_p, sm_count)) return launch_prompt_cluster<T, D, true>(p, G, max_p, sm_count, st);
+        if (tc_takes(p.U, p.w * G, max_p, sm_count)) return launch_prompt_cluster<T, D, true>(p, G, mean_p, max_p, sm_count, st);
     PromptClusterParams pp{};
     pp.p = p;
     while ((1 << pp.log2g) < G) ++pp.log2g;
@@ -1081,12 +1107,9 @@ inline corm_status_t launch_prompt_cluster(const PromptParams& p, int G, int max
     // first version of the kernel (the shapes take 840, 598 and 60 us now, with 2, 8 and 8):
     // 1024 units x 3250 keys 969-1353 (with the slab's stride) / 956-1033 / 1073 / 1365, 128 units x 8192 keys (G 4) 2152 / 1281 / 811 / 752, 32 units x
     // 4096 keys 350 / 192 / 120 / 93.
-    // On tcgen05, one block per SM: one wave where clusters of two or more fit it, else three waves and more (128 units of 2048..
-    // 4096 keys, w 256, with 1 / 2 / 4 / 8: 985 / 967 / 907 / 1197).
     int cs = 1;
-    const bool one_wave = kTc && p.U * 2 <= sm_count;
-    const long long blocks = one_wave ? sm_count / 2 + 1 : (kTc ? 500ll : 1500ll) * sm_count / 148;
-    while (cs < kPcMaxCluster && cs * 2 <= n_words && (long long)p.U * cs < blocks) cs *= 2;
+    if constexpr (kTc) cs = tc_blocks_per_unit(p.U, mean_p, max_p, n_words, sm_count);
+    else while (cs < kPcMaxCluster && cs * 2 <= n_words && (long long)p.U * cs < 1500ll * sm_count / 148) cs *= 2;
     PcSmem lay;
     if constexpr (kTc) lay = tc_smem_layout<D>(pp.rows8); else lay = pc_smem_layout<T, D>(pp.rows8);
     if (lay.total > 227 * 1024) return CORM_ERR_UNSUPPORTED;

@@ -98,7 +98,9 @@ __device__ __forceinline__ void tc_free(uint32_t tmem) { asm volatile("tcgen05.d
 
 // error of a logit of phase A (before the 1/sqrt(d)) per unit of the unit's largest key magnitude; n1, n2, n3: 1-norms of the
 // row and of its second and third pieces (see the head of the file). k2.q3 and r2.q3 are left out; adding the small parts
-// together and scaling rounds twice.
+// together and scaling rounds twice. The small products share an accumulator over all channels, so the bound is up to 1.9 times
+// split_error's, but phase B's own, with 17 roundings per 16 terms, is narrower: logits formed again, here / mma.sync, 32 units x
+// 8192 keys, G 4, w 128, 47982 / 47999 of 1.3e8, 128 x 3390, w 256, 37480 / 37934, one key channel 64 times the others 986301 / 1115750.
 __device__ __forceinline__ float tc_split_error(float n1, float n2, float n3) {
     return 2.0267e-6f * (8.f * n1 * (1.f / 8192.f) + 16.f * n2 * (1.f / 8192.f) + 24.f * n3) * 1.05f +
            1.3e-7f * (n2 * (1.f / 64.f) + n1 * (1.f / 8192.f) + n3) + n3 * (1.f / 60.f);

@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from paper_2404_15949_b200.workload import CONFIGS, generate
-from parity_util import OUT_TOL, assert_states_equal, make_gpu_cache, make_oracle, to_dev
+from parity_util import OUT_TOL, assert_states_equal, make_gpu_cache, make_oracle, sorted_state, stamps_to_ages, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -362,6 +362,16 @@ WIDE_PROMPTS = [
     ("bf16", 64, 1, (600, 700), 256, "one channel"),
     ("bf16", 64, 2, (2040, 2060), 16, "out of range"),
     ("bf16", 128, 1, (1, 40), 5, "out of range"),
+    # (from 96 rows on: on tcgen05; logits of 640 and 662 lie on either side of the largest that plain sums may hold)
+    ("bf16", 128, 4, (1000, 1100), 40, "large logits"),
+    ("bf16", 64, 1, (600, 700), 128, "large logits"),
+    ("bf16", 128, 8, (300, 420), 16, "out of range"),
+    ("bf16", 64, 4, (500, 560), 128, "out of range"),
+    ("bf16", 128, 2, (700, 700), 100, "640"),
+    ("bf16", 128, 1, (256, 330), 128, "662"),
+    ("bf16", 64, 1, (900, 1000), 96, "640"),
+    ("bf16", 64, 8, (400, 450), 32, "662"),
+    ("bf16", 128, 4, (500, 600), 128, "one channel"),
     ("f32", 128, 2, (900, 1000), 40, "large logits"),
     ("f32", 64, 8, (255, 300), 64, "large logits"),
 ]
@@ -374,6 +384,10 @@ def _widen(data, what, dtype):
         kp *= 128.0
     elif what == "out of range":
         kp *= 2.0 ** 58
+    elif what in ("640", "662"):                       # the logit of every query with the sixth key, but for 3 of other channels
+        kp[..., 0], ql[..., 0] = 0.0, 8.0
+        kp[..., 5, 0] = float(what) * np.sqrt(kp.shape[-1]) / 8.0
+        kp = rnd(kp)
     else:
         kp[..., 3] *= 4096.0
         ql[..., 3] /= 4096.0
@@ -398,8 +412,8 @@ def test_prompts_of_wide_range(case):
 
 @pytest.mark.parametrize("what", ["large logits", "one channel"])
 def test_prompts_of_wide_range_take_fp64_time_not_a_pass_per_row(what):
-    """256 rows of 32 units: both phases in fp64 take about four times the ordinary pass; forming each row apart, with two
-    passes over its keys, took more than ten times."""
+    """256 rows of 32 units: both phases in fp64 take about five times the ordinary pass on tcgen05 (184 and 954 us); forming
+    each row apart, with two passes over its keys, took more than ten times."""
     cfg = _cfg("bf16", 128, 1, 8, 4, (2000, 2000), 1, 256, 64)
     data = generate(cfg)
     plain, _ = _prompt_time(cfg, data, "bf16")
@@ -465,7 +479,7 @@ MANY_ROWS = [
     (64, 1, 2, 3, (40, 600), 97),
     (64, 4, 1, 3, (255, 449), 32),
     (64, 8, 1, 2, (1023, 1025), 128),
-    (64, 1, 8, 12, (256, 320), 192),                    # more blocks of 64 channels (clusters of four and eight) than SMs
+    (64, 1, 8, 12, (256, 320), 192),                    # more blocks of 64 channels than SMs
 ]
 
 
@@ -546,3 +560,34 @@ def test_rows_that_move_in_the_step_that_wrote_them(dtype, d, G):
         assert_states_equal(many, orc, 0, B, nkv, f"chained, {s0 + 12}")
     st = one.corm_cache_stats()
     assert st["device_status"] == 0 and st["moved_rows"] > steps * B * nkv // 4, st
+
+
+# many units, or long ones: clusters of one, two and four blocks of 1024 to 2048 keys (16 to 32 tiles), several waves of them
+LONG_BLOCKS = [
+    # head_dim, group, kv heads, batch, prompt range, w, sampled sequences, sampled kv heads
+    (128, 1, 29, 10, (1024, 1024), 192, [0, 9], [3, 28]),
+    (128, 1, 32, 4, (2048, 4096), 256, [1, 3], [0, 17]),
+    (128, 4, 8, 4, (8192, 8192), 128, [2], [5]),
+    (64, 2, 16, 12, (1500, 3000), 128, [4, 11], [7]),
+]
+
+
+@pytest.mark.parametrize("case", LONG_BLOCKS, ids=lambda c: "-".join(str(x) for x in c))
+def test_prompts_of_many_rows_in_long_blocks(case):
+    """Sampled units against the oracle, as they come from a pass over all of them."""
+    d, G, nkv, B, prange, w, seqs, heads = case
+    cfg = _cfg("bf16", d, G, nkv, B, prange, 2, w, 64)
+    data, sub = generate(cfg), generate(cfg, seqs=seqs, kv_heads=heads)
+    orc = make_oracle(cfg, len(seqs), len(heads))
+    orc.set_near_band(1e-11)
+    orc.compress_prompt(0, sub.k_prompt, sub.v_prompt, sub.q_last, sub.prompt_lens)
+    gpu = make_gpu_cache(cfg, B, nkv)
+    gpu.corm_compress_prompt(0, to_dev(data.k_prompt, "bf16"), to_dev(data.v_prompt, "bf16"), to_dev(data.q_last, "bf16"),
+                             data.prompt_lens)
+    for i, b in enumerate(seqs):
+        for j, h in enumerate(heads):
+            g, o = sorted_state(gpu.corm_cache_export_state(0, b, h)), orc.export_unit(0, i, j)
+            assert g["live_len"] == o["live_len"] and np.array_equal(g["pos"], o["pos"]), (b, h)
+            assert np.array_equal(stamps_to_ages(g["word"], g["n_tokens"], w), o["age"]), (b, h)
+            assert np.array_equal(g["k"].astype(np.float64), o["k"]) and np.array_equal(g["v"].astype(np.float64), o["v"]), (b, h)
+    assert gpu.corm_cache_stats()["device_status"] == 0
