@@ -20,7 +20,9 @@
 // again in fp64 by the callers, so results never depend on it.
 #pragma once
 
-#include "corm_fast.cuh"
+#include <cuda.h>
+
+#include "corm_ptx.cuh"
 
 namespace corm {
 

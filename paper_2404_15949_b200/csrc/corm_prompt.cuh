@@ -37,22 +37,12 @@
 #pragma once
 
 #include "corm_fast.cuh"
-#include "corm_mma.cuh"
+#include "corm_prompt_rows.cuh"
+#include "corm_prompt_tc.cuh"
 
 namespace corm {
 
-constexpr int kPcThreads = 256;
-constexpr int kPcWarps = kPcThreads / 32;
-constexpr int kPcKeys = 128;                    // keys per ring buffer
-// ring buffers: three, two where rows are long or the row pieces of a group take the room
-template <typename T, int D> __host__ __device__ constexpr int pc_bufs(int rows8) {
-    return D * Elem<T>::kBytes > 256 || (Elem<T>::kBytes == 2 && D == 128 && rows8 > 16) ? 2 : 3;
-}
-constexpr int kPcGroup = 4;                     // octets of rows (bf16) whose pieces lie on chip at a time in phase A
-constexpr int kPcGroupB = 8;                    // ... whose raw values do in phase B
-constexpr int kPcMaxCluster = 8;
 constexpr int kTcMinRows = 96;                  // rows of a unit from which phases A and B may run on tcgen05
-constexpr double kPcLogitLimit = 650.0;         // exp of anything below stays finite in fp64, also summed over 2^19 keys
 // Bound of a logit's error, times the prompt's keys, beyond which a unit does both phases in fp64: so many verdicts would be
 // left open that most rows are formed apart. us per pass, tensor cores / fp64, one key channel 256 and 1024 times the others:
 // mma.sync 32 units x 32768 keys, G 4, w 16, 6240 / 4210 and 13440 / 4210; 1024 x 3250, w 8, 1570 / 3100 and 3070 / 3180; tcgen05
@@ -67,18 +57,6 @@ struct PromptClusterParams {
     int32_t rows8;           // w G rounded up to a multiple of 8
 };
 
-struct PcSmem { int ring, zs, thr, n1, qe, flags, words, list, stage, frag, misc, tc, total; };
-constexpr int kPcOpenCap = 64;
-struct PcMisc {
-    double red[kPcWarps][2];
-    double mz[2];
-    double zw[kPcWarps][kPcGroup * 8];          // phase A: the warps' sums of a group's rows
-    int count, bad, warp_sum[kPcWarps], fail;
-    int n_open;                                 // verdicts that phase B left open: (row, key)
-    int2 open[kPcOpenCap];
-    uint32_t amax;                              // largest magnitude (bf16 bits) of the block's keys
-    float thr_f[kPcGroupB * 8], err_f[kPcGroupB * 8], slack[kPcGroupB * 8];      // phase B: a group's rows
-};
 template <typename T, int D>
 __host__ __device__ inline PcSmem pc_smem_layout(int rows8) {
     PcSmem s{};
@@ -105,13 +83,6 @@ __host__ __device__ inline PcSmem pc_smem_layout(int rows8) {
 // byte offset of 16-byte chunk c of row r inside a ring buffer (rows of D elements, chunk index XOR row mod 8)
 template <typename T, int D> __device__ __forceinline__ int pc_offset(int r, int c) { return r * (D * Elem<T>::kBytes) + ((c ^ (r & 7)) << 4); }
 
-__device__ __forceinline__ void cp_async16_zfill(uint32_t dst_smem, const void* src_gmem, bool on) {
-    const int n = on ? 16 : 0;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst_smem), "l"(src_gmem), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // One logit before the 1/sqrt(d), in fp64, by a whole warp.
 template <typename T, int D>
 __device__ __forceinline__ double warp_exact_dot(const T* q, const T* k, int lane) {
@@ -124,24 +95,6 @@ __device__ __forceinline__ double warp_exact_dot(const T* q, const T* k, int lan
     for (int i = 0; i < NPL; ++i) part = fma((double)a[i], (double)b[i], part);
     return warp_sum(part);
 }
-
-// What the rows of a unit look like: row r = (rho << log2g) + g is the query of window slot rho, head g, at position
-// P - (w - 1 - rho); it exists iff rho >= w - min(P, w).
-struct PcRows {
-    int rows, log2g, w, P;
-    __device__ __forceinline__ int rho(int r) const { return r >> log2g; }
-    __device__ __forceinline__ int pos(int r) const {       // 0: no such query
-        const int x = rho(r), i = P - (w - 1 - x);
-        return r < rows && i >= 1 ? i : 0;
-    }
-    template <typename T, int D> __device__ __forceinline__ const T* q(const T* q_unit, int r) const {
-        return q_unit + ((size_t)(r & ((1 << log2g) - 1)) * w + rho(r)) * D;
-    }
-};
-
-// A verdict's entry in a key's register: the shift register's bit, or the query's position for wide windows.
-__device__ __forceinline__ uint32_t pc_mark(int w, int rho, int qpos) { return w <= 32 ? 1u << (w - 1 - rho) : (uint32_t)qpos; }
-__device__ __forceinline__ uint32_t pc_join(int w, uint32_t a, uint32_t b) { return w <= 32 ? (a | b) : max(a, b); }
 
 // The marked rows, exactly, by all blocks of the cluster: log-sum-exp in fp64 with a running maximum, then the verdicts that
 // phase B left open (misc->open, or every key where those did not fit). Verdicts that phase B was sure of hold
@@ -193,12 +146,6 @@ __device__ __noinline__ void pc_exact_rows(const PromptParams& p, const PcRows& 
         }
         cluster_sync();                                       // everybody has read mz; the marks of this row are written
     }
-}
-
-__device__ __forceinline__ void pc_leave_open(uint32_t* flags, PcMisc* misc, int row, int j) {
-    atomicOr(flags + (row >> 5), 1u << (row & 31));
-    const int at = atomicAdd(&misc->n_open, 1);
-    if (at < kPcOpenCap) misc->open[at] = make_int2(row, j);
 }
 
 // Units whose logits are too large for plain sums of exponentials (650 and more), whose elements the pieces cannot hold, or
@@ -516,12 +463,6 @@ __device__ __noinline__ void pc_open_verdicts(const PromptParams& p, const PcRow
     }
     if (lane == 0) atomicAdd(p.counters + CNT_NEAR, (unsigned long long)n_near);
 }
-
-}  // namespace corm
-
-#include "corm_prompt_tc.cuh"
-
-namespace corm {
 
 // kTc: phases A and B on tcgen05 (corm_prompt_tc.cuh)
 template <typename T, int D, bool kTc>

@@ -20,8 +20,11 @@
 // before; and few integer ones, which issue as slowly (masks only on the last keys, ballots through shared memory: phase B 173
 // -> 121). us per pass, mma.sync -> here: 128 units x 2048..4096 keys, G 1, w 256, 1580 -> 905; 32 units x 8192 keys, G 4, w
 // 128, 1657 -> 1045; 8 units x 4096, w 128, 160 -> 89. Tried: the products issued by one of the eight warps in turn (the same).
-// (included by corm_prompt.cuh behind the definitions it shares)
 #pragma once
+
+#include <type_traits>
+
+#include "corm_prompt_rows.cuh"
 
 namespace corm {
 
