@@ -3,9 +3,11 @@
 // The cluster's blocks share the unit's live slots (whole 32-slot words each) and do the whole of Algorithm 1:
 //   1. every warp streams 16-key tiles of K and V through its own ring of shared-memory stages (2-D tensor-map copies
 //      with the 128-byte swizzle, mbarriers, bounded waits): logits, probabilities, P.V; no block-wide step in the loop;
-//   -- the blocks exchange {m, Z, acc} per head through distributed shared memory: log-sum-exp, thresholds, outputs
+//   -- the warps push {m, Z} per head to all blocks: log-sum-exp, thresholds; the blocks push their output numerators to the
+//      block that writes them
 //   2. verdicts of the block's slots, register update, keep bits;
-//   -- the blocks exchange their counts of kept slots: new length, places of holes and movers
+//   -- the warps push their counts of kept slots, and keep bits and registers of the unit's last words: new length, places of
+//      holes and movers
 //   3. hole filling, shared over the cluster; the first block publishes the unit's new length.
 //
 // bf16 logits on the tensor cores (corm_mma.cuh): keys cut into pieces k1, k2, r2, queries into q1, q2, q3. An
@@ -21,13 +23,14 @@
 // unit with a key or query element the pieces cannot hold (2^56 and more, infinity, NaN) takes that loop too: its products
 // have no bounds on the tensor cores. So does one whose bounds are too wide to be of use (kDcReach).
 //
-// What bounds it: on units of a few hundred keys the chain of round trips (set-up 2 us, first tiles 2, exchange and
-// thresholds 2.5, verdicts 1, exchange 1, moves 2, launch 2); on long units instruction issue in the streaming loop: about
+// What bounds it: on units of a few hundred keys the chain of round trips (8 units x 170 keys, fp32, at 9.4 us a step:
+// launch and length 2.0, first tiles 1.8, pushes and thresholds 1.5, verdicts 0.8, counts and lists 1.6, moves 1.5), in part
+// instructions that are not in the cache yet (ncu: 1.8 warps of 8.9 wait for them per issue); on long units instruction issue in the streaming loop: about
 // 650 instructions per tile (192 of them the two-element additions that cut the keys), of 5000 cycles per tile and warp
 // with 16 warps on an SM only 270 are spent waiting for its copies. So one stage each for K and V is enough (with two for
 // K: 32 units x 8200 keys 43 us a step instead of 38), and what is smaller leaves more L1. Units differ in length and SMs
 // hold one block or two, which is what keeps the rest of HBM's rate away.
-// Measured, us per step from one call per step, before -> first version -> now:
+// Measured, us per step from one call per step, before -> first version -> before the pushes (now: below):
 //   64 units x 970 keys, G 8, bf16          253 -> 32 -> 27     128 units x 1090 keys, G 4, 64 channels   143 -> 30 -> 26
 //   20 units x 250 keys, G 2, fp32           64 -> 16 -> 13     8 units x 170 keys, G 1, fp32            37.7 -> 14 -> 11
 //   128 units x 2800 keys, G 4, bf16         86 -> 68 -> 54     32 units x 21400 keys, G 4, bf16          133 -> 103 -> 80
@@ -36,9 +39,11 @@
 // block an equal share of all tiles and a second launch for the verdicts, from the block-per-split kernel).
 //
 // What the blocks tell one another is pushed (st.async: value and byte count travel together, one way), each block waiting on
-// its own barriers, instead of cluster barriers and loads from the peers behind them (two round trips and a flush each):
-// 8 units x 170 keys, fp32, 11.0 -> 9.4 us a step, 32 units x 1160 keys, G 1, 19.6 -> 17.0, 128 units x 1090 keys, 64
-// channels, 27.2 -> 25.5, 128 units x 1800 keys, G 4, 54 -> 52 (of which 1-3 us are the lists of row moves).
+// its own barriers, instead of cluster barriers and loads from the peers behind them (two round trips and a flush each). A push
+// orders nothing but itself, so whatever one block needs of another's is in a push (or, where heads are formed again or lists go
+// to scratch, behind a meeting with release and acquire). us per request, cluster barriers -> pushes: one fp32 sequence, 64
+// steps, 767 -> 677; 32 layers 12260 -> 10690; G 8 1490 -> 1400; 64 channels 1536 -> 1400; fp32 G 2 815 -> 720; G 4, 128 units x
+// 1800 keys 5980 -> 5880, paged and chained 6130 -> 6140.
 //
 // Verdicts are the fp64 ones: a slot's logit is kept in fp32, and one that lies within the proven error of its threshold
 // is formed again in fp64. If it then lies within the error of the log-sum-exp itself, the head is marked and the

@@ -25,13 +25,14 @@
 // sums keep the largest logit apart, so that a query at position 1 stays exactly on its threshold.
 //
 // What bounds it: for windows of a few queries HBM and the latency of the gather (K once, the survivors' V in, K and V
-// out); for wide windows the tensor pipe's mma.sync rate in phase A (R P d multiply-adds, seven times).
+// out); for more rows, below those that tc_takes gives to tcgen05, the tensor pipe's mma.sync rate in phase A (R P d
+// multiply-adds, seven times).
 // Measured, us per pass: a two-launch pass (fp64 logits on the CUDA cores; one block per unit gathering; for fp32 or 64
 // channels one block per unit for everything) -> a first cluster pass (a warp per octet of rows, every warp cutting every
-// key; marked rows a key at a time) -> now (of which products without a zeroed addend, fragment addresses from one lane
+// key; marked rows a key at a time) -> now on mma.sync (of which products without a zeroed addend, fragment addresses from one lane
 // constant and exponentials without a range check, which the limit on the logits makes needless: 1755 -> 1699 at w 128):
-//   1024 units x 3250 keys, G 1, w 8    1597 -> 1036 ->  840    128 units x 3390 keys, G 1, w 256    5341 -> 1709 -> 1582
-//   128 units x 8192 keys, G 4, w 8     1821 ->  769 ->  598    32 units x 8192 keys, G 4, w 128     6736 -> 2206 -> 1699
+//   1024 units x 3250 keys, G 1, w 8    1597 -> 1036 ->  840    128 units x 3390 keys, G 1, w 256    5341 -> 1709 -> 1582 (tcgen05: 905)
+//   128 units x 8192 keys, G 4, w 8     1821 ->  769 ->  598    32 units x 8192 keys, G 4, w 128     6736 -> 2206 -> 1699 (tcgen05: 1045)
 //   32 units x 32768 keys, G 4, w 16    4618 -> 2375 -> 1049    32 units x 4096 keys, G 1, w 8        259 ->   65 ->   60
 //   fp32: 20 units x 1300 keys, G 2     2787 ->  103            64 channels: 128 units x 2000, G 4  11037 ->  273 ->  238
 #pragma once
@@ -1044,8 +1045,8 @@ inline corm_status_t launch_prompt_cluster(const PromptParams& p, int G, int mea
     pp.rows8 = (p.w * G + 7) / 8 * 8;
     const int n_words = std::max(1, (max_p + 31) / 32);
     // As many blocks per unit as make the launch at least five waves of resident blocks: fewer leave the machine
-    // to the longest units, more pay each block's fixed chain of round trips more often. us per pass with 1 / 2 / 4 / 8, on the
-    // first version of the kernel (the shapes take 840, 598 and 60 us now, with 2, 8 and 8):
+    // to the longest units, more pay each block's fixed chain of round trips more often (on tcgen05: tc_blocks_per_unit). us per
+    // pass with 1 / 2 / 4 / 8, on the first version of the kernel (the shapes take 840, 598 and 60 us now, with 2, 8 and 8):
     // 1024 units x 3250 keys 969-1353 (with the slab's stride) / 956-1033 / 1073 / 1365, 128 units x 8192 keys (G 4) 2152 / 1281 / 811 / 752, 32 units x
     // 4096 keys 350 / 192 / 120 / 93.
     int cs = 1;

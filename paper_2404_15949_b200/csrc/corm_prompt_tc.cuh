@@ -9,14 +9,14 @@
 // while the block's eight warps cut the next and take the exponentials of the one before. Phase B: one product of the raw
 // values, verdicts by ballot; the logits inside the rounding bound are listed and formed again in fp64, four lanes each.
 //
-// Accumulation on tcgen05, checked on the GPU as for mma.sync: whole numbers up to 2^23.8, chains of 56, random and of one
-// sign, none off by a bit. Accumulators: k1.q1; k1.q2 + k2.q1; k2.q2 (all exact); k1.q3, then r2.q2, then r2.q1. The last one is
+// Accumulation on tcgen05, checked on the GPU as for mma.sync (tests/test_gpu_tc_products.py for what the pieces reach): whole
+// numbers up to 2^23.8, chains of 56, random and of one sign, none off by a bit. Accumulators: k1.q1; k1.q2 + k2.q1; k2.q2 (all exact); k1.q3, then r2.q2, then r2.q1. The last one is
 // rounded: with 17 roundings of 2^-23 a step on what has been added up so far, its eight steps of r2.q1 err by at most
 // 8 x 17 x 2^-23 A |q1|_1 / 8192, the smaller terms before them by 24 and 16 times 17 x 2^-23 of theirs (tc_split_error).
 //
 // What bounds it: fp64 and tensor instructions share a pipe, so phase A takes the products' time plus the exponentials'.
-// 512 rows x 1024 keys a block, us: phase A 302 (without the exponentials 163, without the products 173, without either 75),
-// phase B 121. Hence few fp64 operations per row and key: 13 with a table of 2^(i/16) and the 1/sqrt(d) inside the constants, 20
+// 512 rows x 1024 keys a block, us: phase A 302 (163 with the exponentials left out, 173 with the products left out, 75 with
+// both), phase B 121. Hence few fp64 operations per row and key: 13 with a table of 2^(i/16) and the 1/sqrt(d) inside the constants, 20
 // before; and few integer ones, which issue as slowly (masks only on the last keys, ballots through shared memory: phase B 173
 // -> 121). us per pass, mma.sync -> here: 128 units x 2048..4096 keys, G 1, w 256, 1580 -> 905; 32 units x 8192 keys, G 4, w
 // 128, 1657 -> 1045; 8 units x 4096, w 128, 160 -> 89. Tried: the products issued by one of the eight warps in turn (the same).

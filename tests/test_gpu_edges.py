@@ -40,8 +40,9 @@ def test_bf16_outputs_are_the_exact_ones_rounded(d, G):
     assert total >= 20000 and wrong <= 3e-4 * total, (wrong, total)
 
 
-# one block per unit as long as its list space allows (a split length beyond the unit), so a block owns as many 32-slot
-# words as it can keep track of: 3071 for fp32 / 64 channels, 4096 otherwise; and one word more than that
+# one block per unit as long as its list space allows (a split length beyond the unit), so a block owns about as many 32-slot
+# words as it can keep track of (3583 for fp32 / 64 channels, 4096 otherwise; EVICTED below has exactly as many and one more), or
+# two blocks where a unit may have more than that
 LONG_UNITS = [
     # dtype, head_dim, group, live keys, max_tokens, paged
     ("f32", 64, 1, 98250, 3071 * 32, False),
