@@ -48,8 +48,7 @@ constexpr int kTcMinRows = 96;                  // rows of a unit from which pha
 // left open that most rows are formed apart. us per pass, tensor cores / fp64, one key channel 256 and 1024 times the others:
 // mma.sync 32 units x 32768 keys, G 4, w 16, 6240 / 4210 and 13440 / 4210; 1024 x 3250, w 8, 1570 / 3100 and 3070 / 3180; tcgen05
 // 32 x 8192, G 4, w 128, 10500 / 7360 and 24650 / 7360; 128 x 3390, w 256, 3520 / 6650 and 10360 / 6650; 32 x 2000, w 256, 650 /
-// 950 and 1750 / 950; 16 x 8192, w 128, 1450 / 2010 and 3860 / 2010 (fp64 inside the mma.sync launch, which has twice the blocks
-// per SM or more L1: 8140, 6770, 1060 and 1810).
+// 950 and 1750 / 950; 16 x 8192, w 128, 1450 / 1820 and 3860 / 1820 (fp64 inside the mma.sync launch: 8140, 6770, 1060 and 1810).
 constexpr double kPcReachKeys = 1.2;
 
 struct PromptClusterParams {
@@ -153,10 +152,12 @@ __device__ __noinline__ void pc_exact_rows(const PromptParams& p, const PcRows& 
 // whose error bounds are too wide to be of use: both phases in fp64 on the CUDA cores, with running maxima. A warp owns units
 // of four rows (the queries widened in shared memory), a lane one or two keys; warps share rows by groups of 32 keys where
 // there are fewer than eight row units. On return the thresholds and the scratch registers are there; rows are marked, and
-// their keys listed, for ties only. key_buf: 128 rows of keys, q_stage: 4 rows of doubles per warp, words: 128 registers.
+// their keys listed, for ties only. key_buf: 128 rows of keys, q_stage: room for `room` units of doubles per warp (a warp with no
+// more than that widens its rows once; else for every chunk of keys, which a block on tcgen05, with little L1, pays for: 16 units x
+// 8192 keys, 128 rows, 2007 -> 1817 us), words: 128 registers.
 template <typename T, int D>
 __device__ __noinline__ void pc_fp64_rows(const PromptParams& p, const PcRows& R, const T* Qu, const T* Ku, int k_begin, int n_keys, unsigned char* key_buf,
-                                          double* q_stage, double* zs, double* thr_sm, uint32_t* words, uint32_t* words_g, uint32_t* flags, PcMisc* misc, int cs) {
+                                          double* q_stage, int room, double* zs, double* thr_sm, uint32_t* words, uint32_t* words_g, uint32_t* flags, PcMisc* misc, int cs) {
     constexpr int kRow = D * Elem<T>::kBytes, kChunks = kRow / 16, kEl = 16 / Elem<T>::kBytes, kSubs = kPcKeys / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nc = (n_keys + kPcKeys - 1) / kPcKeys;
     const int n_ru = (R.rows + 3) / 4;
@@ -164,7 +165,8 @@ __device__ __noinline__ void pc_fp64_rows(const PromptParams& p, const PcRows& R
     while (slots < n_ru && slots < kPcWarps) slots *= 2;
     const int groups = min(kPcWarps / slots, kSubs), my_ru = warp % slots, my_kg = warp / slots;
     const bool works = my_ru < n_ru && my_kg < groups;
-    double* const q = q_stage + warp * 4 * D;
+    double* q = q_stage + warp * room * 4 * D;
+    const bool kept = (n_ru + slots - 1) / slots <= room;
     double* const ms = groups > 1 ? zs + 32 : thr_sm;         // running maxima next to the sums (fewer than 32 rows x groups)
     auto load = [&](int c) {
         __syncthreads();                                      // everybody is done with the chunk before
@@ -177,7 +179,9 @@ __device__ __noinline__ void pc_fp64_rows(const PromptParams& p, const PcRows& R
         }
         __syncthreads();
     };
-    auto stage = [&](int ru) {
+    auto stage = [&](int ru, bool first) {                    // unit ru's rows in q
+        q = q_stage + (warp * room + (kept ? ru / slots : 0)) * 4 * D;
+        if (kept && !first) return;
         __syncwarp();
         for (int x = lane; x < 4 * D; x += 32) {
             const int r = ru * 4 + x / D;
@@ -228,7 +232,7 @@ __device__ __noinline__ void pc_fp64_rows(const PromptParams& p, const PcRows& R
         const int n_valid = min(kPcKeys, n_keys - c * kPcKeys);
         if (!works) continue;
         for (int ru = my_ru; ru < n_ru; ru += slots) {
-            if (c == 0 || n_ru > slots) stage(ru);            // a warp with one row unit keeps it staged
+            stage(ru, c == 0);
             double m[4], z[4];
 #pragma unroll
             for (int x = 0; x < 4; ++x) { m[x] = -INFINITY; z[x] = 0.0; }
@@ -289,7 +293,7 @@ __device__ __noinline__ void pc_fp64_rows(const PromptParams& p, const PcRows& R
         const int n_valid = min(kPcKeys, n_keys - c * kPcKeys);
         if (works)
             for (int ru = my_ru; ru < n_ru; ru += slots) {
-                if (n_ru > slots) stage(ru);
+                stage(ru, false);
                 for (int sub = my_kg; sub < kSubs && sub * 32 < n_valid; sub += 2 * groups) {
                     const bool two = sub + groups < kSubs && (sub + groups) * 32 < n_valid;
                     double s[2][4];
@@ -732,7 +736,7 @@ prompt_cluster_kernel(const __grid_constant__ PromptClusterParams pp) {
         cluster_sync();                                       // everybody has read everybody's sums of phase A
         constexpr int kBuf = kPcKeys * kRow;
         static_assert(kPcWarps * 4 * D * 8 <= kBuf, "the widened rows fit a ring buffer");
-        pc_fp64_rows<T, D>(p, R, Qu, Ku, k_begin, n_keys, smem + lay.ring, reinterpret_cast<double*>(smem + lay.ring + kBuf), zs, thr_sm,
+        pc_fp64_rows<T, D>(p, R, Qu, Ku, k_begin, n_keys, smem + lay.ring, reinterpret_cast<double*>(smem + lay.ring + kBuf), kTc ? kTcRowRoom : 1, zs, thr_sm,
                            kBf16 ? reinterpret_cast<uint32_t*>(f12) : words_sm, words_g, flags, misc, cs);
     } else if constexpr (kTc) {
         tc_phase_b<D>(p, block, thr_sm, n1_sm, qe_sm, eps_unit, words_g, flags, misc);

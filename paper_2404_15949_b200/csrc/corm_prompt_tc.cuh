@@ -33,6 +33,7 @@ constexpr int kTcMaxRows = 1024;                 // rows of a unit whose sums an
 constexpr int kTcNearFlush = 2048, kTcNearCap = kTcNearFlush + kTcRows * kTcKeys;      // listed logits: a tile's always fit
 constexpr int kTcThreads = kPcThreads + 32;      // a ninth warp issues phase A's products
 constexpr int kTcStagesB = 4;
+constexpr int kTcRowRoom = 4;                    // units of four rows that a warp of pc_fp64_rows keeps widened (little L1 is left)
 // A block takes all of an SM's tensor memory and keeps it while it meets its cluster. A second one on the SM would wait for
 // columns that the first gives back only after meeting peers that may wait in the same way, without end: so a block asks for
 // more than half of the SM's shared memory (228 KB, of which the system takes 1 KB per block), whatever its operands need.
@@ -546,7 +547,8 @@ __host__ __device__ inline PcSmem tc_smem_layout(int rows8) {
     int off = 0;
     auto take = [&](int bytes) { int at = off; off = (off + bytes + 127) / 128 * 128; return at; };
     s.ring = take(S::kOperands);
-    s.frag = 3 * kPcKeys * D * 2;                // (of pc_fp64_rows, behind its keys and rows)
+    s.frag = kPcKeys * D * 2 + kPcWarps * kTcRowRoom * 4 * D * 8;        // (of pc_fp64_rows: registers behind its keys and rows)
+    static_assert(kPcKeys * D * 2 + kPcWarps * kTcRowRoom * 4 * D * 8 + kPcKeys * 4 <= S::kOperands, "all three fit the operands");
     s.zs = take((rows8 > 64 ? rows8 : 64) * 8);
     s.thr = take(rows8 * 8);
     s.n1 = take(rows8 * 4);
