@@ -1003,17 +1003,21 @@ inline cudaError_t launch_prompt_begin(PromptBeginParams& bp, const int32_t* len
     return cudaSuccess;
 }
 
-// Whether phases A and B of a bf16 pass run on tcgen05. A block has an SM to itself there, so it takes rows enough to fill the
-// 128 lanes, and either few units (whose clusters of eight fit the machine at once) or much work. From 192 rows on it is the
-// faster one for any number of units and keys (32 to 1024 units of 256 to 1000 keys, both head sizes: 1.0 to 6.6 times; the least
-// with 192 rows and 1024 units of 512 keys, 1168 -> 1169 us, 256 keys 693 -> 635, with 256 rows 1570 -> 1184). us per pass, mma.sync ->
-// tcgen05, 128 channels: 32 units x 1000 keys, 96 / 128 / 256 rows, 68 -> 118 / 96 -> 119 / 144 -> 93; 32 x 1500, 128 rows, 127 -> 142;
-// 128 x 3000, 96 / 128 rows, 569 -> 566 / 703 -> 556; 1024 x 3000, 100 rows, 3760 -> 3070; 8 x 256, 96 rows, 46 -> 39; 8 x 4096, 128
-// rows, 160 -> 89; 32 x 300, 192 rows, 85 -> 65; 64 channels: 64 x 2000, 128 rows, 178 -> 192; 32 x 1000, 256 rows, 98 -> 69.
+// Whether phases A and B of a bf16 pass run on tcgen05. The time there follows the groups of 128 rows, on mma.sync the rows, so what
+// counts is how full the groups are; short prompts and few units (whose clusters of eight are resident at once) gain in any
+// case. Time on mma.sync over that on tcgen05, equal prompts of 1000 to 8000 keys, 24 to 512 units, 128 / 64 channels:
+//   rows   96 0.87-1.32 / 0.85-1.26   112 0.97-1.48 / 0.90-1.60   128 1.02-1.49 / 1.09-1.51   129 0.81-1.14 / 0.76-1.04
+//         144 0.80-1.10 / 0.75-1.05   160 0.88-1.20 / 0.82-1.15   192 0.99-1.37 / 0.90-1.32   224 1.11-1.66 / 1.06-1.52
+//         256 1.30-1.78 / 1.01-1.61
+// 256 to 500 keys: 0.96 and more, 96 units x 256 keys 1.7-3.4; 1 to 12 units of any length: 0.86-2.1, 1.3 in
+// the mean. 1024 units x 3000 keys, 100 rows,
+// 3760 -> 3070 us.
 inline bool tc_takes(int n_units, int rows, int max_p, int sm_count) {
     if (rows < kTcMinRows || rows > kTcMaxRows || max_p < 256) return false;
-    if (rows >= 192 || n_units * kPcMaxCluster <= sm_count) return true;
-    return (double)n_units * max_p * rows >= (rows >= 128 ? 2e7 : 2e8);
+    const int groups = (rows + kTcRows - 1) / kTcRows;
+    const double fill = (double)rows / (groups * kTcRows);
+    if (max_p <= 512 || n_units * 148 <= 15 * sm_count || fill >= 0.9) return true;
+    return groups > 1 ? fill >= 0.72 : (double)n_units * max_p * rows >= 2e8;
 }
 
 // Blocks per unit on tcgen05 (one per SM; 33 clusters of four and 15 of eight are resident at once): those that let the pass
