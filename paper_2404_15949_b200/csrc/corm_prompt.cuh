@@ -1009,9 +1009,8 @@ inline cudaError_t launch_prompt_begin(PromptBeginParams& bp, const int32_t* len
 //   rows   96 0.87-1.32 / 0.85-1.26   112 0.97-1.48 / 0.90-1.60   128 1.02-1.49 / 1.09-1.51   129 0.81-1.14 / 0.76-1.04
 //         144 0.80-1.10 / 0.75-1.05   160 0.88-1.20 / 0.82-1.15   192 0.99-1.37 / 0.90-1.32   224 1.11-1.66 / 1.06-1.52
 //         256 1.30-1.78 / 1.01-1.61
-// 256 to 500 keys: 0.96 and more, 96 units x 256 keys 1.7-3.4; 1 to 12 units of any length: 0.86-2.1, 1.3 in
-// the mean. 1024 units x 3000 keys, 100 rows,
-// 3760 -> 3070 us.
+// 256 to 500 keys: 0.96 and more, 96 units x 256 keys 1.7-3.4; 1 to 12 units of any length: 0.86-2.1, 1.3 in the mean. 1024 units
+// x 3000 keys, 100 rows, 3760 -> 3070 us.
 inline bool tc_takes(int n_units, int rows, int max_p, int sm_count) {
     if (rows < kTcMinRows || rows > kTcMaxRows || max_p < 256) return false;
     const int groups = (rows + kTcRows - 1) / kTcRows;
